@@ -21,6 +21,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 # return SP_ERR_OUT_OF_RANGE instead of reading or writing out of bounds).  Much slower; for debugging.
 DEBUG_BOUNDS = os.environ.get("SP_DEBUG_BOUNDS", "") not in ("", "0")
 _LIB_PATH = os.path.join(_HERE, "libsp_debug_bounds.so" if DEBUG_BOUNDS else "libsp.so")
+_TORCH_LIB_PATH = os.path.join(_HERE, "libsp_torch.so")
 
 SYMBOLS = ["sp_status_string", "sp_set_allocator", "sp_pack", "sp_free", "sp_info", "sp_positions",
            "sp_coordinates", "sp_values", "sp_unpack", "sp_spmv", "sp_spmm", "sp_sddmm", "sp_mttkrp",
@@ -35,38 +36,38 @@ class SpError(RuntimeError):
 
 
 def _load():
-    if not os.path.exists(_LIB_PATH):
-        raise ImportError(f"{_LIB_PATH} not found: build it with `python -m paper_2202_04305_b200.build"
-                          f"{' --debug-bounds' if DEBUG_BOUNDS else ''}` (there is no CPU fallback)")
+    for path in (_LIB_PATH, _TORCH_LIB_PATH):
+        if not os.path.exists(path):
+            raise ImportError(f"{path} not found: build it with `python -m paper_2202_04305_b200.build"
+                              f"{' --debug-bounds' if DEBUG_BOUNDS else ''}` (there is no CPU fallback)")
     lib = C.CDLL(_LIB_PATH)
     lib.sp_status_string.restype = C.c_char_p
     lib.sp_status_string.argtypes = [C.c_int]
     for name in SYMBOLS[1:]:
         getattr(lib, name).restype = C.c_int
     lib.sp_launch_count.restype = C.c_int64
-    return lib
+    # argument types stated once: plain integers are then converted in C, without an object per argument
+    p, n, i = C.c_void_p, C.c_int64, C.c_int
+    for name, args in {"sp_pack": [i, p, n, p, i, p, p, p, i, i, C.c_uint, p, p], "sp_free": [p], "sp_info": [p] * 7,
+                       "sp_positions": [p, i, p, p], "sp_coordinates": [p, i, p, p], "sp_values": [p, p, p],
+                       "sp_unpack": [p] * 5, "sp_spmv": [p] * 4, "sp_spmv_static": [p] * 4, "sp_spmm": [p, p, n, n, p, n, p],
+                       "sp_sddmm": [p, p, n, p, n, n, p, p], "sp_mttkrp": [p, p, p, n, p, p], "sp_mttkrp_mode": [p, i, p, n, p, p],
+                       "sp_spmspm": [p, p, i, i, p, p], "sp_convert": [p, p, p, i, i, p, p], "sp_scale": [p, C.c_double, p],
+                       "sp_vec_dot": [p] * 4}.items():
+        getattr(lib, name).argtypes = args
+    side = C.PyDLL(_TORCH_LIB_PATH)
+    side.sp_torch_alloc.restype, side.sp_torch_alloc.argtypes = p, [C.c_size_t, p, p]
+    side.sp_torch_free.restype, side.sp_torch_free.argtypes = None, [p, p, p]
+    side.sp_torch_view.restype, side.sp_torch_view.argtypes = C.py_object, [p, n, i, C.py_object]
+    return lib, side
 
 
-_lib = _load()
+_lib, _torch_lib = _load()
 
 _ALLOC_T = C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p, C.c_void_p)
 _FREE_T = C.CFUNCTYPE(None, C.c_void_p, C.c_void_p, C.c_void_p)
-
-
-def _torch_alloc(nbytes, stream, ctx):
-    try:
-        return torch.cuda.caching_allocator_alloc(max(int(nbytes), 1), stream=int(stream or 0))
-    except Exception:
-        return None
-
-
-def _torch_free(ptr, stream, ctx):
-    if ptr:
-        torch.cuda.caching_allocator_delete(ptr)
-
-
-_alloc_cb = _ALLOC_T(_torch_alloc)
-_free_cb = _FREE_T(_torch_free)
+_torch_alloc, _torch_free = _torch_lib.sp_torch_alloc, _torch_lib.sp_torch_free
+_alloc_cb, _free_cb = C.cast(_torch_alloc, C.c_void_p), C.cast(_torch_free, C.c_void_p)
 _allocator_set = False
 
 
@@ -83,55 +84,64 @@ def _check(code, where):
         raise SpError(code, where)
 
 
+_current_device = torch._C._cuda_getDevice
+_current_stream = torch._C._cuda_getCurrentRawStream
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _current_stream(_current_device())
 
 
 def _dptr(t):
-    return C.c_void_p(t.data_ptr() if t is not None and t.numel() else 0) if t is not None else C.c_void_p(0)
+    return t.data_ptr() if t is not None else 0        # 0 for an empty tensor too
 
 
 def _f64(t, name):
-    if t.dtype != torch.float64 or not t.is_cuda:
+    if t.dtype is not torch.float64 or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA float64 tensor")
     return t
 
 
-class _DevArray:
-    """Zero-copy view of library-owned device memory through __cuda_array_interface__."""
-
-    def __init__(self, ptr, n, typestr, owner):
-        self.__cuda_array_interface__ = {"shape": (n,), "typestr": typestr, "data": (ptr, False), "version": 2}
-        self._owner = owner
+def _view(ptr, n, code, owner):
+    """Zero-copy tensor over library-owned device memory that keeps its owner alive."""
+    v = _torch_lib.sp_torch_view(ptr, n, code, owner)
+    return v if v.get_device() == _current_device() else v.to("cuda")
 
 
-_WIDTH_VIEW = {8: (torch.uint8, "|u1"), 16: (torch.uint16, "<u2"), 32: (torch.int32, "<i4"), 64: (torch.int64, "<i8")}
+_WIDTH_DTYPE = {8: torch.uint8, 16: torch.uint16, 32: torch.int32, 64: torch.int64}
+
+
+def _encoding(rank, dimLevelType, dimOrdering):
+    """The level types and the level order as C arrays (no order = None) and as tuples."""
+    lt = (C.c_int * rank)(*map(int, dimLevelType))
+    if dimOrdering is None:
+        return lt, None, tuple(lt), tuple(range(rank))
+    od = (C.c_int * rank)(*map(int, dimOrdering))
+    return lt, od, tuple(lt), tuple(od)
 
 
 class SpTensor:
     """Owner of an sp_tensor handle."""
 
-    def __init__(self, handle):
+    def __init__(self, handle, known=None):
+        """known: (dims, lt, ord, posBits, crdBits) where the caller has just stated them; asked for otherwise."""
         self._h = handle
-        rank = C.c_int()
-        dims = (C.c_int64 * MAX_RANK)()
-        lt = (C.c_int * MAX_RANK)()
-        od = (C.c_int * MAX_RANK)()
-        pb, cb = C.c_int(), C.c_int()
-        _check(_lib.sp_info(self._h, C.byref(rank), dims, lt, od, C.byref(pb), C.byref(cb)), "sp_info")
-        self.rank = rank.value
-        self.dims = tuple(dims[i] for i in range(self.rank))
-        self.lt = tuple(lt[i] for i in range(self.rank))
-        self.ord = tuple(od[i] for i in range(self.rank))
-        self.pos_bits, self.crd_bits = pb.value, cb.value
+        if known is None:
+            rank = C.c_int()
+            dims, lt, od = (C.c_int64 * MAX_RANK)(), (C.c_int * MAX_RANK)(), (C.c_int * MAX_RANK)()
+            pb, cb = C.c_int(), C.c_int()
+            _check(_lib.sp_info(handle, C.byref(rank), dims, lt, od, C.byref(pb), C.byref(cb)), "sp_info")
+            r = rank.value
+            known = tuple(dims[:r]), tuple(lt[:r]), tuple(od[:r]), pb.value, cb.value
+        self.dims, self.lt, self.ord, self.pos_bits, self.crd_bits = known
+        self.rank = len(self.dims)
 
     def _arr(self, fn, level, bits):
         p, n = C.c_void_p(), C.c_int64()
-        _check(fn(self._h, C.c_int(level), C.byref(p), C.byref(n)), fn.__name__)
-        dt, typestr = _WIDTH_VIEW[bits]
+        _check(fn(self._h, level, C.byref(p), C.byref(n)), fn.__name__)
         if n.value == 0 or not p.value:
-            return torch.empty(0, dtype=dt, device="cuda")
-        return torch.as_tensor(_DevArray(p.value, n.value, typestr, self), device="cuda")
+            return torch.empty(0, dtype=_WIDTH_DTYPE[bits], device="cuda")
+        return _view(p.value, n.value, bits // 8, self)
 
     def positions(self, level):
         """pos[level] as a view of the device array (empty at dense levels): uint8 / uint16 for the
@@ -146,7 +156,7 @@ class SpTensor:
         _check(_lib.sp_values(self._h, C.byref(p), C.byref(n)), "sp_values")
         if n.value == 0:
             return torch.empty(0, dtype=torch.float64, device="cuda")
-        return torch.as_tensor(_DevArray(p.value, n.value, "<f8", self), device="cuda")
+        return _view(p.value, n.value, 0, self)
 
     @property
     def nval(self):
@@ -180,14 +190,13 @@ def sp_pack(dims, coords, vals, dimLevelType, dimOrdering=None, posBits=32, crdB
             raise TypeError("coords must be CUDA tensors of one integer type (int32 or int64)")
         if c.numel() != nnz or not c.is_contiguous():
             raise ValueError("each coords tensor must be contiguous with nnz entries")
-    cptrs = (C.c_void_p * max(rank, 1))(*[c.data_ptr() if nnz else 0 for c in coords])
     h = C.c_void_p()
-    lt = (C.c_int * rank)(*[int(t) for t in dimLevelType])
-    od = (C.c_int * rank)(*[int(o) for o in dimOrdering]) if dimOrdering is not None else None
-    _check(_lib.sp_pack(C.c_int(rank), (C.c_int64 * rank)(*[int(d) for d in dims]), C.c_int64(nnz), cptrs,
-                        C.c_int(bits), _dptr(vals), lt, od, C.c_int(posBits), C.c_int(crdBits), C.c_uint(flags),
-                        _stream(), C.byref(h)), "sp_pack")
-    return SpTensor(h)
+    c_lt, c_od, lt, od = _encoding(rank, dimLevelType, dimOrdering)
+    c_dims = (C.c_int64 * rank)(*map(int, dims))
+    cptrs = (C.c_void_p * max(rank, 1))(*[c.data_ptr() if nnz else 0 for c in coords])
+    _check(_lib.sp_pack(rank, c_dims, nnz, cptrs, bits, vals.data_ptr(), c_lt, c_od, posBits, crdBits, flags, _stream(),
+                        C.byref(h)), "sp_pack")
+    return SpTensor(h, (tuple(c_dims), lt, od, posBits or 64, crdBits or 64))
 
 
 def sp_unpack(t: SpTensor):
@@ -225,7 +234,7 @@ def sp_spmm(A: SpTensor, B, C_out=None):
     N = B.shape[1]
     if C_out is None:
         C_out = torch.empty((A.dims[0], N), dtype=torch.float64, device="cuda")
-    _check(_lib.sp_spmm(A._h, _dptr(B), C.c_int64(N), C.c_int64(B.stride(0)), _dptr(C_out), C.c_int64(C_out.stride(0)),
+    _check(_lib.sp_spmm(A._h, _dptr(B), N, B.stride(0), _dptr(C_out), C_out.stride(0),
                         _stream()), "sp_spmm")
     return C_out
 
@@ -234,8 +243,7 @@ def sp_sddmm(S: SpTensor, A, B, x_vals=None):
     _f64(A, "A"); _f64(B, "B")
     if x_vals is None:
         x_vals = torch.empty(S.nval, dtype=torch.float64, device="cuda")
-    _check(_lib.sp_sddmm(S._h, _dptr(A), C.c_int64(A.stride(0)), _dptr(B), C.c_int64(B.stride(0)),
-                         C.c_int64(A.shape[1]), _dptr(x_vals), _stream()), "sp_sddmm")
+    _check(_lib.sp_sddmm(S._h, _dptr(A), A.stride(0), _dptr(B), B.stride(0), A.shape[1], _dptr(x_vals), _stream()), "sp_sddmm")
     return x_vals
 
 
@@ -246,7 +254,7 @@ def sp_mttkrp(T: SpTensor, B, Cf, M=None):
     R = B.shape[1]
     if M is None:
         M = torch.empty((T.dims[0], R), dtype=torch.float64, device="cuda")
-    _check(_lib.sp_mttkrp(T._h, _dptr(B), _dptr(Cf), C.c_int64(R), _dptr(M), _stream()), "sp_mttkrp")
+    _check(_lib.sp_mttkrp(T._h, _dptr(B), _dptr(Cf), R, _dptr(M), _stream()), "sp_mttkrp")
     return M
 
 
@@ -265,7 +273,7 @@ def sp_mttkrp_mode(T: SpTensor, mode: int, factors, M=None):
     if M is None:
         M = torch.empty((T.dims[mode], R), dtype=torch.float64, device="cuda")
     ptrs = (C.c_void_p * 3)(*[f.data_ptr() if (f is not None and d != mode) else 0 for d, f in enumerate(factors)])
-    _check(_lib.sp_mttkrp_mode(T._h, C.c_int(mode), ptrs, C.c_int64(R), _dptr(M), _stream()), "sp_mttkrp_mode")
+    _check(_lib.sp_mttkrp_mode(T._h, mode, ptrs, R, _dptr(M), _stream()), "sp_mttkrp_mode")
     return M
 
 
@@ -273,7 +281,7 @@ def sp_spmspm(A: SpTensor, B: SpTensor, posBits=32, crdBits=32) -> SpTensor:
     """C = A * B with A, B, C all CSR; returns a new handle."""
     use_torch_allocator()
     h = C.c_void_p()
-    _check(_lib.sp_spmspm(A._h, B._h, C.c_int(posBits), C.c_int(crdBits), _stream(), C.byref(h)), "sp_spmspm")
+    _check(_lib.sp_spmspm(A._h, B._h, posBits, crdBits, _stream(), C.byref(h)), "sp_spmspm")
     return SpTensor(h)
 
 
@@ -281,14 +289,13 @@ def sp_convert(t: SpTensor, dimLevelType, dimOrdering=None, posBits=32, crdBits=
     """Re-encode a tensor through coordinates (unpack + pack on the device)."""
     use_torch_allocator()
     h = C.c_void_p()
-    lt = (C.c_int * t.rank)(*[int(x) for x in dimLevelType])
-    od = (C.c_int * t.rank)(*[int(o) for o in dimOrdering]) if dimOrdering is not None else None
-    _check(_lib.sp_convert(t._h, lt, od, C.c_int(posBits), C.c_int(crdBits), _stream(), C.byref(h)), "sp_convert")
-    return SpTensor(h)
+    c_lt, c_od, lt, od = _encoding(t.rank, dimLevelType, dimOrdering)
+    _check(_lib.sp_convert(t._h, c_lt, c_od, posBits, crdBits, _stream(), C.byref(h)), "sp_convert")
+    return SpTensor(h, (t.dims, lt, od, posBits or 64, crdBits or 64))
 
 
 def sp_scale(x: SpTensor, c: float):
-    _check(_lib.sp_scale(x._h, C.c_double(c), _stream()), "sp_scale")
+    _check(_lib.sp_scale(x._h, c, _stream()), "sp_scale")
     return x
 
 

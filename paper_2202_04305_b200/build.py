@@ -46,6 +46,26 @@ def _compile(src: str, verbose: bool, obj_dir: str = OBJ, extra=()) -> str:
 
 
 LIB_DEBUG = os.path.join(HERE, "libsp_debug_bounds.so")
+LIB_TORCH = os.path.join(HERE, "libsp_torch.so")
+
+
+def build_torch(force: bool = False) -> str:
+    """The binding's torch side (allocator hooks, tensor views); host code only."""
+    src = os.path.join(CSRC, "torch_memory.cpp")
+    if not force and os.path.exists(LIB_TORCH) and os.path.getmtime(LIB_TORCH) >= os.path.getmtime(src):
+        return LIB_TORCH
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
+    cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", LIB_TORCH]
+    for inc in (os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                sysconfig.get_paths()["include"], os.path.join(cuda, "include")):
+        cmd += ["-isystem", inc]
+    cmd += ["-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    subprocess.check_call(cmd)
+    return LIB_TORCH
 
 
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
@@ -59,7 +79,9 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
         for f in os.listdir(obj_dir):
             os.remove(os.path.join(obj_dir, f))
     with cf.ThreadPoolExecutor(max_workers=8) as ex:
+        side = ex.submit(build_torch, force)
         objs = list(ex.map(lambda s: _compile(s, verbose, obj_dir, extra), SOURCES))
+    side.result()
     if force or not os.path.exists(lib) or any(os.path.getmtime(o) > os.path.getmtime(lib) for o in objs):
         subprocess.check_call([_nvcc(), "-Wno-deprecated-gpu-targets", "-shared", "-o", lib] + objs + ["-lcudart"])
     return lib
