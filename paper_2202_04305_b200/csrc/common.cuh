@@ -180,7 +180,9 @@ __device__ __forceinline__ int64_t sp_checked_index(int64_t i, int64_t n, int li
 // its fix-up) are launched as programmatic dependents: the next kernel may be set up on the device
 // while its predecessor drains, and its first statement waits until that predecessor has completed
 // and its writes are visible.  Nothing triggers early: the only thing overlapped is the launch itself.
-// In a kernel launched the ordinary way the wait returns at once.
+// In a kernel launched the ordinary way the wait returns at once.  A pointer to what a predecessor wrote
+// is not `const __restrict__`: loads through such a pointer count as invariant, which leaves the compiler
+// free to move them above the wait whatever memory it says it touches.
 __device__ __forceinline__ void sp_wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
@@ -238,6 +240,11 @@ sp_status sp_get_merge_partition(sp_tensor* t, int64_t items_per_chunk, cudaStre
 // device on first use (one small kernel and one read-back, which waits for the stream) and kept.
 sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out);
 sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t nnz_per_chunk, cudaStream_t stream, sp_partition* out);
+
+// sp_pack for matrices with a compressed inner level and short segments (pack_rows.cu).  SP_ERR_UNSUPPORTED:
+// nothing was built, take the general path.
+sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64_t nnz, const void* outer, const void* inner, int coord_bits,
+                       const double* vals, int posBits, int crdBits, cudaStream_t stream, sp_tensor** out);
 
 // SpMV for rank-2 handles whose inner level is dense (dense_inner.cu).
 sp_status sp_spmv_dense_inner(const sp_tensor* A, const double* x, double* y, cudaStream_t stream);

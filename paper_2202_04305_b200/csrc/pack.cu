@@ -199,7 +199,7 @@ __device__ __forceinline__ uint32_t block256_excl_scan(uint32_t v, uint32_t* sum
 // to 0.59 ms per pass.
 template <int BITS, bool PAY>
 __global__ void __launch_bounds__(kSortThreads)
-k_sort_upsweep(const uint64_t* __restrict__ keys, int64_t n, int shift, uint32_t* __restrict__ tilehist, int64_t ntiles) {
+k_sort_upsweep(const uint64_t* keys, int64_t n, int shift, uint32_t* __restrict__ tilehist, int64_t ntiles) {
     sp_wait_for_previous_kernel();
     constexpr int kSortIpt = SortShape<PAY>::kIpt, kSortTile = SortShape<PAY>::kTile;
     constexpr int RADIX = 1 << BITS;
@@ -252,7 +252,7 @@ __device__ __forceinline__ uint32_t same_value_lanes(uint32_t d) {
 constexpr int kScanChunk = 2048;
 
 __global__ void __launch_bounds__(256)
-k_sort_chunk_totals(const uint32_t* __restrict__ tilehist, int64_t ntiles, int64_t nchunks, uint32_t* __restrict__ chunk_tot) {
+k_sort_chunk_totals(const uint32_t* tilehist, int64_t ntiles, int64_t nchunks, uint32_t* __restrict__ chunk_tot) {
     sp_wait_for_previous_kernel();
     __shared__ uint32_t sums[8];
     const uint32_t* row = tilehist + (int64_t)blockIdx.x * ntiles;
@@ -269,7 +269,7 @@ k_sort_chunk_totals(const uint32_t* __restrict__ tilehist, int64_t ntiles, int64
 }
 
 __global__ void __launch_bounds__(256)
-k_sort_scan(uint32_t* tilehist, int64_t ntiles, int64_t nchunks, const uint32_t* __restrict__ chunk_tot,
+k_sort_scan(uint32_t* tilehist, int64_t ntiles, int64_t nchunks, const uint32_t* chunk_tot,
             uint32_t* __restrict__ digit_total) {
     sp_wait_for_previous_kernel();
     __shared__ uint32_t stage[kScanChunk];
@@ -334,11 +334,11 @@ __device__ __forceinline__ void rank_rounds(const uint64_t (&key)[kSortIpt], int
 // on the way out: keys_out gets key >> split_bits, idx_out the low split_bits bits.
 template <bool PAY, int BITS>
 __global__ void __launch_bounds__(kSortThreads, SortShape<PAY>::kMinBlocks)   // several tiles per SM hide the ranking chain's latency
-k_sort_downsweep(const uint64_t* __restrict__ keys_in, const uint64_t* __restrict__ pay_in,
+k_sort_downsweep(const uint64_t* keys_in, const uint64_t* pay_in,
                  uint64_t* __restrict__ keys_out, uint64_t* __restrict__ pay_out, uint32_t* __restrict__ idx_out,
                  int64_t n, int shift,
-                 const uint32_t* __restrict__ tilehist, int64_t ntiles,
-                 const uint32_t* __restrict__ digit_total, int split_bits) {
+                 const uint32_t* tilehist, int64_t ntiles,
+                 const uint32_t* digit_total, int split_bits) {
     sp_wait_for_previous_kernel();
     constexpr int kSortIpt = SortShape<PAY>::kIpt, kSortTile = SortShape<PAY>::kTile;
     constexpr int RADIX = 1 << BITS;
@@ -541,7 +541,7 @@ __device__ __forceinline__ uint64_t block_excl_scan64(uint64_t v, uint64_t* sums
 // > shift[l], and a count is the population count of a ballot.
 template <int RANK>
 __global__ void __launch_bounds__(kCtThreads)
-k_count_flags(const uint64_t* __restrict__ keys, int64_t n, LevelPlan p, uint64_t* __restrict__ tilesum) {
+k_count_flags(const uint64_t* keys, int64_t n, LevelPlan p, uint64_t* __restrict__ tilesum) {
     sp_wait_for_previous_kernel();
     __shared__ uint32_t wtot[kCtThreads / 32][SP_MAX_RANK];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -589,7 +589,7 @@ static_assert(kField * SP_MAX_RANK <= 64 && (1 << kField) > kCtTile, "packed per
 // Across tiles the counts outgrow the packed fields, so each level is scanned on its own.  A thread
 // owns a run of consecutive tiles, so the block scans once however many tiles there are.
 __global__ void __launch_bounds__(512)
-k_scan_tiles(const uint64_t* __restrict__ tilesum, int64_t ntiles, int rank, int64_t* __restrict__ tileprefix,
+k_scan_tiles(const uint64_t* tilesum, int64_t ntiles, int rank, int64_t* __restrict__ tileprefix,
              int64_t* __restrict__ counts) {
     sp_wait_for_previous_kernel();
     __shared__ uint64_t sums[16];
@@ -816,7 +816,7 @@ __global__ void __launch_bounds__(512) k_rmin_tiles(T* tilemin, int64_t ntiles) 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kCtThreads) k_rmin_apply(T* __restrict__ a, int64_t L, const T* __restrict__ tilecarry) {
+__global__ void __launch_bounds__(kCtThreads) k_rmin_apply(T* a, int64_t L, const T* tilecarry) {
     sp_wait_for_previous_kernel();
     __shared__ T sums[16];
     const T ident = ~(T)0;
@@ -942,6 +942,13 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
     for (int l = 0; l < rank; ++l)
         if (plan.lt[l] == SP_COMPRESSED && (uint64_t)(plan.sz[l] - 1) > max_crd) return SP_ERR_WIDTH_OVERFLOW;
 
+#ifndef SP_BENCH_BUILD
+    if (rank == 2 && plan.lt[1] == SP_COMPRESSED && nnz > 0) {     // short rows (or columns) need no sort by key
+        const sp_status rs = sp_pack_rows(dims, plan.src, plan.lt, nnz, coo_coords[plan.src[0]], coo_coords[plan.src[1]], coo_coord_bits,
+                                          coo_vals, posBits, crdBits, stream, out);
+        if (rs != SP_ERR_UNSUPPORTED) return rs;
+    }
+#endif
     sp_workspace ws(stream);
     PhaseTimer timer(stream, times);
     int npasses_done = 0;

@@ -52,7 +52,7 @@ __device__ __forceinline__ void ld2(const double* p, double* a) {
 template <typename P, typename I, int V, int NCH>
 __global__ void __launch_bounds__(kSThreads)
 k_sddmm(const P* __restrict__ pos, const I* __restrict__ crd, const double* __restrict__ sval,
-        const I* __restrict__ outer, const double* __restrict__ A, int64_t lda, const double* __restrict__ Bt,
+        const I* __restrict__ outer, const double* A, int64_t lda, const double* Bt,
         int64_t ldt, int64_t K, double* __restrict__ xv, const int64_t* __restrict__ prow,
         const int64_t* __restrict__ pnz, int64_t nchunks, int64_t na, int64_t nb) {
     // na, nb: rows of A and of Bt (used by the bounds-checking debug build only)

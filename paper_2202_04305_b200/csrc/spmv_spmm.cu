@@ -173,7 +173,7 @@ k_spmv(const P* __restrict__ pos, const I* __restrict__ crd, const double* __res
 }
 
 template <typename I>
-__global__ void k_spmv_fixup(const double* __restrict__ carry_val, const int64_t* __restrict__ carry_row,
+__global__ void k_spmv_fixup(const double* carry_val, const int64_t* carry_row,
                              int64_t ntiles, const I* __restrict__ outer, double* __restrict__ y, int64_t m) {
     sp_wait_for_previous_kernel();
     int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -528,7 +528,7 @@ k_spmm_scatter(const uint32_t* __restrict__ seg, const I* __restrict__ crd, cons
 }
 
 template <typename I>
-__global__ void k_spmm_fixup(const double* __restrict__ carry, const int64_t* __restrict__ carry_row,
+__global__ void k_spmm_fixup(const double* carry, const int64_t* carry_row,
                              int64_t nchunks, const I* __restrict__ outer, int64_t N, double* __restrict__ C,
                              int64_t ldc, int64_t m) {
     sp_wait_for_previous_kernel();
