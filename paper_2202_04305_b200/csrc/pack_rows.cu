@@ -1,299 +1,335 @@
-// sp_pack for matrices with a compressed inner level and short segments (rows of CSR and DCSR, columns of
-// CSC and DCSC): the entries are counted per outer index, scattered to their segment and put in order
-// inside it, instead of being sorted by a fused key.
+// sp_pack for matrices with a compressed inner level and moderate segments (rows of CSR and DCSR, columns of
+// CSC and DCSC): no sort by key, the entries pass through memory twice.
 //
-//   1. k_rows_count    range check; rank of the entry among those of its outer index seen so far (one atomic)
-//   2. k_rows_sums     per tile of outer indices: entries, non-empty indices, sum of squared lengths
-//      k_rows_offsets  segment starts; pos[1], and for a compressed outer level crd[0] and the packed pos[1]
-//   3. k_rows_scatter  value and both coordinates of every entry as one 16-byte record into its segment
-//   4. k_rows_sort     order inside the segments by counting the smaller coordinates; crd[1], values
+//   1. k_rows_partition  range check; entries into buckets, one per range of outer indices, in any order
+//   2. k_rows_build      a block per bucket: entries per outer index, order inside every segment, and
+//                        everything the bucket contributes to the storage, written in order
+//   3. k_rows_outer      (compressed outer level) the buckets' lists of stored outer indices, joined
 //
-// Every entry is moved twice where the radix sort moves it once per eight key bits, all array sizes are
-// known beforehand (the outer level's are bounded), and the one read-back comes at the end.  Step 4 costs the
-// sum of the squared segment lengths; a device-side check (k_rows_sums) makes the kernels after it return
-// when that or a single segment is too long, and the caller takes the radix path, as it does for
-// duplicate coordinates, whose values have to be summed.
-//
-// Bound: random accesses at L2 (5,000,000 entries by 1,048,576 columns: counting 51 us, scatter 120 us; 100 and
-// 42 G accesses/s).  The whole pack of those entries takes 282 us, by radix sort 341 us; of 10,486 entries 63 us
-// against 85 us.
+// Buckets hold about kAverage entries and at most kCap.  Random accesses are what a GPU is slow at (about 140 G
+// single-lane accesses/s here, hit or miss): this way an entry costs one, its 16-byte store in step 1; every
+// other scattered access stays in shared memory.  Sizes are known beforehand (a compressed outer level's are
+// bounded), so the one read-back comes at the end.  A bucket that overflows (long or very uneven segments)
+// and duplicate coordinates, whose values have to be summed, are found on the device; the kernels after that
+// return and the caller takes the radix path.
 #include "common.cuh"
 
 #include <algorithm>
 
+#ifndef SP_ROWS_MINB
+#define SP_ROWS_MINB 3
+#endif
+#ifndef SP_ROWS_T2
+#define SP_ROWS_T2 300000
+#endif
+#ifndef SP_ROWS_T8
+#define SP_ROWS_T8 3000000
+#endif
+
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kIpt = 8;                         // entries per thread and tile of k_rows_count / k_rows_scatter
-constexpr int kTile = kThreads * kIpt;
-constexpr int kRowIpt = 8;                      // outer indices per thread of the two scan kernels
-constexpr int kRowTile = kThreads * kRowIpt;
-constexpr int kSortTile = 2048;                 // entries whose segments start in a block's share of k_rows_sort
-constexpr int kMaxLen = 2048;                   // longest segment taken
-constexpr int kSortCap = kSortTile + kMaxLen;
-constexpr uint32_t kAbortRank = 4 * kMaxLen;    // a longer segment is not taken, so counting it further is pointless
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kCap = 4096;                      // entries a bucket can hold
+constexpr int kIpt = kCap / kThreads;           // ... per thread of k_rows_build
+constexpr int kAverage = 2048;                  // entries per bucket aimed at: rows of 48 +- 7 and power-law rows stay below twice that
+constexpr int kWidth = 2048;                    // outer indices of a bucket
+constexpr int kMaxBuckets = 4096;
+constexpr int kDense = 24;                      // mean compares per entry above which segments are cut into bins
 
-// What the device reports: word 0 = kErr* bits, 1 = non-empty outer indices, 2 = sum of squared segment lengths.
-// kErrIndex: an index derived from the counters fell outside its array (its access was skipped); never for a sound run.
-constexpr unsigned long long kErrRange = 1, kErrDup = 2, kErrLong = 4, kErrIndex = 8;
+// What the device reports: word 0 = kErr* bits, 1 = non-empty outer indices.
+constexpr unsigned long long kErrRange = 1, kErrDup = 2, kErrLong = 4;
 
-using Rec = uint4;                              // value (low word, high word), inner coordinate, outer coordinate
+using Rec = uint4;                              // value (low, high word), inner coordinate, outer coordinate
 
-// Whether the kernels after k_rows_sums go on.
-__device__ __forceinline__ bool stopped(const unsigned long long* info, unsigned long long most) {
-    return __ldcg(info) != 0 || __ldcg(info + 2) > most;
+// Outer index o lies in bucket o * scale / 2^32; bucket b begins at the first o that the formula gives b for.
+__host__ __device__ __forceinline__ int64_t bucket_begin(int64_t b, uint32_t scale, int64_t no) {
+    const int64_t o = (int64_t)((((uint64_t)b << 32) + scale - 1) / scale);
+    return o < no ? o : no;
 }
 
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-k_rows_count(const CT* __restrict__ oc, const CT* __restrict__ ic, int64_t n, int64_t no, int64_t ni, uint32_t* __restrict__ count,
-             uint32_t* __restrict__ rank, unsigned long long* __restrict__ info) {
-    if (__ldcg(info) != 0) return;              // an earlier block met a bad entry or a very long segment
-    const int64_t base = (int64_t)blockIdx.x * kTile + threadIdx.x;
-    CT o[kIpt], c[kIpt];
-    uint32_t r[kIpt];
+// Whether some block has reported an error, the same answer for all threads of a block.
+__device__ __forceinline__ bool stopped(const unsigned long long* info) {
+    return __syncthreads_or(threadIdx.x == 0 && __ldcg(info) != 0) != 0;
+}
+
+// Exclusive scan over the block of one counter per thread.
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* s_w, uint32_t* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t incl = v;
 #pragma unroll
-    for (int i = 0; i < kIpt; ++i) {
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) s_w[w] = incl;
+    __syncthreads();
+    uint32_t pre = 0, tot = 0;
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) {
+        const uint32_t s = s_w[i];
+        if (i < w) pre += s;
+        tot += s;
+    }
+    __syncthreads();
+    *total = tot;
+    return incl - v + pre;
+}
+
+// In-place exclusive scan of s[0 .. n), n <= PER * kThreads; s[n] = the total.
+template <int PER>
+__device__ __forceinline__ void scan_shared(uint32_t* s, int n, uint32_t* s_w) {
+    const int i0 = threadIdx.x * PER;
+    uint32_t v[PER], mine = 0, tot;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) { v[i] = i0 + i < n ? s[i0 + i] : 0u; mine += v[i]; }
+    uint32_t at = block_scan(mine, s_w, &tot);
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (i0 + i < n) { s[i0 + i] = at; at += v[i]; }
+    if (threadIdx.x == 0) s[n] = tot;
+    __syncthreads();
+}
+
+// A block sends a tile of kThreads * PER entries to their buckets: ranks inside the tile by shared-memory
+// atomics, the tile's place in every bucket by one atomic on the bucket's cursor.
+template <typename CT, int PER>
+__global__ void __launch_bounds__(kThreads)
+k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
+                 uint32_t scale, int nb, uint32_t* __restrict__ cursor, Rec* __restrict__ rec, unsigned long long* __restrict__ info) {
+    extern __shared__ uint32_t s_hist[];
+    if (stopped(info)) return;
+    const int t = threadIdx.x;
+    for (int b = t; b < nb; b += kThreads) s_hist[b] = 0u;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * (kThreads * PER) + t;
+    CT o[PER], c[PER];
+    uint32_t r[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
         const int64_t e = base + i * kThreads;
         o[i] = e < n ? oc[e] : (CT)0;
         c[i] = e < n ? ic[e] : (CT)0;
     }
-    bool bad = false, far = false;
+    bool bad = false;
 #pragma unroll
-    for (int i = 0; i < kIpt; ++i) {
-        const int64_t e = base + i * kThreads;
-        r[i] = 0;
-        if (o[i] < 0 || (int64_t)o[i] >= no || c[i] < 0 || (int64_t)c[i] >= ni) bad = true;
-        else if (e < n) r[i] = atomicAdd(count + o[i], 1u);
+    for (int i = 0; i < PER; ++i) {
+        if (o[i] < 0 || (int64_t)o[i] >= no || c[i] < 0 || (int64_t)c[i] >= ni) { bad = true; o[i] = 0; }
+        r[i] = base + i * kThreads < n ? atomicAdd(&s_hist[__umulhi((uint32_t)o[i], scale)], 1u) : 0u;
     }
-#pragma unroll
-    for (int i = 0; i < kIpt; ++i) {
-        const int64_t e = base + i * kThreads;
-        if (e < n) rank[e] = r[i];
-        far |= r[i] >= kAbortRank;
-    }
-    if (bad) atomicOr(info, kErrRange);
-    if (far) atomicOr(info, kErrLong);
-}
-
-// Block-wide exclusive scan of two counters at once and their totals.
-__device__ __forceinline__ uint2 block_scan2(uint2 v, uint2* s_w, uint2* total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint2 incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t ux = __shfl_up_sync(0xffffffffu, incl.x, o), uy = __shfl_up_sync(0xffffffffu, incl.y, o);
-        if (lane >= o) { incl.x += ux; incl.y += uy; }
-    }
-    if (lane == 31) s_w[w] = incl;
-    __syncthreads();
-    uint2 pre = make_uint2(0, 0), tot = make_uint2(0, 0);
-#pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) {
-        const uint2 s = s_w[i];
-        if (i < w) { pre.x += s.x; pre.y += s.y; }
-        tot.x += s.x; tot.y += s.y;
-    }
-    __syncthreads();
-    *total = tot;
-    return make_uint2(incl.x - v.x + pre.x, incl.y - v.y + pre.y);
-}
-
-// A thread's kRowIpt consecutive counters.
-__device__ __forceinline__ void load_counts(const uint32_t* count, int64_t no, uint32_t* len) {
-    const int64_t q0 = (int64_t)blockIdx.x * kRowTile + (int64_t)threadIdx.x * kRowIpt;
-    if (q0 + kRowIpt <= no) {                   // `count` is 256-byte aligned
-#pragma unroll
-        for (int i = 0; i < kRowIpt; i += 4) {
-            const uint4 v = *reinterpret_cast<const uint4*>(count + q0 + i);
-            len[i] = v.x; len[i + 1] = v.y; len[i + 2] = v.z; len[i + 3] = v.w;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < kRowIpt; ++i) len[i] = q0 + i < no ? count[q0 + i] : 0u;
-    }
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_rows_sums(const uint32_t* count, int64_t no, uint2* __restrict__ tile, unsigned long long* __restrict__ info) {
-    sp_wait_for_previous_kernel();
-    if (__ldcg(info) != 0) return;
-    __shared__ uint2 s_w[kThreads / 32];
-    __shared__ unsigned long long s_sq[kThreads / 32];
-    uint32_t len[kRowIpt];
-    load_counts(count, no, len);
-    uint2 mine = make_uint2(0, 0), tot;
-    unsigned long long sq = 0;
-    bool longer = false;
-#pragma unroll
-    for (int i = 0; i < kRowIpt; ++i) {
-        mine.x += len[i];
-        mine.y += len[i] != 0;
-        sq += (unsigned long long)len[i] * len[i];
-        longer |= len[i] > kMaxLen;
-    }
-    block_scan2(mine, s_w, &tot);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if ((threadIdx.x & 31) == 0) s_sq[threadIdx.x >> 5] = sq;
-    if (__syncthreads_or(longer) && threadIdx.x == 0) atomicOr(info, kErrLong);
-    if (threadIdx.x == 0) {
-        tile[blockIdx.x] = tot;
-        for (int i = 1; i < kThreads / 32; ++i) sq += s_sq[i];
-        atomicAdd(info + 2, sq);
-    }
-}
-
-// start[q] = first entry of outer index q; first[t] = start of the first segment that starts at entry
-// t * kSortTile or later (t = 0 .. the number of sort tiles).  DBL: crd0 / pos1 list the non-empty indices.
-template <typename P, typename I, bool DBL>
-__global__ void __launch_bounds__(kThreads)
-k_rows_offsets(const uint32_t* count, int64_t no, const uint2* tile, int64_t n, unsigned long long most,
-               uint32_t* __restrict__ start, uint32_t* __restrict__ first, P* __restrict__ pos0, I* __restrict__ crd0,
-               P* __restrict__ pos1, int64_t nq, unsigned long long* __restrict__ info) {
-    sp_wait_for_previous_kernel();
-    if (stopped(info, most)) return;
-    const uint32_t stiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
-    bool off = false;
-    __shared__ uint2 s_w[kThreads / 32];
-    uint2 before = make_uint2(0, 0), tot;
-    for (int64_t t = threadIdx.x; t < blockIdx.x; t += kThreads) { const uint2 v = tile[t]; before.x += v.x; before.y += v.y; }
-    block_scan2(before, s_w, &tot);             // every block adds up the tiles before its own
-    before = tot;
-    uint32_t len[kRowIpt];
-    load_counts(count, no, len);
-    uint2 mine = make_uint2(0, 0);
-#pragma unroll
-    for (int i = 0; i < kRowIpt; ++i) { mine.x += len[i]; mine.y += len[i] != 0; }
-    uint2 at = block_scan2(mine, s_w, &tot);
-    at.x += before.x;
-    at.y += before.y;
-    const int64_t q0 = (int64_t)blockIdx.x * kRowTile + (int64_t)threadIdx.x * kRowIpt;
-#pragma unroll
-    for (int i = 0; i < kRowIpt; ++i) {
-        const int64_t q = q0 + i;
-        if (q < no) {
-            start[q] = at.x;
-            if (!DBL) {
-                if (sizeof(P) != 4) pos1[q] = (P)at.x;          // 32-bit positions: start is pos1
-            } else if (len[i]) {
-                if (at.y < nq) {
-                    crd0[at.y] = (I)q;
-                    pos1[at.y] = (P)at.x;
-                } else off = true;
-            }
-            off |= (int64_t)at.x + len[i] > n;
-            for (uint32_t t = at.x / kSortTile + 1; t <= stiles && (int64_t)t * kSortTile <= (int64_t)at.x + len[i]; ++t) first[t] = at.x + len[i];
-            at.x += len[i];
-            at.y += len[i] != 0;
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) first[0] = 0;
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kThreads - 1) {
-        off |= (int64_t)at.x != n || (DBL && (int64_t)at.y > nq);
-        first[stiles] = (uint32_t)n;
-        if (!DBL || (int64_t)at.y <= nq) pos1[DBL ? (int64_t)at.y : no] = (P)n;
-        if (DBL) { pos0[0] = 0; pos0[1] = (P)at.y; info[1] = at.y; }
-    }
-    if (off) atomicOr(info, kErrIndex);
-}
-
-template <typename CT>
-__global__ void __launch_bounds__(kThreads)
-k_rows_scatter(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n,
-               const uint32_t* rank, const uint32_t* start, int64_t no, unsigned long long most,
-               unsigned long long* __restrict__ info, Rec* __restrict__ rec) {
-    sp_wait_for_previous_kernel();
-    if (stopped(info, most)) return;
-    const int64_t base = (int64_t)blockIdx.x * kTile + threadIdx.x;
-    uint32_t o[kIpt], c[kIpt], r[kIpt];
-    double v[kIpt];
-#pragma unroll
-    for (int i = 0; i < kIpt; ++i) {
-        const int64_t e = base + i * kThreads;
-        const bool ok = e < n;
-        o[i] = ok ? (uint32_t)oc[e] : 0u;
-        c[i] = ok ? (uint32_t)ic[e] : 0u;
-        r[i] = ok ? rank[e] : 0u;
-        v[i] = ok ? vals[e] : 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < kIpt; ++i) r[i] += o[i] < no ? start[o[i]] : (uint32_t)n;
-    bool off = false;
-#pragma unroll
-    for (int i = 0; i < kIpt; ++i)
-        if (base + i * kThreads < n) {
-            if (r[i] >= n) { off = true; continue; }
-            rec[r[i]] = make_uint4((uint32_t)__double2loint(v[i]), (uint32_t)__double2hiint(v[i]), c[i], o[i]);
-        }
-    if (off) atomicOr(info, kErrIndex);
-}
-
-// A block puts the segments that start among its kSortTile entries in order.  An entry's place is the number
-// of smaller coordinates in its segment, counted over shared memory: lanes of one segment read the same word.
-template <typename I>
-__global__ void __launch_bounds__(kThreads)
-k_rows_sort(const Rec* rec, const uint32_t* first, int64_t n, unsigned long long most, unsigned long long* __restrict__ info,
-            I* __restrict__ crd, double* __restrict__ val, uint32_t* __restrict__ seg_out) {
-    sp_wait_for_previous_kernel();
-    if (stopped(info, most)) return;
-    __shared__ uint32_t s_c[kSortCap];
-    __shared__ uint32_t s_head[kSortCap / 32 + 1];      // one bit per entry: a segment starts here (and one past the end)
-    __shared__ int s_prev[kSortCap / 32], s_next[kSortCap / 32 + 1];
-    const int64_t e0 = first[blockIdx.x];
-    const int64_t span = (int64_t)first[blockIdx.x + 1] - e0;
-    const int cnt = (int)(span < kSortCap + 1 ? span : kSortCap + 1);
-    if (cnt <= 0) return;
-    if (cnt > kSortCap || e0 + cnt > n) {
-        if (threadIdx.x == 0) atomicOr(info, kErrIndex);
+    if (__syncthreads_or(bad)) {
+        if (t == 0) atomicOr(info, kErrRange);
         return;
     }
-    const int t = threadIdx.x, lane = t & 31;
-    const int words = (cnt + 31) / 32;
-    for (int i = t; i < words * 32; i += kThreads) {
-        uint32_t c = 0, o = 0, ob = 0;
-        if (i < cnt) {
-            const Rec x = rec[e0 + i];
-            c = x.z; o = x.w;
-            if (lane == 0 && i > 0) ob = rec[e0 + i - 1].w;
+    bool full = false;
+    for (int b = t; b < nb; b += kThreads) {
+        const uint32_t k = s_hist[b];
+        if (k) {
+            const uint32_t at = atomicAdd(cursor + b, k);
+            full |= at + k > (uint32_t)kCap;
+            s_hist[b] = at;
         }
-        s_c[i] = c;
-        const uint32_t up = __shfl_up_sync(0xffffffffu, o, 1);
-        const bool head = i < cnt && (i == 0 || o != (lane ? up : ob));
-        const uint32_t m = __ballot_sync(0xffffffffu, head);
-        if (lane == 0) s_head[i / 32] = m;
     }
-    __syncthreads();
-    for (int w = t; w < words; w += kThreads) {         // last head before word w, first head from word w on
-        int p = w - 1;
-        while (p >= 0 && s_head[p] == 0) --p;
-        s_prev[w] = p >= 0 ? p * 32 + 31 - __clz(s_head[p]) : 0;
-        int q = w;
-        while (q < words && s_head[q] == 0) ++q;
-        s_next[w] = q < words ? q * 32 + __ffs(s_head[q]) - 1 : cnt;
+    if (__syncthreads_or(full)) {
+        if (t == 0) atomicOr(info, kErrLong);
+        return;
     }
-    if (t == 0) s_next[words] = cnt;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int64_t e = base + i * kThreads;
+        if (e < n) {
+            const uint32_t b = __umulhi((uint32_t)o[i], scale);
+            const double v = vals[e];
+            rec[(size_t)b * kCap + s_hist[b] + r[i]] =
+                make_uint4((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), (uint32_t)c[i], (uint32_t)o[i]);
+        }
+    }
+}
+
+struct BuildShared {
+    uint32_t count[kWidth + 1];                 // entries, then starts, of the bucket's outer indices; later the entries' outer offsets
+    uint32_t crd[kCap];
+    union {
+        double val[kCap];
+        struct { uint32_t lo[kWidth], hi[kWidth]; };        // smallest and largest coordinate of a segment
+        struct { double unused[kCap / 2]; uint32_t bin[kCap]; };
+    };
+    uint32_t bin_end;                           // bin[kCap] when the bucket is full
+    uint32_t w[kWarps];
+};
+static_assert(sizeof(uint32_t) * 2 * kWidth <= sizeof(double) * kCap / 2, "lo and hi lie before bin");
+static_assert(kWidth * 2 >= kCap, "the starts' space holds a 16-bit number per entry");
+
+// The place of an entry is the start of its segment plus the number of smaller coordinates in it, counted over
+// shared memory.  Where segments are long (more than kDense compares per entry on average) they are first
+// cut into as many bins as they have entries, evenly between their smallest and largest coordinate, and only
+// the entries of one bin are compared.
+template <typename P, typename I, bool DBL>
+__global__ void __launch_bounds__(kThreads, SP_ROWS_MINB)
+k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int nb, unsigned long long* __restrict__ info,
+             P* __restrict__ pos1, I* __restrict__ crd, double* __restrict__ val, uint32_t* __restrict__ seg_out,
+             uint32_t* __restrict__ outer_list, uint32_t* __restrict__ outer_pos, uint32_t* __restrict__ outer_count) {
+    sp_wait_for_previous_kernel();
+    if (stopped(info)) return;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    BuildShared& s = *reinterpret_cast<BuildShared*>(s_raw);
+    const int t = threadIdx.x, b = blockIdx.x;
+    const int cnt = (int)cursor[b];
+    const int64_t lo = bucket_begin(b, scale, no), hi = b + 1 < nb ? bucket_begin(b + 1, scale, no) : no;
+    const int width = (int)(hi - lo);
+    // entries of this thread, requested first; the values are fetched again at the end (registers)
+    const Rec* mine = rec + (size_t)b * kCap + t;
+    uint32_t c[kIpt], qr[kIpt];                 // inner coordinate; outer offset << 16 | rank, later the place
+#pragma unroll
+    for (int i = 0; i < kIpt; ++i) {
+        c[i] = qr[i] = 0u;
+        if (i * kThreads + t < cnt) { const Rec x = mine[i * kThreads]; c[i] = x.z; qr[i] = x.w - (uint32_t)lo; }
+    }
+    uint32_t before = 0, base;
+    for (int q = t; q < b; q += kThreads) before += cursor[q];
+    for (int q = t; q < width; q += kThreads) { s.count[q] = 0u; s.lo[q] = ~0u; s.hi[q] = 0u; }
+    block_scan(before, s.w, &base);             // (also the barrier after the zeroing)
+#pragma unroll
+    for (int i = 0; i < kIpt; ++i)
+        if (i * kThreads + t < cnt) qr[i] = qr[i] << 16 | atomicAdd(&s.count[qr[i]], 1u);
     __syncthreads();
+    // mean number of compares without bins; outer level
+    uint32_t sq = 0, filled = 0, tot_sq, tot_filled;
+    constexpr int kPerW = kWidth / kThreads;
+#pragma unroll
+    for (int i = 0; i < kPerW; ++i) {
+        const int q = t * kPerW + i;
+        const uint32_t k = q < width ? s.count[q] : 0u;
+        sq += k * k;                            // at most kCap^2 in all
+        filled += k != 0;
+    }
+    const uint32_t at_filled = block_scan(filled, s.w, &tot_filled);
+    block_scan(sq, s.w, &tot_sq);
+    const bool bins = tot_sq > (uint32_t)kDense * (uint32_t)cnt;
+    if (DBL) {
+        uint32_t k = 0;                         // the stored indices of this thread's kPerW, in order
+#pragma unroll
+        for (int i = 0; i < kPerW; ++i) {
+            const int q = t * kPerW + i;
+            if (q < width && s.count[q]) { outer_list[lo + at_filled + k] = (uint32_t)(lo + q); ++k; }
+        }
+        if (t == 0) outer_count[b] = tot_filled;
+        __syncthreads();
+        uint32_t len[kPerW];
+#pragma unroll
+        for (int i = 0; i < kPerW; ++i) { const int q = t * kPerW + i; len[i] = q < width ? s.count[q] : 0u; }
+        scan_shared<kPerW>(s.count, width, s.w);
+        k = 0;
+#pragma unroll
+        for (int i = 0; i < kPerW; ++i)
+            if (len[i]) { outer_pos[lo + at_filled + k] = base + s.count[t * kPerW + i]; ++k; }
+    } else {
+        scan_shared<kPerW>(s.count, width, s.w);
+        for (int q = t; q < width; q += kThreads) pos1[lo + q] = (P)(base + s.count[q]);
+        if (b == nb - 1 && t == 0) pos1[no] = (P)n;
+    }
+    // place of coordinate c among s.crd[j .. e)
     bool dup = false;
-    for (int i = t; i < cnt; i += kThreads) {
-        const uint32_t h = s_head[i / 32], below = h & (0xffffffffu >> (31 - lane)), above = lane == 31 ? 0u : h >> (lane + 1);
-        const int s = below ? (i & ~31) + 31 - __clz(below) : s_prev[i / 32];
-        const int e = above ? i + __ffs(above) : s_next[i / 32 + 1];
-        const Rec x = rec[e0 + i];
-        const uint32_t c = x.z;
-        int less = 0, same = 0;
-        for (int j = s; j < e; ++j) {
-            const uint32_t cj = s_c[j];
-            less += cj < c;
-            same += cj == c;
+    auto place_of = [&](int j, int e, uint32_t cc) {
+        int at = j, same = 0;
+        for (; j < e; ++j) {
+            const uint32_t cj = s.crd[j];
+            at += cj < cc;
+            same += cj == cc;
         }
         dup |= same > 1;
-        const int64_t p = e0 + s + less;
-        crd[p] = (I)c;
-        val[p] = __hiloint2double((int)x.y, (int)x.x);
-        if (seg_out) seg_out[p] = x.w;
+        return at;
+    };
+    uint32_t to[kIpt];                          // outer offset << 16 | place
+    if (!bins) {
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i)
+            if (i * kThreads + t < cnt) s.crd[s.count[qr[i] >> 16] + (qr[i] & 0xffffu)] = c[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i)
+            if (i * kThreads + t < cnt) {
+                const uint32_t q = qr[i] >> 16;
+                to[i] = q << 16 | (uint32_t)place_of((int)s.count[q], (int)s.count[q + 1], c[i]);
+            }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i)
+            if (i * kThreads + t < cnt) {
+                atomicMin(&s.lo[qr[i] >> 16], c[i]);
+                atomicMax(&s.hi[qr[i] >> 16], c[i]);
+            }
+        for (int j = t; j < cnt; j += kThreads) s.bin[j] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i)
+            if (i * kThreads + t < cnt) {
+                const uint32_t q = qr[i] >> 16, first = s.count[q], len = s.count[q + 1] - first, c0 = s.lo[q];
+                // not decreasing in the coordinate: the factor is the segment's, and rounding keeps the order
+                const uint32_t k = (uint32_t)((float)(c[i] - c0) * ((float)len / ((float)(s.hi[q] - c0) + 1.0f)));
+                const uint32_t g = first + (k < len ? k : len - 1u);
+                to[i] = g << 16 | atomicAdd(&s.bin[g], 1u);
+            }
+        __syncthreads();
+        scan_shared<kIpt>(s.bin, cnt, s.w);     // the total lands in bin[cnt], which is bin_end for a full bucket
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i)
+            if (i * kThreads + t < cnt) s.crd[s.bin[to[i] >> 16] + (to[i] & 0xffffu)] = c[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i)
+            if (i * kThreads + t < cnt) {
+                const uint32_t g = to[i] >> 16;
+                to[i] = (qr[i] & 0xffff0000u) | (uint32_t)place_of((int)s.bin[g], (int)s.bin[g + 1], c[i]);
+            }
     }
-    if (dup) atomicOr(info, kErrDup);
+    if (__syncthreads_or(dup)) {
+        if (t == 0) atomicOr(info, kErrDup);
+        return;
+    }
+    // everyone has read the coordinates, starts and bins: their space takes the sorted bucket
+    uint16_t* s_seg = reinterpret_cast<uint16_t*>(s.count);
+#pragma unroll
+    for (int i = 0; i < kIpt; ++i)
+        if (i * kThreads + t < cnt) {
+            const uint2 v = *reinterpret_cast<const uint2*>(mine + i * kThreads);
+            const uint32_t p = to[i] & 0xffffu;
+            s.crd[p] = c[i];
+            s.val[p] = __hiloint2double((int)v.y, (int)v.x);
+            if (seg_out) s_seg[p] = (uint16_t)(to[i] >> 16);
+        }
+    __syncthreads();
+    for (int j = t; j < cnt; j += kThreads) {
+        crd[base + j] = (I)s.crd[j];
+        val[base + j] = s.val[j];
+        if (seg_out) seg_out[base + j] = (uint32_t)lo + s_seg[j];
+    }
+}
+
+// Joins the buckets' lists of non-empty outer indices and of their first entries: crd[0] and pos[1].
+template <typename P, typename I>
+__global__ void __launch_bounds__(kThreads)
+k_rows_outer(const uint32_t* outer_list, const uint32_t* outer_pos, const uint32_t* outer_count, int64_t n, int64_t no, uint32_t scale, int nb,
+             unsigned long long* __restrict__ info, P* __restrict__ pos0, I* __restrict__ crd0, P* __restrict__ pos1) {
+    sp_wait_for_previous_kernel();
+    if (stopped(info)) return;
+    __shared__ uint32_t s_w[kWarps];
+    const int t = threadIdx.x, b = blockIdx.x;
+    uint32_t before = 0, base;
+    for (int q = t; q < b; q += kThreads) before += outer_count[q];
+    block_scan(before, s_w, &base);
+    const int64_t lo = bucket_begin(b, scale, no);
+    const uint32_t cnt = outer_count[b];
+    for (uint32_t q = t; q < cnt; q += kThreads) {
+        crd0[base + q] = (I)outer_list[lo + q];
+        pos1[base + q] = (P)outer_pos[lo + q];
+    }
+    if (b == nb - 1 && t == 0) {
+        pos1[base + cnt] = (P)n;
+        pos0[0] = 0;
+        pos0[1] = (P)(base + cnt);
+        info[1] = base + cnt;
+    }
 }
 
 }  // namespace
@@ -302,29 +338,31 @@ k_rows_sort(const Rec* rec, const uint32_t* first, int64_t n, unsigned long long
 sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64_t n, const void* outer, const void* inner, int coord_bits,
                        const double* vals, int posBits, int crdBits, cudaStream_t stream, sp_tensor** out) {
     const int64_t no = dims[ord[0]], ni = dims[ord[1]];
-    // Counters, starts and one scan over the outer indices are paid whatever they hold, so there may be at
-    // most four per entry; records hold 32-bit coordinates; narrow positions need the radix path's width checks.
-    if (posBits < 32 || crdBits < 32 || no > 4 * n + 65536 || no >= ((int64_t)1 << 31) || ni >= ((int64_t)1 << 32) || n >= ((int64_t)1 << 31))
-        return SP_ERR_UNSUPPORTED;
-    // an average this long cannot pass the check below
-    const unsigned long long most = 200000000ull + 128ull * (unsigned long long)n;
-    if ((double)n * (double)n > (double)most * (double)no) return SP_ERR_UNSUPPORTED;
+    // narrow positions need the radix path's width checks; records hold 32-bit coordinates
+    if (posBits < 32 || crdBits < 32 || no >= ((int64_t)1 << 31) || ni >= ((int64_t)1 << 32)) return SP_ERR_UNSUPPORTED;
+    // enough buckets for the entries and for the outer indices, no more than there are outer indices
+    int64_t buckets = std::max(sp_ceil_div(n, kAverage), sp_ceil_div(no, kWidth - 48));
+    if (buckets > kMaxBuckets) return SP_ERR_UNSUPPORTED;
+    if (buckets > no) {
+        if (n > no * kCap) return SP_ERR_UNSUPPORTED;
+        buckets = no;
+    }
+    const int nb = (int)buckets;
+    const uint32_t scale = (uint32_t)std::min<uint64_t>(((uint64_t)nb << 32) / (uint64_t)no, 0xffffffffull);
+    for (int64_t b : {(int64_t)0, (int64_t)nb - 1})      // the last range also takes what rounding leaves over
+        if ((b + 1 < nb ? bucket_begin(b + 1, scale, no) : no) - bucket_begin(b, scale, no) > kWidth) return SP_ERR_UNSUPPORTED;
     const bool dbl = lt[0] == SP_COMPRESSED;
-    const int64_t rtiles = sp_ceil_div(no, kRowTile), stiles = sp_ceil_div(n, kSortTile);
     const size_t pw = posBits / 8, cw = crdBits / 8;
-    const bool alias = !dbl && posBits == 32;           // pos[1] is the array of segment starts
     sp_workspace ws(stream);
-    const size_t counters = sp_workspace::bytes_for<uint32_t>((size_t)no), infob = sp_workspace::bytes_for<unsigned long long>(4);
-    ws.reserve(counters + infob + sp_workspace::bytes_for<uint32_t>((size_t)n) + sp_workspace::bytes_for<Rec>((size_t)n) +
-               sp_workspace::bytes_for<uint2>((size_t)rtiles) + sp_workspace::bytes_for<uint32_t>((size_t)stiles + 2) +
-               (alias ? 0 : sp_workspace::bytes_for<uint32_t>((size_t)no)));
-    uint32_t* count = ws.get<uint32_t>((size_t)no);
-    unsigned long long* info = ws.get<unsigned long long>(4);
-    uint32_t* rank = ws.get<uint32_t>((size_t)n);
-    Rec* rec = ws.get<Rec>((size_t)n);
-    uint2* tile = ws.get<uint2>((size_t)rtiles);
-    uint32_t* first = ws.get<uint32_t>((size_t)stiles + 2);
-    uint32_t* start = alias ? nullptr : ws.get<uint32_t>((size_t)no);
+    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb), infob = sp_workspace::bytes_for<unsigned long long>(2);
+    ws.reserve(cursors + infob + sp_workspace::bytes_for<Rec>((size_t)nb * kCap) +
+               (dbl ? 2 * sp_workspace::bytes_for<uint32_t>((size_t)no) + cursors : 0));
+    uint32_t* cursor = ws.get<uint32_t>((size_t)nb);
+    unsigned long long* info = ws.get<unsigned long long>(2);
+    Rec* rec = ws.get<Rec>((size_t)nb * kCap);
+    uint32_t* outer_list = dbl ? ws.get<uint32_t>((size_t)no) : nullptr;
+    uint32_t* outer_pos = dbl ? ws.get<uint32_t>((size_t)no) : nullptr;
+    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb) : nullptr;
     if (ws.failed) return SP_ERR_ALLOC;
 
     sp_tensor* t = new sp_tensor();
@@ -355,48 +393,48 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         seg_out = reinterpret_cast<uint32_t*>(sg.aux);
         t->parts[(uint64_t)SP_PART_SEGIDS << 56] = sg;
     }
-    if (alias) start = static_cast<uint32_t*>(t->pos[1]);
 
-    cudaError_t e = cudaMemsetAsync(count, 0, counters + infob, stream);
-    const dim3 tiles((unsigned)sp_ceil_div(n, kTile)), threads(kThreads);
-#define SP_ROWS_LAUNCH(kernel, grid, ...) \
-    (e = e != cudaSuccess ? e : sp_launch_dependent(kernel, grid, threads, 0, stream, __VA_ARGS__))
-    if (e == cudaSuccess) {                             // the first of the chain: an ordinary launch
-        if (coord_bits == 32)
-            k_rows_count<int32_t><<<tiles, threads, 0, stream>>>(static_cast<const int32_t*>(outer), static_cast<const int32_t*>(inner), n, no, ni, count, rank, info);
-        else
-            k_rows_count<int64_t><<<tiles, threads, 0, stream>>>(static_cast<const int64_t*>(outer), static_cast<const int64_t*>(inner), n, no, ni, count, rank, info);
+    cudaError_t e = cudaMemsetAsync(cursor, 0, cursors + infob, stream);
+    if (e == cudaSuccess) {
+#define SP_ROWS_PARTITION(CT, PER)                                                                                        \
+    k_rows_partition<CT, PER><<<(unsigned)sp_ceil_div(n, kThreads * PER), kThreads, (size_t)nb * sizeof(uint32_t), stream>>>( \
+        static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, info)
+        const int per = n < SP_ROWS_T2 ? 2 : n < SP_ROWS_T8 ? 8 : 16;
+        if (coord_bits == 32) { if (per == 2) SP_ROWS_PARTITION(int32_t, 2); else if (per == 8) SP_ROWS_PARTITION(int32_t, 8); else SP_ROWS_PARTITION(int32_t, 16); }
+        else { if (per == 2) SP_ROWS_PARTITION(int64_t, 2); else if (per == 8) SP_ROWS_PARTITION(int64_t, 8); else SP_ROWS_PARTITION(int64_t, 16); }
+#undef SP_ROWS_PARTITION
         e = cudaGetLastError();
     }
-    SP_ROWS_LAUNCH(k_rows_sums, dim3((unsigned)rtiles), (const uint32_t*)count, no, tile, info);
+#define SP_ROWS_LAUNCH(kernel, smem, ...) \
+    (e = e != cudaSuccess ? e : sp_launch_dependent(kernel, dim3((unsigned)nb), dim3(kThreads), smem, stream, __VA_ARGS__))
+#define SP_ROWS_BUILD(DBL)                                                                                                \
+    do {                                                                                                                  \
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows_build<P, I, DBL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BuildShared)); \
+        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), (const Rec*)rec, (const uint32_t*)cursor, n, no, scale, nb, info, pos1, \
+                       crd1, t->val, seg_out, outer_list, outer_pos, outer_count);                                        \
+    } while (0)
     SP_DISPATCH_WIDTHS(t, {
         P* pos0 = static_cast<P*>(t->pos[0]);
         I* crd0 = static_cast<I*>(t->crd[0]);
         P* pos1 = static_cast<P*>(t->pos[1]);
-        if (dbl) SP_ROWS_LAUNCH((k_rows_offsets<P, I, true>), dim3((unsigned)rtiles), (const uint32_t*)count, no, (const uint2*)tile, n, most, start, first, pos0, crd0, pos1, nq, info);
-        else SP_ROWS_LAUNCH((k_rows_offsets<P, I, false>), dim3((unsigned)rtiles), (const uint32_t*)count, no, (const uint2*)tile, n, most, start, first, pos0, crd0, pos1, nq, info);
+        I* crd1 = static_cast<I*>(t->crd[1]);
+        if (dbl) {
+            SP_ROWS_BUILD(true);
+            SP_ROWS_LAUNCH((k_rows_outer<P, I>), 0, (const uint32_t*)outer_list, (const uint32_t*)outer_pos, (const uint32_t*)outer_count, n, no,
+                           scale, nb, info, pos0, crd0, pos1);
+        } else {
+            SP_ROWS_BUILD(false);
+        }
     });
-    if (coord_bits == 32)
-        SP_ROWS_LAUNCH(k_rows_scatter<int32_t>, tiles, static_cast<const int32_t*>(outer), static_cast<const int32_t*>(inner), vals, n,
-                       (const uint32_t*)rank, (const uint32_t*)start, no, most, info, rec);
-    else
-        SP_ROWS_LAUNCH(k_rows_scatter<int64_t>, tiles, static_cast<const int64_t*>(outer), static_cast<const int64_t*>(inner), vals, n,
-                       (const uint32_t*)rank, (const uint32_t*)start, no, most, info, rec);
-    if (crdBits == 32)
-        SP_ROWS_LAUNCH(k_rows_sort<uint32_t>, dim3((unsigned)stiles), (const Rec*)rec, (const uint32_t*)first, n, most, info,
-                       static_cast<uint32_t*>(t->crd[1]), t->val, seg_out);
-    else
-        SP_ROWS_LAUNCH(k_rows_sort<uint64_t>, dim3((unsigned)stiles), (const Rec*)rec, (const uint32_t*)first, n, most, info,
-                       static_cast<uint64_t*>(t->crd[1]), t->val, seg_out);
+#undef SP_ROWS_BUILD
 #undef SP_ROWS_LAUNCH
-    sp_count_launches(5);
-    unsigned long long back[3] = {};
+    sp_count_launches(dbl ? 3 : 2);
+    unsigned long long back[2] = {};
     if (e == cudaSuccess) e = cudaMemcpyAsync(back, info, sizeof back, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return fail(SP_ERR_CUDA);
-    if (back[0] & kErrIndex) return fail(SP_ERR_CUDA);
     if (back[0] & kErrRange) return fail(SP_ERR_OUT_OF_RANGE);
-    if (back[0] != 0 || back[2] > most) return fail(SP_ERR_UNSUPPORTED);
+    if (back[0] != 0) return fail(SP_ERR_UNSUPPORTED);
     t->npos[1] = (dbl ? (int64_t)back[1] : no) + 1;
     if (dbl) t->ncrd[0] = (int64_t)back[1];
     *out = t;

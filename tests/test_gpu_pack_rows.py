@@ -1,5 +1,5 @@
-"""Packing matrices with short segments: lengths at the edges of the tiles and of the range that is packed
-without a sort by key, and the inputs that have to fall back to it."""
+"""Packing matrices without a sort by key: segment lengths at the edges of buckets and tiles, and the inputs
+that have to take the radix path (a bucket that overflows, duplicates)."""
 import numpy as np
 import pytest
 
@@ -23,15 +23,17 @@ def _matrix(lens, n, seed, repeat=0):
 CASES = {
     "one_entry": ([1], 1, 0),
     "one_row": ([70], 90, 0),
-    "tile_edge": ([2047, 1, 2048, 0, 0, 1, 2047, 2], 2100, 0),      # segments that end on, before and after a tile's edge
-    "longest_taken": ([5, 2048, 7], 2100, 0),
-    "too_long": ([5, 2049, 7], 2100, 0),
-    "far_too_long": ([3, 20000, 3], 30000, 0),                      # counting gives up
+    "full_bucket": ([4096], 5000, 0),
+    "overfull_bucket": ([4097], 5000, 0),
+    "full_among_others": ([5, 4000, 7] + [0] * 1990, 5000, 0),
+    "far_too_long": ([3, 20000, 3], 30000, 0),
     "many_empty": ([0] * 5000 + [3] + [0] * 60000 + [1], 10, 0),
-    "empty_tiles": ([1] * 2048 + [0] * 4096 + [1] * 2049, 50, 0),
-    "words": ([31, 33, 32, 64, 1, 0, 65] * 40, 300, 0),
+    "empty_buckets": ([1] * 2048 + [0] * 4096 + [1] * 2049, 50, 0),
+    "bucket_edges": ([1, 2047, 2049, 0, 0, 1, 2047, 2, 2048] * 3, 2100, 0),
+    "long_rows": ([500] * 40 + [0, 1, 2] * 20 + [1500] * 20, 1600, 0),       # cut into bins
+    "many_tiles": ([30] * 20000, 60, 0),                                    # the larger tiles of entries
     "duplicates": ([20] * 300, 64, 17),
-    "squares_too_many": ([1500] * 100, 1600, 0),                    # within the longest segment, but too much counting
+    "duplicates_in_bins": ([300] * 30, 400, 2),
 }
 
 
@@ -56,3 +58,18 @@ def test_pack_rows(oracle, name, enc):
     with pytest.raises(sp().SpError) as e:
         sp().sp_pack(coo.dims, coords, vals, lt, od)
     assert e.value.code == 3
+
+
+def test_pack_rows_clustered_columns(oracle):
+    """Long rows whose columns lie close together, at both ends of a wide matrix."""
+    rng = np.random.default_rng(8)
+    n = (1 << 32) - 1                                                # the widest that 32-bit coordinates hold
+    rows = np.repeat(np.arange(12), 300)
+    near = np.where(rows % 2 == 0, 0, n - 400)
+    cols = np.concatenate([rng.choice(400, 300, replace=False) for _ in range(12)]) + near
+    cols[5] = n - 1                                                  # one far away: all others of its row in one bin
+    order = rng.permutation(rows.size)
+    coo = I.Coo((12, n), [rows[order].astype(np.int64), cols[order].astype(np.int64)], I.uniform_pm1(8, 5, rows.size))
+    coords, vals = to_dev(coo, 64)
+    for lt in ((0, 1), (1, 1)):
+        assert_storage_equal(sp().sp_pack(coo.dims, coords, vals, lt), oracle.pack(coo.dims, coo.coords, coo.vals, lt, (0, 1)))
