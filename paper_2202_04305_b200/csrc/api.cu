@@ -28,6 +28,24 @@ void sp_dev_free(void* p, cudaStream_t stream) {
     if (stream) cudaFreeAsync(p, stream); else cudaFree(p);
 }
 
+unsigned long long* sp_host_words() {
+    struct Words {
+        unsigned long long* p = nullptr;
+        ~Words() { if (p) cudaFreeHost(p); }
+    };
+    static thread_local Words w;
+    if (!w.p) {
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, kHostWords * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        w.p = static_cast<unsigned long long*>(p);
+    }
+    for (int i = 0; i < kHostWords; ++i) w.p[i] = 0;
+    return w.p;
+}
+
 sp_status sp_check_device(const sp_tensor* t) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return SP_ERR_CUDA;

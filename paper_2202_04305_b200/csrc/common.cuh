@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -111,7 +112,25 @@ struct sp_workspace {
     }
 };
 
+// A few words of pinned host memory of the calling thread, zeroed: the target of a call's read-back, or, being
+// mapped, of what its kernels report themselves.  Valid until the thread's next call that asks for them;
+// such calls wait for their stream before they return.  nullptr: no memory.  (A read-back into ordinary host
+// memory is staged by the runtime, 5 to 8 us more per call.)
+constexpr int kHostWords = 16;
+unsigned long long* sp_host_words();
+
 void sp_count_launches(int n);
+
+// Raises a kernel's dynamic shared-memory limit, once per device.
+template <auto Kernel>
+inline cudaError_t sp_allow_shared(int device, size_t bytes) {
+    static std::atomic<uint64_t> done{0};
+    const uint64_t bit = (uint64_t)1 << (device & 63);
+    if (device < 64 && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && device < 64) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
 
 // One NVTX range per API call (visible in Nsight Systems / Compute timelines; a no-op costing a
 // few nanoseconds when no tool is attached).

@@ -1049,10 +1049,12 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
         SP_LAUNCH_CHECK();
         timer.mark(kPhCount);
         sp_count_launches(3);
-        int64_t h_back[SP_MAX_RANK + 1] = {};          // one read-back: the counts and the error word
-        SP_CUDA(cudaMemcpyAsync(h_back, d_counts, sizeof h_back, cudaMemcpyDeviceToHost, stream));
+        unsigned long long* h_back = sp_host_words();  // one read-back: the counts and the error word
+        if (!h_back) return SP_ERR_ALLOC;
+        static_assert(SP_MAX_RANK + 1 <= kHostWords, "the read-back fits");
+        SP_CUDA(cudaMemcpyAsync(h_back, d_counts, (SP_MAX_RANK + 1) * sizeof *h_back, cudaMemcpyDeviceToHost, stream));
         SP_CUDA(cudaStreamSynchronize(stream));
-        for (int l = 0; l < SP_MAX_RANK; ++l) counts[l] = h_back[l];
+        for (int l = 0; l < SP_MAX_RANK; ++l) counts[l] = (int64_t)h_back[l];
         const int h_err = (int)(h_back[SP_MAX_RANK] & 0xffffffff);
         if (h_err & kErrRange) return SP_ERR_OUT_OF_RANGE;
         if ((flags & SP_DUP_ERROR) && counts[rank - 1] != n) return SP_ERR_DUPLICATE;

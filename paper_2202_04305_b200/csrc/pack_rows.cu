@@ -16,29 +16,25 @@
 
 #include <algorithm>
 
-#ifndef SP_ROWS_MINB
-#define SP_ROWS_MINB 3
-#endif
-#ifndef SP_ROWS_T2
-#define SP_ROWS_T2 300000
-#endif
-#ifndef SP_ROWS_T8
-#define SP_ROWS_T8 3000000
-#endif
-
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
+constexpr int kThreads = 512;                   // of k_rows_partition
+constexpr int kBThreads = 512;                  // of k_rows_build and k_rows_outer
+constexpr int kWarps = kBThreads / 32;
 constexpr int kCap = 4096;                      // entries a bucket can hold
-constexpr int kIpt = kCap / kThreads;           // ... per thread of k_rows_build
+constexpr int kIpt = kCap / kBThreads;          // ... per thread of k_rows_build
 constexpr int kAverage = 2048;                  // entries per bucket aimed at: rows of 48 +- 7 and power-law rows stay below twice that
 constexpr int kWidth = 2048;                    // outer indices of a bucket
 constexpr int kMaxBuckets = 4096;
 constexpr int kDense = 24;                      // mean compares per entry above which segments are cut into bins
 
-// What the device reports: word 0 = kErr* bits, 1 = non-empty outer indices.
-constexpr unsigned long long kErrRange = 1, kErrDup = 2, kErrLong = 4;
+// What the device reports, straight into the caller's pinned words: one word per event, then the number of
+// non-empty outer indices.  `stop` is the device's own copy: later blocks and kernels return once it is set.
+enum { kErrRange = 0, kErrDup, kErrLong, kOuterCount };
+__device__ __forceinline__ void report(int what, uint32_t* stop, unsigned long long* host) {
+    *static_cast<volatile unsigned long long*>(host + what) = 1;
+    *static_cast<volatile uint32_t*>(stop) = 1;
+}
 
 using Rec = uint4;                              // value (low, high word), inner coordinate, outer coordinate
 
@@ -49,8 +45,8 @@ __host__ __device__ __forceinline__ int64_t bucket_begin(int64_t b, uint32_t sca
 }
 
 // Whether some block has reported an error, the same answer for all threads of a block.
-__device__ __forceinline__ bool stopped(const unsigned long long* info) {
-    return __syncthreads_or(threadIdx.x == 0 && __ldcg(info) != 0) != 0;
+__device__ __forceinline__ bool stopped(const uint32_t* stop) {
+    return __syncthreads_or(threadIdx.x == 0 && __ldcg(stop) != 0) != 0;
 }
 
 // Exclusive scan over the block of one counter per thread.
@@ -76,7 +72,7 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* s_w, uint32
     return incl - v + pre;
 }
 
-// In-place exclusive scan of s[0 .. n), n <= PER * kThreads; s[n] = the total.
+// In-place exclusive scan of s[0 .. n), n <= PER * kBThreads; s[n] = the total.
 template <int PER>
 __device__ __forceinline__ void scan_shared(uint32_t* s, int n, uint32_t* s_w) {
     const int i0 = threadIdx.x * PER;
@@ -94,11 +90,11 @@ __device__ __forceinline__ void scan_shared(uint32_t* s, int n, uint32_t* s_w) {
 // A block sends a tile of kThreads * PER entries to their buckets: ranks inside the tile by shared-memory
 // atomics, the tile's place in every bucket by one atomic on the bucket's cursor.
 template <typename CT, int PER>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
-                 uint32_t scale, int nb, uint32_t* __restrict__ cursor, Rec* __restrict__ rec, unsigned long long* __restrict__ info) {
+                 uint32_t scale, int nb, uint32_t* __restrict__ cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
     extern __shared__ uint32_t s_hist[];
-    if (stopped(info)) return;
+    if (stopped(stop)) return;
     const int t = threadIdx.x;
     for (int b = t; b < nb; b += kThreads) s_hist[b] = 0u;
     __syncthreads();
@@ -118,20 +114,27 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
         r[i] = base + i * kThreads < n ? atomicAdd(&s_hist[__umulhi((uint32_t)o[i], scale)], 1u) : 0u;
     }
     if (__syncthreads_or(bad)) {
-        if (t == 0) atomicOr(info, kErrRange);
+        if (t == 0) report(kErrRange, stop, host);
         return;
     }
-    bool full = false;
-    for (int b = t; b < nb; b += kThreads) {
-        const uint32_t k = s_hist[b];
-        if (k) {
-            const uint32_t at = atomicAdd(cursor + b, k);
-            full |= at + k > (uint32_t)kCap;
-            s_hist[b] = at;
-        }
+    // all cursors of a thread at once: one wait, not one per bucket
+    constexpr int kPerB = kMaxBuckets / kThreads;
+    uint32_t k[kPerB], at[kPerB];
+#pragma unroll
+    for (int q = 0; q < kPerB; ++q) {
+        const int b = t + q * kThreads;
+        k[q] = b < nb ? s_hist[b] : 0u;
+        at[q] = k[q] ? atomicAdd(cursor + b, k[q]) : 0u;
     }
+    bool full = false;
+#pragma unroll
+    for (int q = 0; q < kPerB; ++q)
+        if (k[q]) {
+            full |= at[q] + k[q] > (uint32_t)kCap;
+            s_hist[t + q * kThreads] = at[q];
+        }
     if (__syncthreads_or(full)) {
-        if (t == 0) atomicOr(info, kErrLong);
+        if (t == 0) report(kErrLong, stop, host);
         return;
     }
 #pragma unroll
@@ -165,12 +168,12 @@ static_assert(kWidth * 2 >= kCap, "the starts' space holds a 16-bit number per e
 // cut into as many bins as they have entries, evenly between their smallest and largest coordinate, and only
 // the entries of one bin are compared.
 template <typename P, typename I, bool DBL>
-__global__ void __launch_bounds__(kThreads, SP_ROWS_MINB)
-k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int nb, unsigned long long* __restrict__ info,
+__global__ void __launch_bounds__(kBThreads, 2)
+k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int nb, uint32_t* stop, unsigned long long* host,
              P* __restrict__ pos1, I* __restrict__ crd, double* __restrict__ val, uint32_t* __restrict__ seg_out,
              uint32_t* __restrict__ outer_list, uint32_t* __restrict__ outer_pos, uint32_t* __restrict__ outer_count) {
     sp_wait_for_previous_kernel();
-    if (stopped(info)) return;
+    if (stopped(stop)) return;
     extern __shared__ __align__(16) unsigned char s_raw[];
     BuildShared& s = *reinterpret_cast<BuildShared*>(s_raw);
     const int t = threadIdx.x, b = blockIdx.x;
@@ -183,19 +186,19 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
 #pragma unroll
     for (int i = 0; i < kIpt; ++i) {
         c[i] = qr[i] = 0u;
-        if (i * kThreads + t < cnt) { const Rec x = mine[i * kThreads]; c[i] = x.z; qr[i] = x.w - (uint32_t)lo; }
+        if (i * kBThreads + t < cnt) { const Rec x = mine[i * kBThreads]; c[i] = x.z; qr[i] = x.w - (uint32_t)lo; }
     }
     uint32_t before = 0, base;
-    for (int q = t; q < b; q += kThreads) before += cursor[q];
-    for (int q = t; q < width; q += kThreads) { s.count[q] = 0u; s.lo[q] = ~0u; s.hi[q] = 0u; }
+    for (int q = t; q < b; q += kBThreads) before += cursor[q];
+    for (int q = t; q < width; q += kBThreads) { s.count[q] = 0u; s.lo[q] = ~0u; s.hi[q] = 0u; }
     block_scan(before, s.w, &base);             // (also the barrier after the zeroing)
 #pragma unroll
     for (int i = 0; i < kIpt; ++i)
-        if (i * kThreads + t < cnt) qr[i] = qr[i] << 16 | atomicAdd(&s.count[qr[i]], 1u);
+        if (i * kBThreads + t < cnt) qr[i] = qr[i] << 16 | atomicAdd(&s.count[qr[i]], 1u);
     __syncthreads();
     // mean number of compares without bins; outer level
     uint32_t sq = 0, filled = 0, tot_sq, tot_filled;
-    constexpr int kPerW = kWidth / kThreads;
+    constexpr int kPerW = kWidth / kBThreads;
 #pragma unroll
     for (int i = 0; i < kPerW; ++i) {
         const int q = t * kPerW + i;
@@ -225,45 +228,46 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
             if (len[i]) { outer_pos[lo + at_filled + k] = base + s.count[t * kPerW + i]; ++k; }
     } else {
         scan_shared<kPerW>(s.count, width, s.w);
-        for (int q = t; q < width; q += kThreads) pos1[lo + q] = (P)(base + s.count[q]);
+        for (int q = t; q < width; q += kBThreads) pos1[lo + q] = (P)(base + s.count[q]);
         if (b == nb - 1 && t == 0) pos1[no] = (P)n;
     }
-    // place of coordinate c among s.crd[j .. e)
-    bool dup = false;
+    // place of coordinate c among s.crd[j .. e), and the sum of the thread's places
+    uint32_t sum = 0;
     auto place_of = [&](int j, int e, uint32_t cc) {
-        int at = j, same = 0;
-        for (; j < e; ++j) {
-            const uint32_t cj = s.crd[j];
-            at += cj < cc;
-            same += cj == cc;
+        uint32_t at = (uint32_t)j;
+        for (; j + 1 < e; j += 2) {
+            const uint32_t c0 = s.crd[j], c1 = s.crd[j + 1];
+            at += c0 < cc;
+            at += c1 < cc;
         }
-        dup |= same > 1;
+        if (j < e) at += s.crd[j] < cc;
+        sum += at;
         return at;
     };
     uint32_t to[kIpt];                          // outer offset << 16 | place
     if (!bins) {
 #pragma unroll
         for (int i = 0; i < kIpt; ++i)
-            if (i * kThreads + t < cnt) s.crd[s.count[qr[i] >> 16] + (qr[i] & 0xffffu)] = c[i];
+            if (i * kBThreads + t < cnt) s.crd[s.count[qr[i] >> 16] + (qr[i] & 0xffffu)] = c[i];
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kIpt; ++i)
-            if (i * kThreads + t < cnt) {
+            if (i * kBThreads + t < cnt) {
                 const uint32_t q = qr[i] >> 16;
-                to[i] = q << 16 | (uint32_t)place_of((int)s.count[q], (int)s.count[q + 1], c[i]);
+                to[i] = q << 16 | place_of((int)s.count[q], (int)s.count[q + 1], c[i]);
             }
     } else {
 #pragma unroll
         for (int i = 0; i < kIpt; ++i)
-            if (i * kThreads + t < cnt) {
+            if (i * kBThreads + t < cnt) {
                 atomicMin(&s.lo[qr[i] >> 16], c[i]);
                 atomicMax(&s.hi[qr[i] >> 16], c[i]);
             }
-        for (int j = t; j < cnt; j += kThreads) s.bin[j] = 0u;
+        for (int j = t; j < cnt; j += kBThreads) s.bin[j] = 0u;
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kIpt; ++i)
-            if (i * kThreads + t < cnt) {
+            if (i * kBThreads + t < cnt) {
                 const uint32_t q = qr[i] >> 16, first = s.count[q], len = s.count[q + 1] - first, c0 = s.lo[q];
                 // not decreasing in the coordinate: the factor is the segment's, and rounding keeps the order
                 const uint32_t k = (uint32_t)((float)(c[i] - c0) * ((float)len / ((float)(s.hi[q] - c0) + 1.0f)));
@@ -274,32 +278,34 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
         scan_shared<kIpt>(s.bin, cnt, s.w);     // the total lands in bin[cnt], which is bin_end for a full bucket
 #pragma unroll
         for (int i = 0; i < kIpt; ++i)
-            if (i * kThreads + t < cnt) s.crd[s.bin[to[i] >> 16] + (to[i] & 0xffffu)] = c[i];
+            if (i * kBThreads + t < cnt) s.crd[s.bin[to[i] >> 16] + (to[i] & 0xffffu)] = c[i];
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kIpt; ++i)
-            if (i * kThreads + t < cnt) {
+            if (i * kBThreads + t < cnt) {
                 const uint32_t g = to[i] >> 16;
-                to[i] = (qr[i] & 0xffff0000u) | (uint32_t)place_of((int)s.bin[g], (int)s.bin[g + 1], c[i]);
+                to[i] = (qr[i] & 0xffff0000u) | place_of((int)s.bin[g], (int)s.bin[g + 1], c[i]);
             }
     }
-    if (__syncthreads_or(dup)) {
-        if (t == 0) atomicOr(info, kErrDup);
+    // Distinct coordinates take the places 0 .. cnt - 1; of equal ones all get the lowest, so the sum falls short.
+    uint32_t tot_sum;
+    block_scan(sum, s.w, &tot_sum);             // also the barrier after which coordinates, starts and bins are dead
+    if (tot_sum != (uint32_t)(cnt * (cnt - 1) / 2)) {
+        if (t == 0) report(kErrDup, stop, host);
         return;
     }
-    // everyone has read the coordinates, starts and bins: their space takes the sorted bucket
     uint16_t* s_seg = reinterpret_cast<uint16_t*>(s.count);
 #pragma unroll
     for (int i = 0; i < kIpt; ++i)
-        if (i * kThreads + t < cnt) {
-            const uint2 v = *reinterpret_cast<const uint2*>(mine + i * kThreads);
+        if (i * kBThreads + t < cnt) {
+            const uint2 v = *reinterpret_cast<const uint2*>(mine + i * kBThreads);
             const uint32_t p = to[i] & 0xffffu;
             s.crd[p] = c[i];
             s.val[p] = __hiloint2double((int)v.y, (int)v.x);
             if (seg_out) s_seg[p] = (uint16_t)(to[i] >> 16);
         }
     __syncthreads();
-    for (int j = t; j < cnt; j += kThreads) {
+    for (int j = t; j < cnt; j += kBThreads) {
         crd[base + j] = (I)s.crd[j];
         val[base + j] = s.val[j];
         if (seg_out) seg_out[base + j] = (uint32_t)lo + s_seg[j];
@@ -308,19 +314,19 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
 
 // Joins the buckets' lists of non-empty outer indices and of their first entries: crd[0] and pos[1].
 template <typename P, typename I>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kBThreads)
 k_rows_outer(const uint32_t* outer_list, const uint32_t* outer_pos, const uint32_t* outer_count, int64_t n, int64_t no, uint32_t scale, int nb,
-             unsigned long long* __restrict__ info, P* __restrict__ pos0, I* __restrict__ crd0, P* __restrict__ pos1) {
+             uint32_t* stop, unsigned long long* host, P* __restrict__ pos0, I* __restrict__ crd0, P* __restrict__ pos1) {
     sp_wait_for_previous_kernel();
-    if (stopped(info)) return;
+    if (stopped(stop)) return;
     __shared__ uint32_t s_w[kWarps];
     const int t = threadIdx.x, b = blockIdx.x;
     uint32_t before = 0, base;
-    for (int q = t; q < b; q += kThreads) before += outer_count[q];
+    for (int q = t; q < b; q += kBThreads) before += outer_count[q];
     block_scan(before, s_w, &base);
     const int64_t lo = bucket_begin(b, scale, no);
     const uint32_t cnt = outer_count[b];
-    for (uint32_t q = t; q < cnt; q += kThreads) {
+    for (uint32_t q = t; q < cnt; q += kBThreads) {
         crd0[base + q] = (I)outer_list[lo + q];
         pos1[base + q] = (P)outer_pos[lo + q];
     }
@@ -328,7 +334,7 @@ k_rows_outer(const uint32_t* outer_list, const uint32_t* outer_pos, const uint32
         pos1[base + cnt] = (P)n;
         pos0[0] = 0;
         pos0[1] = (P)(base + cnt);
-        info[1] = base + cnt;
+        *static_cast<volatile unsigned long long*>(host + kOuterCount) = base + cnt;
     }
 }
 
@@ -354,16 +360,17 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     const bool dbl = lt[0] == SP_COMPRESSED;
     const size_t pw = posBits / 8, cw = crdBits / 8;
     sp_workspace ws(stream);
-    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb), infob = sp_workspace::bytes_for<unsigned long long>(2);
-    ws.reserve(cursors + infob + sp_workspace::bytes_for<Rec>((size_t)nb * kCap) +
+    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb + 1);
+    ws.reserve(cursors + sp_workspace::bytes_for<Rec>((size_t)nb * kCap) +
                (dbl ? 2 * sp_workspace::bytes_for<uint32_t>((size_t)no) + cursors : 0));
-    uint32_t* cursor = ws.get<uint32_t>((size_t)nb);
-    unsigned long long* info = ws.get<unsigned long long>(2);
+    uint32_t* cursor = ws.get<uint32_t>((size_t)nb + 1);
     Rec* rec = ws.get<Rec>((size_t)nb * kCap);
     uint32_t* outer_list = dbl ? ws.get<uint32_t>((size_t)no) : nullptr;
     uint32_t* outer_pos = dbl ? ws.get<uint32_t>((size_t)no) : nullptr;
-    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb) : nullptr;
-    if (ws.failed) return SP_ERR_ALLOC;
+    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb + 1) : nullptr;
+    unsigned long long* host = sp_host_words();
+    if (ws.failed || !host) return SP_ERR_ALLOC;
+    uint32_t* stop = cursor + nb;
 
     sp_tensor* t = new sp_tensor();
     auto fail = [&](sp_status s) { sp_free(t); return s; };
@@ -394,23 +401,24 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         t->parts[(uint64_t)SP_PART_SEGIDS << 56] = sg;
     }
 
-    cudaError_t e = cudaMemsetAsync(cursor, 0, cursors + infob, stream);
+    cudaError_t e = cudaMemsetAsync(cursor, 0, (size_t)(nb + 1) * sizeof(uint32_t), stream);
     if (e == cudaSuccess) {
 #define SP_ROWS_PARTITION(CT, PER)                                                                                        \
     k_rows_partition<CT, PER><<<(unsigned)sp_ceil_div(n, kThreads * PER), kThreads, (size_t)nb * sizeof(uint32_t), stream>>>( \
-        static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, info)
-        const int per = n < SP_ROWS_T2 ? 2 : n < SP_ROWS_T8 ? 8 : 16;
-        if (coord_bits == 32) { if (per == 2) SP_ROWS_PARTITION(int32_t, 2); else if (per == 8) SP_ROWS_PARTITION(int32_t, 8); else SP_ROWS_PARTITION(int32_t, 16); }
-        else { if (per == 2) SP_ROWS_PARTITION(int64_t, 2); else if (per == 8) SP_ROWS_PARTITION(int64_t, 8); else SP_ROWS_PARTITION(int64_t, 16); }
+        static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, stop, host)
+        // small inputs need the blocks, large ones the fewer cursor updates (5 M entries: 8 per thread 215 us, 2 252, 16 270)
+        const bool small = n < 300000;
+        if (coord_bits == 32) { if (small) SP_ROWS_PARTITION(int32_t, 2); else SP_ROWS_PARTITION(int32_t, 8); }
+        else { if (small) SP_ROWS_PARTITION(int64_t, 2); else SP_ROWS_PARTITION(int64_t, 8); }
 #undef SP_ROWS_PARTITION
         e = cudaGetLastError();
     }
 #define SP_ROWS_LAUNCH(kernel, smem, ...) \
-    (e = e != cudaSuccess ? e : sp_launch_dependent(kernel, dim3((unsigned)nb), dim3(kThreads), smem, stream, __VA_ARGS__))
+    (e = e != cudaSuccess ? e : sp_launch_dependent(kernel, dim3((unsigned)nb), dim3(kBThreads), smem, stream, __VA_ARGS__))
 #define SP_ROWS_BUILD(DBL)                                                                                                \
     do {                                                                                                                  \
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k_rows_build<P, I, DBL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BuildShared)); \
-        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), (const Rec*)rec, (const uint32_t*)cursor, n, no, scale, nb, info, pos1, \
+        if (e == cudaSuccess) e = sp_allow_shared<k_rows_build<P, I, DBL>>(t->device, sizeof(BuildShared));             \
+        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), (const Rec*)rec, (const uint32_t*)cursor, n, no, scale, nb, stop, host, pos1, \
                        crd1, t->val, seg_out, outer_list, outer_pos, outer_count);                                        \
     } while (0)
     SP_DISPATCH_WIDTHS(t, {
@@ -421,7 +429,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         if (dbl) {
             SP_ROWS_BUILD(true);
             SP_ROWS_LAUNCH((k_rows_outer<P, I>), 0, (const uint32_t*)outer_list, (const uint32_t*)outer_pos, (const uint32_t*)outer_count, n, no,
-                           scale, nb, info, pos0, crd0, pos1);
+                           scale, nb, stop, host, pos0, crd0, pos1);
         } else {
             SP_ROWS_BUILD(false);
         }
@@ -429,14 +437,12 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
 #undef SP_ROWS_BUILD
 #undef SP_ROWS_LAUNCH
     sp_count_launches(dbl ? 3 : 2);
-    unsigned long long back[2] = {};
-    if (e == cudaSuccess) e = cudaMemcpyAsync(back, info, sizeof back, cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return fail(SP_ERR_CUDA);
-    if (back[0] & kErrRange) return fail(SP_ERR_OUT_OF_RANGE);
-    if (back[0] != 0) return fail(SP_ERR_UNSUPPORTED);
-    t->npos[1] = (dbl ? (int64_t)back[1] : no) + 1;
-    if (dbl) t->ncrd[0] = (int64_t)back[1];
+    if (host[kErrRange]) return fail(SP_ERR_OUT_OF_RANGE);
+    if (host[kErrDup] || host[kErrLong]) return fail(SP_ERR_UNSUPPORTED);
+    t->npos[1] = (dbl ? (int64_t)host[kOuterCount] : no) + 1;
+    if (dbl) t->ncrd[0] = (int64_t)host[kOuterCount];
     *out = t;
     return SP_OK;
 }

@@ -94,10 +94,11 @@ sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out) {
     else k_max_segment<uint64_t><<<blocks, 256, 0, stream>>>(static_cast<const uint64_t*>(t->pos[last]), nseg, d);
     SP_LAUNCH_CHECK();
     sp_count_launches(1);
-    unsigned long long h = 0;
-    SP_CUDA(cudaMemcpyAsync(&h, d, sizeof h, cudaMemcpyDeviceToHost, stream));
+    unsigned long long* h = sp_host_words();
+    if (!h) return SP_ERR_ALLOC;
+    SP_CUDA(cudaMemcpyAsync(h, d, sizeof *h, cudaMemcpyDeviceToHost, stream));
     SP_CUDA(cudaStreamSynchronize(stream));
-    t->max_seg = (int64_t)h;
+    t->max_seg = (int64_t)*h;
     *out = t->max_seg;
     return SP_OK;
 }

@@ -247,10 +247,12 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     k_row_offsets<<<1, kPThreads, 0, stream>>>(rowlen, m, C->pos[1], posBits, d_count);
     if (cudaGetLastError() != cudaSuccess) return fail(SP_ERR_CUDA);
     sp_count_launches(2);
-    int64_t count = 0;
-    if (cudaMemcpyAsync(&count, d_count, sizeof count, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+    unsigned long long* h_count = sp_host_words();
+    if (!h_count) return fail(SP_ERR_ALLOC);
+    if (cudaMemcpyAsync(h_count, d_count, sizeof *h_count, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)
         return fail(SP_ERR_CUDA);
+    const int64_t count = (int64_t)*h_count;
     if ((uint64_t)count > sp_width_max(posBits)) return fail(SP_ERR_WIDTH_OVERFLOW);
     C->ncrd[1] = count;
     C->nval = count;
