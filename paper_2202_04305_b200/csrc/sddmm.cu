@@ -6,19 +6,14 @@
 // j = crd[1][p]; x[p] = S.val[p] * dot(A[i,:], B[:,j]).  B is given K x n row-major,
 // so a column is K elements a whole row apart; it is transposed once per call into
 // a workspace so each entry reads one contiguous K-vector.  The (row end, entry)
-// merge path is cut into equal pieces, one per warp; a warp keeps A[i,:] in
-// registers across the entries of a row and reduces each dot product with shuffles.
+// merge path is cut into equal pieces, one per lane group (k_sddmm_group).
 #include "common.cuh"
 
 namespace {
 
-// Warps share nothing, so blocks are kept small (two warps): 0.328 ms on the 2,000,000-entry sample against
-// 0.331 ms with four warps and 0.337 ms with eight.
-#ifndef SP_SDDMM_THREADS
-#define SP_SDDMM_THREADS 64
-#endif
-constexpr int kSThreads = SP_SDDMM_THREADS;
+constexpr int kSThreads = 64;
 constexpr int kSItems = 64;   // merge items per warp
+constexpr int kGThreads = 64;  // of k_sddmm_group (32: the same; 128: 265 us against 262)
 
 __global__ void __launch_bounds__(256)
 k_transpose(const double* __restrict__ B, int64_t ldb, int64_t K, int64_t n, double* __restrict__ Bt, int64_t ldt) {
@@ -34,22 +29,19 @@ k_transpose(const double* __restrict__ B, int64_t ldb, int64_t K, int64_t n, dou
 #pragma unroll
     for (int r = ty; r < 32; r += 8) {
         int64_t j = j0 + r, k = k0 + tx;
-        if (j < n && k < K) Bt[j * ldt + k] = tile[tx][r];
+        if (j < n && k < ldt) Bt[j * ldt + k] = tile[tx][r];      // zeros from K up to ldt
     }
 }
 
 template <int V>
 __device__ __forceinline__ void ld2(const double* p, double* a) {
-    if (V == 4) {           // one 32-byte load (p is 32-byte aligned)
-        asm volatile("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-                     : "=d"(a[0]), "=d"(a[V > 1 ? 1 : 0]), "=d"(a[V > 2 ? 2 : 0]), "=d"(a[V > 3 ? 3 : 0]) : "l"(p));
-    } else if (V == 2) { double2 q = *reinterpret_cast<const double2*>(p); a[0] = q.x; a[V - 1] = q.y; }
+    if (V == 2) { const double2 q = *reinterpret_cast<const double2*>(p); a[0] = q.x; a[V - 1] = q.y; }
     else a[0] = *p;
 }
 
-// NCH > 0: A[i,:] lives in NCH register chunks of 32*V columns (K <= NCH*32*V).
-// NCH == 0: any K, A is re-read (from L1) for every entry.
-template <typename P, typename I, int V, int NCH>
+// K > 512: a warp per merge-path piece, one dot product at a time; the operand row is re-read (from L1) for
+// every entry.
+template <typename P, typename I, int V>
 __global__ void __launch_bounds__(kSThreads)
 k_sddmm(const P* __restrict__ pos, const I* __restrict__ crd, const double* __restrict__ sval,
         const I* __restrict__ outer, const double* A, int64_t lda, const double* Bt,
@@ -62,10 +54,6 @@ k_sddmm(const P* __restrict__ pos, const I* __restrict__ crd, const double* __re
     const int lane = threadIdx.x & 31;
     const int64_t i0 = prow[w], j0 = pnz[w], i1 = prow[w + 1], j1 = pnz[w + 1];
     if (j1 == j0) return;
-
-    constexpr int NA = NCH > 0 ? NCH : 1;
-    double a[NA][V];
-    bool a_ready = false;
     int64_t row = i0, p = j0, rbase = i0, nzbase = j0;
     int64_t E = (rbase + lane < i1) ? (int64_t)pos[rbase + lane + 1] : j1;
     I c_l = (nzbase + lane < j1) ? crd[nzbase + lane] : (I)0;
@@ -74,20 +62,7 @@ k_sddmm(const P* __restrict__ pos, const I* __restrict__ crd, const double* __re
 
     while (true) {
         const int64_t rend = row < i1 ? __shfl_sync(0xffffffffu, E, (int)(row - rbase)) : j1;
-        const double* arow = nullptr;
-        if (p < rend) {
-            arow = A + SP_IDX(outer ? (int64_t)outer[row] : row, na) * lda;
-            if (NCH > 0 && !a_ready) {
-#pragma unroll
-                for (int ch = 0; ch < NA; ++ch) {
-                    const int64_t kk = (int64_t)ch * 32 * V + lane * V;
-#pragma unroll
-                    for (int q = 0; q < V; ++q) a[ch][q] = 0.0;
-                    if (kk < K) ld2<V>(arow + kk, a[ch]);
-                }
-                a_ready = true;
-            }
-        }
+        const double* arow = p < rend ? A + SP_IDX(outer ? (int64_t)outer[row] : row, na) * lda : nullptr;
         while (p < rend) {
             int off = (int)(p - nzbase);
             if (off == 32) {
@@ -98,73 +73,166 @@ k_sddmm(const P* __restrict__ pos, const I* __restrict__ crd, const double* __re
                 off = 0;
             }
             const int cnt = (int)min(rend - p, (int64_t)(32 - off));
-#ifndef SP_SDDMM_BATCH
-#define SP_SDDMM_BATCH 2
-#endif
-            if (NCH > 0) {
-                // kB entries at a time: all their operand loads are requested before the first of the
-                // (dependent) warp reductions starts; a batch's tail repeats its last entry
-                constexpr int kB = SP_SDDMM_BATCH;
-                for (int t = 0; t < cnt; t += kB) {
-                    double b[kB][NA][V];
+            for (int t = 0; t < cnt; ++t) {
+                const int64_t j = SP_IDX(__shfl_sync(0xffffffffu, c_l, off + t), nb);
+                const double* brow = Bt + j * ldt;
+                double part = 0.0;
+                for (int64_t kk = (int64_t)lane * V; kk < K; kk += 32 * V) {
+                    double b[V], aa[V];
+                    ld2<V>(brow + kk, b);
+                    ld2<V>(arow + kk, aa);
 #pragma unroll
-                    for (int u = 0; u < kB; ++u) {
-                        const int tt = t + u < cnt ? t + u : cnt - 1;
-                        const int64_t j = SP_IDX(__shfl_sync(0xffffffffu, c_l, off + tt), nb);
-                        const double* brow = Bt + j * ldt;
-#pragma unroll
-                        for (int ch = 0; ch < NA; ++ch) {
-                            const int64_t kk = (int64_t)ch * 32 * V + lane * V;
-#pragma unroll
-                            for (int q = 0; q < V; ++q) b[u][ch][q] = 0.0;
-                            if (kk < K) ld2<V>(brow + kk, b[u][ch]);
-                        }
-                    }
-                    double part[kB];
-#pragma unroll
-                    for (int u = 0; u < kB; ++u) {
-                        part[u] = 0.0;
-#pragma unroll
-                        for (int ch = 0; ch < NA; ++ch)
-#pragma unroll
-                            for (int q = 0; q < V; ++q) part[u] = fma(a[ch][q], b[u][ch][q], part[u]);
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                        for (int u = 0; u < kB; ++u) part[u] += __shfl_xor_sync(0xffffffffu, part[u], o);
-#pragma unroll
-                    for (int u = 0; u < kB; ++u)
-                        if (t + u < cnt && lane == off + t + u) res = part[u];
+                    for (int q = 0; q < V; ++q) part = fma(aa[q], b[q], part);
                 }
-            } else {
-                for (int t = 0; t < cnt; ++t) {
-                    const int64_t j = SP_IDX(__shfl_sync(0xffffffffu, c_l, off + t), nb);
-                    const double* brow = Bt + j * ldt;
-                    double part = 0.0;
-                    for (int64_t kk = (int64_t)lane * V; kk < K; kk += 32 * V) {
-                        double b[V], aa[V];
-                        ld2<V>(brow + kk, b);
-                        ld2<V>(arow + kk, aa);
 #pragma unroll
-                        for (int q = 0; q < V; ++q) part = fma(aa[q], b[q], part);
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-                    if (lane == off + t) res = part;
-                }
+                for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+                if (lane == off + t) res = part;
             }
             p += cnt;
         }
         if (row >= i1) break;
         ++row;
-        a_ready = false;
         if (row - rbase == 32) {
             rbase += 32;
             E = (rbase + lane < i1) ? (int64_t)pos[rbase + lane + 1] : j1;
         }
     }
     if (nzbase + lane < j1) xv[nzbase + lane] = v_l * res;
+}
+
+// K <= 512: a group of L lanes owns a merge-path piece and V factors a lane (K <= L * V), W of them adjacent.  The
+// operand row of the piece's current row sits in registers; the gathered rows of the next kDepth entries
+// are on their way into shared memory by asynchronous copies, every lane into slots of its own (nobody else
+// reads them, so nothing is synchronised and nothing in flight holds a register).  The dot products of
+// kDepth entries are folded over the group together, each exchange halving the number of sums a lane
+// carries, and the groups of a warp share the loop's instructions.
+// 2,000,000 samples, K = 128, operands of 134 MB: 262 us with the transpose, 304 us when a warp took one dot
+// product at a time; L = 8, 16, 32: 290, 262, 270 (fewer lanes, fewer copies of the loop in flight; more,
+// more instructions).  Bound: HBM, since the gathered operand does not fit L2 (1.1 GB for 0.3 GB of
+// operands; 64 % of the HBM rate).  Operand rows kept in registers and loaded ahead cost 190 and more
+// registers (342 us); requested through the ring as well, twice the shared memory (273 us).
+constexpr int kDepth = 4;
+
+template <int W>
+__device__ __forceinline__ void copy_async(double* dst, const double* src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (W == 2) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
+template <typename P, typename I, int L, int V, int W, bool FULL>
+__global__ void __launch_bounds__(kGThreads)
+k_sddmm_group(const P* __restrict__ pos, const I* __restrict__ crd, const double* __restrict__ sval,
+              const I* __restrict__ outer, const double* A, int64_t lda, int avec, const double* G, int64_t ldg, int K,
+              double* __restrict__ xv, const int64_t* __restrict__ prow, const int64_t* __restrict__ pnz, int64_t nchunks,
+              int64_t nseg, int64_t na, int64_t nb) {
+    // na, nb: rows of A and of G (used by the bounds-checking debug build only)
+    sp_wait_for_previous_kernel();                  // the transpose that wrote one of the operands
+    extern __shared__ __align__(16) double s_ring[];            // [kDepth][V / W][threads] runs of W
+    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / L;
+    if (w >= nchunks) return;                       // shuffles below stay inside a group
+    const int gl = threadIdx.x % L;
+    const unsigned gmask = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u) << (sp_lane() / L * L);
+    const int64_t i0 = prow[w], j0 = pnz[w];
+    const int nrows = (int)(prow[w + 1] - i0), nz = (int)(pnz[w + 1] - j0);
+    if (nz == 0) return;
+    const P* ends = pos + i0 + 1;                   // row r of the piece ends at entry ends[r]; the open row at nz
+    const I* cl = crd + j0;
+    const double* vl = sval + j0;
+    double* xl = xv + j0;
+    double* slot = s_ring + threadIdx.x * W;
+    int koff[V / W];
+    bool on[V / W];
+#pragma unroll
+    for (int j = 0; j < V / W; ++j) {
+        const int k = (j * L + gl) * W;
+        on[j] = FULL || k < K;
+        koff[j] = on[j] ? k : 0;
+    }
+    auto request = [&](int u, I k) {                // entry's row of G into ring position u
+        const double* row = G + (int64_t)SP_IDX(k, nb) * ldg;
+#pragma unroll
+        for (int j = 0; j < V / W; ++j)
+            if (on[j]) copy_async<W>(slot + (u * (V / W) + j) * (kGThreads * W), row + koff[j]);
+    };
+    double a[V];
+    auto load_row = [&](int r) {
+        const double* arow = A + SP_IDX(outer ? (int64_t)outer[i0 + r] : i0 + r, na) * lda;
+#pragma unroll
+        for (int j = 0; j < V / W; ++j) {
+            if (W == 2 && avec) {
+                const double2 x = *reinterpret_cast<const double2*>(arow + koff[j]);
+                a[j * W] = on[j] ? x.x : 0.0;
+                a[j * W + W - 1] = on[j] ? x.y : 0.0;
+            } else {
+#pragma unroll
+                for (int q = 0; q < W; ++q) a[j * W + q] = on[j] && koff[j] + q < K ? arow[koff[j] + q] : 0.0;
+            }
+        }
+    };
+    auto end_of = [&](int r) { return r < nrows ? (int)((int64_t)ends[r] - j0) : nz; };
+    int row = 0, rend = end_of(0);
+    while (rend == 0) rend = end_of(++row);         // rows without entries; nz > 0 ends this
+    I kn[kDepth];
+#pragma unroll
+    for (int u = 0; u < kDepth; ++u) {
+        if (u < nz) request(u, cl[u]);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    load_row(row);
+#pragma unroll
+    for (int u = 0; u < kDepth; ++u) kn[u] = cl[kDepth + u < nz ? kDepth + u : nz - 1];
+    constexpr int kSpan = L / kDepth < 1 ? 1 : L / kDepth;      // lanes that end up with the same entry's sum
+    const int mine = gl / kSpan;
+    for (int p = 0; p < nz; p += kDepth) {
+        const bool writer = gl % kSpan == 0 && p + mine < nz;
+        const double sv = writer ? vl[p + mine] : 0.0;
+        double part[kDepth];
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kDepth - 1) : "memory");
+            part[u] = 0.0;
+            if (p + u < nz) {
+                if (p + u == rend) {                // the next row with entries
+                    do rend = end_of(++row); while (rend == p + u);
+                    load_row(row);
+                }
+#pragma unroll
+                for (int j = 0; j < V / W; ++j) {
+                    const double* x = slot + (u * (V / W) + j) * (kGThreads * W);
+                    if (W == 2) {
+                        double2 t = *reinterpret_cast<const double2*>(x);
+                        if (!FULL && !on[j]) t = make_double2(0.0, 0.0);
+                        part[u] = fma(a[j * W], t.x, part[u]);
+                        part[u] = fma(a[j * W + W - 1], t.y, part[u]);
+                    } else if (FULL || on[j]) {
+                        part[u] = fma(a[j], *x, part[u]);
+                    }
+                }
+                if (p + kDepth + u < nz) request(u, kn[u]);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        }
+#pragma unroll
+        for (int u = 0; u < kDepth; ++u) kn[u] = cl[p + 2 * kDepth + u < nz ? p + 2 * kDepth + u : nz - 1];
+        int o = L / 2;
+        {
+            const bool h = gl & o;
+            const double s0 = __shfl_xor_sync(gmask, h ? part[0] : part[2], o), s1 = __shfl_xor_sync(gmask, h ? part[1] : part[3], o);
+            part[0] = (h ? part[2] : part[0]) + s0;
+            part[1] = (h ? part[3] : part[1]) + s1;
+            o >>= 1;
+        }
+        {
+            const bool h = gl & o;
+            const double s0 = __shfl_xor_sync(gmask, h ? part[0] : part[1], o);
+            part[0] = (h ? part[1] : part[0]) + s0;
+            o >>= 1;
+        }
+#pragma unroll
+        for (; o > 0; o >>= 1) part[0] += __shfl_xor_sync(gmask, part[0], o);
+        if (writer) xl[p + mine] = sv * part[0];
+    }
 }
 
 // S with a dense inner level ((dense|compressed, dense), either ordering): every cell of a stored
@@ -265,6 +333,67 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
     if (!x_vals) return SP_ERR_INVALID_ARG;
     const bool dbl = S->lt[0] == SP_COMPRESSED;
 
+    const bool pair_a = K % 2 == 0 && lda % 2 == 0 && reinterpret_cast<uintptr_t>(A) % 16 == 0;
+    if (K <= 512) {
+        sp_workspace ws(stream);
+        const int64_t nseg = S->npos[1] - 1, ldt = (K + 1) & ~(int64_t)1;
+        double* Bt = ws.get<double>((size_t)n * ldt + 2);
+        if (ws.failed) return SP_ERR_ALLOC;
+        Bt = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Bt) + 15) & ~(uintptr_t)15);
+        k_transpose<<<dim3((unsigned)sp_ceil_div(n, 32), (unsigned)sp_ceil_div(ldt, 32)), 256, 0, stream>>>(B, ldb, K, n, Bt, ldt);
+        SP_LAUNCH_CHECK();
+        sp_partition part;
+        // shorter pieces where there are few (30,000 to 115,000 entries: 10 against 14 us; 240,000 and up: no gain)
+        const sp_status st = sp_get_merge_partition(S, nseg + nnz < 200000 ? 16 : 32, stream, &part);
+        if (st != SP_OK) return st;
+        // row in registers / gathered row: A and B^T, or for column-major S the other way round
+        const double *reg = colmajor ? Bt : A, *gat = colmajor ? A : Bt;
+        const int64_t ldreg = colmajor ? ldt : lda, ldgat = colmajor ? lda : ldt;
+        const bool pairs = !colmajor || pair_a;
+        const int avec = colmajor || pair_a;
+        cudaError_t e = cudaSuccess;
+#define SP_SG_LAUNCH(L, V, W, FULL)                                                                                       \
+    do {                                                                                                                   \
+        constexpr size_t ring = (size_t)kDepth * V * kGThreads * sizeof(double);                                           \
+        e = sp_allow_shared<k_sddmm_group<P, I, L, V, W, FULL>>(S->device, ring);                                          \
+        if (e == cudaSuccess)                                                                                              \
+            e = sp_launch_dependent(k_sddmm_group<P, I, L, V, W, FULL>, dim3((unsigned)sp_ceil_div(part.nchunks * L, kGThreads)), \
+                                    dim3(kGThreads), ring, stream, pos, crd, (const double*)S->val, outer, reg, ldreg, avec, gat, ldgat, \
+                                    (int)K, x_vals, (const int64_t*)part.row, (const int64_t*)part.nz, part.nchunks, nseg, \
+                                    S->dims[S->ord[0]], S->dims[S->ord[1]]);                                               \
+    } while (0)
+        SP_DISPATCH_WIDTHS(S, {
+            const P* pos = static_cast<const P*>(S->pos[1]);
+            const I* crd = static_cast<const I*>(S->crd[1]);
+            const I* outer = dbl ? static_cast<const I*>(S->crd[0]) : nullptr;
+            if (pairs) {
+                if (K == 128) SP_SG_LAUNCH(16, 8, 2, true);
+                else if (K == 96) SP_SG_LAUNCH(16, 6, 2, true);
+                else if (K == 64) SP_SG_LAUNCH(16, 4, 2, true);
+                else if (K == 32) SP_SG_LAUNCH(8, 4, 2, true);
+                else if (K <= 16) SP_SG_LAUNCH(4, 4, 2, false);
+                else if (K < 32) SP_SG_LAUNCH(8, 4, 2, false);
+                else if (K < 64) SP_SG_LAUNCH(16, 4, 2, false);
+                else if (K < 96) SP_SG_LAUNCH(16, 6, 2, false);
+                else if (K < 128) SP_SG_LAUNCH(16, 8, 2, false);
+                else if (K <= 256) SP_SG_LAUNCH(16, 16, 2, false);
+                else SP_SG_LAUNCH(32, 16, 2, false);
+            } else {
+                if (K <= 16) SP_SG_LAUNCH(4, 4, 1, false);
+                else if (K <= 32) SP_SG_LAUNCH(8, 4, 1, false);
+                else if (K <= 64) SP_SG_LAUNCH(8, 8, 1, false);
+                else if (K <= 128) SP_SG_LAUNCH(16, 8, 1, false);
+                else if (K <= 256) SP_SG_LAUNCH(32, 8, 1, false);
+                else SP_SG_LAUNCH(32, 16, 1, false);
+            }
+        });
+#undef SP_SG_LAUNCH
+        SP_CUDA(e);
+        SP_LAUNCH_CHECK();
+        sp_count_launches(2);
+        SP_BOUNDS_RETURN(stream);
+        return SP_OK;
+    }
     sp_workspace ws(stream);
     const int64_t ldt = (K + 1) & ~(int64_t)1;   // even, so rows stay 16-byte aligned
     int64_t ldt_k = ldt;                         // leading dimension of the gathered operand in the kernel
@@ -279,9 +408,6 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
     if (st != SP_OK) return st;
     const bool vec2 = (K % 2 == 0) && (lda % 2 == 0) && (reinterpret_cast<uintptr_t>(A) % 16 == 0) &&
                       (reinterpret_cast<uintptr_t>(Bt) % 16 == 0);
-    // 32-byte loads when every operand row starts on a 32-byte boundary and K is a multiple of four
-    const bool vec4 = vec2 && (K % 4 == 0) && (lda % 4 == 0) && (ldt % 4 == 0) && (reinterpret_cast<uintptr_t>(A) % 32 == 0) &&
-                      (reinterpret_cast<uintptr_t>(Bt) % 32 == 0);
     const unsigned blocks = (unsigned)sp_ceil_div(part.nchunks * 32, kSThreads);
     // The kernel keeps the operand row of the outer (segment) index in registers and gathers the
     // row of the inner index: for column-major S the two operands simply trade places
@@ -290,8 +416,8 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
         const double* ta = A; A = Bt; Bt = const_cast<double*>(ta);
         const int64_t tl = lda; lda = ldt; ldt_k = tl;
     }
-#define SP_SDDMM_LAUNCH(V, NCH)                                                                                     \
-    sddmm_launch_st = sp_launch_dependent(k_sddmm<P, I, V, NCH>, dim3(blocks), dim3(kSThreads), 0, stream, pos, crd,  \
+#define SP_SDDMM_LAUNCH(V)                                                                                     \
+    sddmm_launch_st = sp_launch_dependent(k_sddmm<P, I, V>, dim3(blocks), dim3(kSThreads), 0, stream, pos, crd,  \
                                           (const double*)S->val, outer, (const double*)A, lda, (const double*)Bt, ldt_k, K, \
                                           x_vals, (const int64_t*)part.row, (const int64_t*)part.nz, part.nchunks,        \
                                           S->dims[S->ord[0]], S->dims[S->ord[1]])
@@ -300,18 +426,7 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
         const P* pos = static_cast<const P*>(S->pos[1]);
         const I* crd = static_cast<const I*>(S->crd[1]);
         const I* outer = dbl ? static_cast<const I*>(S->crd[0]) : nullptr;
-        if (vec4 && K > 64 && K <= 512) {
-            if (K <= 128) SP_SDDMM_LAUNCH(4, 1);
-            else if (K <= 256) SP_SDDMM_LAUNCH(4, 2);
-            else SP_SDDMM_LAUNCH(4, 4);
-        } else if (vec2) {
-            if (K <= 64) SP_SDDMM_LAUNCH(2, 1);
-            else if (K <= 128) SP_SDDMM_LAUNCH(2, 2);
-            else if (K <= 256) SP_SDDMM_LAUNCH(2, 4);
-            else SP_SDDMM_LAUNCH(2, 0);
-        } else {
-            SP_SDDMM_LAUNCH(1, 0);
-        }
+        if (vec2) SP_SDDMM_LAUNCH(2); else SP_SDDMM_LAUNCH(1);
     });
 #undef SP_SDDMM_LAUNCH
     SP_CUDA(sddmm_launch_st);
