@@ -2,18 +2,17 @@
 // (dense, compressed) - the SpMSpM kernel of Section 4.3, measured in Section 6.2 (Table 2).
 //
 // The paper's loop nest expands each row of C into a dense workspace (values + "filled" flags),
-// records which columns were touched, and compresses the row back in index order.  Here a block
-// owns a row at a time: its warps walk the entries A[i,k] (one per warp), lanes walk row k of B
-// and add a*b into the block's workspace row with atomics, setting one bit per touched column in
-// a bitmap.  Compression reads the bitmap words in order, so the columns come out sorted without
-// a sort; a block-wide scan of the words' bit counts gives every column its slot.  The kernel runs
-// twice: a symbolic pass that only counts (row lengths -> positions by a scan -> sizes of C's
-// arrays, read back once), and a numeric pass that fills coordinates and values.
-// Cost per row is proportional to its products plus dims[1]/32 bitmap words.
-// When a dense row of C and its bitmap fit in shared memory (dims[1] up to about 25,000) the
-// workspace lives there and the expansion's atomics never leave the SM; wider results use one
-// workspace row per block in global memory (L2-resident).
+// records which columns were touched, and compresses the row back in index order.  Both paths below
+// keep that shape, with the flags as a bitmap whose words, read in order, give the columns sorted.  The
+// product runs in two passes: a symbolic one (row lengths -> positions by a scan -> sizes of C's arrays,
+// read back once) and a numeric one.  Results of up to 32,768 columns whose operand rows are not too
+// sparse take the bitmap path (k_row_bitmaps, k_symbolic, k_numeric).  Otherwise a block owns a row at a
+// time (k_spmspm): warps walk the entries A[i,k], lanes walk row k of B and add into the block's workspace
+// row with atomics, in shared memory when a row of C fits there (dims[1] up to about 25,000), else in
+// one workspace row per block in global memory (L2-resident).
 #include "common.cuh"
+
+#include <algorithm>
 
 namespace {
 
@@ -128,15 +127,23 @@ k_spmspm(const P* __restrict__ apos, const I* __restrict__ acrd, const double* _
 }
 
 // Single block: pos[0] = 0, pos[i+1] = rowlen[0] + .. + rowlen[i]; total to *count.
-__global__ void __launch_bounds__(kPThreads)
-k_row_offsets(const int64_t* __restrict__ rowlen, int64_t m, void* __restrict__ pos, int posBits, int64_t* __restrict__ count) {
-    __shared__ unsigned long long s_w[kPThreads / 32];
+constexpr int kOffThreads = 1024, kOffPer = 8;
+__global__ void __launch_bounds__(kOffThreads)
+k_row_offsets(const int64_t* rowlen, int64_t m, void* __restrict__ pos, int posBits, int64_t* __restrict__ count) {
+    sp_wait_for_previous_kernel();
+    __shared__ unsigned long long s_w[kOffThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned long long run = 0;
     if (threadIdx.x == 0) sp_store_uint(pos, 0, 0, posBits);
-    for (int64_t b = 0; b < m; b += kPThreads) {
-        const int64_t i = b + threadIdx.x;
-        unsigned long long v = i < m ? (unsigned long long)rowlen[i] : 0ull, incl = v;
+    for (int64_t b = 0; b < m; b += kOffThreads * kOffPer) {
+        const int64_t i0 = b + (int64_t)threadIdx.x * kOffPer;
+        unsigned long long v[kOffPer], mine = 0;
+#pragma unroll
+        for (int u = 0; u < kOffPer; ++u) {
+            v[u] = i0 + u < m ? (unsigned long long)rowlen[i0 + u] : 0ull;
+            mine += v[u];
+        }
+        unsigned long long incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, o);
@@ -144,13 +151,238 @@ k_row_offsets(const int64_t* __restrict__ rowlen, int64_t m, void* __restrict__ 
         }
         if (lane == 31) s_w[w] = incl;
         __syncthreads();
-        unsigned long long pre = 0, tot = 0;
-        for (int q = 0; q < kPThreads / 32; ++q) { if (q < w) pre += s_w[q]; tot += s_w[q]; }
+        if (w == 0) {
+            unsigned long long x = s_w[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long u = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += u;
+            }
+            s_w[lane] = x;
+        }
         __syncthreads();
-        if (i < m) sp_store_uint(pos, i + 1, run + pre + incl, posBits);
-        run += tot;
+        unsigned long long at = run + (w ? s_w[w - 1] : 0ull) + incl - mine;
+#pragma unroll
+        for (int u = 0; u < kOffPer; ++u) {
+            at += v[u];
+            if (i0 + u < m) sp_store_uint(pos, i0 + u + 1, at, posBits);
+        }
+        run += s_w[kOffThreads / 32 - 1];
+        __syncthreads();
     }
     if (threadIdx.x == 0) *count = (int64_t)run;
+}
+
+// ---- results of up to kMaxCols columns whose operand rows are not too sparse --------------------------
+// Which columns a row of C holds is the union of the rows of B that it meets: with every row of B as a
+// bitmap (k_row_bitmaps) that is an OR of whole words, read 16 bytes a lane (k_symbolic), and the union
+// is kept for the numeric pass.  That pass gives a warp a row of C and a block of kColBlk columns, whose
+// sums lie in shared memory that no other warp touches: the columns of a row of B are distinct, so the
+// lanes of an instruction never meet, and no atomic is needed.
+// 8192 x 8192 at density 0.01 (55 M products, 37.5 M results): 463 us for the call, 580 us with one block per row,
+// atomics on a shared-memory row and the bitmap built twice (symbolic 112 -> 48 us with the bitmaps, offsets
+// 26 -> 10, numeric 434 -> 400).  Bound: the shared-memory pipe, 72 % busy: two accesses of 8 bytes per product.
+constexpr int64_t kMaxCols = 32768;
+constexpr int kColBlk = 1024;                   // columns of a warp of k_numeric (2048, half the warps: 494 us against 463 below)
+constexpr int kBitWarps = 4, kOrWarps = 4, kNumWarps = 4;
+
+// One warp per row of B: its bitmap (stride words, a multiple of four), and split[k * (nblk + 1) + c] =
+// the first entry of row k whose column is at least c * kColBlk.
+template <typename P, typename I>
+__global__ void __launch_bounds__(kBitWarps * 32)
+k_row_bitmaps(const P* __restrict__ pos, const I* __restrict__ crd, int64_t rows, int64_t n, int stride, int nblk,
+              uint32_t* __restrict__ bits, uint32_t* __restrict__ split) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t* mine = reinterpret_cast<uint32_t*>(s_dyn) + (size_t)w * stride;
+    const int64_t k = (int64_t)blockIdx.x * kBitWarps + w;
+    if (k >= rows) return;
+    for (int x = lane; x < stride; x += 32) mine[x] = 0u;
+    __syncwarp();
+    const int64_t b0 = (int64_t)pos[k], b1 = (int64_t)pos[k + 1];
+    uint32_t* sp = split + k * (nblk + 1);
+    for (int64_t q = b0 + lane; q < b1; q += 32) {
+        const uint32_t j = (uint32_t)SP_IDX(crd[q], n);
+        atomicOr(mine + (j >> 5), 1u << (j & 31));
+        const int cb = (int)(j / kColBlk);
+        for (int c = q > b0 ? (int)((uint32_t)SP_IDX(crd[q - 1], n) / kColBlk) + 1 : 0; c <= cb; ++c) sp[c] = (uint32_t)q;
+        if (q == b1 - 1)
+            for (int c = cb + 1; c <= nblk; ++c) sp[c] = (uint32_t)b1;
+    }
+    if (b1 == b0)
+        for (int c = lane; c <= nblk; c += 32) sp[c] = (uint32_t)b0;
+    __syncwarp();
+    for (int x = lane * 4; x < stride; x += 128)
+        *reinterpret_cast<uint4*>(bits + k * stride + x) = *reinterpret_cast<const uint4*>(mine + x);
+}
+
+// One warp per row of C: the OR of the bitmaps of the rows of B that row i of A names, and its bit count.
+template <typename P, typename I>
+__global__ void __launch_bounds__(kOrWarps * 32)
+k_symbolic(const P* __restrict__ apos, const I* __restrict__ acrd, const uint32_t* bits, int64_t m, int64_t kdim, int stride,
+           uint32_t* __restrict__ cbits, int64_t* __restrict__ rowlen) {
+    sp_wait_for_previous_kernel();
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * kOrWarps + (threadIdx.x >> 5);
+    if (i >= m) return;
+    const int64_t a0 = (int64_t)apos[i], a1 = (int64_t)apos[i + 1];
+    constexpr int kQ = 2, kE = 4;                   // 16-byte runs per lane and entry, entries in flight
+    uint32_t total = 0;
+    for (int x0 = 0; x0 < stride; x0 += 128 * kQ) {
+        uint4 acc[kQ];
+#pragma unroll
+        for (int t = 0; t < kQ; ++t) acc[t] = make_uint4(0u, 0u, 0u, 0u);
+        for (int64_t base = a0; base < a1; base += 32) {
+            const int cnt = a1 - base < 32 ? (int)(a1 - base) : 32;
+            const uint32_t k_l = lane < cnt ? (uint32_t)SP_IDX(acrd[base + lane], kdim) : 0u;
+            for (int e = 0; e < cnt; e += kE) {
+                uint4 v[kE][kQ];
+#pragma unroll
+                for (int u = 0; u < kE; ++u) {
+                    const uint32_t k = __shfl_sync(0xffffffffu, k_l, e + u < cnt ? e + u : cnt - 1);   // the tail repeats an entry
+                    const uint32_t* row = bits + (int64_t)k * stride + x0 + lane * 4;
+#pragma unroll
+                    for (int t = 0; t < kQ; ++t)
+                        v[u][t] = x0 + t * 128 + lane * 4 < stride ? *reinterpret_cast<const uint4*>(row + t * 128)
+                                                                   : make_uint4(0u, 0u, 0u, 0u);
+                }
+#pragma unroll
+                for (int u = 0; u < kE; ++u)
+#pragma unroll
+                    for (int t = 0; t < kQ; ++t) {
+                        acc[t].x |= v[u][t].x; acc[t].y |= v[u][t].y; acc[t].z |= v[u][t].z; acc[t].w |= v[u][t].w;
+                    }
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kQ; ++t) {
+            if (x0 + t * 128 + lane * 4 < stride)
+                *reinterpret_cast<uint4*>(cbits + i * stride + x0 + t * 128 + lane * 4) = acc[t];
+            total += (uint32_t)(__popc(acc[t].x) + __popc(acc[t].y) + __popc(acc[t].z) + __popc(acc[t].w));
+        }
+    }
+    total = __reduce_add_sync(0xffffffffu, total);
+    if (lane == 0) rowlen[i] = (int64_t)total;
+}
+
+// C32: C's coordinates are 32 bits wide (a plain store instead of a width switch).
+template <typename P, typename I, bool C32>
+__global__ void __launch_bounds__(kNumWarps * 32)
+k_numeric(const P* __restrict__ apos, const I* __restrict__ acrd, const double* __restrict__ aval,
+          const uint32_t* __restrict__ split, const I* __restrict__ bcrd, const double* __restrict__ bval, int64_t m,
+          int nblk, int stride, const uint32_t* __restrict__ cbits, const void* __restrict__ cpos, int cposBits,
+          void* __restrict__ ccrd, int ccrdBits, double* __restrict__ cval, int64_t kdim, int64_t n) {
+    // per warp: its columns' sums; the segments of the next 32 entries of A and their factors, read back as
+    // broadcasts (a shuffle per word costs the same pipe as a shared-memory access of all of them)
+    struct __align__(16) Seg { uint32_t first, len; double a; };
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ Seg s_seg[kNumWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double* acc = reinterpret_cast<double*>(s_dyn) + (size_t)w * kColBlk;
+    for (int x = lane; x < kColBlk; x += 32) acc[x] = 0.0;
+    __syncwarp();
+    const int64_t items = m * nblk;
+    const uint32_t below = (1u << lane) - 1u;
+    constexpr int kE = 8;                           // segments of B rows fetched together (4: 477 us, 2: 498)
+    for (int64_t item = (int64_t)blockIdx.x * kNumWarps + w; item < items; item += (int64_t)gridDim.x * kNumWarps) {
+        const int64_t i = item / nblk;
+        const int cb = (int)(item - i * nblk);
+        const int64_t a0 = (int64_t)apos[i], a1 = (int64_t)apos[i + 1];
+        const uint32_t* row = cbits + i * stride;
+        const int wb = cb * (kColBlk / 32);
+        double* accl = acc - cb * kColBlk;              // indexed by column
+        const Seg* seg = s_seg[w];
+        for (int64_t base = a0; base < a1; base += 32) {
+            const int cnt = a1 - base < 32 ? (int)(a1 - base) : 32;
+            Seg mine;
+            mine.first = mine.len = 0;                  // past the row's end: empty segments
+            mine.a = 0.0;
+            if (lane < cnt) {
+                const int64_t k = SP_IDX((int64_t)acrd[base + lane], kdim);
+                mine.a = aval[base + lane];
+                mine.first = split[k * (nblk + 1) + cb];
+                mine.len = split[k * (nblk + 1) + cb + 1] - mine.first;
+            }
+            s_seg[w][lane] = mine;
+            const bool any_long = __any_sync(0xffffffffu, mine.len > 32);
+            __syncwarp();
+            // software pipeline: the next kE segments are requested before these are added
+            uint32_t jc[kE], jn[kE];
+            double vc[kE], vn[kE];
+            auto fetch = [&](int e, uint32_t (&j)[kE], double (&v)[kE]) {
+#pragma unroll
+                for (int u = 0; u < kE; ++u) {
+                    const uint2 sl = *reinterpret_cast<const uint2*>(&seg[e + u]);
+                    j[u] = ~0u;
+                    if ((uint32_t)lane < sl.y) {
+                        j[u] = (uint32_t)SP_IDX(bcrd[sl.x + lane], n);
+                        v[u] = bval[sl.x + lane];
+                    }
+                }
+            };
+            auto add = [&](int e, const uint32_t (&j)[kE], const double (&v)[kE]) {
+#pragma unroll
+                for (int u = 0; u < kE; ++u) {
+                    if (j[u] != ~0u) accl[j[u]] = fma(seg[e + u].a, v[u], accl[j[u]]);
+                    __syncwarp();
+                }
+                if (any_long)                           // segments of more than 32 entries
+                    for (int u = 0; u < kE; ++u) {
+                        const Seg g = seg[e + u];
+                        for (uint32_t q = 32; q < g.len; q += 32) {
+                            if (q + lane < g.len) {
+                                const int jj = (int)SP_IDX(bcrd[g.first + q + lane], n);
+                                accl[jj] = fma(g.a, bval[g.first + q + lane], accl[jj]);
+                            }
+                            __syncwarp();
+                        }
+                    }
+            };
+            fetch(0, jc, vc);
+            for (int e = 0; e < cnt; e += 2 * kE) {
+                fetch((e + kE) & 31, jn, vn);           // wraps at 32: a repeated fetch that nobody adds
+                add(e, jc, vc);
+                if (e + kE >= cnt) break;
+                fetch((e + 2 * kE) & 31, jc, vc);
+                add(e + kE, jn, vn);
+            }
+            __syncwarp();                               // s_seg is written again
+        }
+        // the block's columns in order
+        uint32_t before = 0;                            // columns of the row in earlier blocks
+        for (int x = lane; x < wb; x += 32) before += (uint32_t)__popc(row[x]);
+        before = __reduce_add_sync(0xffffffffu, before);
+        int64_t slot = (int64_t)sp_load_uint(cpos, i, cposBits) + before;
+#pragma unroll 1
+        for (int h = 0; h < kColBlk / 1024; ++h) {
+            const int x = wb + h * 32 + lane;
+            const uint32_t bits = x < stride ? row[x] : 0u;
+            uint32_t at = (uint32_t)__popc(bits), tot = at;     // exclusive prefix over the 32 words
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, tot, o);
+                if (lane >= o) tot += u;
+            }
+            at = tot - at;
+            tot = __shfl_sync(0xffffffffu, tot, 31);
+            double* sums = acc + h * 1024 + lane;
+            double* cv = cval + slot;
+#pragma unroll 8
+            for (int q = 0; q < 32; ++q) {
+                const uint32_t wbits = __shfl_sync(0xffffffffu, bits, q), o = __shfl_sync(0xffffffffu, at, q);
+                if ((wbits >> lane) & 1u) {
+                    const uint32_t to = o + (uint32_t)__popc(wbits & below);
+                    const uint32_t col = (uint32_t)(cb * kColBlk + h * 1024 + q * 32 + lane);
+                    if (C32) static_cast<uint32_t*>(ccrd)[slot + to] = col;
+                    else sp_store_uint(ccrd, slot + to, (uint64_t)col, ccrdBits);
+                    cv[to] = sums[q * 32];
+                    sums[q * 32] = 0.0;
+                }
+            }
+            slot += tot;
+        }
+        __syncwarp();
+    }
 }
 
 }  // namespace
@@ -189,6 +421,13 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     SP_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t shm_sym = (size_t)((words * 4 + 7) & ~(int64_t)7);
     const size_t shm_num = shm_sym + (size_t)n * sizeof(double);
+    // The bitmap path reads a bitmap row per entry of A where the other one walks a row of B: rows of B
+    // of at least a sixteenth of a bitmap row's words, and bitmaps of at most 256 MB.
+    const int stride = (int)((words + 3) & ~(int64_t)3);          // words of a bitmap row
+    const int64_t kdim = B->dims[0];
+    const bool bitmaps = n <= kMaxCols && m > 0 && kdim > 0 && B->nval < ((int64_t)1 << 32) &&
+                         (m + kdim) * stride * 4 <= ((int64_t)256 << 20) && stride * kdim <= 16 * (B->nval + kdim);
+    const int nblk = (int)sp_ceil_div(n, kColBlk);
     const bool in_smem = shm_num + 2048 <= (size_t)smem_max;
     auto blocks_for = [&](size_t shm) {
         int64_t per_sm = (int64_t)((size_t)smem_max / (shm + 1024));
@@ -203,14 +442,19 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     sp_workspace ws(stream);
     double* wsrow = nullptr;
     uint32_t* bm = nullptr;
-    if (!in_smem) {
+    uint32_t *bbits = nullptr, *cbits = nullptr, *split = nullptr;
+    if (bitmaps) {
+        bbits = ws.get<uint32_t>((size_t)kdim * stride);
+        cbits = ws.get<uint32_t>((size_t)m * stride);
+        split = ws.get<uint32_t>((size_t)kdim * (nblk + 1));
+    } else if (!in_smem) {
         wsrow = ws.get<double>((size_t)nblocks * n);
         bm = ws.get<uint32_t>((size_t)nblocks * words);
     }
     int64_t* rowlen = ws.get<int64_t>((size_t)m + 1);
     int64_t* d_count = ws.get<int64_t>(1);
     if (ws.failed) return SP_ERR_ALLOC;
-    if (!in_smem) {
+    if (!bitmaps && !in_smem) {
         SP_CUDA(cudaMemsetAsync(wsrow, 0, (size_t)nblocks * n * sizeof(double), stream));
         SP_CUDA(cudaMemsetAsync(bm, 0, (size_t)nblocks * words * sizeof(uint32_t), stream));
     }
@@ -243,8 +487,22 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
             k_spmspm<P, I, NUM, false><<<(unsigned)nblocks, kPThreads, 0, stream>>>(SP_SPMSPM_ARGS);              \
         }                                                                                                         \
     })
-    if (m > 0) SP_SPMSPM_LAUNCH(false);
-    k_row_offsets<<<1, kPThreads, 0, stream>>>(rowlen, m, C->pos[1], posBits, d_count);
+    if (bitmaps) {
+        SP_DISPATCH_WIDTHS(A, {
+            const size_t shm = (size_t)kBitWarps * stride * sizeof(uint32_t);
+            k_row_bitmaps<P, I><<<(unsigned)sp_ceil_div(kdim, kBitWarps), kBitWarps * 32, shm, stream>>>(
+                static_cast<const P*>(B->pos[1]), static_cast<const I*>(B->crd[1]), kdim, n, stride, nblk, bbits, split);
+            if (sp_launch_dependent(k_symbolic<P, I>, dim3((unsigned)sp_ceil_div(m, kOrWarps)), dim3(kOrWarps * 32), 0, stream,
+                                    static_cast<const P*>(A->pos[1]), static_cast<const I*>(A->crd[1]), (const uint32_t*)bbits, m,
+                                    kdim, stride, cbits, rowlen) != cudaSuccess)
+                return fail(SP_ERR_CUDA);
+        });
+        sp_count_launches(1);
+    } else if (m > 0) {
+        SP_SPMSPM_LAUNCH(false);
+    }
+    if (sp_launch_dependent(k_row_offsets, dim3(1), dim3(kOffThreads), 0, stream, (const int64_t*)rowlen, m, C->pos[1], posBits, d_count) != cudaSuccess)
+        return fail(SP_ERR_CUDA);
     if (cudaGetLastError() != cudaSuccess) return fail(SP_ERR_CUDA);
     sp_count_launches(2);
     unsigned long long* h_count = sp_host_words();
@@ -260,7 +518,24 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     C->val = static_cast<double*>(sp_dev_alloc((size_t)(count ? count : 1) * sizeof(double), stream));
     if (!C->crd[1] || !C->val) return fail(SP_ERR_ALLOC);
     if (m > 0 && count > 0) {
-        SP_SPMSPM_LAUNCH(true);
+        if (bitmaps) {
+            constexpr size_t shm = (size_t)kNumWarps * kColBlk * sizeof(double);
+            const int64_t items = m * nblk;
+            const unsigned blocks = (unsigned)std::min<int64_t>(sp_ceil_div(items, kNumWarps), (int64_t)sms * (smem_max / (shm + 1024)));
+#define SP_NUMERIC(C32)                                                                                                       \
+    do {                                                                                                                      \
+        if (sp_allow_shared<k_numeric<P, I, C32>>(dev, shm) != cudaSuccess) return fail(SP_ERR_CUDA);                         \
+        k_numeric<P, I, C32><<<blocks, kNumWarps * 32, shm, stream>>>(                                                        \
+            static_cast<const P*>(A->pos[1]), static_cast<const I*>(A->crd[1]), A->val, split, static_cast<const I*>(B->crd[1]), B->val, m, \
+            nblk, stride, cbits, C->pos[1], posBits, C->crd[1], crdBits, C->val, kdim, n);                                    \
+    } while (0)
+            SP_DISPATCH_WIDTHS(A, {
+                if (crdBits == 32) SP_NUMERIC(true); else SP_NUMERIC(false);
+            });
+#undef SP_NUMERIC
+        } else {
+            SP_SPMSPM_LAUNCH(true);
+        }
         if (cudaGetLastError() != cudaSuccess) return fail(SP_ERR_CUDA);
         sp_count_launches(1);
     }

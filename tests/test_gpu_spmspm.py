@@ -68,3 +68,16 @@ def test_exact_integers_and_errors(oracle):
     with pytest.raises(b.SpError) as e:          # inner dimensions differ (200 x 150 times 200 x 150)
         b.sp_spmspm(csr, csr)
     assert e.value.code == 1
+
+
+@pytest.mark.parametrize("m,k,n,na,nb", [(40, 30, 1023, 300, 30 * 1023), (40, 30, 1024, 400, 9000), (33, 70, 1025, 2310, 60000),
+                                         (20, 40, 2049, 500, 40 * 2049), (12, 9, 32768, 60, 100000), (12, 9, 32769, 60, 100000),
+                                         (1, 1, 1, 1, 1), (50, 64, 4000, 50 * 64, 30000), (3, 200, 31, 600, 3000)])
+def test_bitmap_path_edges(oracle, m, k, n, na, nb):
+    """Column blocks just full, one over and one short, full operand rows (segments of more than a warp), rows of
+    exactly 32 and 64 entries, and the widest result of the bitmap path beside the first that is too wide."""
+    A, B = I.uniform_matrix(m, k, na, seed=m + n), I.uniform_matrix(k, n, nb, seed=n + 1)
+    _check(oracle, A, B)
+    if n <= 4000:
+        _check(oracle, A, B, 64, 64, 64)
+        _check(oracle, A, B, 32, 16)
