@@ -893,6 +893,79 @@ __global__ void k_unpack(UnpackArgs a) {
     }
 }
 
+// Matrices with a compressed inner level and 32- or 64-bit arrays: a block unpacks kUnpackTile consecutive
+// entries.  Two searches, by the warps together, find the segments that the tile touches; each of those
+// marks its first entry, and an entry's segment is the last mark at or before it.  (A search of its own
+// per entry, 17 dependent loads for 70,000 rows, took 33 us on 1,500,007 entries; this takes 12.)
+constexpr int kUnpackThreads = 256;
+constexpr int kUnpackTile = 1024;
+
+// Last q in [0, n) with pos[q] <= p, found by a warp, 32 probes at a time (pos[0] <= p).
+template <typename P>
+__device__ __forceinline__ int64_t warp_last_at_most(const P* __restrict__ pos, int64_t n, int64_t p) {
+    int64_t lo = 0, hi = n;                       // the answer is in [lo, hi)
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) >> 5, q = lo + step * (int64_t)sp_lane();
+        const unsigned m = __ballot_sync(0xffffffffu, q < hi && (int64_t)pos[q] <= p);      // a run of ones from lane 0
+        const int64_t at = lo + step * (31 - __clz(m));
+        hi = at + step < hi ? at + step : hi;
+        lo = at;
+    }
+    return lo;
+}
+
+template <typename P, typename I>
+__global__ void __launch_bounds__(kUnpackThreads)
+k_unpack_rows(const P* __restrict__ pos, const I* __restrict__ crd, const double* __restrict__ val, const I* __restrict__ outer,
+              int64_t nseg, int64_t n, int64_t* __restrict__ out_outer, int64_t* __restrict__ out_inner, double* __restrict__ vals_out) {
+    __shared__ uint32_t s_seg[kUnpackTile];       // 1 + offset (from the tile's first segment) of the segment that starts here
+    __shared__ int64_t s_range[2];
+    __shared__ uint32_t s_w[kUnpackThreads / 32];
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const int64_t e0 = (int64_t)blockIdx.x * kUnpackTile;
+    const int cnt = (int)(n - e0 < kUnpackTile ? n - e0 : kUnpackTile);
+    constexpr int kPer = kUnpackTile / kUnpackThreads;
+    for (int i = t; i < kUnpackTile; i += kUnpackThreads) s_seg[i] = 0u;
+    if (w < 2) {
+        const int64_t q = warp_last_at_most(pos, nseg, w ? e0 + cnt - 1 : e0);
+        if (lane == 0) s_range[w] = q;
+    }
+    __syncthreads();
+    const int64_t q0 = s_range[0], q1 = s_range[1];
+    for (int64_t q = q0 + 1 + t; q <= q1; q += kUnpackThreads) {
+        const int64_t i = (int64_t)pos[q] - e0;   // empty segments share their start with the next; the largest wins
+        if (i < cnt) atomicMax(&s_seg[i], (uint32_t)(q - q0));
+    }
+    __syncthreads();
+    uint32_t m[kPer];                             // running maximum over a thread's consecutive entries, then over the block
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        m[i] = s_seg[t * kPer + i];
+        if (i && m[i] < m[i - 1]) m[i] = m[i - 1];
+    }
+    uint32_t run = m[kPer - 1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o && u > run) run = u;
+    }
+    if (lane == 31) s_w[w] = run;
+    uint32_t before = __shfl_up_sync(0xffffffffu, run, 1);
+    if (lane == 0) before = 0;
+    __syncthreads();
+    for (int i = 0; i < w; ++i)
+        if (s_w[i] > before) before = s_w[i];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) s_seg[t * kPer + i] = m[i] > before ? m[i] : before;
+    __syncthreads();
+    for (int i = t; i < cnt; i += kUnpackThreads) {
+        const int64_t q = q0 + s_seg[i];
+        out_outer[e0 + i] = outer ? (int64_t)outer[q] : q;
+        out_inner[e0 + i] = (int64_t)crd[e0 + i];
+        vals_out[e0 + i] = val[e0 + i];
+    }
+}
+
 int ceil_log2(int64_t v) {   // bits needed for coordinates 0..v-1
     int b = 0;
     while (b < 63 && ((int64_t)1 << b) < v) ++b;
@@ -1222,7 +1295,17 @@ extern "C" sp_status sp_unpack(const sp_tensor* t, void* const* coo_coords_out, 
     a.crdBits = t->crdBits;
     a.vals_out = vals_out;
     *nnz_out = t->nval;
-    if (t->nval > 0) {
+    if (t->nval > 0 && t->rank == 2 && t->lt[1] == SP_COMPRESSED && t->posBits >= 32 && t->crdBits >= 32 && t->npos[1] - 1 < ((int64_t)1 << 32)) {
+        const unsigned tiles = (unsigned)sp_ceil_div(t->nval, kUnpackTile);
+        SP_DISPATCH_WIDTHS(t, {
+            k_unpack_rows<P, I><<<tiles, kUnpackThreads, 0, stream>>>(
+                static_cast<const P*>(t->pos[1]), static_cast<const I*>(t->crd[1]), t->val,
+                t->lt[0] == SP_COMPRESSED ? static_cast<const I*>(t->crd[0]) : nullptr, t->npos[1] - 1, t->nval, a.out[t->ord[0]], a.out[t->ord[1]],
+                vals_out);
+        });
+        sp_count_launches(1);
+        SP_LAUNCH_CHECK();
+    } else if (t->nval > 0) {
         k_unpack<<<(unsigned)sp_ceil_div(t->nval, 256), 256, 0, stream>>>(a);
         sp_count_launches(1);
         SP_LAUNCH_CHECK();

@@ -24,6 +24,7 @@ constexpr int kWarps = kBThreads / 32;
 constexpr int kCap = 4096;                      // entries a bucket can hold
 constexpr int kIpt = kCap / kBThreads;          // ... per thread of k_rows_build
 constexpr int kAverage = 2048;                  // entries per bucket aimed at: rows of 48 +- 7 and power-law rows stay below twice that
+constexpr int kAverageSmall = 256;               // ... of a small input, for more blocks (10,486 entries: 37 us; 2048: 39)
 constexpr int kWidth = 2048;                    // outer indices of a bucket
 constexpr int kMaxBuckets = 4096;
 constexpr int kDense = 24;                      // mean compares per entry above which segments are cut into bins
@@ -347,7 +348,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     // narrow positions need the radix path's width checks; records hold 32-bit coordinates
     if (posBits < 32 || crdBits < 32 || no >= ((int64_t)1 << 31) || ni >= ((int64_t)1 << 32)) return SP_ERR_UNSUPPORTED;
     // enough buckets for the entries and for the outer indices, no more than there are outer indices
-    int64_t buckets = std::max(sp_ceil_div(n, kAverage), sp_ceil_div(no, kWidth - 48));
+    int64_t buckets = std::max(sp_ceil_div(n, n < 300000 ? kAverageSmall : kAverage), sp_ceil_div(no, kWidth - 48));
     if (buckets > kMaxBuckets) return SP_ERR_UNSUPPORTED;
     if (buckets > no) {
         if (n > no * kCap) return SP_ERR_UNSUPPORTED;
