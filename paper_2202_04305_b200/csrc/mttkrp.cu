@@ -15,10 +15,11 @@
 
 #include <limits.h>
 
+#include <algorithm>
+
 namespace {
 
 constexpr int kTThreads = 256;
-constexpr int kTPer = 512;   // entries per warp
 
 // One nnz batch = up to 32 consecutive entries held one per lane (coordinate, value).
 // The ends of the fibres that fall inside the batch are turned into a 32-bit mask, so the
@@ -177,8 +178,6 @@ struct __align__(16) Staged {
     uint32_t bw;     // (level-1 factor row offset << 1) | close-after-this-entry
     double v;
 };
-
-constexpr int kFastPer = 1024;   // entries per warp
 
 // A lane's S columns are S/2 pairs; pair n sits at column offset coff[n] of the 32-column tile,
 // laid out so that the lanes of a group read one contiguous run per 16-byte load.
@@ -451,7 +450,11 @@ static sp_status mttkrp_levels(sp_tensor* T, const double* F1, const double* F2,
     const bool fast = (R % 2 == 0) && maxdim * R < ((int64_t)1 << 31) && reinterpret_cast<uintptr_t>(B) % 16 == 0 &&
                       reinterpret_cast<uintptr_t>(C) % 16 == 0 && reinterpret_cast<uintptr_t>(M) % 16 == 0;
     sp_partition part;
-    sp_status st = sp_get_mttkrp_partition(T, fast ? kFastPer : kTPer, stream, &part);
+    // Entries per warp: enough warps for the GPU (two waves of 16 per SM) before long ranges.  38,175 entries 241 ->
+    // 28 us, 451,180 entries 77 -> 38 us against 1,024 per warp throughout; 20 M entries: 256 543 us, 512 520,
+    // 1,024 521; 5 M, R = 50: 512 312 us, 1,024 343.
+    const int64_t per = std::max<int64_t>(32, std::min<int64_t>(512, sp_ceil_div(sp_ceil_div(nnz, 4736), 32) * 32));
+    sp_status st = sp_get_mttkrp_partition(T, per, stream, &part);
     if (st != SP_OK) return st;
     const unsigned blocks = (unsigned)sp_ceil_div(part.nchunks * 32, fast ? kFThreads : kTThreads);
     if (fast) {
