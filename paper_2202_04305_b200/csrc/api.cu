@@ -104,6 +104,7 @@ sp_status sp_free(sp_tensor* t) {
         sp_dev_free(kv.second.row, nullptr);
         sp_dev_free(kv.second.nz, nullptr);
         sp_dev_free(kv.second.aux, nullptr);
+        sp_dev_free(kv.second.marks, nullptr);
     }
     delete t;
     cudaSetDevice(prev);

@@ -26,6 +26,7 @@ struct sp_partition {
     int64_t* row = nullptr;   // nchunks + 1 entries (device)
     int64_t* nz = nullptr;    // nchunks + 1 entries (device)
     int64_t* aux = nullptr;   // kernel-specific (MTTKRP: slice of each chunk start)
+    uint32_t* marks = nullptr;   // MTTKRP: one word per entry, see k_mttkrp_group
 };
 
 struct sp_tensor {
@@ -250,7 +251,7 @@ static inline sp_status sp_bounds_result(cudaStream_t stream) {
     } while (0)
 
 // Partition tables (partition.cu).  kind distinguishes the position array used.
-enum { SP_PART_MERGE_LAST = 1, SP_PART_MTTKRP = 2, SP_PART_SEGIDS = 3 };
+enum { SP_PART_MERGE_LAST = 1, SP_PART_MTTKRP = 2, SP_PART_SEGIDS = 3, SP_PART_MTTKRP_MARKS = 4 };
 // For rank-2 (x, compressed) storage: the logical level-0 coordinate of every stored entry
 // (the expanded "outer" index), uint32, cached in the handle.  Needs dims < 2^32.
 sp_status sp_get_segment_ids(sp_tensor* t, cudaStream_t stream, const uint32_t** out);
@@ -258,7 +259,8 @@ sp_status sp_get_merge_partition(sp_tensor* t, int64_t items_per_chunk, cudaStre
 // Length of the longest last-level segment (row of CSR, stored row of DCSR, ...), measured on the
 // device on first use (one small kernel and one read-back, which waits for the stream) and kept.
 sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out);
-sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t nnz_per_chunk, cudaStream_t stream, sp_partition* out);
+// with_marks: the entries' words too (level-1 size below 2^29); the tables are cached together or not at all.
+sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t nnz_per_chunk, bool with_marks, cudaStream_t stream, sp_partition* out);
 
 // sp_pack for matrices with a compressed inner level and short segments (pack_rows.cu).  SP_ERR_UNSUPPORTED:
 // nothing was built, take the general path.

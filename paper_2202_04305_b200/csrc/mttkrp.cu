@@ -407,6 +407,159 @@ k_mttkrp_fast(const P* __restrict__ pos1, const I* __restrict__ crd0, const P* _
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Lane groups.  marks[p] (laid out once per handle) says for entry p: level-1 coordinate of its fibre << 2 |
+// "the slice ends here" << 1 | "the fibre ends here".
+//
+// A group of L lanes owns a range of consecutive entries and V columns a lane (L * V columns per blockIdx.y), W of
+// them adjacent and fetched by one load.  The leaf rows of kU entries, and the level-1 rows of the fibres that end
+// among them, are requested together; closing a fibre is accs += F1[j,:] * accf, closing a slice stores its
+// row of M.  The range's last entry closes its fibre in any case: sums are linear, so a fibre may be closed in
+// pieces.  Slices that reach beyond the range go through shared memory, where a block adds up what its
+// groups hold of the same slice, and from there into M (zeroed first) with one atomic per column.
+// Against the staged warps of k_mttkrp_fast: 38,175 entries 27 -> 12 us, 451,180 entries with R = 48 37 -> 28,
+// 5 M entries with R = 48 306 -> 238, 3 M with R = 17 (which that one cannot take) 303 -> 114.  But 20 M entries with
+// R = 32 551 against 520: a group that closes a fibre holds up the other groups of its warp, and 120 registers
+// leave 16 warps per SM.  (kU = 2, 3, 4, 6 there: 604, 551, 644, 860.)
+template <int W>
+__device__ __forceinline__ void ld_run(const double* p, double* a) {
+    if (W == 2) { const double2 t = *reinterpret_cast<const double2*>(p); a[0] = t.x; a[W - 1] = t.y; }
+    else a[0] = *p;
+}
+
+constexpr int kGThreads = 64;     // 300,000 to 1 M entries: 128 threads 10 % slower, 256 60 %
+template <typename P, typename I, int L, int V, int W, int kU>
+__global__ void __launch_bounds__(kGThreads)
+k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, const double* __restrict__ val,
+               const P* __restrict__ pos1, const I* __restrict__ crd0, const double* __restrict__ F1,
+               const double* __restrict__ F2, int64_t R, double* __restrict__ M, const int64_t* __restrict__ pfiber,
+               const int64_t* __restrict__ pnz, const int64_t* __restrict__ pslice, int64_t nchunks, int64_t nslice,
+               int64_t d0, int64_t d1, int64_t d2) {
+    // d0, d1, d2: rows of M, F1, F2 (used by the bounds-checking debug build only)
+    constexpr int kGroups = kGThreads / L, kSlots = 2 * kGroups;
+    __shared__ double s_sum[kSlots][L * V];         // slot 2 g: the slice group g's range begins in, 2 g + 1: the one it ends in
+    __shared__ int64_t s_id[kSlots];                // its row of M, -1 = nothing
+    const int g = threadIdx.x / L, gl = threadIdx.x % L;
+    const int64_t w = (int64_t)blockIdx.x * kGroups + g;
+    const int64_t p0 = w < nchunks ? pnz[w] : 0;
+    const int nz = w < nchunks ? (int)(pnz[w + 1] - p0) : 0;
+    const int64_t cb = (int64_t)blockIdx.y * (L * V);
+    int coff[V / W];                                // idle lanes read the tile's first run and never write
+    bool on[V / W];
+#pragma unroll
+    for (int j = 0; j < V / W; ++j) {
+        const int c = (j * L + gl) * W;
+        on[j] = cb + c < R;
+        coff[j] = on[j] ? c : 0;
+    }
+    auto slot_put = [&](int slot, const double (&a)[V], int64_t id) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) s_sum[slot][(j / W * L + gl) * W + j % W] = a[j];
+        if (gl == 0) s_id[slot] = id;
+    };
+    if (gl == 0) s_id[2 * g] = s_id[2 * g + 1] = -1;
+    if (nz > 0) {
+        const double *F1g = F1 + cb, *F2g = F2 + cb;
+        const uint32_t* ml = marks + p0;
+        const I* cl = crd2 + p0;
+        const double* vl = val + p0;
+        int64_t s = pslice[w], f = pfiber[w];
+        int64_t i = SP_IDX(crd0 ? (int64_t)crd0[s] : s, d0);
+        bool first = true, open = true;
+        double accf[V], accs[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) accf[j] = accs[j] = 0.0;
+        uint32_t mn[kU];
+        I kn[kU];
+        double vn[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {              // the group's lanes read the same word: one transaction
+            const int q = u < nz ? u : nz - 1;
+            mn[u] = ml[q] | (q == nz - 1 ? 4u << 29 : 0u);
+            kn[u] = cl[q];
+            vn[u] = vl[q];
+        }
+        for (int p = 0; p < nz; p += kU) {
+            double c[kU][V], b[kU][V], v[kU];
+            uint32_t mk[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                mk[u] = mn[u];
+                v[u] = vn[u];
+                const double* row = F2g + (int64_t)SP_IDX(kn[u], d2) * R;
+#pragma unroll
+                for (int j = 0; j < V / W; ++j) ld_run<W>(row + coff[j], c[u] + j * W);
+                if (mk[u] & (1u | 1u << 31)) {      // bit 31: the range's last entry
+                    const double* brow = F1g + (int64_t)SP_IDX((mk[u] >> 2) & 0x1fffffffu, d1) * R;
+#pragma unroll
+                    for (int j = 0; j < V / W; ++j) ld_run<W>(brow + coff[j], b[u] + j * W);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int q = p + kU + u < nz ? p + kU + u : nz - 1;
+                mn[u] = ml[q] | (q == nz - 1 ? 4u << 29 : 0u);
+                kn[u] = cl[q];
+                vn[u] = vl[q];
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                if (p + u < nz) {
+#pragma unroll
+                    for (int j = 0; j < V; ++j) accf[j] = fma(v[u], c[u][j], accf[j]);
+                    if (mk[u] & (1u | 1u << 31)) {
+#pragma unroll
+                        for (int j = 0; j < V; ++j) { accs[j] = fma(b[u][j], accf[j], accs[j]); accf[j] = 0.0; }
+                        f += mk[u] & 1u;
+                        if (mk[u] & 2u) {           // the slice is complete
+                            if (first) {
+                                slot_put(2 * g, accs, i);
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < V / W; ++j)
+                                    if (on[j]) {
+                                        double* m = M + i * R + cb + coff[j];
+                                        if (W == 2) *reinterpret_cast<double2*>(m) = make_double2(accs[j * W], accs[j * W + W - 1]);
+                                        else *m = accs[j];
+                                    }
+                            }
+                            first = false;
+#pragma unroll
+                            for (int j = 0; j < V; ++j) accs[j] = 0.0;
+                            ++s;
+                            if (!crd0) while (s < nslice && (int64_t)pos1[s + 1] <= f) ++s;      // slices with no fibres
+                            open = p + u + 1 < nz;
+                            if (open) i = SP_IDX(crd0 ? (int64_t)crd0[s] : s, d0);
+                        }
+                    }
+                }
+            }
+        }
+        if (open) slot_put(first ? 2 * g : 2 * g + 1, accs, i);
+    }
+    __syncthreads();
+    for (int e = g; e < kSlots; e += kGroups) {     // the first of a run of equal slices adds them all up
+        const int64_t id = s_id[e];
+        if (id < 0) continue;
+        int q = e - 1;
+        while (q >= 0 && s_id[q] < 0) --q;
+        if (q >= 0 && s_id[q] == id) continue;
+        double sum[V];
+#pragma unroll
+        for (int j = 0; j < V; ++j) sum[j] = 0.0;
+        for (int u = e; u < kSlots; ++u) {
+            const int64_t d = s_id[u];
+            if (d < 0) continue;
+            if (d != id) break;
+#pragma unroll
+            for (int j = 0; j < V; ++j) sum[j] += s_sum[u][(j / W * L + gl) * W + j % W];
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (on[j / W]) atomicAdd(M + id * R + cb + coff[j / W] + j % W, sum[j]);
+    }
+}
+
 }  // namespace
 
 // F1 / F2: factor matrices of the dimensions stored at levels 1 / 2; M: rows of the level-0 dimension.
@@ -449,12 +602,50 @@ static sp_status mttkrp_levels(sp_tensor* T, const double* F1, const double* F2,
     const int64_t maxdim = d1 > d2 ? d1 : d2;
     const bool fast = (R % 2 == 0) && maxdim * R < ((int64_t)1 << 31) && reinterpret_cast<uintptr_t>(B) % 16 == 0 &&
                       reinterpret_cast<uintptr_t>(C) % 16 == 0 && reinterpret_cast<uintptr_t>(M) % 16 == 0;
+    // Large tensors with 8 < R <= 32 stay on the staged warps: R = 16, 24, 32 and 5 M entries 162, 167, 159 us against
+    // 165, 197, 189; R = 8 162 against 125; 1 M entries, R = 32: 43 against 44.
+    const bool staged = fast && nnz >= 1000000 && R > 8 && R <= 32;
+    if (!staged && d1 < ((int64_t)1 << 29)) {
+        sp_partition part;
+        const int64_t per = std::max<int64_t>(16, std::min<int64_t>(256, sp_ceil_div(sp_ceil_div(nnz, 18944), 16) * 16));   // per group, as below per warp
+        sp_status st = sp_get_mttkrp_partition(T, per, true, stream, &part);
+        if (st != SP_OK) return st;
+        const bool pairs = R % 2 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0 &&
+                           reinterpret_cast<uintptr_t>(M) % 16 == 0;
+#define SP_MTTKRP_GROUP(L, V, W, U)                                                                                        \
+    k_mttkrp_group<P, I, L, V, W, U><<<dim3((unsigned)sp_ceil_div(part.nchunks * L, kGThreads), (unsigned)sp_ceil_div(R, L * V)), kGThreads, 0, stream>>>( \
+        part.marks, static_cast<const I*>(T->crd[2]), T->val, static_cast<const P*>(T->pos[1]),                                 \
+        T->lt[0] == SP_COMPRESSED ? static_cast<const I*>(T->crd[0]) : nullptr, F1, F2, R, M, part.row, part.nz, part.aux, \
+        part.nchunks, T->npos[1] - 1, T->dims[T->ord[0]], d1, d2)
+        SP_DISPATCH_WIDTHS(T, {
+            if (pairs) {
+                if (R <= 8) SP_MTTKRP_GROUP(4, 2, 2, 6);
+                else if (R <= 16) SP_MTTKRP_GROUP(4, 4, 2, 3);
+                else if (R <= 24) SP_MTTKRP_GROUP(4, 6, 2, 2);
+                else if (R <= 32) SP_MTTKRP_GROUP(8, 4, 2, 3);
+                else if (R <= 48) SP_MTTKRP_GROUP(8, 6, 2, 2);
+                else SP_MTTKRP_GROUP(16, 4, 2, 3);
+            } else {
+                if (R <= 8) SP_MTTKRP_GROUP(4, 2, 1, 6);
+                else if (R <= 16) SP_MTTKRP_GROUP(8, 2, 1, 6);
+                else if (R <= 24) SP_MTTKRP_GROUP(8, 3, 1, 3);
+                else if (R <= 32) SP_MTTKRP_GROUP(8, 4, 1, 3);
+                else if (R <= 48) SP_MTTKRP_GROUP(16, 3, 1, 3);
+                else SP_MTTKRP_GROUP(16, 4, 1, 3);
+            }
+        });
+#undef SP_MTTKRP_GROUP
+        SP_LAUNCH_CHECK();
+        sp_count_launches(1);
+        SP_BOUNDS_RETURN(stream);
+        return SP_OK;
+    }
     sp_partition part;
     // Entries per warp: enough warps for the GPU (two waves of 16 per SM) before long ranges.  38,175 entries 241 ->
     // 28 us, 451,180 entries 77 -> 38 us against 1,024 per warp throughout; 20 M entries: 256 543 us, 512 520,
     // 1,024 521; 5 M, R = 50: 512 312 us, 1,024 343.
     const int64_t per = std::max<int64_t>(32, std::min<int64_t>(512, sp_ceil_div(sp_ceil_div(nnz, 4736), 32) * 32));
-    sp_status st = sp_get_mttkrp_partition(T, per, stream, &part);
+    sp_status st = sp_get_mttkrp_partition(T, per, false, stream, &part);
     if (st != SP_OK) return st;
     const unsigned blocks = (unsigned)sp_ceil_div(part.nchunks * 32, fast ? kFThreads : kTThreads);
     if (fast) {

@@ -77,6 +77,75 @@ __global__ void k_max_segment(const P* __restrict__ pos, int64_t nseg, unsigned 
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
 }
 
+// MTTKRP's word per entry: level-1 coordinate of its fibre << 2 | "the fibre ends here".  A block takes a tile of
+// entries: two searches give the fibres that it touches, each of those marks its first entry, and an entry's fibre
+// is the last mark at or before it.
+constexpr int kMarkThreads = 256, kMarkTile = 1024;
+template <typename P, typename I>
+__global__ void __launch_bounds__(kMarkThreads)
+k_mttkrp_marks(const P* __restrict__ pos2, const I* __restrict__ crd1, int64_t nfiber, int64_t nnz, uint32_t* __restrict__ marks) {
+    __shared__ uint32_t s_at[kMarkTile + 1];
+    __shared__ int64_t s_range[2];
+    __shared__ uint32_t s_w[kMarkThreads / 32];
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const int64_t e0 = (int64_t)blockIdx.x * kMarkTile;
+    const int cnt = (int)(nnz - e0 < kMarkTile ? nnz - e0 : kMarkTile);
+    constexpr int kPer = kMarkTile / kMarkThreads;
+    for (int i = t; i <= kMarkTile; i += kMarkThreads) s_at[i] = 0u;
+    if (w < 2) {                                    // the fibres that hold the tile's first and last entry
+        const int64_t p = w ? e0 + cnt - 1 : e0;
+        int64_t lo = 0, hi = nfiber;
+        while (hi - lo > 1) {
+            const int64_t step = (hi - lo + 31) >> 5, q = lo + step * (int64_t)lane;
+            const unsigned m = __ballot_sync(0xffffffffu, q < hi && (int64_t)pos2[q] <= p);
+            const int64_t at = lo + step * (31 - __clz(m));
+            hi = at + step < hi ? at + step : hi;
+            lo = at;
+        }
+        if (lane == 0) s_range[w] = lo;
+    }
+    __syncthreads();
+    const int64_t f0 = s_range[0], f1 = s_range[1];
+    for (int64_t f = f0 + 1 + t; f <= f1; f += kMarkThreads) s_at[(int64_t)pos2[f] - e0] = (uint32_t)(f - f0);   // fibres are not empty
+    if (t == 0 && (int64_t)pos2[f1 + 1] == e0 + cnt) s_at[cnt] = 1u;
+    __syncthreads();
+    uint32_t m[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        m[i] = s_at[t * kPer + i];
+        if (i && m[i] < m[i - 1]) m[i] = m[i - 1];
+    }
+    uint32_t run = m[kPer - 1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o && u > run) run = u;
+    }
+    if (lane == 31) s_w[w] = run;
+    uint32_t before = __shfl_up_sync(0xffffffffu, run, 1);
+    if (lane == 0) before = 0;
+    __syncthreads();
+    for (int i = 0; i < w; ++i)
+        if (s_w[i] > before) before = s_w[i];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int e = t * kPer + i;
+        if (e < cnt) {
+            const uint32_t fo = m[i] > before ? m[i] : before;
+            marks[e0 + e] = (uint32_t)crd1[f0 + fo] << 2 | (s_at[e + 1] != 0u ? 1u : 0u);
+        }
+    }
+}
+
+// ... and | 2 at the last entry of every slice.
+template <typename P>
+__global__ void k_mttkrp_slice_marks(const P* __restrict__ pos1, const P* __restrict__ pos2, int64_t nslice, uint32_t* __restrict__ marks) {
+    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (s >= nslice) return;
+    const int64_t f0 = (int64_t)pos1[s], f1 = (int64_t)pos1[s + 1];
+    if (f1 > f0) marks[(int64_t)pos2[f1] - 1] |= 2u;
+}
+
 }  // namespace
 
 sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out) {
@@ -218,9 +287,9 @@ sp_status sp_widened(sp_tensor* t, cudaStream_t stream, sp_tensor** out) {
     return SP_OK;
 }
 
-sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, cudaStream_t stream, sp_partition* out) {
+sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, bool with_marks, cudaStream_t stream, sp_partition* out) {
     std::lock_guard<std::mutex> lock(t->mu);
-    const uint64_t key = ((uint64_t)SP_PART_MTTKRP << 56) | (uint64_t)per;
+    const uint64_t key = ((uint64_t)(with_marks ? SP_PART_MTTKRP_MARKS : SP_PART_MTTKRP) << 56) | (uint64_t)per;
     auto it = t->parts.find(key);
     if (it != t->parts.end()) { *out = it->second; return SP_OK; }
     const int64_t nnz = t->ncrd[2];
@@ -232,8 +301,9 @@ sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, cudaStream_t stream
     p.row = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
     p.nz = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
     p.aux = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
-    auto drop = [&](sp_status s) { sp_dev_free(p.row, stream); sp_dev_free(p.nz, stream); sp_dev_free(p.aux, stream); return s; };
-    if (!p.row || !p.nz || !p.aux) return drop(SP_ERR_ALLOC);
+    if (with_marks) p.marks = static_cast<uint32_t*>(sp_dev_alloc((size_t)(nnz ? nnz : 1) * sizeof(uint32_t), stream));
+    auto drop = [&](sp_status s) { sp_dev_free(p.row, stream); sp_dev_free(p.nz, stream); sp_dev_free(p.aux, stream); sp_dev_free(p.marks, stream); return s; };
+    if (!p.row || !p.nz || !p.aux || (with_marks && !p.marks)) return drop(SP_ERR_ALLOC);
     const unsigned blocks = (unsigned)sp_ceil_div(p.nchunks + 1, 256);
     if (t->posBits == 32)
         k_mttkrp_partition<uint32_t><<<blocks, 256, 0, stream>>>(
@@ -243,6 +313,15 @@ sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, cudaStream_t stream
         k_mttkrp_partition<uint64_t><<<blocks, 256, 0, stream>>>(
             static_cast<const uint64_t*>(t->pos[1]), nslice, static_cast<const uint64_t*>(t->pos[2]), nfiber, nnz, per,
             p.nchunks, p.row, p.nz, p.aux);
+    if (with_marks && nnz > 0) {
+        SP_DISPATCH_WIDTHS(t, {
+            k_mttkrp_marks<P, I><<<(unsigned)sp_ceil_div(nnz, kMarkTile), kMarkThreads, 0, stream>>>(
+                static_cast<const P*>(t->pos[2]), static_cast<const I*>(t->crd[1]), nfiber, nnz, p.marks);
+            k_mttkrp_slice_marks<P><<<(unsigned)sp_ceil_div(nslice, 256), 256, 0, stream>>>(static_cast<const P*>(t->pos[1]),
+                                                                                           static_cast<const P*>(t->pos[2]), nslice, p.marks);
+        });
+        sp_count_launches(2);
+    }
     if (cudaGetLastError() != cudaSuccess) return drop(SP_ERR_CUDA);
     sp_count_launches(1);
     if (sp_partition_built(stream) != SP_OK) return drop(SP_ERR_CUDA);
