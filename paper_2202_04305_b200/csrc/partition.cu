@@ -77,73 +77,127 @@ __global__ void k_max_segment(const P* __restrict__ pos, int64_t nseg, unsigned 
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
 }
 
-// MTTKRP's word per entry: level-1 coordinate of its fibre << 2 | "the fibre ends here".  A block takes a tile of
-// entries: two searches give the fibres that it touches, each of those marks its first entry, and an entry's fibre
-// is the last mark at or before it.
-constexpr int kMarkThreads = 256, kMarkTile = 1024;
-template <typename P, typename I>
-__global__ void __launch_bounds__(kMarkThreads)
-k_mttkrp_marks(const P* __restrict__ pos2, const I* __restrict__ crd1, int64_t nfiber, int64_t nnz, uint32_t* __restrict__ marks) {
-    __shared__ uint32_t s_at[kMarkTile + 1];
-    __shared__ int64_t s_range[2];
-    __shared__ uint32_t s_w[kMarkThreads / 32];
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const int64_t e0 = (int64_t)blockIdx.x * kMarkTile;
-    const int cnt = (int)(nnz - e0 < kMarkTile ? nnz - e0 : kMarkTile);
-    constexpr int kPer = kMarkTile / kMarkThreads;
-    for (int i = t; i <= kMarkTile; i += kMarkThreads) s_at[i] = 0u;
-    if (w < 2) {                                    // the fibres that hold the tile's first and last entry
-        const int64_t p = w ? e0 + cnt - 1 : e0;
-        int64_t lo = 0, hi = nfiber;
-        while (hi - lo > 1) {
-            const int64_t step = (hi - lo + 31) >> 5, q = lo + step * (int64_t)lane;
-            const unsigned m = __ballot_sync(0xffffffffu, q < hi && (int64_t)pos2[q] <= p);
-            const int64_t at = lo + step * (31 - __clz(m));
-            hi = at + step < hi ? at + step : hi;
-            lo = at;
-        }
-        if (lane == 0) s_range[w] = lo;
+// Last i in [0, n) with pos[i] <= v (pos[0] <= v < pos[n]), by a whole warp: 32 probes a round.
+template <typename P>
+__device__ __forceinline__ int64_t warp_last_le(const P* __restrict__ pos, int64_t n, int64_t v) {
+    int64_t lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) >> 5, i = lo + ((threadIdx.x & 31) + 1) * step;
+        const int le = __popc(__ballot_sync(0xffffffffu, i < hi && (int64_t)pos[i] <= v));
+        lo += le * step;
+        hi = lo + step < hi ? lo + step : hi;
     }
-    __syncthreads();
-    const int64_t f0 = s_range[0], f1 = s_range[1];
-    for (int64_t f = f0 + 1 + t; f <= f1; f += kMarkThreads) s_at[(int64_t)pos2[f] - e0] = (uint32_t)(f - f0);   // fibres are not empty
-    if (t == 0 && (int64_t)pos2[f1 + 1] == e0 + cnt) s_at[cnt] = 1u;
-    __syncthreads();
-    uint32_t m[kPer];
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        m[i] = s_at[t * kPer + i];
-        if (i && m[i] < m[i - 1]) m[i] = m[i - 1];
-    }
-    uint32_t run = m[kPer - 1];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t u = __shfl_up_sync(0xffffffffu, run, o);
-        if (lane >= o && u > run) run = u;
-    }
-    if (lane == 31) s_w[w] = run;
-    uint32_t before = __shfl_up_sync(0xffffffffu, run, 1);
-    if (lane == 0) before = 0;
-    __syncthreads();
-    for (int i = 0; i < w; ++i)
-        if (s_w[i] > before) before = s_w[i];
-#pragma unroll
-    for (int i = 0; i < kPer; ++i) {
-        const int e = t * kPer + i;
-        if (e < cnt) {
-            const uint32_t fo = m[i] > before ? m[i] : before;
-            marks[e0 + e] = (uint32_t)crd1[f0 + fo] << 2 | (s_at[e + 1] != 0u ? 1u : 0u);
-        }
-    }
+    return lo;
 }
 
-// ... and | 2 at the last entry of every slice.
-template <typename P>
-__global__ void k_mttkrp_slice_marks(const P* __restrict__ pos1, const P* __restrict__ pos2, int64_t nslice, uint32_t* __restrict__ marks) {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= nslice) return;
-    const int64_t f0 = (int64_t)pos1[s], f1 = (int64_t)pos1[s + 1];
-    if (f1 > f0) marks[(int64_t)pos2[f1] - 1] |= 2u;
+// MTTKRP's word per entry, level-1 coordinate of its fibre << 2 | "the slice ends here" << 1 | "the fibre ends here",
+// and the slice that every chunk begins in, with its row.  A block takes a run of tiles of whole chunks: two warps
+// look up the fibres and slices at its ends, then each fibre of a tile marks its first entry and an entry's fibre is
+// the last mark at or before it, the next tile's fibres being on their way meanwhile.  The look-up is a chain of
+// some ten loads: 20 M entries 112 us with a block per tile, 77 with one wave of blocks (for 250 MB read and written).
+// The slices of chunks are looked up after the last tile: inside the loop that took 25 us more.
+constexpr int kMarkThreads = 256, kMarkTile = 1024, kMarkBlocks = 148 * 6;
+template <typename P, typename I>
+__global__ void __launch_bounds__(kMarkThreads, 6)
+k_mttkrp_marks(const P* __restrict__ pos1, const I* __restrict__ crd0, int64_t nslice, const P* __restrict__ pos2,
+               const I* __restrict__ crd1, int64_t nfiber, int64_t nnz, int64_t per, int64_t nchunks, int64_t chunks,
+               int64_t* __restrict__ chunk_slice, int64_t* __restrict__ chunk_row, uint32_t* __restrict__ marks) {
+    constexpr int kPer = 4;
+    static_assert(kMarkTile == kPer * kMarkThreads, "a thread owns four entries");
+    __shared__ uint4 s_at4[kMarkTile / 4 + 1];
+    __shared__ uint32_t s_crd[kMarkTile];
+    __shared__ uint32_t s_w[kMarkThreads / 32];
+    __shared__ int64_t s_f[2], s_s[2];
+    uint32_t* const s_at = reinterpret_cast<uint32_t*>(s_at4);
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const int64_t c0 = blockIdx.x * chunks, c1 = c0 + chunks < nchunks ? c0 + chunks : nchunks;
+    const int64_t e1 = c1 * per < nnz ? c1 * per : nnz;
+    const int tile = kMarkTile / (int)per * (int)per;
+    int64_t e0 = c0 * per;
+    if (w < 2) {
+        const int64_t e = w ? e1 : e0;
+        const int64_t f = e < nnz ? warp_last_le(pos2, nfiber, e) : nfiber;
+        const int64_t q = f < nfiber ? warp_last_le(pos1, nslice, f) : nslice - 1;
+        if (lane == 0) { s_f[w] = f; s_s[w] = q; }
+    }
+    __syncthreads();
+    int64_t f0 = s_f[0];
+    const int64_t s0 = s_s[0], s1 = s_s[1], fend = s_f[1] + 1 < nfiber ? s_f[1] + 1 : nfiber;
+    uint32_t cr[kPer];
+    int64_t next[kPer];
+    auto load = [&]() {                     // fibres are not empty: kMarkTile of them reach past any tile
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int64_t f = f0 + t + k * kMarkThreads;
+            cr[k] = f < fend ? (uint32_t)crd1[f] : 0u;
+            next[k] = f < fend ? (int64_t)pos2[f + 1] : nnz + 1 + kMarkTile;
+        }
+    };
+    load();
+    for (; e0 < e1; e0 += tile) {
+        const int cnt = (int)(e1 - e0 < tile ? e1 - e0 : tile);
+        s_at4[t] = make_uint4(0u, 0u, 0u, 0u);
+        if (t == 0) s_at[kMarkTile] = 0u;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            s_crd[t + k * kMarkThreads] = cr[k];
+            if (next[k] - e0 <= cnt) s_at[next[k] - e0] = (uint32_t)(t + k * kMarkThreads + 1);
+        }
+        __syncthreads();
+        const uint4 q = s_at4[t];
+        const uint32_t here[kPer + 1] = {q.x, q.y, q.z, q.w, s_at[t * kPer + kPer]};
+        uint32_t m[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) m[i] = i && here[i] < m[i - 1] ? m[i - 1] : here[i];
+        uint32_t run = m[kPer - 1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o && u > run) run = u;
+        }
+        if (lane == 31) s_w[w] = run;
+        uint32_t before = __shfl_up_sync(0xffffffffu, run, 1);
+        if (lane == 0) before = 0;
+        __syncthreads();
+        uint32_t nf = s_at[kMarkTile];      // fibres that end in the tile
+#pragma unroll
+        for (int i = 0; i < kMarkThreads / 32; ++i) {
+            const uint32_t u = s_w[i];
+            if (i < w && u > before) before = u;
+            if (u > nf) nf = u;
+        }
+        const int64_t ft = f0;
+        f0 += nf;
+        if (e0 + tile < e1) load();
+        uint32_t word[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const uint32_t fo = m[i] > before ? m[i] : before;
+            word[i] = t * kPer + i < cnt ? s_crd[fo] << 2 | (here[i + 1] != 0u ? 1u : 0u) : 0u;
+        }
+        if (t * kPer + kPer <= cnt)
+            reinterpret_cast<uint4*>(marks + e0)[t] = make_uint4(word[0], word[1], word[2], word[3]);
+        else
+            for (int i = 0; t * kPer + i < cnt; ++i) marks[e0 + t * kPer + i] = word[i];
+        if (t * kPer < cnt && t * kPer % (int)per == 0)             // chunks are multiples of four entries
+            chunk_slice[e0 / per + t * kPer / (int)per] = ft + (m[0] > before ? m[0] : before);     // the fibre, for now
+        __syncthreads();
+    }
+    for (int64_t c = c0 + t; c < c1; c += kMarkThreads) {
+        const int64_t f = chunk_slice[c];
+        int64_t lo = s0, hi = s1 + 1;
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((int64_t)pos1[mid] <= f) lo = mid; else hi = mid;
+        }
+        chunk_slice[c] = lo;
+        chunk_row[c] = crd0 ? (int64_t)crd0[lo] : lo;
+    }
+    for (int64_t q = s0 + t; q <= s1; q += kMarkThreads) {          // the last entry of every slice, once the words are written
+        const int64_t f = (int64_t)pos1[q + 1];
+        if (f > (int64_t)pos1[q] && (int64_t)pos2[f] <= e1) marks[(int64_t)pos2[f] - 1] |= 2u;
+    }
 }
 
 }  // namespace
@@ -298,30 +352,25 @@ sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, bool with_marks, cu
     sp_partition p;
     p.nchunks = sp_ceil_div(nnz, per);
     if (p.nchunks < 1) p.nchunks = 1;
+    // With marks a chunk's entries are known, per of them from chunk * per on, and row is the row of M it begins in.
     p.row = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
-    p.nz = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
     p.aux = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
     if (with_marks) p.marks = static_cast<uint32_t*>(sp_dev_alloc((size_t)(nnz ? nnz : 1) * sizeof(uint32_t), stream));
+    else p.nz = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
     auto drop = [&](sp_status s) { sp_dev_free(p.row, stream); sp_dev_free(p.nz, stream); sp_dev_free(p.aux, stream); sp_dev_free(p.marks, stream); return s; };
-    if (!p.row || !p.nz || !p.aux || (with_marks && !p.marks)) return drop(SP_ERR_ALLOC);
+    if (!p.row || !p.aux || (with_marks ? !p.marks : !p.nz)) return drop(SP_ERR_ALLOC);
     const unsigned blocks = (unsigned)sp_ceil_div(p.nchunks + 1, 256);
-    if (t->posBits == 32)
-        k_mttkrp_partition<uint32_t><<<blocks, 256, 0, stream>>>(
-            static_cast<const uint32_t*>(t->pos[1]), nslice, static_cast<const uint32_t*>(t->pos[2]), nfiber, nnz, per,
-            p.nchunks, p.row, p.nz, p.aux);
-    else
-        k_mttkrp_partition<uint64_t><<<blocks, 256, 0, stream>>>(
-            static_cast<const uint64_t*>(t->pos[1]), nslice, static_cast<const uint64_t*>(t->pos[2]), nfiber, nnz, per,
-            p.nchunks, p.row, p.nz, p.aux);
-    if (with_marks && nnz > 0) {
-        SP_DISPATCH_WIDTHS(t, {
-            k_mttkrp_marks<P, I><<<(unsigned)sp_ceil_div(nnz, kMarkTile), kMarkThreads, 0, stream>>>(
-                static_cast<const P*>(t->pos[2]), static_cast<const I*>(t->crd[1]), nfiber, nnz, p.marks);
-            k_mttkrp_slice_marks<P><<<(unsigned)sp_ceil_div(nslice, 256), 256, 0, stream>>>(static_cast<const P*>(t->pos[1]),
-                                                                                           static_cast<const P*>(t->pos[2]), nslice, p.marks);
-        });
-        sp_count_launches(2);
-    }
+    const int64_t in_tile = kMarkTile / per, run = sp_ceil_div(sp_ceil_div(p.nchunks, in_tile), kMarkBlocks) * in_tile;
+    SP_DISPATCH_WIDTHS(t, {
+        const P* const pos1 = static_cast<const P*>(t->pos[1]);
+        const P* const pos2 = static_cast<const P*>(t->pos[2]);
+        if (!with_marks)
+            k_mttkrp_partition<P><<<blocks, 256, 0, stream>>>(pos1, nslice, pos2, nfiber, nnz, per, p.nchunks, p.row, p.nz, p.aux);
+        else if (nnz > 0)
+            k_mttkrp_marks<P, I><<<(unsigned)sp_ceil_div(p.nchunks, run), kMarkThreads, 0, stream>>>(
+                pos1, t->lt[0] == SP_COMPRESSED ? static_cast<const I*>(t->crd[0]) : nullptr, nslice, pos2,
+                static_cast<const I*>(t->crd[1]), nfiber, nnz, per, p.nchunks, run, p.aux, p.row, p.marks);
+    });
     if (cudaGetLastError() != cudaSuccess) return drop(SP_ERR_CUDA);
     sp_count_launches(1);
     if (sp_partition_built(stream) != SP_OK) return drop(SP_ERR_CUDA);
