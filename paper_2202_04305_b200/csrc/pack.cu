@@ -87,11 +87,15 @@ constexpr int kSortThreads = 256;
 #ifndef SP_SORT_PAY_BLOCKS
 #define SP_SORT_PAY_BLOCKS 4
 #endif
-template <bool PAY>
+// Few entries (up to kFewTiles tiles of 1024 keys, index in the key): 4 keys per thread, for more blocks and a
+// shorter chain of ranking rounds (30,000 entries of a rank-3 tensor: pack 76 us; 8 keys 80, 2 keys 80).
+enum { kShapeIndex, kShapeValue, kShapeSmall };     // index in the key; value beside the key; index in the key, few entries
+template <int S>
 struct SortShape {
-    static constexpr int kIpt = PAY ? SP_SORT_PAY_IPT : 16;
+    static constexpr bool kPay = S == kShapeValue;
+    static constexpr int kIpt = S == kShapeValue ? SP_SORT_PAY_IPT : S == kShapeSmall ? 4 : 16;
     static constexpr int kTile = kSortThreads * kIpt;
-    static constexpr int kMinBlocks = PAY ? SP_SORT_PAY_BLOCKS : 3;
+    static constexpr int kMinBlocks = S == kShapeValue ? SP_SORT_PAY_BLOCKS : 3;
 };
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kMaxRadix = 256;
@@ -102,11 +106,11 @@ constexpr int kMaxRadix = 256;
 // idx_bits > 0: the entry index rides in the low idx_bits bits of the key itself (the sort then
 // moves 8 bytes per entry).  Otherwise the entry's value travels beside its key from the first
 // pass on (which reads it from the input, where value e belongs to key e), so no index exists.
-template <typename CT, bool PAY>
+template <typename CT, int S>
 __global__ void __launch_bounds__(kSortThreads)
 k_build_keys(LevelCoords lc, int64_t n, LevelPlan p, uint64_t* keys, int idx_bits, int* err,
              int shift0, uint32_t mask0, uint32_t* __restrict__ tilehist, int64_t ntiles) {
-    constexpr int kSortIpt = SortShape<PAY>::kIpt, kSortTile = SortShape<PAY>::kTile;
+    constexpr int kSortIpt = SortShape<S>::kIpt, kSortTile = SortShape<S>::kTile;
     __shared__ uint32_t hist[kSortWarps][kMaxRadix];
     const int t = threadIdx.x, w = t >> 5;
     for (int i = t; i < kSortWarps * kMaxRadix; i += kSortThreads) (&hist[0][0])[i] = 0;
@@ -197,11 +201,11 @@ __device__ __forceinline__ uint32_t block256_excl_scan(uint32_t v, uint32_t* sum
 // Counting them inside the previous pass's scatter, with global atomics where the keys land, was
 // measured: skewed digits pile onto few counters and the 20,000,000-entry scatter went from 0.145 ms
 // to 0.59 ms per pass.
-template <int BITS, bool PAY>
+template <int BITS, int S>
 __global__ void __launch_bounds__(kSortThreads)
 k_sort_upsweep(const uint64_t* keys, int64_t n, int shift, uint32_t* __restrict__ tilehist, int64_t ntiles) {
     sp_wait_for_previous_kernel();
-    constexpr int kSortIpt = SortShape<PAY>::kIpt, kSortTile = SortShape<PAY>::kTile;
+    constexpr int kSortIpt = SortShape<S>::kIpt, kSortTile = SortShape<S>::kTile;
     constexpr int RADIX = 1 << BITS;
     constexpr uint32_t mask = RADIX - 1;
     __shared__ uint32_t hist[kSortWarps][RADIX];     // one histogram per warp: conflicts only inside a warp
@@ -300,9 +304,15 @@ k_sort_scan(uint32_t* tilehist, int64_t ntiles, int64_t nchunks, const uint32_t*
     if (threadIdx.x == 0 && blockIdx.y == nchunks - 1) digit_total[blockIdx.x] = before + tot;
 }
 
-constexpr size_t down_smem(bool pay, int bits) {
-    return (size_t)(pay ? SortShape<true>::kTile : SortShape<false>::kTile) * (pay ? 16 : 8) + (size_t)kSortWarps * ((1 << bits) + 1) * 4 +
-           (size_t)(1 << bits) * 4 + 64;
+// Up to so many tiles need no scan kernels: a scatter block adds up its digits' tile counts itself, a thread per
+// digit (packs of 30,000, 60,000 and 100,000 entries 97 -> 76, 109 -> 85, 102 -> 92 us with the small tiles above;
+// with 128 tiles 300,000 and 500,000 entries get slower, 113 -> 116 and 112 -> 151).
+constexpr int64_t kFewTiles = 64;
+static_assert(kMaxRadix <= kSortThreads, "a thread per digit");
+
+template <int S, int BITS>
+constexpr size_t down_smem() {
+    return (size_t)SortShape<S>::kTile * (SortShape<S>::kPay ? 16 : 8) + (size_t)kSortWarps * ((1 << BITS) + 1) * 4 + (size_t)(1 << BITS) * 4 + 64;
 }
 
 // Ranks the warp's rounds of 32 keys: rank i = number of earlier keys of this warp with the same
@@ -332,15 +342,16 @@ __device__ __forceinline__ void rank_rounds(const uint64_t (&key)[kSortIpt], int
 // PAY: a 64-bit payload (the entry's value, moved as bits) travels beside every key.  Without it the
 // entry index sits in the key's low bits; the last pass (split_bits >= 0) then separates the two again
 // on the way out: keys_out gets key >> split_bits, idx_out the low split_bits bits.
-template <bool PAY, int BITS>
-__global__ void __launch_bounds__(kSortThreads, SortShape<PAY>::kMinBlocks)   // several tiles per SM hide the ranking chain's latency
+template <int S, int BITS>
+__global__ void __launch_bounds__(kSortThreads, SortShape<S>::kMinBlocks)   // several tiles per SM hide the ranking chain's latency
 k_sort_downsweep(const uint64_t* keys_in, const uint64_t* pay_in,
                  uint64_t* __restrict__ keys_out, uint64_t* __restrict__ pay_out, uint32_t* __restrict__ idx_out,
                  int64_t n, int shift,
                  const uint32_t* tilehist, int64_t ntiles,
                  const uint32_t* digit_total, int split_bits) {
     sp_wait_for_previous_kernel();
-    constexpr int kSortIpt = SortShape<PAY>::kIpt, kSortTile = SortShape<PAY>::kTile;
+    constexpr bool PAY = SortShape<S>::kPay;
+    constexpr int kSortIpt = SortShape<S>::kIpt, kSortTile = SortShape<S>::kTile;
     constexpr int RADIX = 1 << BITS;
     constexpr uint32_t mask = RADIX - 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -368,6 +379,16 @@ k_sort_downsweep(const uint64_t* keys_in, const uint64_t* pay_in,
 #ifdef SP_SORT_PAY_EARLY
         if (PAY) pay[i] = li < tile_n ? pay_in[base + li] : 0;
 #endif
+    }
+    uint32_t few_before = 0, few_total = 0;          // few tiles: this thread's digit in the tiles before this one, and in all
+    if (!digit_total && t < RADIX) {
+        const uint32_t* row = tilehist + (int64_t)t * ntiles;
+#pragma unroll 8
+        for (int q = 0; q < (int)ntiles; ++q) {
+            const uint32_t c = row[q];
+            few_total += c;
+            if (q < (int)blockIdx.x) few_before += c;
+        }
     }
     if (tile_n == kSortTile) rank_rounds<BITS, BITS, kSortIpt>(key, shift, w, lane, tile_n, mycnt, rank);
     else rank_rounds<BITS, BITS + 1, kSortIpt>(key, shift, w, lane, tile_n, mycnt, rank);
@@ -401,7 +422,7 @@ k_sort_downsweep(const uint64_t* keys_in, const uint64_t* pay_in,
                 run += c;
             }
             tot_d[q] = run;
-            gtot_d[q] = digit_total[d];
+            gtot_d[q] = digit_total ? digit_total[d] : few_total;
         }
         mine += tot_d[q];
         gmine += gtot_d[q];
@@ -425,7 +446,7 @@ k_sort_downsweep(const uint64_t* keys_in, const uint64_t* pay_in,
             // key needs one table look-up
             for (int ww = 0; ww < kSortWarps; ++ww) wcnt[ww * (RADIX + 1) + d] += ex;
             // global base of digit d = totals of smaller digits + this tile's prefix within the digit
-            goff[d] = gex + tilehist[(int64_t)d * ntiles + blockIdx.x] - ex;
+            goff[d] = gex + (digit_total ? tilehist[(int64_t)d * ntiles + blockIdx.x] : few_before) - ex;
             ex += tot_d[q];
             gex += gtot_d[q];
         }
@@ -463,17 +484,19 @@ k_sort_downsweep(const uint64_t* keys_in, const uint64_t* pay_in,
 
 // One radix pass (tile histograms unless they exist already, per-digit scans, ranked scatter) for a
 // digit of BITS bits at `shift`.
-template <int BITS>
+template <int S, int BITS>
 sp_status sort_pass(const uint64_t* kin, const uint64_t* pin, uint64_t* kout, uint64_t* pout, uint32_t* iout, int64_t n, int shift,
-                    uint32_t* tilehist, int64_t stiles, uint32_t* digit_total, uint32_t* chunk_tot, bool fused, int split_bits,
+                    uint32_t* tilehist, int64_t stiles, uint32_t* digit_total, uint32_t* chunk_tot, int split_bits,
                     bool have_hist, cudaStream_t stream, PhaseTimer& timer) {
     if (!have_hist) {
-        if (fused) SP_CUDA(sp_launch_dependent(k_sort_upsweep<BITS, false>, dim3((unsigned)stiles), dim3(kSortThreads), 0, stream, kin, n, shift, tilehist, stiles));
-        else SP_CUDA(sp_launch_dependent(k_sort_upsweep<BITS, true>, dim3((unsigned)stiles), dim3(kSortThreads), 0, stream, kin, n, shift, tilehist, stiles));
+        SP_CUDA(sp_launch_dependent(k_sort_upsweep<BITS, S>, dim3((unsigned)stiles), dim3(kSortThreads), 0, stream, kin, n, shift, tilehist, stiles));
         sp_count_launches(1);
     }
     timer.mark(kPhUpsweep);
-    {
+    const bool few = stiles <= kFewTiles;
+    if (few) {
+        digit_total = nullptr;
+    } else {
         const int64_t nchunks = sp_ceil_div(stiles, kScanChunk);
         dim3 grid(1u << BITS, (unsigned)nchunks);
         if (nchunks > 1) {
@@ -481,24 +504,15 @@ sp_status sort_pass(const uint64_t* kin, const uint64_t* pin, uint64_t* kout, ui
             sp_count_launches(1);
         }
         SP_CUDA(sp_launch_dependent(k_sort_scan, grid, dim3(256), 0, stream, tilehist, stiles, nchunks, chunk_tot, digit_total));
+        sp_count_launches(1);
     }
     timer.mark(kPhScan);
-    if (fused) {
-        SP_CUDA(cudaFuncSetAttribute(k_sort_downsweep<false, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)down_smem(false, BITS)));
-        SP_CUDA(sp_launch_dependent(k_sort_downsweep<false, BITS>, dim3((unsigned)stiles), dim3(kSortThreads), down_smem(false, BITS), stream,
-                                 kin, (const uint64_t*)nullptr, kout, (uint64_t*)nullptr, iout, n, shift, (const uint32_t*)tilehist, stiles,
-                                 (const uint32_t*)digit_total, split_bits));
-    } else {
-        SP_CUDA(cudaFuncSetAttribute(k_sort_downsweep<true, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)down_smem(true, BITS)));
-        SP_CUDA(sp_launch_dependent(k_sort_downsweep<true, BITS>, dim3((unsigned)stiles), dim3(kSortThreads), down_smem(true, BITS), stream,
-                                 kin, pin, kout, pout, (uint32_t*)nullptr, n, shift, (const uint32_t*)tilehist, stiles,
-                                 (const uint32_t*)digit_total, -1));
-    }
+    SP_CUDA(cudaFuncSetAttribute(k_sort_downsweep<S, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)down_smem<S, BITS>()));
+    SP_CUDA(sp_launch_dependent(k_sort_downsweep<S, BITS>, dim3((unsigned)stiles), dim3(kSortThreads), down_smem<S, BITS>(), stream, kin, pin, kout,
+                                pout, iout, n, shift, (const uint32_t*)tilehist, stiles, (const uint32_t*)digit_total, split_bits));
     SP_LAUNCH_CHECK();
     timer.mark(kPhDownsweep);
-    sp_count_launches(2);
+    sp_count_launches(1);
     return SP_OK;
 }
 
@@ -1041,7 +1055,9 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
         int idx_bits = 0;
         while (((int64_t)1 << idx_bits) < n) ++idx_bits;
         const bool fused = npasses > 0 && idx_bits > 0 && total_bits + idx_bits <= 64;
-        const int64_t stiles = sp_ceil_div(n, fused ? SortShape<false>::kTile : SortShape<true>::kTile);
+        const int shape = !fused ? kShapeValue : n <= kFewTiles * SortShape<kShapeSmall>::kTile ? kShapeSmall : kShapeIndex;
+        const int64_t stiles = sp_ceil_div(n, shape == kShapeValue ? SortShape<kShapeValue>::kTile
+                                              : shape == kShapeSmall ? SortShape<kShapeSmall>::kTile : SortShape<kShapeIndex>::kTile);
         ct_tiles = sp_ceil_div(n, kCtTile);
         const size_t nscan = (size_t)sp_ceil_div(stiles, kScanChunk) << kMaxDigitBits;
         // every buffer of the pack in one allocation
@@ -1078,11 +1094,12 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
         }
         const int shift0 = npasses ? shifts[0] : 0;
         const uint32_t mask0 = npasses ? (1u << widths[0]) - 1u : 0u;
-#define SP_BUILD_KEYS(CT, PAY)                                                                                       \
-    k_build_keys<CT, PAY><<<(unsigned)stiles, kSortThreads, 0, stream>>>(lc, n, plan, kbuf[0], fused ? idx_bits : 0,         \
+#define SP_BUILD_KEYS(CT, S)                                                                                       \
+    k_build_keys<CT, S><<<(unsigned)stiles, kSortThreads, 0, stream>>>(lc, n, plan, kbuf[0], fused ? idx_bits : 0,         \
                                                                         d_err, shift0, mask0, tilehist, stiles)
-        if (coo_coord_bits == 32) { if (fused) SP_BUILD_KEYS(int32_t, false); else SP_BUILD_KEYS(int32_t, true); }
-        else { if (fused) SP_BUILD_KEYS(int64_t, false); else SP_BUILD_KEYS(int64_t, true); }
+        if (shape == kShapeValue) { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeValue); else SP_BUILD_KEYS(int64_t, kShapeValue); }
+        else if (shape == kShapeSmall) { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeSmall); else SP_BUILD_KEYS(int64_t, kShapeSmall); }
+        else { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeIndex); else SP_BUILD_KEYS(int64_t, kShapeIndex); }
 #undef SP_BUILD_KEYS
         SP_LAUNCH_CHECK();
         sp_count_launches(1);
@@ -1092,17 +1109,20 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
             const bool last = ps == npasses - 1;
             const int split = (fused && last) ? idx_bits : -1;
             sp_status ps_st = SP_ERR_UNSUPPORTED;
+#define SP_SORT_PASS_OF(S, B)                                                                                       \
+    sort_pass<S, B>(kbuf[cur], ps == 0 ? reinterpret_cast<const uint64_t*>(coo_vals) : pbuf[cur], kbuf[cur ^ 1],     \
+                    pbuf[cur ^ 1], isorted, n, shifts[ps], tilehist, stiles, digit_total, chunk_tot, split, ps == 0, stream, timer)
 #define SP_SORT_PASS(B)                                                                                             \
     case B:                                                                                                         \
-        ps_st = sort_pass<B>(kbuf[cur], ps == 0 ? reinterpret_cast<const uint64_t*>(coo_vals) : pbuf[cur],          \
-                             kbuf[cur ^ 1], pbuf[cur ^ 1], isorted, n, shifts[ps], tilehist, stiles,                 \
-                             digit_total, chunk_tot, fused, split, ps == 0, stream, timer);                          \
+        ps_st = shape == kShapeValue ? SP_SORT_PASS_OF(kShapeValue, B)                                               \
+                : shape == kShapeSmall ? SP_SORT_PASS_OF(kShapeSmall, B) : SP_SORT_PASS_OF(kShapeIndex, B);          \
         break;
             switch (widths[ps]) {
                 SP_SORT_PASS(1) SP_SORT_PASS(2) SP_SORT_PASS(3) SP_SORT_PASS(4) SP_SORT_PASS(5)
                 SP_SORT_PASS(6) SP_SORT_PASS(7) SP_SORT_PASS(8)
             }
 #undef SP_SORT_PASS
+#undef SP_SORT_PASS_OF
             if (ps_st != SP_OK) return ps_st;
             cur ^= 1;
         }
