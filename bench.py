@@ -239,9 +239,9 @@ def secondary_bounds(probes, torch, model):
 NCU_LEVELS = {
     "spmm_dcsr": {"lts_bytes": 2.402e9, "dram_bytes": 1.211e9, "source": "profiles/spmv_spmm_sddmm_full_configs.md"},
     "spmv_dcsr": {"lts_bytes": 333.8e6, "dram_bytes": 71.6e6, "source": "profiles/spmv_spmm_sddmm_full_configs.md"},
-    "spmm_csr": {"lts_bytes": 0.672e9, "dram_bytes": 63.0e6, "source": "profiles/spmv_spmm_sddmm_full_configs.md"},
-    "sddmm_csr": {"lts_bytes": 3.070e9, "dram_bytes": 1.186e9, "source": "profiles/spmv_spmm_sddmm_full_configs.md"},
-    "mttkrp_csf": {"lts_bytes": 3.679e9, "dram_bytes": 0.2944e9, "source": "profiles/k_mttkrp_16384cube_20M.md"},
+    "spmm_csr": {"lts_bytes": 0.671e9, "dram_bytes": 58.9e6, "source": "profiles/lane_group_kernels_full_configs.md"},
+    "sddmm_csr": {"lts_bytes": 3.160e9, "dram_bytes": 1.219e9, "source": "profiles/lane_group_kernels_full_configs.md"},
+    "mttkrp_csf": {"lts_bytes": 4.360e9, "dram_bytes": 0.3410e9, "source": "profiles/lane_group_kernels_full_configs.md"},
 }
 
 
