@@ -1,13 +1,13 @@
 // sp_pack for matrices with a compressed inner level and moderate segments (rows of CSR and DCSR, columns of
 // CSC and DCSC): no sort by key, the entries pass through memory twice.
 //
-//   1. k_rows_partition  range check; entries into buckets, one per range of outer indices, in any order
+//   1. k_rows_partition  (k_rows_partition_tiles from 300,000 entries on) range check; entries into buckets, one per range of outer indices, in any order
 //   2. k_rows_build      a block per bucket: entries per outer index, order inside every segment, and
 //                        everything the bucket contributes to the storage, written in order
 //   3. k_rows_outer      (compressed outer level) the buckets' lists of stored outer indices, joined
 //
 // Buckets hold about kAverage entries and at most kCap.  Random accesses are what a GPU is slow at (about 140 G
-// single-lane accesses/s here, hit or miss): this way an entry costs one, its 16-byte store in step 1; every
+// single-lane accesses/s here, hit or miss): this way an entry costs at most one, its 16-byte store in step 1; every
 // other scattered access stays in shared memory.  Sizes are known beforehand (a compressed outer level's are
 // bounded), so the one read-back comes at the end.  A bucket that overflows (long or very uneven segments)
 // and duplicate coordinates, whose values have to be summed, are found on the device; the kernels after that
@@ -147,6 +147,104 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
             rec[(size_t)b * kCap + s_hist[b] + r[i]] =
                 make_uint4((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), (uint32_t)c[i], (uint32_t)o[i]);
         }
+    }
+}
+
+// The same for large inputs, the tile being put in order by bucket in shared memory first: a bucket's entries then
+// leave side by side and one store instruction touches fewer lines, and the values, requested with the coordinates,
+// are no longer waited for at the end.  5 M entries: pack 190 us, 205 with every entry stored from where it was
+// read; 1.5 M with 64-bit coordinates (convert) 98 against 106; 2.5 M 128 against 146.  Tiles of 4096 entries spill
+// (188, 102), 1024 threads with 6 entries each 190, 98, 8 entries 192, 102, three blocks per SM 204, 103.
+constexpr int kTIpt = 6, kTTile = kThreads * kTIpt;
+struct TileShared {
+    Rec rec[kTTile];
+    uint32_t count[kMaxBuckets];                // entries of the tile, then where they begin in rec
+    uint32_t shift[kMaxBuckets];                // place in the bucket minus place in rec
+    uint32_t w[kThreads / 32];
+};
+
+template <typename CT>
+__global__ void __launch_bounds__(kThreads, 2)
+k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
+                       uint32_t scale, int nb, uint32_t* __restrict__ cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    TileShared& s = *reinterpret_cast<TileShared*>(s_raw);
+    if (stopped(stop)) return;
+    const int t = threadIdx.x;
+    for (int b = t; b < nb; b += kThreads) s.count[b] = 0u;
+    const int64_t base = (int64_t)blockIdx.x * kTTile;
+    const int cnt = (int)(n - base < kTTile ? n - base : kTTile);
+    uint32_t o[kTIpt], c[kTIpt], r[kTIpt];
+    double v[kTIpt];
+    bool bad = false;
+    CT oo[kTIpt], cc[kTIpt];
+#pragma unroll
+    for (int i = 0; i < kTIpt; ++i) {
+        const int j = i * kThreads + t;
+        oo[i] = j < cnt ? oc[base + j] : (CT)0;
+        cc[i] = j < cnt ? ic[base + j] : (CT)0;
+        v[i] = j < cnt ? vals[base + j] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kTIpt; ++i) {
+        const bool out = oo[i] < 0 || (int64_t)oo[i] >= no || cc[i] < 0 || (int64_t)cc[i] >= ni;
+        bad |= out;
+        o[i] = out ? 0u : (uint32_t)oo[i];
+        c[i] = (uint32_t)cc[i];
+        r[i] = i * kThreads + t < cnt ? atomicAdd(&s.count[__umulhi(o[i], scale)], 1u) : 0u;
+    }
+    if (__syncthreads_or(bad)) {
+        if (t == 0) report(kErrRange, stop, host);
+        return;
+    }
+    // all cursors of a thread at once: one wait, not one per bucket
+    constexpr int kPerB = (kMaxBuckets + kThreads - 1) / kThreads;
+    uint32_t k[kPerB], at[kPerB], mine = 0;
+#pragma unroll
+    for (int q = 0; q < kPerB; ++q) {
+        const int b = t + q * kThreads;
+        k[q] = b < nb ? s.count[b] : 0u;
+        at[q] = k[q] ? atomicAdd(cursor + b, k[q]) : 0u;
+        mine += k[q];
+    }
+    const int lane = t & 31, w = t >> 5;
+    uint32_t incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += u;
+    }
+    if (lane == 31) s.w[w] = incl;
+    __syncthreads();
+    uint32_t from = incl - mine;
+#pragma unroll
+    for (int i = 0; i < kThreads / 32; ++i) from += i < w ? s.w[i] : 0u;
+    bool full = false;
+#pragma unroll
+    for (int q = 0; q < kPerB; ++q)
+        if (k[q]) {
+            const int b = t + q * kThreads;
+            full |= at[q] + k[q] > (uint32_t)kCap;
+            s.count[b] = from;
+            s.shift[b] = at[q] - from;
+            from += k[q];
+        }
+    if (__syncthreads_or(full)) {
+        if (t == 0) report(kErrLong, stop, host);
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < kTIpt; ++i)
+        if (i * kThreads + t < cnt)
+            s.rec[s.count[__umulhi(o[i], scale)] + r[i]] =
+                make_uint4((uint32_t)__double2loint(v[i]), (uint32_t)__double2hiint(v[i]), c[i], o[i]);
+    __syncthreads();
+#pragma unroll 4
+    for (int j = t; j < cnt; j += kThreads) {
+        const Rec x = s.rec[j];
+        const uint32_t b = __umulhi(x.w, scale);
+        rec[(size_t)b * kCap + (s.shift[b] + (uint32_t)j)] = x;
     }
 }
 
@@ -407,12 +505,20 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
 #define SP_ROWS_PARTITION(CT, PER)                                                                                        \
     k_rows_partition<CT, PER><<<(unsigned)sp_ceil_div(n, kThreads * PER), kThreads, (size_t)nb * sizeof(uint32_t), stream>>>( \
         static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, stop, host)
-        // small inputs need the blocks, large ones the fewer cursor updates (5 M entries: 8 per thread 215 us, 2 252, 16 270)
+        // small inputs need the blocks (and have few entries per tile and bucket): 10,486 entries 36.9 us, 38.6 in tiles
         const bool small = n < 300000;
-        if (coord_bits == 32) { if (small) SP_ROWS_PARTITION(int32_t, 2); else SP_ROWS_PARTITION(int32_t, 8); }
-        else { if (small) SP_ROWS_PARTITION(int64_t, 2); else SP_ROWS_PARTITION(int64_t, 8); }
+#define SP_ROWS_TILES(CT)                                                                                                 \
+    do {                                                                                                                  \
+        e = sp_allow_shared<k_rows_partition_tiles<CT>>(t->device, sizeof(TileShared));                                 \
+        if (e == cudaSuccess)                                                                                             \
+            k_rows_partition_tiles<CT><<<(unsigned)sp_ceil_div(n, kTTile), kThreads, sizeof(TileShared), stream>>>(      \
+                static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, stop, host); \
+    } while (0)
+        if (coord_bits == 32) { if (small) SP_ROWS_PARTITION(int32_t, 2); else SP_ROWS_TILES(int32_t); }
+        else { if (small) SP_ROWS_PARTITION(int64_t, 2); else SP_ROWS_TILES(int64_t); }
+#undef SP_ROWS_TILES
 #undef SP_ROWS_PARTITION
-        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaGetLastError();
     }
 #define SP_ROWS_LAUNCH(kernel, smem, ...) \
     (e = e != cudaSuccess ? e : sp_launch_dependent(kernel, dim3((unsigned)nb), dim3(kBThreads), smem, stream, __VA_ARGS__))
