@@ -21,9 +21,12 @@ namespace {
 constexpr int kThreads = 512;                   // of k_rows_partition
 constexpr int kBThreads = 512;                  // of k_rows_build and k_rows_outer
 constexpr int kWarps = kBThreads / 32;
-constexpr int kCap = 4096;                      // entries a bucket can hold
+// Entries a bucket can hold.  4096 is faster where no bucket overflows (5 M uniform entries 188 us against 196, 6144 204),
+// but power-law rows (mean 16, deviation 54) overflow it and then pay for both paths: 3.2 M of them 279 us against 150,
+// a conversion of 2 M 190 against 123.  5120 is five deviations from their mean.
+constexpr int kCap = 5120;
 constexpr int kIpt = kCap / kBThreads;          // ... per thread of k_rows_build
-constexpr int kAverage = 2048;                  // entries per bucket aimed at: rows of 48 +- 7 and power-law rows stay below twice that
+constexpr int kAverage = 2048;                  // entries per bucket aimed at
 constexpr int kAverageSmall = 256;               // ... of a small input, for more blocks (10,486 entries: 37 us; 2048: 39)
 constexpr int kWidth = 2048;                    // outer indices of a bucket
 constexpr int kMaxBuckets = 4096;
@@ -152,7 +155,7 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
 
 // The same for large inputs, the tile being put in order by bucket in shared memory first: a bucket's entries then
 // leave side by side and one store instruction touches fewer lines, and the values, requested with the coordinates,
-// are no longer waited for at the end.  5 M entries: pack 190 us, 205 with every entry stored from where it was
+// are no longer waited for at the end.  5 M entries: pack 190 us (196 with the present kCap), 205 with every entry stored from where it was
 // read; 1.5 M with 64-bit coordinates (convert) 98 against 106; 2.5 M 128 against 146.  Tiles of 4096 entries spill
 // (188, 102), 1024 threads with 6 entries each 190, 98, 8 entries 192, 102, three blocks per SM 204, 103.
 constexpr int kTIpt = 6, kTTile = kThreads * kTIpt;
@@ -249,7 +252,7 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
 }
 
 struct BuildShared {
-    uint32_t count[kWidth + 1];                 // entries, then starts, of the bucket's outer indices; later the entries' outer offsets
+    uint32_t count[(kCap / 2 > kWidth ? kCap / 2 : kWidth) + 1];    // entries, then starts, of the bucket's outer indices; later the entries' outer offsets
     uint32_t crd[kCap];
     union {
         double val[kCap];
@@ -260,7 +263,7 @@ struct BuildShared {
     uint32_t w[kWarps];
 };
 static_assert(sizeof(uint32_t) * 2 * kWidth <= sizeof(double) * kCap / 2, "lo and hi lie before bin");
-static_assert(kWidth * 2 >= kCap, "the starts' space holds a 16-bit number per entry");
+static_assert(sizeof(BuildShared::count) >= sizeof(uint16_t) * kCap, "the starts' space holds a 16-bit number per entry");
 
 // The place of an entry is the start of its segment plus the number of smaller coordinates in it, counted over
 // shared memory.  Where segments are long (more than kDense compares per entry on average) they are first

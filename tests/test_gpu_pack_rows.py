@@ -32,9 +32,11 @@ CASES = {
     "bucket_edges": ([1, 2047, 2049, 0, 0, 1, 2047, 2, 2048] * 3, 2100, 0),
     "long_rows": ([500] * 40 + [0, 1, 2] * 20 + [1500] * 20, 1600, 0),       # cut into bins
     "many_tiles": ([30] * 20000, 60, 0),                                    # the larger tiles of entries
-    "whole_tiles": ([32] * 10240, 40, 0),                                   # 40 tiles of 8192
-    "one_entry_over": ([32] * 10240 + [1], 40, 0),
-    "many_tiles_overfull": ([30] * 11000 + [5000] + [30] * 100, 6000, 0),
+    "full_at_capacity": ([5120], 6000, 0),
+    "over_capacity": ([5, 5121, 3], 6000, 0),
+    "whole_tiles": ([32] * 12288, 40, 0),                                   # 128 tiles of 3072
+    "one_entry_over": ([32] * 12288 + [1], 40, 0),
+    "many_tiles_overfull": ([30] * 11000 + [5500] + [30] * 100, 6000, 0),
     "duplicates": ([20] * 300, 64, 17),
     "duplicates_in_bins": ([300] * 30, 400, 2),
 }
