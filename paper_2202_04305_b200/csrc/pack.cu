@@ -911,8 +911,12 @@ __global__ void k_unpack(UnpackArgs a) {
 // entries.  Two searches, by the warps together, find the segments that the tile touches; each of those
 // marks its first entry, and an entry's segment is the last mark at or before it.  (A search of its own
 // per entry, 17 dependent loads for 70,000 rows, took 33 us on 1,500,007 entries; this takes 12.)
+// A tile that spans more than kUnpackWalk segments, nearly all of them empty, searches per entry all the same,
+// within its span: going over them is work without a bound (by the host clock: 1,000 entries in 10^7 rows 7.7 ms, now 31 us; 100,000
+// entries in 2^20 rows, 10,500 of them to a tile, 33.7 us, now 24.3).
 constexpr int kUnpackThreads = 256;
 constexpr int kUnpackTile = 1024;
+constexpr int kUnpackWalk = 4 * kUnpackTile;
 
 // Last q in [0, n) with pos[q] <= p, found by a warp, 32 probes at a time (pos[0] <= p).
 template <typename P>
@@ -946,6 +950,27 @@ k_unpack_rows(const P* __restrict__ pos, const I* __restrict__ crd, const double
     }
     __syncthreads();
     const int64_t q0 = s_range[0], q1 = s_range[1];
+    if (q1 - q0 > kUnpackWalk) {                  // the last segment that starts at or before each entry
+        int64_t q[kPer];
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) q[i] = q0;
+        for (int64_t len = q1 - q0 + 1; len > 1;) {
+            const int64_t half = len >> 1;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)        // a thread's searches side by side
+                if ((int64_t)pos[q[i] + half] <= e0 + i * kUnpackThreads + t) q[i] += half;
+            len -= half;
+        }
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int64_t e = e0 + i * kUnpackThreads + t;
+            if (e >= n) break;
+            out_outer[e] = outer ? (int64_t)outer[q[i]] : q[i];
+            out_inner[e] = (int64_t)crd[e];
+            vals_out[e] = val[e];
+        }
+        return;
+    }
     for (int64_t q = q0 + 1 + t; q <= q1; q += kUnpackThreads) {
         const int64_t i = (int64_t)pos[q] - e0;   // empty segments share their start with the next; the largest wins
         if (i < cnt) atomicMax(&s_seg[i], (uint32_t)(q - q0));
