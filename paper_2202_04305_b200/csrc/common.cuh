@@ -199,11 +199,14 @@ __device__ __forceinline__ int64_t sp_checked_index(int64_t i, int64_t n, int li
 // Chains of short kernels in which each needs the one before it (the packer's passes, a kernel and
 // its fix-up) are launched as programmatic dependents: the next kernel may be set up on the device
 // while its predecessor drains, and its first statement waits until that predecessor has completed
-// and its writes are visible.  Nothing triggers early: the only thing overlapped is the launch itself.
+// and its writes are visible.  The only thing overlapped is the launch itself, except where a kernel says
+// sp_release_next_kernel(): once all its blocks have, the next kernel's may start and run up to their wait,
+// before which they touch nothing that any kernel of the chain writes.
 // In a kernel launched the ordinary way the wait returns at once.  A pointer to what a predecessor wrote
 // is not `const __restrict__`: loads through such a pointer count as invariant, which leaves the compiler
 // free to move them above the wait whatever memory it says it touches.
 __device__ __forceinline__ void sp_wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void sp_release_next_kernel() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
 cudaError_t sp_launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

@@ -1,33 +1,46 @@
 // sp_pack for matrices with a compressed inner level and moderate segments (rows of CSR and DCSR, columns of
 // CSC and DCSC): no sort by key, the entries pass through memory twice.
 //
-//   1. k_rows_partition  (k_rows_partition_tiles from 300,000 entries on) range check; entries into buckets, one per range of outer indices, in any order
-//   2. k_rows_build      a block per bucket: entries per outer index, order inside every segment, and
+//   1. k_rows_count      (where slots of kCap records would not follow the entries, and from kCountFrom entries on)
+//                        entries per bucket, a bucket being a range of outer indices, and where every bucket begins
+//   2. k_rows_partition  (k_rows_partition_tiles from kSmall entries on) range check; entries to their buckets, in any order
+//   3. k_rows_build      a block per bucket: entries per outer index, order inside every segment, and
 //                        everything the bucket contributes to the storage, written in order
-//   3. k_rows_outer      (compressed outer level) the buckets' lists of stored outer indices, joined
+//   4. k_rows_outer      (compressed outer level) the buckets' lists of stored outer indices, joined
 //
 // Buckets hold about kAverage entries and at most kCap.  Random accesses are what a GPU is slow at (about 140 G
-// single-lane accesses/s here, hit or miss): this way an entry costs at most one, its 16-byte store in step 1; every
+// single-lane accesses/s here, hit or miss): this way an entry costs at most one, its 16-byte store in step 2; every
 // other scattered access stays in shared memory.  Sizes are known beforehand (a compressed outer level's are
 // bounded), so the one read-back comes at the end.  A bucket that overflows (long or very uneven segments)
 // and duplicate coordinates, whose values have to be summed, are found on the device; the kernels after that
 // return and the caller takes the radix path.
+//
+// Without step 1 a bucket has a slot of kCap records, 2.5 times what it holds on average and 16 times in small inputs;
+// with it the scratch is 16 bytes an entry, less than the radix path's, however many rows there are (1,000 entries in
+// 8 M rows: 0.1 MB, 336 MB in slots; 5 M entries: 80 MB, 200 in slots).  It costs 3 us of 40 and more (300,000 entries
+// 43.5 us against 40.0, 1 M 67 against 64) and next to nothing of a large pack, where buckets side by side spare every
+// block the sum over the ones before (5 M entries 194 to 198 us against 195).  An overflow is then known before the
+// entries move: 3.2 M entries with a row of 6,000 284 us against 295, 5 M with a row of 20,000 368 against 373, with a
+// row of 1 M, whose counters collide, 382 against 376 (by radix alone 252, 343, 348).
 #include "common.cuh"
 
 #include <algorithm>
 
 namespace {
 
+constexpr int kCThreads = 1024, kCBlocks = 148; // of k_rows_count
+constexpr int64_t kCountFrom = 2000000;         // entries from which on it runs
 constexpr int kThreads = 512;                   // of k_rows_partition
 constexpr int kBThreads = 512;                  // of k_rows_build and k_rows_outer
 constexpr int kWarps = kBThreads / 32;
-// Entries a bucket can hold.  4096 is faster where no bucket overflows (5 M uniform entries 188 us against 196, 6144 204),
-// but power-law rows (mean 16, deviation 54) overflow it and then pay for both paths: 3.2 M of them 279 us against 150,
-// a conversion of 2 M 190 against 123.  5120 is five deviations from their mean.
+// Entries a bucket can hold: a block orders them in shared memory, two blocks to an SM.  With 4096, 5 M uniform entries
+// took 188 us against 196, but power-law rows (mean 16, deviation 54) overflow such buckets and take the radix path: 3.2 M
+// of them 279 us against 150, a conversion of 2 M 190 against 123.
 constexpr int kCap = 5120;
 constexpr int kIpt = kCap / kBThreads;          // ... per thread of k_rows_build
 constexpr int kAverage = 2048;                  // entries per bucket aimed at
-constexpr int kAverageSmall = 256;               // ... of a small input, for more blocks (10,486 entries: 37 us; 2048: 39)
+constexpr int kAverageSmall = 320;               // ... of a small input, for more blocks (10,486 entries: 37 us; 2048: 39)
+constexpr int64_t kSmall = 300000;              // entries below which an input counts as small
 constexpr int kWidth = 2048;                    // outer indices of a bucket
 constexpr int kMaxBuckets = 4096;
 constexpr int kDense = 24;                      // mean compares per entry above which segments are cut into bins
@@ -38,6 +51,11 @@ enum { kErrRange = 0, kErrDup, kErrLong, kOuterCount };
 __device__ __forceinline__ void report(int what, uint32_t* stop, unsigned long long* host) {
     *static_cast<volatile unsigned long long*>(host + what) = 1;
     *static_cast<volatile uint32_t*>(stop) = 1;
+}
+
+// Where bucket b's records begin, its slot being the b-th of `slot` records (0: buckets side by side, ends in cursor).
+__device__ __forceinline__ uint32_t records_of(uint32_t b, uint32_t slot, const uint32_t* cursor) {
+    return slot ? b * slot : b ? cursor[b - 1] : 0u;
 }
 
 using Rec = uint4;                              // value (low, high word), inner coordinate, outer coordinate
@@ -53,7 +71,8 @@ __device__ __forceinline__ bool stopped(const uint32_t* stop) {
     return __syncthreads_or(threadIdx.x == 0 && __ldcg(stop) != 0) != 0;
 }
 
-// Exclusive scan over the block of one counter per thread.
+// Exclusive scan over a block of WARPS warps of one counter per thread.
+template <int WARPS = kWarps>
 __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* s_w, uint32_t* total) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t incl = v;
@@ -66,7 +85,7 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* s_w, uint32
     __syncthreads();
     uint32_t pre = 0, tot = 0;
 #pragma unroll
-    for (int i = 0; i < kWarps; ++i) {
+    for (int i = 0; i < WARPS; ++i) {
         const uint32_t s = s_w[i];
         if (i < w) pre += s;
         tot += s;
@@ -91,14 +110,66 @@ __device__ __forceinline__ void scan_shared(uint32_t* s, int n, uint32_t* s_w) {
     __syncthreads();
 }
 
+// Entries per bucket, in shared memory per block and then added up in cursor (cleared before), and, by the last block,
+// where the buckets begin: cursor[b], which the partition advances to where bucket b ends.  Few blocks, since each
+// adds up to kMaxBuckets counters.
+template <typename CT>
+__global__ void __launch_bounds__(kCThreads)
+k_rows_count(const CT* __restrict__ oc, int64_t n, int64_t no, uint32_t scale, int nb, uint32_t* cursor, uint32_t* stop, uint32_t* ticket,
+             unsigned long long* host) {
+    constexpr int kU = 16, kPerB = kMaxBuckets / kCThreads;
+    __shared__ uint32_t s_hist[kMaxBuckets];
+    __shared__ uint32_t s_w[kCThreads / 32];
+    __shared__ bool s_last;
+    sp_release_next_kernel();                       // it ranks its entries before it waits for the cursors
+    const int t = threadIdx.x;
+    for (int b = t; b < nb; b += kCThreads) s_hist[b] = 0u;
+    __syncthreads();
+    for (int64_t base = (int64_t)blockIdx.x * (kCThreads * kU); base < n; base += (int64_t)gridDim.x * (kCThreads * kU)) {
+        CT o[kU];
+#pragma unroll
+        for (int i = 0; i < kU; ++i) o[i] = base + i * kCThreads + t < n ? oc[base + i * kCThreads + t] : (CT)-1;
+#pragma unroll
+        for (int i = 0; i < kU; ++i)                // the partition reports what is out of range
+            if (o[i] >= 0 && (int64_t)o[i] < no) atomicAdd(&s_hist[__umulhi((uint32_t)o[i], scale)], 1u);
+    }
+    __syncthreads();
+    for (int b = t; b < nb; b += kCThreads)
+        if (s_hist[b]) atomicAdd(cursor + b, s_hist[b]);
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int b = t; b < nb; b += kCThreads) s_hist[b] = __ldcg(cursor + b);
+    __syncthreads();
+    uint32_t k[kPerB], mine = 0, tot;
+    bool full = false;
+#pragma unroll
+    for (int q = 0; q < kPerB; ++q) {
+        const int b = t * kPerB + q;
+        k[q] = b < nb ? s_hist[b] : 0u;
+        full |= k[q] > (uint32_t)kCap;
+        mine += k[q];
+    }
+    uint32_t at = block_scan<kCThreads / 32>(mine, s_w, &tot);
+#pragma unroll
+    for (int q = 0; q < kPerB; ++q) {
+        const int b = t * kPerB + q;
+        if (b < nb) cursor[b] = at;
+        at += k[q];
+    }
+    if (__syncthreads_or(full) && t == 0) report(kErrLong, stop, host);
+}
+
 // A block sends a tile of kThreads * PER entries to their buckets: ranks inside the tile by shared-memory
 // atomics, the tile's place in every bucket by one atomic on the bucket's cursor.
 template <typename CT, int PER>
 __global__ void __launch_bounds__(kThreads, 2)
 k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
-                 uint32_t scale, int nb, uint32_t* __restrict__ cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
+                 uint32_t scale, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
     extern __shared__ uint32_t s_hist[];
-    if (stopped(stop)) return;
     const int t = threadIdx.x;
     for (int b = t; b < nb; b += kThreads) s_hist[b] = 0u;
     __syncthreads();
@@ -117,7 +188,10 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
         if (o[i] < 0 || (int64_t)o[i] >= no || c[i] < 0 || (int64_t)c[i] >= ni) { bad = true; o[i] = 0; }
         r[i] = base + i * kThreads < n ? atomicAdd(&s_hist[__umulhi((uint32_t)o[i], scale)], 1u) : 0u;
     }
-    if (__syncthreads_or(bad)) {
+    bad = __syncthreads_or(bad) != 0;
+    sp_wait_for_previous_kernel();
+    if (stopped(stop)) return;
+    if (bad) {
         if (t == 0) report(kErrRange, stop, host);
         return;
     }
@@ -134,8 +208,9 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
 #pragma unroll
     for (int q = 0; q < kPerB; ++q)
         if (k[q]) {
-            full |= at[q] + k[q] > (uint32_t)kCap;
-            s_hist[t + q * kThreads] = at[q];
+            const uint32_t b = t + q * kThreads;
+            full |= slot && at[q] + k[q] > slot;
+            s_hist[b] = at[q] + b * slot;
         }
     if (__syncthreads_or(full)) {
         if (t == 0) report(kErrLong, stop, host);
@@ -147,7 +222,7 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
         if (e < n) {
             const uint32_t b = __umulhi((uint32_t)o[i], scale);
             const double v = vals[e];
-            rec[(size_t)b * kCap + s_hist[b] + r[i]] =
+            rec[s_hist[b] + r[i]] =
                 make_uint4((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), (uint32_t)c[i], (uint32_t)o[i]);
         }
     }
@@ -162,17 +237,16 @@ constexpr int kTIpt = 6, kTTile = kThreads * kTIpt;
 struct TileShared {
     Rec rec[kTTile];
     uint32_t count[kMaxBuckets];                // entries of the tile, then where they begin in rec
-    uint32_t shift[kMaxBuckets];                // place in the bucket minus place in rec
+    uint32_t shift[kMaxBuckets];                // place among the records minus place in rec
     uint32_t w[kThreads / 32];
 };
 
 template <typename CT>
 __global__ void __launch_bounds__(kThreads, 2)
 k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
-                       uint32_t scale, int nb, uint32_t* __restrict__ cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
+                       uint32_t scale, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     TileShared& s = *reinterpret_cast<TileShared*>(s_raw);
-    if (stopped(stop)) return;
     const int t = threadIdx.x;
     for (int b = t; b < nb; b += kThreads) s.count[b] = 0u;
     const int64_t base = (int64_t)blockIdx.x * kTTile;
@@ -197,7 +271,10 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
         c[i] = (uint32_t)cc[i];
         r[i] = i * kThreads + t < cnt ? atomicAdd(&s.count[__umulhi(o[i], scale)], 1u) : 0u;
     }
-    if (__syncthreads_or(bad)) {
+    bad = __syncthreads_or(bad) != 0;
+    sp_wait_for_previous_kernel();
+    if (stopped(stop)) return;
+    if (bad) {
         if (t == 0) report(kErrRange, stop, host);
         return;
     }
@@ -227,10 +304,10 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
 #pragma unroll
     for (int q = 0; q < kPerB; ++q)
         if (k[q]) {
-            const int b = t + q * kThreads;
-            full |= at[q] + k[q] > (uint32_t)kCap;
+            const uint32_t b = t + q * kThreads;
+            full |= slot && at[q] + k[q] > slot;
             s.count[b] = from;
-            s.shift[b] = at[q] - from;
+            s.shift[b] = at[q] + b * slot - from;
             from += k[q];
         }
     if (__syncthreads_or(full)) {
@@ -247,12 +324,12 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
     for (int j = t; j < cnt; j += kThreads) {
         const Rec x = s.rec[j];
         const uint32_t b = __umulhi(x.w, scale);
-        rec[(size_t)b * kCap + (s.shift[b] + (uint32_t)j)] = x;
+        rec[s.shift[b] + (uint32_t)j] = x;
     }
 }
 
 struct BuildShared {
-    uint32_t count[(kCap / 2 > kWidth ? kCap / 2 : kWidth) + 1];    // entries, then starts, of the bucket's outer indices; later the entries' outer offsets
+    uint32_t count[kWidth + 1];                 // entries, then starts, of the bucket's outer indices
     uint32_t crd[kCap];
     union {
         double val[kCap];
@@ -261,9 +338,9 @@ struct BuildShared {
     };
     uint32_t bin_end;                           // bin[kCap] when the bucket is full
     uint32_t w[kWarps];
+    uint16_t seg[kCap];                         // outer offsets of the entries, in order
 };
 static_assert(sizeof(uint32_t) * 2 * kWidth <= sizeof(double) * kCap / 2, "lo and hi lie before bin");
-static_assert(sizeof(BuildShared::count) >= sizeof(uint16_t) * kCap, "the starts' space holds a 16-bit number per entry");
 
 // The place of an entry is the start of its segment plus the number of smaller coordinates in it, counted over
 // shared memory.  Where segments are long (more than kDense compares per entry on average) they are first
@@ -271,29 +348,32 @@ static_assert(sizeof(BuildShared::count) >= sizeof(uint16_t) * kCap, "the starts
 // the entries of one bin are compared.
 template <typename P, typename I, bool DBL>
 __global__ void __launch_bounds__(kBThreads, 2)
-k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int nb, uint32_t* stop, unsigned long long* host,
-             P* __restrict__ pos1, I* __restrict__ crd, double* __restrict__ val, uint32_t* __restrict__ seg_out,
-             uint32_t* __restrict__ outer_list, uint32_t* __restrict__ outer_pos, uint32_t* __restrict__ outer_count) {
+k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int nb, uint32_t slot, uint32_t* stop, unsigned long long* host,
+             P* __restrict__ pos1, I* __restrict__ crd, double* __restrict__ val, uint32_t* __restrict__ seg_out, uint32_t* __restrict__ outer_count) {
     sp_wait_for_previous_kernel();
     if (stopped(stop)) return;
     extern __shared__ __align__(16) unsigned char s_raw[];
     BuildShared& s = *reinterpret_cast<BuildShared*>(s_raw);
     const int t = threadIdx.x, b = blockIdx.x;
-    const int cnt = (int)cursor[b];
+    const uint32_t place = records_of(b, slot, cursor);
+    const int cnt = (int)(slot ? cursor[b] : cursor[b] - place);
     const int64_t lo = bucket_begin(b, scale, no), hi = b + 1 < nb ? bucket_begin(b + 1, scale, no) : no;
     const int width = (int)(hi - lo);
     // entries of this thread, requested first; the values are fetched again at the end (registers)
-    const Rec* mine = rec + (size_t)b * kCap + t;
+    const Rec* mine = rec + place + t;
     uint32_t c[kIpt], qr[kIpt];                 // inner coordinate; outer offset << 16 | rank, later the place
 #pragma unroll
     for (int i = 0; i < kIpt; ++i) {
         c[i] = qr[i] = 0u;
         if (i * kBThreads + t < cnt) { const Rec x = mine[i * kBThreads]; c[i] = x.z; qr[i] = x.w - (uint32_t)lo; }
     }
-    uint32_t before = 0, base;
-    for (int q = t; q < b; q += kBThreads) before += cursor[q];
     for (int q = t; q < width; q += kBThreads) { s.count[q] = 0u; s.lo[q] = ~0u; s.hi[q] = 0u; }
-    block_scan(before, s.w, &base);             // (also the barrier after the zeroing)
+    uint32_t before = 0, base = place;          // base: entries in the buckets before
+    if (slot) {
+        for (int q = t; q < b; q += kBThreads) before += cursor[q];
+        block_scan(before, s.w, &base);
+    }
+    __syncthreads();
 #pragma unroll
     for (int i = 0; i < kIpt; ++i)
         if (i * kBThreads + t < cnt) qr[i] = qr[i] << 16 | atomicAdd(&s.count[qr[i]], 1u);
@@ -311,25 +391,8 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
     const uint32_t at_filled = block_scan(filled, s.w, &tot_filled);
     block_scan(sq, s.w, &tot_sq);
     const bool bins = tot_sq > (uint32_t)kDense * (uint32_t)cnt;
-    if (DBL) {
-        uint32_t k = 0;                         // the stored indices of this thread's kPerW, in order
-#pragma unroll
-        for (int i = 0; i < kPerW; ++i) {
-            const int q = t * kPerW + i;
-            if (q < width && s.count[q]) { outer_list[lo + at_filled + k] = (uint32_t)(lo + q); ++k; }
-        }
-        if (t == 0) outer_count[b] = tot_filled;
-        __syncthreads();
-        uint32_t len[kPerW];
-#pragma unroll
-        for (int i = 0; i < kPerW; ++i) { const int q = t * kPerW + i; len[i] = q < width ? s.count[q] : 0u; }
-        scan_shared<kPerW>(s.count, width, s.w);
-        k = 0;
-#pragma unroll
-        for (int i = 0; i < kPerW; ++i)
-            if (len[i]) { outer_pos[lo + at_filled + k] = base + s.count[t * kPerW + i]; ++k; }
-    } else {
-        scan_shared<kPerW>(s.count, width, s.w);
+    scan_shared<kPerW>(s.count, width, s.w);
+    if (!DBL) {
         for (int q = t; q < width; q += kBThreads) pos1[lo + q] = (P)(base + s.count[q]);
         if (b == nb - 1 && t == 0) pos1[no] = (P)n;
     }
@@ -391,12 +454,11 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
     }
     // Distinct coordinates take the places 0 .. cnt - 1; of equal ones all get the lowest, so the sum falls short.
     uint32_t tot_sum;
-    block_scan(sum, s.w, &tot_sum);             // also the barrier after which coordinates, starts and bins are dead
+    block_scan(sum, s.w, &tot_sum);             // also the barrier after which coordinates and bins are dead
     if (tot_sum != (uint32_t)(cnt * (cnt - 1) / 2)) {
         if (t == 0) report(kErrDup, stop, host);
         return;
     }
-    uint16_t* s_seg = reinterpret_cast<uint16_t*>(s.count);
 #pragma unroll
     for (int i = 0; i < kIpt; ++i)
         if (i * kBThreads + t < cnt) {
@@ -404,20 +466,30 @@ k_rows_build(const Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint
             const uint32_t p = to[i] & 0xffffu;
             s.crd[p] = c[i];
             s.val[p] = __hiloint2double((int)v.y, (int)v.x);
-            if (seg_out) s_seg[p] = (uint16_t)(to[i] >> 16);
+            if (seg_out) s.seg[p] = (uint16_t)(to[i] >> 16);
         }
     __syncthreads();
     for (int j = t; j < cnt; j += kBThreads) {
         crd[base + j] = (I)s.crd[j];
         val[base + j] = s.val[j];
-        if (seg_out) seg_out[base + j] = (uint32_t)lo + s_seg[j];
+        if (seg_out) seg_out[base + j] = (uint32_t)lo + s.seg[j];
+    }
+    if (DBL) {                                  // the stored indices and their first entries, in order, where the records were
+        uint32_t k = at_filled;
+#pragma unroll
+        for (int i = 0; i < kPerW; ++i) {
+            const int q = t * kPerW + i;
+            if (q < width && s.count[q + 1] != s.count[q])
+                *reinterpret_cast<uint2*>(rec + place + k++) = make_uint2((uint32_t)(lo + q), base + s.count[q]);
+        }
+        if (t == 0) outer_count[b] = tot_filled;
     }
 }
 
 // Joins the buckets' lists of non-empty outer indices and of their first entries: crd[0] and pos[1].
 template <typename P, typename I>
 __global__ void __launch_bounds__(kBThreads)
-k_rows_outer(const uint32_t* outer_list, const uint32_t* outer_pos, const uint32_t* outer_count, int64_t n, int64_t no, uint32_t scale, int nb,
+k_rows_outer(const Rec* rec, const uint32_t* cursor, const uint32_t* outer_count, int64_t n, int nb, uint32_t slot,
              uint32_t* stop, unsigned long long* host, P* __restrict__ pos0, I* __restrict__ crd0, P* __restrict__ pos1) {
     sp_wait_for_previous_kernel();
     if (stopped(stop)) return;
@@ -426,11 +498,12 @@ k_rows_outer(const uint32_t* outer_list, const uint32_t* outer_pos, const uint32
     uint32_t before = 0, base;
     for (int q = t; q < b; q += kBThreads) before += outer_count[q];
     block_scan(before, s_w, &base);
-    const int64_t lo = bucket_begin(b, scale, no);
+    const Rec* list = rec + records_of(b, slot, cursor);
     const uint32_t cnt = outer_count[b];
     for (uint32_t q = t; q < cnt; q += kBThreads) {
-        crd0[base + q] = (I)outer_list[lo + q];
-        pos1[base + q] = (P)outer_pos[lo + q];
+        const uint2 x = *reinterpret_cast<const uint2*>(list + q);
+        crd0[base + q] = (I)x.x;
+        pos1[base + q] = (P)x.y;
     }
     if (b == nb - 1 && t == 0) {
         pos1[base + cnt] = (P)n;
@@ -449,7 +522,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     // narrow positions need the radix path's width checks; records hold 32-bit coordinates
     if (posBits < 32 || crdBits < 32 || no >= ((int64_t)1 << 31) || ni >= ((int64_t)1 << 32)) return SP_ERR_UNSUPPORTED;
     // enough buckets for the entries and for the outer indices, no more than there are outer indices
-    int64_t buckets = std::max(sp_ceil_div(n, n < 300000 ? kAverageSmall : kAverage), sp_ceil_div(no, kWidth - 48));
+    int64_t buckets = std::max(sp_ceil_div(n, n < kSmall ? kAverageSmall : kAverage), sp_ceil_div(no, kWidth - 48));
     if (buckets > kMaxBuckets) return SP_ERR_UNSUPPORTED;
     if (buckets > no) {
         if (n > no * kCap) return SP_ERR_UNSUPPORTED;
@@ -462,20 +535,34 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     const bool dbl = lt[0] == SP_COMPRESSED;
     const size_t pw = posBits / 8, cw = crdBits / 8;
     sp_workspace ws(stream);
-    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb + 1);
-    ws.reserve(cursors + sp_workspace::bytes_for<Rec>((size_t)nb * kCap) +
-               (dbl ? 2 * sp_workspace::bytes_for<uint32_t>((size_t)no) + cursors : 0));
-    uint32_t* cursor = ws.get<uint32_t>((size_t)nb + 1);
-    Rec* rec = ws.get<Rec>((size_t)nb * kCap);
-    uint32_t* outer_list = dbl ? ws.get<uint32_t>((size_t)no) : nullptr;
-    uint32_t* outer_pos = dbl ? ws.get<uint32_t>((size_t)no) : nullptr;
-    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb + 1) : nullptr;
+    const bool counted = n >= kCountFrom || (int64_t)nb * kCap > 16 * n + 65536;
+    const uint32_t slot = counted ? 0u : (uint32_t)kCap;
+    const size_t records = counted ? (size_t)n : (size_t)nb * kCap;
+    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb + 2);
+    ws.reserve(cursors + sp_workspace::bytes_for<Rec>(records) + (dbl ? cursors : 0));
+    uint32_t* cursor = ws.get<uint32_t>((size_t)nb + 2);
+    Rec* rec = ws.get<Rec>(records);
+    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb + 2) : nullptr;
     unsigned long long* host = sp_host_words();
     if (ws.failed || !host) return SP_ERR_ALLOC;
-    uint32_t* stop = cursor + nb;
+    uint32_t *stop = cursor + nb, *ticket = cursor + nb + 1;
+
+    // counted while the host prepares the rest
+    SP_CUDA(cudaMemsetAsync(cursor, 0, (size_t)(nb + 2) * sizeof(uint32_t), stream));
+    if (counted) {
+        const unsigned blocks = (unsigned)std::min<int64_t>(kCBlocks, sp_ceil_div(n, kCThreads * 16));
+        if (coord_bits == 32) k_rows_count<int32_t><<<blocks, kCThreads, 0, stream>>>(static_cast<const int32_t*>(outer), n, no, scale, nb, cursor, stop, ticket, host);
+        else k_rows_count<int64_t><<<blocks, kCThreads, 0, stream>>>(static_cast<const int64_t*>(outer), n, no, scale, nb, cursor, stop, ticket, host);
+        SP_LAUNCH_CHECK();
+        sp_count_launches(1);
+    }
 
     sp_tensor* t = new sp_tensor();
-    auto fail = [&](sp_status s) { sp_free(t); return s; };
+    auto fail = [&](sp_status s) {              // what is under way may still write to the host's words
+        cudaStreamSynchronize(stream);
+        sp_free(t);
+        return s;
+    };
     cudaGetDevice(&t->device);
     t->rank = 2;
     t->posBits = posBits;
@@ -503,33 +590,32 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         t->parts[(uint64_t)SP_PART_SEGIDS << 56] = sg;
     }
 
-    cudaError_t e = cudaMemsetAsync(cursor, 0, (size_t)(nb + 1) * sizeof(uint32_t), stream);
-    if (e == cudaSuccess) {
-#define SP_ROWS_PARTITION(CT, PER)                                                                                        \
-    k_rows_partition<CT, PER><<<(unsigned)sp_ceil_div(n, kThreads * PER), kThreads, (size_t)nb * sizeof(uint32_t), stream>>>( \
-        static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, stop, host)
-        // small inputs need the blocks (and have few entries per tile and bucket): 10,486 entries 36.9 us, 38.6 in tiles
-        const bool small = n < 300000;
-#define SP_ROWS_TILES(CT)                                                                                                 \
+    // small inputs need the blocks (and have few entries per tile and bucket): 10,486 entries 36.9 us, 38.6 in tiles
+    const bool small = n < kSmall;
+    cudaError_t e = cudaSuccess;
+#define SP_ROWS_PARTITION(CT)                                                                                             \
     do {                                                                                                                  \
-        e = sp_allow_shared<k_rows_partition_tiles<CT>>(t->device, sizeof(TileShared));                                 \
-        if (e == cudaSuccess)                                                                                             \
-            k_rows_partition_tiles<CT><<<(unsigned)sp_ceil_div(n, kTTile), kThreads, sizeof(TileShared), stream>>>(      \
-                static_cast<const CT*>(outer), static_cast<const CT*>(inner), vals, n, no, ni, scale, nb, cursor, rec, stop, host); \
+        const CT *oc = static_cast<const CT*>(outer), *ic = static_cast<const CT*>(inner);                                \
+        if (small) {                                                                                                      \
+            e = sp_launch_dependent(k_rows_partition<CT, 2>, dim3((unsigned)sp_ceil_div(n, kThreads * 2)), dim3(kThreads), \
+                                    (size_t)nb * sizeof(uint32_t), stream, oc, ic, vals, n, no, ni, scale, nb, slot, cursor, rec, stop, host); \
+        } else {                                                                                                          \
+            e = sp_allow_shared<k_rows_partition_tiles<CT>>(t->device, sizeof(TileShared));                               \
+            if (e == cudaSuccess)                                                                                         \
+                e = sp_launch_dependent(k_rows_partition_tiles<CT>, dim3((unsigned)sp_ceil_div(n, kTTile)), dim3(kThreads), sizeof(TileShared), \
+                                        stream, oc, ic, vals, n, no, ni, scale, nb, slot, cursor, rec, stop, host);             \
+        }                                                                                                                 \
     } while (0)
-        if (coord_bits == 32) { if (small) SP_ROWS_PARTITION(int32_t, 2); else SP_ROWS_TILES(int32_t); }
-        else { if (small) SP_ROWS_PARTITION(int64_t, 2); else SP_ROWS_TILES(int64_t); }
-#undef SP_ROWS_TILES
+    if (coord_bits == 32) SP_ROWS_PARTITION(int32_t);
+    else SP_ROWS_PARTITION(int64_t);
 #undef SP_ROWS_PARTITION
-        if (e == cudaSuccess) e = cudaGetLastError();
-    }
 #define SP_ROWS_LAUNCH(kernel, smem, ...) \
     (e = e != cudaSuccess ? e : sp_launch_dependent(kernel, dim3((unsigned)nb), dim3(kBThreads), smem, stream, __VA_ARGS__))
 #define SP_ROWS_BUILD(DBL)                                                                                                \
     do {                                                                                                                  \
         if (e == cudaSuccess) e = sp_allow_shared<k_rows_build<P, I, DBL>>(t->device, sizeof(BuildShared));             \
-        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), (const Rec*)rec, (const uint32_t*)cursor, n, no, scale, nb, stop, host, pos1, \
-                       crd1, t->val, seg_out, outer_list, outer_pos, outer_count);                                        \
+        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), rec, (const uint32_t*)cursor, n, no, scale, nb, slot, stop, host, pos1, \
+                       crd1, t->val, seg_out, outer_count);                                        \
     } while (0)
     SP_DISPATCH_WIDTHS(t, {
         P* pos0 = static_cast<P*>(t->pos[0]);
@@ -538,8 +624,8 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         I* crd1 = static_cast<I*>(t->crd[1]);
         if (dbl) {
             SP_ROWS_BUILD(true);
-            SP_ROWS_LAUNCH((k_rows_outer<P, I>), 0, (const uint32_t*)outer_list, (const uint32_t*)outer_pos, (const uint32_t*)outer_count, n, no,
-                           scale, nb, stop, host, pos0, crd0, pos1);
+            SP_ROWS_LAUNCH((k_rows_outer<P, I>), 0, (const Rec*)rec, (const uint32_t*)cursor, (const uint32_t*)outer_count, n, nb, slot, stop, host,
+                           pos0, crd0, pos1);
         } else {
             SP_ROWS_BUILD(false);
         }

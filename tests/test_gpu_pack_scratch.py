@@ -1,0 +1,57 @@
+"""What packing a matrix asks of the allocator follows its entries, however many rows it has."""
+import pytest
+import torch
+
+from gpu_util import MATRIX_ENCODINGS, sp
+
+pytestmark = pytest.mark.gpu
+
+
+class Meter:
+    """An allocator that keeps count: bytes held now and at most."""
+
+    def __init__(self):
+        self.b, self.live, self.held, self.peak = sp(), {}, 0, 0
+
+        def alloc(nbytes, stream, ctx):
+            p = torch.cuda.caching_allocator_alloc(max(int(nbytes), 1), stream=int(stream or 0))
+            self.live[p] = int(nbytes)
+            self.held += int(nbytes)
+            self.peak = max(self.peak, self.held)
+            return p
+
+        def free(ptr, stream, ctx):
+            if ptr:
+                self.held -= self.live.pop(ptr)
+                torch.cuda.caching_allocator_delete(ptr)
+
+        self._a, self._f = self.b._ALLOC_T(alloc), self.b._FREE_T(free)
+
+    def __enter__(self):
+        self.b.use_torch_allocator()
+        assert self.b._lib.sp_set_allocator(self._a, self._f, None) == 0
+        return self
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        self.b._lib.sp_set_allocator(self.b._alloc_cb, self.b._free_cb, None)
+
+
+@pytest.mark.parametrize("enc", list(MATRIX_ENCODINGS))
+@pytest.mark.parametrize("outer,nnz", [(1 << 20, 1000), (8_000_000, 1000), (8_000_000, 299_999), (1 << 20, 90_000), (2_000, 69_999), (20_000, 300_000), (200_000, 1_999_999), (200_000, 2_000_000)])
+def test_scratch_follows_the_entries(enc, outer, nnz):
+    lt, od = MATRIX_ENCODINGS[enc]
+    inner = 4096
+    e = torch.arange(nnz, device="cuda", dtype=torch.int64)
+    key = e * (outer * inner // nnz) + e % 7
+    o, i = (key // inner).int(), (key % inner).int()
+    dims, coords = ((outer, inner), [o, i]) if od == (0, 1) else ((inner, outer), [i, o])
+    vals = e.double()
+    with Meter() as m:
+        A = sp().sp_pack(dims, coords, vals, lt, od)
+        handle = m.held
+        # 40 bytes an entry, 256 in inputs so small that it does not matter
+        assert m.peak - handle <= (40 * nnz if nnz >= 100_000 else 256 * nnz) + (2 << 20), f"{m.peak - handle} bytes of scratch"
+        # stored: 12 bytes an entry (16 with the column ids of column-major storage), 8 an outer index that may be stored
+        assert handle <= 16 * nnz + 8 * min(nnz, outer) * lt[0] + 4 * (outer + 1) * (1 - lt[0]) + (8 << 10)
+        A.free()
