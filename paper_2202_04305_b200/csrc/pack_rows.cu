@@ -39,8 +39,11 @@ constexpr int kWarps = kBThreads / 32;
 constexpr int kCap = 5120;
 constexpr int kIpt = kCap / kBThreads;          // ... per thread of k_rows_build
 constexpr int kAverage = 2048;                  // entries per bucket aimed at
-constexpr int kAverageSmall = 320;               // ... of a small input, for more blocks (10,486 entries: 37 us; 2048: 39)
-constexpr int64_t kSmall = 300000;              // entries below which an input counts as small
+constexpr int kAverageSmall = 320;               // ... of a small input, for more blocks
+// Entries below which an input counts as small: buckets of kAverageSmall entries, stored from where they were read.  60,000
+// entries in rows of 16 and of 100: 36.4 and 38 us, the other way 38 and 39; 80,000: 40.2 and 43.2, 39.5 and 39.4;
+// 200,000: 51.5 and 56.4, 39.3 and 39.7; 299,999: 60.6 and 67.9, 40.0 and 40.5.
+constexpr int64_t kSmall = 80000;
 constexpr int kWidth = 2048;                    // outer indices of a bucket
 constexpr int kMaxBuckets = 4096;
 constexpr int kDense = 24;                      // mean compares per entry above which segments are cut into bins
@@ -590,7 +593,6 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         t->parts[(uint64_t)SP_PART_SEGIDS << 56] = sg;
     }
 
-    // small inputs need the blocks (and have few entries per tile and bucket): 10,486 entries 36.9 us, 38.6 in tiles
     const bool small = n < kSmall;
     cudaError_t e = cudaSuccess;
 #define SP_ROWS_PARTITION(CT)                                                                                             \
