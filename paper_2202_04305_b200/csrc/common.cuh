@@ -268,7 +268,7 @@ sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t nnz_per_chunk, bool with
 // sp_pack for matrices with a compressed inner level and short segments (pack_rows.cu).  SP_ERR_UNSUPPORTED:
 // nothing was built, take the general path.
 sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64_t nnz, const void* outer, const void* inner, int coord_bits,
-                       const double* vals, int posBits, int crdBits, cudaStream_t stream, sp_tensor** out);
+                       const double* vals, int posBits, int crdBits, unsigned flags, cudaStream_t stream, sp_tensor** out);
 
 // SpMV for rank-2 handles whose inner level is dense (dense_inner.cu).
 sp_status sp_spmv_dense_inner(const sp_tensor* A, const double* x, double* y, cudaStream_t stream);

@@ -1057,7 +1057,7 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
 #ifndef SP_BENCH_BUILD
     if (rank == 2 && plan.lt[1] == SP_COMPRESSED && nnz > 0) {     // short rows (or columns) need no sort by key
         const sp_status rs = sp_pack_rows(dims, plan.src, plan.lt, nnz, coo_coords[plan.src[0]], coo_coords[plan.src[1]], coo_coord_bits,
-                                          coo_vals, posBits, crdBits, stream, out);
+                                          coo_vals, posBits, crdBits, flags, stream, out);
         if (rs != SP_ERR_UNSUPPORTED) return rs;
     }
 #endif

@@ -7,13 +7,16 @@
 //   3. k_rows_build      a block per bucket: entries per outer index, order inside every segment, and
 //                        everything the bucket contributes to the storage, written in order
 //   4. k_rows_outer      (compressed outer level) the buckets' lists of stored outer indices, joined
+//   5. k_rows_close_up   (duplicate coordinates only) the buckets' entries moved together
 //
 // Buckets hold about kAverage entries and at most kCap.  Random accesses are what a GPU is slow at (about 140 G
 // single-lane accesses/s here, hit or miss): this way an entry costs at most one, its 16-byte store in step 2; every
 // other scattered access stays in shared memory.  Sizes are known beforehand (a compressed outer level's are
-// bounded), so the one read-back comes at the end.  A bucket that overflows (long or very uneven segments)
-// and duplicate coordinates, whose values have to be summed, are found on the device; the kernels after that
-// return and the caller takes the radix path.
+// bounded), so the one read-back comes at the end.  Duplicate coordinates are found and their values summed, in input
+// order, inside the bucket's block; what it stores then ends short of its place, and step 5 closes the gaps, in
+// arrays of the right size: 5 M entries with one coordinate repeated 270 us, four times each 385, by radix 330
+// and 416; 10,486 entries 62 and 99.  A bucket that overflows (long or very uneven segments) is found on the device
+// too; the kernels after that return and the caller takes the radix path.
 //
 // Without step 1 a bucket has a slot of kCap records, 2.5 times what it holds on average and 16 times in small inputs;
 // with it the scratch is 16 bytes an entry, less than the radix path's, however many rows there are (1,000 entries in
@@ -49,8 +52,8 @@ constexpr int kMaxBuckets = 4096;
 constexpr int kDense = 24;                      // mean compares per entry above which segments are cut into bins
 
 // What the device reports, straight into the caller's pinned words: one word per event, then the number of
-// non-empty outer indices.  `stop` is the device's own copy: later blocks and kernels return once it is set.
-enum { kErrRange = 0, kErrDup, kErrLong, kOuterCount };
+// non-empty outer indices; the last is where the number of duplicates is read back to.  `stop` is the device's own copy: later blocks and kernels return once it is set.
+enum { kErrRange = 0, kErrDup, kErrLong, kOuterCount, kLost };
 __device__ __forceinline__ void report(int what, uint32_t* stop, unsigned long long* host) {
     *static_cast<volatile unsigned long long*>(host + what) = 1;
     *static_cast<volatile uint32_t*>(stop) = 1;
@@ -61,7 +64,15 @@ __device__ __forceinline__ uint32_t records_of(uint32_t b, uint32_t slot, const 
     return slot ? b * slot : b ? cursor[b - 1] : 0u;
 }
 
-using Rec = uint4;                              // value (low, high word), inner coordinate, outer coordinate
+// Value (low, high word) and 64 bits: the low kOffBits of the outer coordinate, which tell a bucket's apart, the
+// entry's number in the input, the inner coordinate in its inner_bits (low, high word).
+using Rec = uint4;
+constexpr int kOffBits = 11, kOffShift = 64 - kOffBits;
+static_assert(1 << kOffBits == kWidth, "a bucket's outer indices differ in their low bits");
+__device__ __forceinline__ Rec make_rec(double v, uint32_t outer, uint32_t number, uint32_t inner, int inner_bits) {
+    return make_uint4((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), __funnelshift_lc(0u, number, inner_bits) | inner,
+                      outer << (kOffShift - 32) | __funnelshift_lc(number, 0u, inner_bits));
+}
 
 // Outer index o lies in bucket o * scale / 2^32; bucket b begins at the first o that the formula gives b for.
 __host__ __device__ __forceinline__ int64_t bucket_begin(int64_t b, uint32_t scale, int64_t no) {
@@ -171,7 +182,7 @@ k_rows_count(const CT* __restrict__ oc, int64_t n, int64_t no, uint32_t scale, i
 template <typename CT, int PER>
 __global__ void __launch_bounds__(kThreads, 2)
 k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
-                 uint32_t scale, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
+                 uint32_t scale, int inner_bits, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
     extern __shared__ uint32_t s_hist[];
     const int t = threadIdx.x;
     for (int b = t; b < nb; b += kThreads) s_hist[b] = 0u;
@@ -225,8 +236,7 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
         if (e < n) {
             const uint32_t b = __umulhi((uint32_t)o[i], scale);
             const double v = vals[e];
-            rec[s_hist[b] + r[i]] =
-                make_uint4((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), (uint32_t)c[i], (uint32_t)o[i]);
+            rec[s_hist[b] + r[i]] = make_rec(v, (uint32_t)o[i], (uint32_t)e, (uint32_t)c[i], inner_bits);
         }
     }
 }
@@ -241,13 +251,14 @@ struct TileShared {
     Rec rec[kTTile];
     uint32_t count[kMaxBuckets];                // entries of the tile, then where they begin in rec
     uint32_t shift[kMaxBuckets];                // place among the records minus place in rec
+    uint32_t to[kTTile];                        // where an entry goes among the records
     uint32_t w[kThreads / 32];
 };
 
 template <typename CT>
 __global__ void __launch_bounds__(kThreads, 2)
 k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, const double* __restrict__ vals, int64_t n, int64_t no, int64_t ni,
-                       uint32_t scale, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
+                       uint32_t scale, int inner_bits, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     TileShared& s = *reinterpret_cast<TileShared*>(s_raw);
     const int t = threadIdx.x;
@@ -283,13 +294,13 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
     }
     // all cursors of a thread at once: one wait, not one per bucket
     constexpr int kPerB = (kMaxBuckets + kThreads - 1) / kThreads;
-    uint32_t k[kPerB], at[kPerB], mine = 0;
+    uint32_t at[kPerB], mine = 0;
 #pragma unroll
     for (int q = 0; q < kPerB; ++q) {
         const int b = t + q * kThreads;
-        k[q] = b < nb ? s.count[b] : 0u;
-        at[q] = k[q] ? atomicAdd(cursor + b, k[q]) : 0u;
-        mine += k[q];
+        const uint32_t k = b < nb ? s.count[b] : 0u;
+        at[q] = k ? atomicAdd(cursor + b, k) : 0u;
+        mine += k;
     }
     const int lane = t & 31, w = t >> 5;
     uint32_t incl = mine;
@@ -305,29 +316,31 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
     for (int i = 0; i < kThreads / 32; ++i) from += i < w ? s.w[i] : 0u;
     bool full = false;
 #pragma unroll
-    for (int q = 0; q < kPerB; ++q)
-        if (k[q]) {
-            const uint32_t b = t + q * kThreads;
-            full |= slot && at[q] + k[q] > slot;
+    for (int q = 0; q < kPerB; ++q) {
+        const int b = t + q * kThreads;
+        const uint32_t k = b < nb ? s.count[b] : 0u;    // read again: registers
+        if (k) {
+            full |= slot && at[q] + k > slot;
             s.count[b] = from;
-            s.shift[b] = at[q] + b * slot - from;
-            from += k[q];
+            s.shift[b] = at[q] + (uint32_t)b * slot - from;
+            from += k;
         }
+    }
     if (__syncthreads_or(full)) {
         if (t == 0) report(kErrLong, stop, host);
         return;
     }
 #pragma unroll
     for (int i = 0; i < kTIpt; ++i)
-        if (i * kThreads + t < cnt)
-            s.rec[s.count[__umulhi(o[i], scale)] + r[i]] =
-                make_uint4((uint32_t)__double2loint(v[i]), (uint32_t)__double2hiint(v[i]), c[i], o[i]);
+        if (i * kThreads + t < cnt) {
+            const uint32_t b = __umulhi(o[i], scale), at = s.count[b] + r[i];
+            s.rec[at] = make_rec(v[i], o[i], blockIdx.x * (uint32_t)kTTile + i * kThreads + t, c[i], inner_bits);
+            s.to[at] = s.shift[b] + at;
+        }
     __syncthreads();
 #pragma unroll 4
     for (int j = t; j < cnt; j += kThreads) {
-        const Rec x = s.rec[j];
-        const uint32_t b = __umulhi(x.w, scale);
-        rec[s.shift[b] + (uint32_t)j] = x;
+        rec[s.to[j]] = s.rec[j];
     }
 }
 
@@ -338,9 +351,11 @@ struct BuildShared {
         double val[kCap];
         struct { uint32_t lo[kWidth], hi[kWidth]; };        // smallest and largest coordinate of a segment
         struct { double unused[kCap / 2]; uint32_t bin[kCap]; };
+        struct { uint32_t times[kCap], number[kCap]; };     // of equal coordinates, at their place: how many, and which in the input
     };
     uint32_t bin_end;                           // bin[kCap] when the bucket is full
     uint32_t w[kWarps];
+    uint32_t compares, places;                  // sums over the block
     uint16_t seg[kCap];                         // outer offsets of the entries, in order
 };
 static_assert(sizeof(uint32_t) * 2 * kWidth <= sizeof(double) * kCap / 2, "lo and hi lie before bin");
@@ -348,10 +363,11 @@ static_assert(sizeof(uint32_t) * 2 * kWidth <= sizeof(double) * kCap / 2, "lo an
 // The place of an entry is the start of its segment plus the number of smaller coordinates in it, counted over
 // shared memory.  Where segments are long (more than kDense compares per entry on average) they are first
 // cut into as many bins as they have entries, evenly between their smallest and largest coordinate, and only
-// the entries of one bin are compared.
+// the entries of one bin are compared.  first[b]: the entries before bucket b; lost[b]: the duplicates in it; *total: in all.
 template <typename P, typename I, bool DBL>
 __global__ void __launch_bounds__(kBThreads, 2)
-k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int nb, uint32_t slot, uint32_t* stop, unsigned long long* host,
+k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t scale, int inner_bits, int nb, uint32_t slot, uint32_t* stop, uint32_t* __restrict__ first, uint32_t* lost,
+             uint32_t* total, unsigned long long* host,
              P* __restrict__ pos1, I* __restrict__ crd, double* __restrict__ val, uint32_t* __restrict__ seg_out, uint32_t* __restrict__ outer_count) {
     sp_wait_for_previous_kernel();
     if (stopped(stop)) return;
@@ -360,17 +376,23 @@ k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t s
     const int t = threadIdx.x, b = blockIdx.x;
     const uint32_t place = records_of(b, slot, cursor);
     const int cnt = (int)(slot ? cursor[b] : cursor[b] - place);
-    const int64_t lo = bucket_begin(b, scale, no), hi = b + 1 < nb ? bucket_begin(b + 1, scale, no) : no;
-    const int width = (int)(hi - lo);
+    const uint32_t lo = (uint32_t)bucket_begin(b, scale, no);
+    const int width = (int)((b + 1 < nb ? bucket_begin(b + 1, scale, no) : no) - lo);
     // entries of this thread, requested first; the values are fetched again at the end (registers)
     const Rec* mine = rec + place + t;
+    const uint32_t inner_mask = inner_bits < 32 ? (1u << inner_bits) - 1u : ~0u;
     uint32_t c[kIpt], qr[kIpt];                 // inner coordinate; outer offset << 16 | rank, later the place
 #pragma unroll
     for (int i = 0; i < kIpt; ++i) {
         c[i] = qr[i] = 0u;
-        if (i * kBThreads + t < cnt) { const Rec x = mine[i * kBThreads]; c[i] = x.z; qr[i] = x.w - (uint32_t)lo; }
+        if (i * kBThreads + t < cnt) {
+            const Rec x = mine[i * kBThreads];
+            c[i] = x.z & inner_mask;
+            qr[i] = ((x.w >> (kOffShift - 32)) - lo) & (kWidth - 1);
+        }
     }
     for (int q = t; q < width; q += kBThreads) { s.count[q] = 0u; s.lo[q] = ~0u; s.hi[q] = 0u; }
+    if (t == 0) s.compares = s.places = 0u;
     uint32_t before = 0, base = place;          // base: entries in the buckets before
     if (slot) {
         for (int q = t; q < b; q += kBThreads) before += cursor[q];
@@ -381,20 +403,18 @@ k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t s
     for (int i = 0; i < kIpt; ++i)
         if (i * kBThreads + t < cnt) qr[i] = qr[i] << 16 | atomicAdd(&s.count[qr[i]], 1u);
     __syncthreads();
-    // mean number of compares without bins; outer level
-    uint32_t sq = 0, filled = 0, tot_sq, tot_filled;
+    uint32_t sq = 0;                            // mean number of compares without bins
     constexpr int kPerW = kWidth / kBThreads;
 #pragma unroll
     for (int i = 0; i < kPerW; ++i) {
         const int q = t * kPerW + i;
         const uint32_t k = q < width ? s.count[q] : 0u;
         sq += k * k;                            // at most kCap^2 in all
-        filled += k != 0;
     }
-    const uint32_t at_filled = block_scan(filled, s.w, &tot_filled);
-    block_scan(sq, s.w, &tot_sq);
-    const bool bins = tot_sq > (uint32_t)kDense * (uint32_t)cnt;
-    scan_shared<kPerW>(s.count, width, s.w);
+    sq = __reduce_add_sync(0xffffffffu, sq);
+    if (sp_lane() == 0) atomicAdd(&s.compares, sq);
+    scan_shared<kPerW>(s.count, width, s.w);    // (also the barrier after that)
+    const bool bins = s.compares > (uint32_t)kDense * (uint32_t)cnt;
     if (!DBL) {
         for (int q = t; q < width; q += kBThreads) pos1[lo + q] = (P)(base + s.count[q]);
         if (b == nb - 1 && t == 0) pos1[no] = (P)n;
@@ -456,11 +476,35 @@ k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t s
             }
     }
     // Distinct coordinates take the places 0 .. cnt - 1; of equal ones all get the lowest, so the sum falls short.
-    uint32_t tot_sum;
-    block_scan(sum, s.w, &tot_sum);             // also the barrier after which coordinates and bins are dead
-    if (tot_sum != (uint32_t)(cnt * (cnt - 1) / 2)) {
-        if (t == 0) report(kErrDup, stop, host);
-        return;
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (sp_lane() == 0) atomicAdd(&s.places, sum);
+    __syncthreads();                            // coordinates and bins are dead from here on
+    const bool dups = s.places != (uint32_t)(cnt * (cnt - 1) / 2);
+    if (dups) {                                 // equal ones take successive places in the order of the input
+        for (int j = t; j < cnt; j += kBThreads) s.times[j] = 0u;
+        __syncthreads();
+        auto number_of = [&](int j) {
+            const uint2 k = reinterpret_cast<const uint2*>(rec + place + j)[1];
+            return (uint32_t)((((uint64_t)k.y << 32 | k.x) << kOffBits) >> (kOffBits + inner_bits));
+        };
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i) s.crd[i * kBThreads + t] = to[i];       // kept there: the loops are not unrolled
+#pragma unroll 1
+        for (int j = t; j < cnt; j += kBThreads) {
+            const uint32_t p = s.crd[j] & 0xffffu;
+            s.number[p + atomicAdd(&s.times[p], 1u)] = number_of(j);
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int j = t; j < cnt; j += kBThreads) {
+            const uint32_t p = s.crd[j] & 0xffffu, number = number_of(j);
+            uint32_t smaller = 0;
+            for (uint32_t k = 0; k < s.times[p]; ++k) smaller += s.number[p + k] < number;
+            s.crd[j] += smaller;
+        }
+#pragma unroll
+        for (int i = 0; i < kIpt; ++i) to[i] = s.crd[i * kBThreads + t];
+        __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < kIpt; ++i)
@@ -469,36 +513,114 @@ k_rows_build(Rec* rec, const uint32_t* cursor, int64_t n, int64_t no, uint32_t s
             const uint32_t p = to[i] & 0xffffu;
             s.crd[p] = c[i];
             s.val[p] = __hiloint2double((int)v.y, (int)v.x);
-            if (seg_out) s.seg[p] = (uint16_t)(to[i] >> 16);
+            if (seg_out || dups) s.seg[p] = (uint16_t)(to[i] >> 16);
         }
     __syncthreads();
-    for (int j = t; j < cnt; j += kBThreads) {
-        crd[base + j] = (I)s.crd[j];
-        val[base + j] = s.val[j];
-        if (seg_out) seg_out[base + j] = (uint32_t)lo + s.seg[j];
+    uint32_t distinct = (uint32_t)cnt;
+    if (!dups) {
+        for (int j = t; j < cnt; j += kBThreads) {
+            crd[base + j] = (I)s.crd[j];
+            val[base + j] = s.val[j];
+            if (seg_out) seg_out[base + j] = lo + s.seg[j];
+        }
+    } else {
+        // the first of equal ones adds the others up and is stored; each thread takes kIpt adjacent entries
+        const int j0 = t * kIpt;
+        uint32_t heads = 0;
+#pragma unroll 1
+        for (int j = j0; j < j0 + kIpt && j < cnt; ++j)
+            if (j == 0 || s.crd[j] != s.crd[j - 1] || s.seg[j] != s.seg[j - 1]) heads |= 1u << (j - j0);
+        const uint32_t stored = block_scan(__popc(heads), s.w, &distinct);
+        uint32_t at = base + stored;
+#pragma unroll 1
+        for (int j = j0; j < j0 + kIpt && j < cnt; ++j)
+            if (heads >> (j - j0) & 1u) {
+                double sum = s.val[j];
+                for (int k = j + 1; k < cnt && s.crd[k] == s.crd[j] && s.seg[k] == s.seg[j]; ++k) sum += s.val[k];
+                crd[at] = (I)s.crd[j];
+                val[at] = sum;
+                if (seg_out) seg_out[at] = lo + s.seg[j];
+                ++at;
+            }
+        __syncthreads();
+        at = stored;                            // from here on crd[j] is the number of entries stored before entry j
+#pragma unroll 1
+        for (int j = j0; j < j0 + kIpt && j < cnt; ++j) {
+            s.crd[j] = at;
+            at += heads >> (j - j0) & 1u;
+        }
+        __syncthreads();
+        for (int q = t; q <= width; q += kBThreads) {
+            const uint32_t j = s.count[q];
+            s.count[q] = j < (uint32_t)cnt ? s.crd[j] : distinct;
+            if (!DBL && q < width) pos1[lo + q] = (P)(base + s.count[q]);
+        }
+        __syncthreads();
+        if (t == 0) {
+            atomicAdd(total, (uint32_t)cnt - distinct);
+            *static_cast<volatile unsigned long long*>(host + kErrDup) = 1;
+        }
     }
+    if (t == 0) { first[b] = base; lost[b] = (uint32_t)cnt - distinct; }
     if (DBL) {                                  // the stored indices and their first entries, in order, where the records were
-        uint32_t k = at_filled;
+        uint32_t filled = 0, all;
+#pragma unroll
+        for (int i = 0; i < kPerW; ++i) {
+            const int q = t * kPerW + i;
+            filled += q < width && s.count[q + 1] != s.count[q];
+        }
+        uint32_t k = block_scan(filled, s.w, &all);
 #pragma unroll
         for (int i = 0; i < kPerW; ++i) {
             const int q = t * kPerW + i;
             if (q < width && s.count[q + 1] != s.count[q])
-                *reinterpret_cast<uint2*>(rec + place + k++) = make_uint2((uint32_t)(lo + q), base + s.count[q]);
+                *reinterpret_cast<uint2*>(rec + place + k++) = make_uint2(lo + q, base + s.count[q]);
         }
-        if (t == 0) outer_count[b] = tot_filled;
+        if (t == 0) outer_count[b] = all;
     }
 }
 
-// Joins the buckets' lists of non-empty outer indices and of their first entries: crd[0] and pos[1].
+// After duplicates: the entries that every bucket stored, moved to where they belong; first and lost as k_rows_build left them.
+template <typename P, typename I, bool DBL>
+__global__ void __launch_bounds__(kBThreads)
+k_rows_close_up(const uint32_t* __restrict__ first, const uint32_t* __restrict__ lost, int64_t n, int64_t stored, int64_t no, uint32_t scale, int nb,
+                const P* __restrict__ pos1, const I* __restrict__ crd, const double* __restrict__ val, const uint32_t* __restrict__ seg,
+                P* __restrict__ pos1_out, I* __restrict__ crd_out, double* __restrict__ val_out, uint32_t* __restrict__ seg_out) {
+    __shared__ uint32_t s_w[kWarps];
+    const int t = threadIdx.x, b = blockIdx.x;
+    uint32_t mine = 0, before;
+    for (int q = t; q < b; q += kBThreads) mine += lost[q];
+    block_scan(mine, s_w, &before);
+    const uint32_t from = first[b], to = from - before;
+    const int cnt = (int)((b + 1 < nb ? first[b + 1] : (uint32_t)n) - from - lost[b]);
+    for (int j = t; j < cnt; j += kBThreads) {
+        crd_out[to + j] = crd[from + j];
+        val_out[to + j] = val[from + j];
+        if (seg) seg_out[to + j] = seg[from + j];
+    }
+    if (!DBL) {
+        const int64_t lo = bucket_begin(b, scale, no), hi = b + 1 < nb ? bucket_begin(b + 1, scale, no) : no;
+        for (int64_t o = lo + t; o < hi; o += kBThreads) pos1_out[o] = pos1[o] - (P)before;
+        if (b == nb - 1 && t == 0) pos1_out[no] = (P)stored;
+    }
+}
+
+// Joins the buckets' lists of non-empty outer indices and of their first entries: crd[0] and pos[1].  lost: entries
+// that buckets hold less than they take up, nullptr = none.
 template <typename P, typename I>
 __global__ void __launch_bounds__(kBThreads)
-k_rows_outer(const Rec* rec, const uint32_t* cursor, const uint32_t* outer_count, int64_t n, int nb, uint32_t slot,
+k_rows_outer(const Rec* rec, const uint32_t* cursor, const uint32_t* outer_count, const uint32_t* lost, int64_t n, int nb, uint32_t slot,
              uint32_t* stop, unsigned long long* host, P* __restrict__ pos0, I* __restrict__ crd0, P* __restrict__ pos1) {
     sp_wait_for_previous_kernel();
     if (stopped(stop)) return;
     __shared__ uint32_t s_w[kWarps];
     const int t = threadIdx.x, b = blockIdx.x;
-    uint32_t before = 0, base;
+    uint32_t before = 0, base, gone = 0;
+    if (lost) {
+        for (int q = t; q < b; q += kBThreads) before += lost[q];
+        block_scan(before, s_w, &gone);
+        before = 0;
+    }
     for (int q = t; q < b; q += kBThreads) before += outer_count[q];
     block_scan(before, s_w, &base);
     const Rec* list = rec + records_of(b, slot, cursor);
@@ -506,7 +628,7 @@ k_rows_outer(const Rec* rec, const uint32_t* cursor, const uint32_t* outer_count
     for (uint32_t q = t; q < cnt; q += kBThreads) {
         const uint2 x = *reinterpret_cast<const uint2*>(list + q);
         crd0[base + q] = (I)x.x;
-        pos1[base + q] = (P)x.y;
+        pos1[base + q] = (P)(x.y - gone);
     }
     if (b == nb - 1 && t == 0) {
         pos1[base + cnt] = (P)n;
@@ -520,7 +642,7 @@ k_rows_outer(const Rec* rec, const uint32_t* cursor, const uint32_t* outer_count
 
 // Returns SP_OK with *out set; an error; or SP_ERR_UNSUPPORTED when the caller should take the radix path.
 sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64_t n, const void* outer, const void* inner, int coord_bits,
-                       const double* vals, int posBits, int crdBits, cudaStream_t stream, sp_tensor** out) {
+                       const double* vals, int posBits, int crdBits, unsigned flags, cudaStream_t stream, sp_tensor** out) {
     const int64_t no = dims[ord[0]], ni = dims[ord[1]];
     // narrow positions need the radix path's width checks; records hold 32-bit coordinates
     if (posBits < 32 || crdBits < 32 || no >= ((int64_t)1 << 31) || ni >= ((int64_t)1 << 32)) return SP_ERR_UNSUPPORTED;
@@ -532,6 +654,10 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         buckets = no;
     }
     const int nb = (int)buckets;
+    int inner_bits = 1, number_bits = 1;                 // what a record holds beside the value has to fit
+    while (((int64_t)1 << inner_bits) < ni) ++inner_bits;
+    while (((int64_t)1 << number_bits) < n) ++number_bits;
+    if (inner_bits + number_bits > kOffShift) return SP_ERR_UNSUPPORTED;
     const uint32_t scale = (uint32_t)std::min<uint64_t>(((uint64_t)nb << 32) / (uint64_t)no, 0xffffffffull);
     for (int64_t b : {(int64_t)0, (int64_t)nb - 1})      // the last range also takes what rounding leaves over
         if ((b + 1 < nb ? bucket_begin(b + 1, scale, no) : no) - bucket_begin(b, scale, no) > kWidth) return SP_ERR_UNSUPPORTED;
@@ -541,17 +667,18 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     const bool counted = n >= kCountFrom || (int64_t)nb * kCap > 16 * n + 65536;
     const uint32_t slot = counted ? 0u : (uint32_t)kCap;
     const size_t records = counted ? (size_t)n : (size_t)nb * kCap;
-    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb + 2);
-    ws.reserve(cursors + sp_workspace::bytes_for<Rec>(records) + (dbl ? cursors : 0));
-    uint32_t* cursor = ws.get<uint32_t>((size_t)nb + 2);
+    const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb + 3);
+    ws.reserve(3 * cursors + sp_workspace::bytes_for<Rec>(records) + (dbl ? cursors : 0));
+    uint32_t* cursor = ws.get<uint32_t>((size_t)nb + 3);
     Rec* rec = ws.get<Rec>(records);
-    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb + 2) : nullptr;
+    uint32_t *first = ws.get<uint32_t>((size_t)nb + 3), *lost = ws.get<uint32_t>((size_t)nb + 3);
+    uint32_t* outer_count = dbl ? ws.get<uint32_t>((size_t)nb + 3) : nullptr;
     unsigned long long* host = sp_host_words();
     if (ws.failed || !host) return SP_ERR_ALLOC;
-    uint32_t *stop = cursor + nb, *ticket = cursor + nb + 1;
+    uint32_t *stop = cursor + nb, *ticket = cursor + nb + 1, *total = cursor + nb + 2;
 
     // counted while the host prepares the rest
-    SP_CUDA(cudaMemsetAsync(cursor, 0, (size_t)(nb + 2) * sizeof(uint32_t), stream));
+    SP_CUDA(cudaMemsetAsync(cursor, 0, (size_t)(nb + 3) * sizeof(uint32_t), stream));
     if (counted) {
         const unsigned blocks = (unsigned)std::min<int64_t>(kCBlocks, sp_ceil_div(n, kCThreads * 16));
         if (coord_bits == 32) k_rows_count<int32_t><<<blocks, kCThreads, 0, stream>>>(static_cast<const int32_t*>(outer), n, no, scale, nb, cursor, stop, ticket, host);
@@ -571,27 +698,31 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     t->posBits = posBits;
     t->crdBits = crdBits;
     for (int l = 0; l < 2; ++l) { t->dims[l] = dims[l]; t->lt[l] = lt[l]; t->ord[l] = ord[l]; }
-    // one allocation for the handle's arrays; a compressed outer level's are sized for its bound
-    const int64_t nq = dbl ? std::min(no, n) : no;
-    const size_t b_pos0 = dbl ? sp_workspace::padded(2 * pw) : 0, b_crd0 = dbl ? sp_workspace::padded((size_t)nq * cw) : 0;
-    const size_t b_pos1 = sp_workspace::padded((size_t)(nq + 1) * pw), b_crd1 = sp_workspace::padded((size_t)n * cw);
-    t->block = sp_dev_alloc(b_pos0 + b_crd0 + b_pos1 + b_crd1 + sp_workspace::padded((size_t)n * sizeof(double)), stream);
-    if (!t->block) return fail(SP_ERR_ALLOC);
-    char* p = static_cast<char*>(t->block);
-    if (dbl) { t->pos[0] = p; t->crd[0] = p + b_pos0; t->npos[0] = 2; }
-    p += b_pos0 + b_crd0;
-    t->pos[1] = p;
-    t->crd[1] = p + b_pos1;
-    t->val = reinterpret_cast<double*>(p + b_pos1 + b_crd1);
-    t->ncrd[1] = t->nval = n;
-    uint32_t* seg_out = nullptr;
-    if (ord[0] == 1) {                                  // column-major: the column of every entry, for SpMM
-        sp_partition sg;
-        sg.aux = static_cast<int64_t*>(sp_dev_alloc((size_t)n * sizeof(uint32_t), stream));
-        if (!sg.aux) return fail(SP_ERR_ALLOC);
-        seg_out = reinterpret_cast<uint32_t*>(sg.aux);
-        t->parts[(uint64_t)SP_PART_SEGIDS << 56] = sg;
-    }
+    // the handle's arrays, one allocation, for `entries` stored entries and `outers` outer indices (a compressed outer
+    // level's are at first sized for their bound)
+    auto arrays = [&](int64_t entries, int64_t outers) {
+        const size_t b_pos0 = dbl ? sp_workspace::padded(2 * pw) : 0, b_crd0 = dbl ? sp_workspace::padded((size_t)outers * cw) : 0;
+        const size_t b_pos1 = sp_workspace::padded((size_t)(outers + 1) * pw), b_crd1 = sp_workspace::padded((size_t)entries * cw);
+        t->block = sp_dev_alloc(b_pos0 + b_crd0 + b_pos1 + b_crd1 + sp_workspace::padded((size_t)entries * sizeof(double)), stream);
+        if (!t->block) return false;
+        char* p = static_cast<char*>(t->block);
+        if (dbl) { t->pos[0] = p; t->crd[0] = p + b_pos0; t->npos[0] = 2; }
+        p += b_pos0 + b_crd0;
+        t->pos[1] = p;
+        t->crd[1] = p + b_pos1;
+        t->val = reinterpret_cast<double*>(p + b_pos1 + b_crd1);
+        t->ncrd[1] = t->nval = entries;
+        if (ord[0] == 1) {                              // column-major: the column of every entry, for SpMM
+            sp_partition sg;
+            sg.aux = static_cast<int64_t*>(sp_dev_alloc((size_t)entries * sizeof(uint32_t), stream));
+            if (!sg.aux) return false;
+            t->parts[(uint64_t)SP_PART_SEGIDS << 56] = sg;
+        }
+        return true;
+    };
+    auto columns = [&]() { return ord[0] == 1 ? reinterpret_cast<uint32_t*>(t->parts[(uint64_t)SP_PART_SEGIDS << 56].aux) : nullptr; };
+    if (!arrays(n, dbl ? std::min(no, n) : no)) return fail(SP_ERR_ALLOC);
+    uint32_t* seg_out = columns();
 
     const bool small = n < kSmall;
     cudaError_t e = cudaSuccess;
@@ -600,12 +731,12 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         const CT *oc = static_cast<const CT*>(outer), *ic = static_cast<const CT*>(inner);                                \
         if (small) {                                                                                                      \
             e = sp_launch_dependent(k_rows_partition<CT, 2>, dim3((unsigned)sp_ceil_div(n, kThreads * 2)), dim3(kThreads), \
-                                    (size_t)nb * sizeof(uint32_t), stream, oc, ic, vals, n, no, ni, scale, nb, slot, cursor, rec, stop, host); \
+                                    (size_t)nb * sizeof(uint32_t), stream, oc, ic, vals, n, no, ni, scale, inner_bits, nb, slot, cursor, rec, stop, host); \
         } else {                                                                                                          \
             e = sp_allow_shared<k_rows_partition_tiles<CT>>(t->device, sizeof(TileShared));                               \
             if (e == cudaSuccess)                                                                                         \
                 e = sp_launch_dependent(k_rows_partition_tiles<CT>, dim3((unsigned)sp_ceil_div(n, kTTile)), dim3(kThreads), sizeof(TileShared), \
-                                        stream, oc, ic, vals, n, no, ni, scale, nb, slot, cursor, rec, stop, host);             \
+                                        stream, oc, ic, vals, n, no, ni, scale, inner_bits, nb, slot, cursor, rec, stop, host);             \
         }                                                                                                                 \
     } while (0)
     if (coord_bits == 32) SP_ROWS_PARTITION(int32_t);
@@ -616,7 +747,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
 #define SP_ROWS_BUILD(DBL)                                                                                                \
     do {                                                                                                                  \
         if (e == cudaSuccess) e = sp_allow_shared<k_rows_build<P, I, DBL>>(t->device, sizeof(BuildShared));             \
-        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), rec, (const uint32_t*)cursor, n, no, scale, nb, slot, stop, host, pos1, \
+        SP_ROWS_LAUNCH((k_rows_build<P, I, DBL>), sizeof(BuildShared), rec, (const uint32_t*)cursor, n, no, scale, inner_bits, nb, slot, stop, first, lost, total, host, pos1, \
                        crd1, t->val, seg_out, outer_count);                                        \
     } while (0)
     SP_DISPATCH_WIDTHS(t, {
@@ -626,7 +757,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         I* crd1 = static_cast<I*>(t->crd[1]);
         if (dbl) {
             SP_ROWS_BUILD(true);
-            SP_ROWS_LAUNCH((k_rows_outer<P, I>), 0, (const Rec*)rec, (const uint32_t*)cursor, (const uint32_t*)outer_count, n, nb, slot, stop, host,
+            SP_ROWS_LAUNCH((k_rows_outer<P, I>), 0, (const Rec*)rec, (const uint32_t*)cursor, (const uint32_t*)outer_count, (const uint32_t*)nullptr, n, nb, slot, stop, host,
                            pos0, crd0, pos1);
         } else {
             SP_ROWS_BUILD(false);
@@ -638,9 +769,43 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return fail(SP_ERR_CUDA);
     if (host[kErrRange]) return fail(SP_ERR_OUT_OF_RANGE);
-    if (host[kErrDup] || host[kErrLong]) return fail(SP_ERR_UNSUPPORTED);
-    t->npos[1] = (dbl ? (int64_t)host[kOuterCount] : no) + 1;
-    if (dbl) t->ncrd[0] = (int64_t)host[kOuterCount];
+    if (host[kErrLong]) return fail(SP_ERR_UNSUPPORTED);
+    const int64_t outers = dbl ? (int64_t)host[kOuterCount] : no;
+    if (host[kErrDup]) {
+        if (flags & SP_DUP_ERROR) return fail(SP_ERR_DUPLICATE);
+        if (cudaMemcpyAsync(host + kLost, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+            cudaStreamSynchronize(stream) != cudaSuccess)
+            return fail(SP_ERR_CUDA);
+        const int64_t stored = n - (int64_t)(uint32_t)host[kLost];
+        const void *pos1_was = t->pos[1], *crd_was = t->crd[1], *block_was = t->block;
+        const double* val_was = t->val;
+        t->block = nullptr;                             // the first arrays go back with the scratch
+        ws.ptrs.push_back(const_cast<void*>(block_was));
+        if (seg_out) ws.ptrs.push_back(seg_out);
+        t->parts.clear();
+        for (int l = 0; l < 2; ++l) t->pos[l] = t->crd[l] = nullptr;
+        t->val = nullptr;
+        if (!arrays(stored, outers)) return fail(SP_ERR_ALLOC);
+        SP_DISPATCH_WIDTHS(t, {
+            const P* const pos1_in = static_cast<const P*>(pos1_was);
+            const I* const crd_in = static_cast<const I*>(crd_was);
+            P* const pos1 = static_cast<P*>(t->pos[1]);
+            I* const crd1 = static_cast<I*>(t->crd[1]);
+            if (dbl) {
+                k_rows_close_up<P, I, true><<<(unsigned)nb, kBThreads, 0, stream>>>(first, lost, n, stored, no, scale, nb, pos1_in, crd_in, val_was,
+                                                                                   seg_out, pos1, crd1, t->val, columns());
+                k_rows_outer<P, I><<<(unsigned)nb, kBThreads, 0, stream>>>(rec, cursor, outer_count, lost, stored, nb, slot, stop, host,
+                                                                           static_cast<P*>(t->pos[0]), static_cast<I*>(t->crd[0]), pos1);
+            } else {
+                k_rows_close_up<P, I, false><<<(unsigned)nb, kBThreads, 0, stream>>>(first, lost, n, stored, no, scale, nb, pos1_in, crd_in, val_was,
+                                                                                    seg_out, pos1, crd1, t->val, columns());
+            }
+        });
+        if (cudaGetLastError() != cudaSuccess) return fail(SP_ERR_CUDA);
+        sp_count_launches(dbl ? 2 : 1);
+    }
+    t->npos[1] = outers + 1;
+    if (dbl) t->ncrd[0] = outers;
     *out = t;
     return SP_OK;
 }
