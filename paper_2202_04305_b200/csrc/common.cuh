@@ -262,7 +262,8 @@ sp_status sp_get_merge_partition(sp_tensor* t, int64_t items_per_chunk, cudaStre
 // Length of the longest last-level segment (row of CSR, stored row of DCSR, ...), measured on the
 // device on first use (one small kernel and one read-back, which waits for the stream) and kept.
 sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out);
-// with_marks: the entries' words too (level-1 size below 2^29); the tables are cached together or not at all.
+// with_marks: the entries' words too (level-1 size below 2^29); the tables are cached together or not at all, and
+// once per handle: every call on a handle asks for the same nnz_per_chunk, whatever its number of columns.
 sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t nnz_per_chunk, bool with_marks, cudaStream_t stream, sp_partition* out);
 
 // sp_pack for matrices with a compressed inner level and short segments (pack_rows.cu).  SP_ERR_UNSUPPORTED:

@@ -207,8 +207,9 @@ __global__ void __launch_bounds__(kFThreads, 8)
 k_mttkrp_staged(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, const double* __restrict__ val,
                 const P* __restrict__ pos1, const I* __restrict__ crd0, const double* __restrict__ F1,
                 const double* __restrict__ F2, int64_t R, double* __restrict__ M, const int64_t* __restrict__ pslice,
-                int64_t nnz, int64_t nchunks, int64_t nslice,
+                int64_t nnz, int chunks, int64_t nranges, int64_t nslice,
                 int64_t d0, int64_t d1, int64_t d2) {
+    // chunks: chunks of the table in a group's range
     // d0, d1, d2: rows of M, F1, F2 (used by the bounds-checking debug build only)
     constexpr int GL = 32 / S;      // lanes per group = entries per group and batch
     constexpr int kStep = 2;       // entries of a group in flight
@@ -219,7 +220,7 @@ k_mttkrp_staged(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, 
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, gw = lane / GL, hl = lane % GL, g = threadIdx.x / GL;
     const int64_t w = (int64_t)blockIdx.x * kGroups + g;
     const int64_t p0 = w * kFPer;
-    const int nz = w < nchunks ? (int)(nnz - p0 < kFPer ? nnz - p0 : kFPer) : 0;
+    const int nz = w < nranges ? (int)(nnz - p0 < kFPer ? nnz - p0 : kFPer) : 0;
     const int nmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)nz);
     const uint32_t rbytes = (uint32_t)R * 8u;
     const int64_t rb = (int64_t)blockIdx.y * 32;
@@ -234,7 +235,7 @@ k_mttkrp_staged(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, 
     auto column = [&](int q) { return (W256 ? 4 * hl + 2 * (q / 2) : (q / 2) * 2 * GL + 2 * hl) + (q & 1); };
     if (hl == 0) s_id[2 * g] = s_id[2 * g + 1] = -1;
     const char *F1g = reinterpret_cast<const char*>(F1 + rb), *F2g = reinterpret_cast<const char*>(F2 + rb);
-    int64_t s = nz > 0 ? pslice[w] : 0;
+    int64_t s = nz > 0 ? pslice[w * chunks] : 0;
     bool first = true;
     double accf[S], accs[S];
 #pragma unroll
@@ -370,8 +371,9 @@ __global__ void __launch_bounds__(kGThreads, L == 8 && V == 3 ? 8 : 1)      // 1
 k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, const double* __restrict__ val,
                const P* __restrict__ pos1, const I* __restrict__ crd0, const double* __restrict__ F1,
                const double* __restrict__ F2, int64_t R, double* __restrict__ M, const int64_t* __restrict__ pslice,
-               const int64_t* __restrict__ prow, int64_t nnz, int per, int64_t nchunks, int64_t nslice,
+               const int64_t* __restrict__ prow, int64_t nnz, int per, int chunks, int64_t nranges, int64_t nslice,
                int64_t d0, int64_t d1, int64_t d2) {
+    // chunks: chunks of the table in a group's range of per entries
     // d0, d1, d2: rows of M, F1, F2 (used by the bounds-checking debug build only)
     constexpr int kGroups = kGThreads / L, kSlots = 2 * kGroups;
     __shared__ double s_sum[kSlots][L * V];         // slot 2 g: the slice group g's range begins in, 2 g + 1: the one it ends in
@@ -379,7 +381,7 @@ k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, c
     const int g = threadIdx.x / L, gl = threadIdx.x % L;
     const int64_t w = (int64_t)blockIdx.x * kGroups + g;
     const int64_t p0 = w * per;
-    const int nz = w < nchunks ? (int)(nnz - p0 < per ? nnz - p0 : per) : 0;
+    const int nz = w < nranges ? (int)(nnz - p0 < per ? nnz - p0 : per) : 0;
     const int64_t cb = (int64_t)blockIdx.y * (L * V);
     int coff[V / W];                                // idle lanes read the tile's first run and never write
     bool on[V / W];
@@ -400,8 +402,8 @@ k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, c
         const uint32_t* ml = marks + p0;
         const I* cl = crd2 + p0;
         const double* vl = val + p0;
-        int64_t s = pslice[w];
-        int64_t i = SP_IDX(prow[w], d0);
+        int64_t s = pslice[w * chunks];
+        int64_t i = SP_IDX(prow[w * chunks], d0);
         bool first = true, open = true;
         double accf[V], accs[V];
 #pragma unroll
@@ -544,18 +546,23 @@ static sp_status mttkrp_levels(sp_tensor* T, const double* F1, const double* F2,
     // Large tensors with 8 < R <= 32 take the staged warps: R = 16, 24, 32 and 5 M entries 141, 146, 145 us against
     // 165, 197, 189; 1 M entries, R = 32: 38 against 44.  R = 8 goes to lane groups, whose four lanes all have columns.
     const bool staged = fast && nnz >= 1000000 && R > 8 && R <= 32;
+    // Entries per group, as below per warp.  The table says where chunks begin that both this range and the staged one are
+    // whole numbers of, so that every R finds what it needs in the handle's one table.  (Ranges of whole 64s instead, for
+    // longer chunks: 1.3 to 4 M entries, R = 17 and 48, 4 to 12 % slower.)
+    const int64_t per = std::max<int64_t>(16, std::min<int64_t>(256, sp_ceil_div(sp_ceil_div(nnz, 18944), 16) * 16));
+    const int64_t chunk = std::min<int64_t>(per & -per, kFPer);
     if (!staged && d1 < ((int64_t)1 << 29)) {
         sp_partition part;
-        const int64_t per = std::max<int64_t>(16, std::min<int64_t>(256, sp_ceil_div(sp_ceil_div(nnz, 18944), 16) * 16));   // per group, as below per warp
-        sp_status st = sp_get_mttkrp_partition(T, per, true, stream, &part);
+        sp_status st = sp_get_mttkrp_partition(T, chunk, true, stream, &part);
         if (st != SP_OK) return st;
+        const int64_t ranges = sp_ceil_div(nnz, per);
         const bool pairs = R % 2 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0 &&
                            reinterpret_cast<uintptr_t>(M) % 16 == 0;
 #define SP_MTTKRP_GROUP(L, V, W, U)                                                                                        \
-    k_mttkrp_group<P, I, L, V, W, U><<<dim3((unsigned)sp_ceil_div(part.nchunks * L, kGThreads), (unsigned)sp_ceil_div(R, L * V)), kGThreads, 0, stream>>>( \
+    k_mttkrp_group<P, I, L, V, W, U><<<dim3((unsigned)sp_ceil_div(ranges * L, kGThreads), (unsigned)sp_ceil_div(R, L * V)), kGThreads, 0, stream>>>( \
         part.marks, static_cast<const I*>(T->crd[2]), T->val, static_cast<const P*>(T->pos[1]),                                 \
         T->lt[0] == SP_COMPRESSED ? static_cast<const I*>(T->crd[0]) : nullptr, F1, F2, R, M, part.aux, part.row, nnz, (int)per, \
-        part.nchunks, T->npos[1] - 1, T->dims[T->ord[0]], d1, d2)
+        (int)(per / chunk), ranges, T->npos[1] - 1, T->dims[T->ord[0]], d1, d2)
         SP_DISPATCH_WIDTHS(T, {
             if (pairs) {
                 if (R <= 8) SP_MTTKRP_GROUP(4, 2, 2, 6);
@@ -581,12 +588,13 @@ static sp_status mttkrp_levels(sp_tensor* T, const double* F1, const double* F2,
     }
     sp_partition part;
     if (staged) {
-        sp_status st = sp_get_mttkrp_partition(T, kFPer, true, stream, &part);
+        sp_status st = sp_get_mttkrp_partition(T, chunk, true, stream, &part);
         if (st != SP_OK) return st;
+        const int64_t ranges = sp_ceil_div(nnz, kFPer);
 #define SP_MTTKRP_STAGED(S, W)                                                                                             \
-    k_mttkrp_staged<P, I, S, W><<<dim3((unsigned)sp_ceil_div(part.nchunks * (32 / S), kFThreads), (unsigned)sp_ceil_div(R, 32)), kFThreads, 0, stream>>>( \
+    k_mttkrp_staged<P, I, S, W><<<dim3((unsigned)sp_ceil_div(ranges * (32 / S), kFThreads), (unsigned)sp_ceil_div(R, 32)), kFThreads, 0, stream>>>( \
         part.marks, static_cast<const I*>(T->crd[2]), T->val, static_cast<const P*>(T->pos[1]),                            \
-        T->lt[0] == SP_COMPRESSED ? static_cast<const I*>(T->crd[0]) : nullptr, F1, F2, R, M, part.aux, nnz, part.nchunks, \
+        T->lt[0] == SP_COMPRESSED ? static_cast<const I*>(T->crd[0]) : nullptr, F1, F2, R, M, part.aux, nnz, (int)(kFPer / chunk), ranges, \
         T->npos[1] - 1, T->dims[T->ord[0]], d1, d2)
         // one 32-byte load per lane and factor row when every lane has its four columns and rows are 32-byte aligned
         const bool w256 = R % 32 == 0 && reinterpret_cast<uintptr_t>(F1) % 32 == 0 && reinterpret_cast<uintptr_t>(F2) % 32 == 0;
@@ -602,8 +610,8 @@ static sp_status mttkrp_levels(sp_tensor* T, const double* F1, const double* F2,
         return SP_OK;
     }
     // Level-1 sizes of 2^29 and more: entries per warp as above
-    const int64_t per = std::max<int64_t>(32, std::min<int64_t>(512, sp_ceil_div(sp_ceil_div(nnz, 4736), 32) * 32));
-    sp_status st = sp_get_mttkrp_partition(T, per, false, stream, &part);
+    const int64_t wper = std::max<int64_t>(32, std::min<int64_t>(512, sp_ceil_div(sp_ceil_div(nnz, 4736), 32) * 32));
+    sp_status st = sp_get_mttkrp_partition(T, wper, false, stream, &part);
     if (st != SP_OK) return st;
     const unsigned blocks = (unsigned)sp_ceil_div(part.nchunks * 32, kTThreads);
     SP_DISPATCH_WIDTHS(T, {

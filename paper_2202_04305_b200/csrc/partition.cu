@@ -343,7 +343,8 @@ sp_status sp_widened(sp_tensor* t, cudaStream_t stream, sp_tensor** out) {
 
 sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, bool with_marks, cudaStream_t stream, sp_partition* out) {
     std::lock_guard<std::mutex> lock(t->mu);
-    const uint64_t key = ((uint64_t)(with_marks ? SP_PART_MTTKRP_MARKS : SP_PART_MTTKRP) << 56) | (uint64_t)per;
+    // the words do not depend on per: a handle has one table of them, and per is the same for all its calls
+    const uint64_t key = with_marks ? (uint64_t)SP_PART_MTTKRP_MARKS << 56 : ((uint64_t)SP_PART_MTTKRP << 56) | (uint64_t)per;
     auto it = t->parts.find(key);
     if (it != t->parts.end()) { *out = it->second; return SP_OK; }
     const int64_t nnz = t->ncrd[2];
