@@ -370,10 +370,10 @@ template <typename P, typename I, int L, int V, int W, int kU>
 __global__ void __launch_bounds__(kGThreads, L == 8 && V == 3 ? 8 : 1)      // 112 registers there, 96 unasked: 113 us, 133
 k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, const double* __restrict__ val,
                const P* __restrict__ pos1, const I* __restrict__ crd0, const double* __restrict__ F1,
-               const double* __restrict__ F2, int64_t R, double* __restrict__ M, const int64_t* __restrict__ pslice,
+               const double* __restrict__ F2, int64_t R, int64_t cols, double* __restrict__ M, const int64_t* __restrict__ pslice,
                const int64_t* __restrict__ prow, int64_t nnz, int per, int chunks, int64_t nranges, int64_t nslice,
                int64_t d0, int64_t d1, int64_t d2) {
-    // chunks: chunks of the table in a group's range of per entries
+    // cols of the R columns, from where F1, F2 and M point on; chunks: of the table, in a group's range of per entries
     // d0, d1, d2: rows of M, F1, F2 (used by the bounds-checking debug build only)
     constexpr int kGroups = kGThreads / L, kSlots = 2 * kGroups;
     __shared__ double s_sum[kSlots][L * V];         // slot 2 g: the slice group g's range begins in, 2 g + 1: the one it ends in
@@ -388,7 +388,7 @@ k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, c
 #pragma unroll
     for (int j = 0; j < V / W; ++j) {
         const int c = (j * L + gl) * W;
-        on[j] = cb + c < R;
+        on[j] = cb + c < cols;
         coff[j] = on[j] ? c : 0;
     }
     auto slot_put = [&](int slot, const double (&a)[V], int64_t id) {
@@ -558,11 +558,14 @@ static sp_status mttkrp_levels(sp_tensor* T, const double* F1, const double* F2,
         const int64_t ranges = sp_ceil_div(nnz, per);
         const bool pairs = R % 2 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0 &&
                            reinterpret_cast<uintptr_t>(M) % 16 == 0;
+        // a launch covers at most 65,535 tiles of columns
 #define SP_MTTKRP_GROUP(L, V, W, U)                                                                                        \
-    k_mttkrp_group<P, I, L, V, W, U><<<dim3((unsigned)sp_ceil_div(ranges * L, kGThreads), (unsigned)sp_ceil_div(R, L * V)), kGThreads, 0, stream>>>( \
-        part.marks, static_cast<const I*>(T->crd[2]), T->val, static_cast<const P*>(T->pos[1]),                                 \
-        T->lt[0] == SP_COMPRESSED ? static_cast<const I*>(T->crd[0]) : nullptr, F1, F2, R, M, part.aux, part.row, nnz, (int)per, \
-        (int)(per / chunk), ranges, T->npos[1] - 1, T->dims[T->ord[0]], d1, d2)
+    for (int64_t c0 = 0; c0 < R; c0 += (int64_t)65535 * (L * V))                                                           \
+    k_mttkrp_group<P, I, L, V, W, U><<<dim3((unsigned)sp_ceil_div(ranges * L, kGThreads),                                  \
+                                            (unsigned)std::min<int64_t>(65535, sp_ceil_div(R - c0, L * V))), kGThreads, 0, stream>>>( \
+        part.marks, static_cast<const I*>(T->crd[2]), T->val, static_cast<const P*>(T->pos[1]),                            \
+        T->lt[0] == SP_COMPRESSED ? static_cast<const I*>(T->crd[0]) : nullptr, F1 + c0, F2 + c0, R, R - c0, M + c0,       \
+        part.aux, part.row, nnz, (int)per, (int)(per / chunk), ranges, T->npos[1] - 1, T->dims[T->ord[0]], d1, d2)
         SP_DISPATCH_WIDTHS(T, {
             if (pairs) {
                 if (R <= 8) SP_MTTKRP_GROUP(4, 2, 2, 6);
