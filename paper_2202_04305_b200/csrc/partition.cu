@@ -101,7 +101,8 @@ template <typename P, typename I>
 __global__ void __launch_bounds__(kMarkThreads, 6)
 k_mttkrp_marks(const P* __restrict__ pos1, const I* __restrict__ crd0, int64_t nslice, const P* __restrict__ pos2,
                const I* __restrict__ crd1, int64_t nfiber, int64_t nnz, int64_t per, int64_t nchunks, int64_t chunks,
-               int64_t* __restrict__ chunk_slice, int64_t* __restrict__ chunk_row, uint32_t* __restrict__ marks) {
+               int64_t* __restrict__ chunk_slice, int64_t* __restrict__ chunk_row, uint32_t* __restrict__ marks, int64_t d0, int64_t d1) {
+    // d0, d1: sizes of levels 0 and 1 (used by the bounds-checking debug build only)
     constexpr int kPer = 4;
     static_assert(kMarkTile == kPer * kMarkThreads, "a thread owns four entries");
     __shared__ uint4 s_at4[kMarkTile / 4 + 1];
@@ -129,7 +130,7 @@ k_mttkrp_marks(const P* __restrict__ pos1, const I* __restrict__ crd0, int64_t n
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
             const int64_t f = f0 + t + k * kMarkThreads;
-            cr[k] = f < fend ? (uint32_t)crd1[f] : 0u;
+            cr[k] = f < fend ? (uint32_t)SP_IDX(crd1[f], d1) : 0u;
             next[k] = f < fend ? (int64_t)pos2[f + 1] : nnz + 1 + kMarkTile;
         }
     };
@@ -192,7 +193,7 @@ k_mttkrp_marks(const P* __restrict__ pos1, const I* __restrict__ crd0, int64_t n
             if ((int64_t)pos1[mid] <= f) lo = mid; else hi = mid;
         }
         chunk_slice[c] = lo;
-        chunk_row[c] = crd0 ? (int64_t)crd0[lo] : lo;
+        chunk_row[c] = SP_IDX(crd0 ? (int64_t)crd0[lo] : lo, d0);
     }
     for (int64_t q = s0 + t; q <= s1; q += kMarkThreads) {          // the last entry of every slice, once the words are written
         const int64_t f = (int64_t)pos1[q + 1];
@@ -370,9 +371,13 @@ sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t per, bool with_marks, cu
         else if (nnz > 0)
             k_mttkrp_marks<P, I><<<(unsigned)sp_ceil_div(p.nchunks, run), kMarkThreads, 0, stream>>>(
                 pos1, t->lt[0] == SP_COMPRESSED ? static_cast<const I*>(t->crd[0]) : nullptr, nslice, pos2,
-                static_cast<const I*>(t->crd[1]), nfiber, nnz, per, p.nchunks, run, p.aux, p.row, p.marks);
+                static_cast<const I*>(t->crd[1]), nfiber, nnz, per, p.nchunks, run, p.aux, p.row, p.marks,
+                t->dims[t->ord[0]], t->dims[t->ord[1]]);
     });
     if (cudaGetLastError() != cudaSuccess) return drop(SP_ERR_CUDA);
+#ifdef SP_DEBUG_BOUNDS
+    { const sp_status b = sp_bounds_result(stream); if (b != SP_OK) return drop(b); }
+#endif
     sp_count_launches(1);
     if (sp_partition_built(stream) != SP_OK) return drop(SP_ERR_CUDA);
     t->parts[key] = p;
