@@ -258,7 +258,9 @@ enum { SP_PART_MERGE_LAST = 1, SP_PART_MTTKRP = 2, SP_PART_SEGIDS = 3, SP_PART_M
 // For rank-2 (x, compressed) storage: the logical level-0 coordinate of every stored entry
 // (the expanded "outer" index), uint32, cached in the handle.  Needs dims < 2^32.
 sp_status sp_get_segment_ids(sp_tensor* t, cudaStream_t stream, const uint32_t** out);
-sp_status sp_get_merge_partition(sp_tensor* t, int64_t items_per_chunk, cudaStream_t stream, sp_partition* out);
+// max_seg: also the length of the longest last-level segment, with one wait for both.  Where it is not known and the
+// stream is being captured, INT64_MAX: the caller then takes the route for segments of any length.
+sp_status sp_get_merge_partition(sp_tensor* t, int64_t items_per_chunk, cudaStream_t stream, sp_partition* out, int64_t* max_seg = nullptr);
 // Length of the longest last-level segment (row of CSR, stored row of DCSR, ...), measured on the
 // device on first use (one small kernel and one read-back, which waits for the stream) and kept.
 sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out);

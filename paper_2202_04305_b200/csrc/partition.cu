@@ -203,26 +203,36 @@ k_mttkrp_marks(const P* __restrict__ pos1, const I* __restrict__ crd0, int64_t n
 
 }  // namespace
 
-sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out) {
-    std::lock_guard<std::mutex> lock(t->mu);
-    if (t->max_seg >= 0) { *out = t->max_seg; return SP_OK; }
+// Enqueues the measuring of the longest last-level segment into *host (of sp_host_words), unless it is known or there are none.
+static sp_status measure_max_segment(sp_tensor* t, sp_workspace& ws, cudaStream_t stream, unsigned long long** host) {
+    *host = nullptr;
     const int last = t->rank - 1;
     const int64_t nseg = t->npos[last] - 1;
-    if (nseg <= 0 || t->ncrd[last] == 0) { t->max_seg = 0; *out = 0; return SP_OK; }
-    sp_workspace ws(stream);
-    unsigned long long* d = ws.get<unsigned long long>(1);
-    if (ws.failed) return SP_ERR_ALLOC;
+    if (t->max_seg >= 0) return SP_OK;
+    if (nseg <= 0 || t->ncrd[last] == 0) { t->max_seg = 0; return SP_OK; }
+    unsigned long long *d = ws.get<unsigned long long>(1), *h = sp_host_words();
+    if (ws.failed || !h) return SP_ERR_ALLOC;
     SP_CUDA(cudaMemsetAsync(d, 0, sizeof *d, stream));
     const unsigned blocks = (unsigned)std::min<int64_t>(sp_ceil_div(nseg, 256), 148 * 8);
     if (t->posBits == 32) k_max_segment<uint32_t><<<blocks, 256, 0, stream>>>(static_cast<const uint32_t*>(t->pos[last]), nseg, d);
     else k_max_segment<uint64_t><<<blocks, 256, 0, stream>>>(static_cast<const uint64_t*>(t->pos[last]), nseg, d);
     SP_LAUNCH_CHECK();
     sp_count_launches(1);
-    unsigned long long* h = sp_host_words();
-    if (!h) return SP_ERR_ALLOC;
     SP_CUDA(cudaMemcpyAsync(h, d, sizeof *h, cudaMemcpyDeviceToHost, stream));
-    SP_CUDA(cudaStreamSynchronize(stream));
-    t->max_seg = (int64_t)*h;
+    *host = h;
+    return SP_OK;
+}
+
+sp_status sp_get_max_segment(sp_tensor* t, cudaStream_t stream, int64_t* out) {
+    std::lock_guard<std::mutex> lock(t->mu);
+    sp_workspace ws(stream);
+    unsigned long long* h = nullptr;
+    const sp_status st = measure_max_segment(t, ws, stream, &h);
+    if (st != SP_OK) return st;
+    if (h) {
+        SP_CUDA(cudaStreamSynchronize(stream));
+        t->max_seg = (int64_t)*h;
+    }
     *out = t->max_seg;
     return SP_OK;
 }
@@ -253,33 +263,52 @@ sp_status sp_get_segment_ids(sp_tensor* t, cudaStream_t stream, const uint32_t**
     return SP_OK;
 }
 
-sp_status sp_get_merge_partition(sp_tensor* t, int64_t items, cudaStream_t stream, sp_partition* out) {
+sp_status sp_get_merge_partition(sp_tensor* t, int64_t items, cudaStream_t stream, sp_partition* out, int64_t* max_seg) {
     std::lock_guard<std::mutex> lock(t->mu);
     const uint64_t key = ((uint64_t)SP_PART_MERGE_LAST << 56) | (uint64_t)items;
     auto it = t->parts.find(key);
-    if (it != t->parts.end()) { *out = it->second; return SP_OK; }
+    if (it != t->parts.end()) {
+        *out = it->second;
+        if (!max_seg) return SP_OK;
+        *max_seg = t->max_seg;
+        if (t->max_seg >= 0) return SP_OK;
+        // Not known, and not to be measured in a capture: as if rows were long.
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        SP_CUDA(cudaStreamIsCapturing(stream, &capture));
+        if (capture != cudaStreamCaptureStatusNone) { *max_seg = INT64_MAX; return SP_OK; }
+    }
+    sp_workspace ws(stream);
+    unsigned long long* h = nullptr;
+    sp_partition p;
     const int last = t->rank - 1;
     const int64_t nseg = t->npos[last] - 1;
     const int64_t nnz = t->ncrd[last];
-    sp_partition p;
-    p.nchunks = sp_ceil_div(nseg + nnz, items);
-    if (p.nchunks < 1) p.nchunks = 1;
-    p.row = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
-    p.nz = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
+    const bool missing = it == t->parts.end();
     auto drop = [&](sp_status s) { sp_dev_free(p.row, stream); sp_dev_free(p.nz, stream); return s; };
-    if (!p.row || !p.nz) return drop(SP_ERR_ALLOC);
-    const unsigned blocks = (unsigned)sp_ceil_div(p.nchunks + 1, 256);
-    if (t->posBits == 32)
-        k_merge_partition<uint32_t><<<blocks, 256, 0, stream>>>(static_cast<const uint32_t*>(t->pos[last]), nseg, nnz,
-                                                                 items, p.nchunks, p.row, p.nz);
-    else
-        k_merge_partition<uint64_t><<<blocks, 256, 0, stream>>>(static_cast<const uint64_t*>(t->pos[last]), nseg, nnz,
-                                                                 items, p.nchunks, p.row, p.nz);
-    if (cudaGetLastError() != cudaSuccess) return drop(SP_ERR_CUDA);
-    sp_count_launches(1);
+    if (missing) {
+        p.nchunks = sp_ceil_div(nseg + nnz, items);
+        if (p.nchunks < 1) p.nchunks = 1;
+        p.row = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
+        p.nz = static_cast<int64_t*>(sp_dev_alloc((size_t)(p.nchunks + 1) * sizeof(int64_t), stream));
+        if (!p.row || !p.nz) return drop(SP_ERR_ALLOC);
+        const unsigned blocks = (unsigned)sp_ceil_div(p.nchunks + 1, 256);
+        if (t->posBits == 32)
+            k_merge_partition<uint32_t><<<blocks, 256, 0, stream>>>(static_cast<const uint32_t*>(t->pos[last]), nseg, nnz,
+                                                                     items, p.nchunks, p.row, p.nz);
+        else
+            k_merge_partition<uint64_t><<<blocks, 256, 0, stream>>>(static_cast<const uint64_t*>(t->pos[last]), nseg, nnz,
+                                                                     items, p.nchunks, p.row, p.nz);
+        if (cudaGetLastError() != cudaSuccess) return drop(SP_ERR_CUDA);
+        sp_count_launches(1);
+    }
+    if (max_seg) {
+        const sp_status st = measure_max_segment(t, ws, stream, &h);
+        if (st != SP_OK) return drop(st);
+    }
     if (sp_partition_built(stream) != SP_OK) return drop(SP_ERR_CUDA);
-    t->parts[key] = p;
-    *out = p;
+    if (h) t->max_seg = (int64_t)*h;
+    if (max_seg) *max_seg = t->max_seg;
+    if (missing) t->parts[key] = *out = p;
     return SP_OK;
 }
 

@@ -671,11 +671,20 @@ extern "C" sp_status sp_spmm(sp_tensor* A, const double* B, int64_t N, int64_t l
     // entries) of at least 16 entries with N = 16 or 32: B's rows come from HBM, and what counts is how many of
     // them are in flight: 1,048,576 columns, rows of 48, N = 32: 217 us here, 242 us with k_spmm_merge.  Everything
     // else is faster there (N = 64: 228 against 250 us, rows of 5: 251 against 264, B in L2: 88 against 99 and less).
-    if (rowmajor && (N == 16 || N == 32) && A->dims[1] * ldb * 8 > ((int64_t)100 << 20) && A->ncrd[1] >= 16 * nseg && ldb % 2 == 0 &&
-        ldc % 2 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0) {
-        int64_t max_seg = 0;
-        st = sp_get_max_segment(A, stream, &max_seg);
+    const bool by_rows = rowmajor && (N == 16 || N == 32) && A->dims[1] * ldb * 8 > ((int64_t)100 << 20) && A->ncrd[1] >= 16 * nseg &&
+                         ldb % 2 == 0 && ldc % 2 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0;
+    int64_t max_seg = 0;
+    sp_partition part;
+    if (rowmajor) {
+        // Shorter pieces where there would be too few to fill the GPU (about 10,000 groups are resident).
+        // Measured, 32 against 64 items: 175,000 entries, N = 50, 18.5 against 22.5 us; 430,000 entries,
+        // N = 50, 32.5 against 28.7; 1,050,000 entries, N = 64, 59.6 against 56.9 (16: 67.6, 128: 57.1).
+        // Looked up for every N, also where the route below needs none: the handle's first product makes it, and one that is
+        // captured later, with another N, finds it.
+        st = sp_get_merge_partition(A, nseg + A->ncrd[1] < 300000 ? 32 : 64, stream, &part, by_rows ? &max_seg : nullptr);
         if (st != SP_OK) return st;
+    }
+    if (by_rows) {
         const int64_t mean = A->ncrd[1] / nseg;
         if (max_seg <= 4096 && max_seg <= 4 * mean + 32) {
 #define SP_SPMM_ROWS(L, V)                                                                                              \
@@ -699,7 +708,6 @@ extern "C" sp_status sp_spmm(sp_tensor* A, const double* B, int64_t N, int64_t l
         st = clear_C();
         if (st != SP_OK) return st;
     }
-    sp_partition part;
     sp_workspace ws(stream);
     double* carry = nullptr;
     int64_t* crow = nullptr;
@@ -713,11 +721,6 @@ extern "C" sp_status sp_spmm(sp_tensor* A, const double* B, int64_t N, int64_t l
         st = sp_get_segment_ids(A, stream, &segs);
         if (st != SP_OK) return st;
     } else {
-        // Shorter pieces where there would be too few to fill the GPU (about 10,000 groups are resident).
-        // Measured, 32 against 64 items: 175,000 entries, N = 50, 18.5 against 22.5 us; 430,000 entries,
-        // N = 50, 32.5 against 28.7; 1,050,000 entries, N = 64, 59.6 against 56.9 (16: 67.6, 128: 57.1).
-        st = sp_get_merge_partition(A, nseg + A->ncrd[1] < 300000 ? 32 : 64, stream, &part);
-        if (st != SP_OK) return st;
         gblocks = sp_ceil_div(part.nchunks * lanes, kMThreads);
         // the open row of every block's pieces: N partial sums and the row number, scratch of this call alone
         carry = ws.get<double>((size_t)gblocks * N + 1);
