@@ -12,7 +12,6 @@
 namespace {
 
 constexpr int kSThreads = 64;
-constexpr int kSItems = 64;   // merge items per warp
 constexpr int kGThreads = 64;  // of k_sddmm_group (32: the same; 128: 265 us against 262)
 
 __global__ void __launch_bounds__(256)
@@ -333,18 +332,21 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
     if (!x_vals) return SP_ERR_INVALID_ARG;
     const bool dbl = S->lt[0] == SP_COMPRESSED;
 
+    // The pieces of either kernel, so that a handle has one table whatever K is: shorter ones where there are few (30,000 to
+    // 115,000 entries, K <= 512: 10 against 14 us; 240,000 and up: no gain).
+    const int64_t nseg = S->npos[1] - 1;
+    const int64_t items = nseg + nnz < 200000 ? 16 : 32;
     const bool pair_a = K % 2 == 0 && lda % 2 == 0 && reinterpret_cast<uintptr_t>(A) % 16 == 0;
     if (K <= 512) {
         sp_workspace ws(stream);
-        const int64_t nseg = S->npos[1] - 1, ldt = (K + 1) & ~(int64_t)1;
+        const int64_t ldt = (K + 1) & ~(int64_t)1;
         double* Bt = ws.get<double>((size_t)n * ldt + 2);
         if (ws.failed) return SP_ERR_ALLOC;
         Bt = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(Bt) + 15) & ~(uintptr_t)15);
         k_transpose<<<dim3((unsigned)sp_ceil_div(n, 32), (unsigned)sp_ceil_div(ldt, 32)), 256, 0, stream>>>(B, ldb, K, n, Bt, ldt);
         SP_LAUNCH_CHECK();
         sp_partition part;
-        // shorter pieces where there are few (30,000 to 115,000 entries: 10 against 14 us; 240,000 and up: no gain)
-        const sp_status st = sp_get_merge_partition(S, nseg + nnz < 200000 ? 16 : 32, stream, &part);
+        const sp_status st = sp_get_merge_partition(S, items, stream, &part);
         if (st != SP_OK) return st;
         // row in registers / gathered row: A and B^T, or for column-major S the other way round
         const double *reg = colmajor ? Bt : A, *gat = colmajor ? A : Bt;
@@ -404,7 +406,7 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
     SP_LAUNCH_CHECK();
 
     sp_partition part;
-    sp_status st = sp_get_merge_partition(S, kSItems, stream, &part);
+    sp_status st = sp_get_merge_partition(S, items, stream, &part);
     if (st != SP_OK) return st;
     const bool vec2 = (K % 2 == 0) && (lda % 2 == 0) && (reinterpret_cast<uintptr_t>(A) % 16 == 0) &&
                       (reinterpret_cast<uintptr_t>(Bt) % 16 == 0);

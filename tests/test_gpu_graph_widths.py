@@ -45,3 +45,23 @@ def test_spmm(oracle, enc, warm, then):
     torch.cuda.synchronize()
     ref, bound = oracle.spmm(m, coo.coords[0], compact, coo.vals, host)
     assert_close(C.cpu().numpy(), ref, bound, f"{enc} N={then} after N={warm}")
+
+
+@pytest.mark.parametrize("warm,then", [(64, 600), (600, 64), (17, 513)])
+@pytest.mark.parametrize("enc", list(MATRIX_ENCODINGS))
+def test_sddmm(oracle, enc, warm, then):
+    coo = I.uniform_matrix(150, 140, 2500, seed=5)
+    S = sp().sp_pack(coo.dims, *to_dev(coo), *MATRIX_ENCODINGS[enc])
+    x = torch.empty(S.nval, dtype=torch.float64, device="cuda")
+    ops = {K: (I.dense_operand(3, K, 150, K), I.dense_operand(4, K, K, 140)) for K in (warm, then)}
+    d = {K: (dev(a), dev(b)) for K, (a, b) in ops.items()}
+    sp().sp_sddmm(S, *d[warm], x)
+    g = _captured(lambda: sp().sp_sddmm(S, *d[then], x))
+    x.fill_(float("nan"))
+    g.replay()
+    torch.cuda.synchronize()
+    e, b = oracle.sddmm(coo.coords[0], coo.coords[1], coo.vals, *ops[then])
+    at = oracle.pack(coo.dims, coo.coords, coo.vals, *MATRIX_ENCODINGS[enc]).entry_pos
+    ref, bound = np.empty_like(e), np.empty_like(b)
+    ref[at], bound[at] = e, b
+    assert_close(x.cpu().numpy(), ref, bound, f"{enc} K={then} after K={warm}")
