@@ -5,9 +5,9 @@
 // records which columns were touched, and compresses the row back in index order.  Both paths below
 // keep that shape, with the flags as a bitmap whose words, read in order, give the columns sorted.  The
 // product runs in two passes: a symbolic one (row lengths -> positions by a scan -> sizes of C's arrays,
-// read back once) and a numeric one.  Results of up to 32,768 columns whose operand rows are not too
-// sparse take the bitmap path (k_row_bitmaps, k_symbolic, k_numeric).  Otherwise a block owns a row at a
-// time (k_spmspm): warps walk the entries A[i,k], lanes walk row k of B and add into the block's workspace
+// read back once) and a numeric one.  Results of up to 32,768 columns with enough products for their size
+// take the bitmap path (k_row_bitmaps, k_symbolic, k_numeric), but for rows of A much longer than the
+// others.  Otherwise a block owns a row at a time (k_spmspm): warps walk the entries A[i,k], lanes walk row k of B and add into the block's workspace
 // row with atomics, in shared memory when a row of C fits there (dims[1] up to about 25,000), else in
 // one workspace row per block in global memory (L2-resident).
 #include "common.cuh"
@@ -42,13 +42,17 @@ __device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t* su
 
 // NUMERIC = false: rowlen[i] = number of distinct columns of row i.
 // NUMERIC = true : crd / val of C filled at cpos[i].. ; the workspace row is left zeroed.
-template <typename P, typename I, bool NUMERIC, bool SMEM>
+// LONG: only the rows that k_symbolic put in list, *nlong of them.
+template <typename P, typename I, bool NUMERIC, bool SMEM, bool LONG>
 __global__ void __launch_bounds__(kPThreads)
 k_spmspm(const P* __restrict__ apos, const I* __restrict__ acrd, const double* __restrict__ aval,
          const P* __restrict__ bpos, const I* __restrict__ bcrd, const double* __restrict__ bval, int64_t m,
          int64_t n, double* __restrict__ ws_all, uint32_t* __restrict__ bm_all, int64_t* __restrict__ rowlen,
          const void* __restrict__ cpos, int cposBits, void* __restrict__ ccrd, int ccrdBits,
-         double* __restrict__ cval, int64_t kdim) {
+         double* __restrict__ cval, int64_t kdim, const uint32_t* list, const unsigned long long* nlong) {
+    sp_wait_for_previous_kernel();
+    const int64_t rows = LONG ? (int64_t)*nlong : m;
+    if (LONG && blockIdx.x >= rows) return;
     __shared__ uint32_t sums[kPThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t words = (n + 31) >> 5;
@@ -67,7 +71,8 @@ k_spmspm(const P* __restrict__ apos, const I* __restrict__ acrd, const double* _
         bm = bm_all + (int64_t)blockIdx.x * words;
     }
 
-    for (int64_t i = blockIdx.x; i < m; i += gridDim.x) {
+    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+        const int64_t i = LONG ? (int64_t)list[r] : r;
         // expand: every product of row i lands in the workspace
         const int64_t a0 = (int64_t)apos[i], a1 = (int64_t)apos[i + 1];
         for (int64_t p = a0 + w; p < a1; p += kPThreads / 32) {
@@ -191,7 +196,8 @@ constexpr int kBitWarps = 4, kOrWarps = 4, kNumWarps = 4;
 template <typename P, typename I>
 __global__ void __launch_bounds__(kBitWarps * 32)
 k_row_bitmaps(const P* __restrict__ pos, const I* __restrict__ crd, int64_t rows, int64_t n, int stride, int nblk,
-              uint32_t* __restrict__ bits, uint32_t* __restrict__ split) {
+              uint32_t* __restrict__ bits, uint32_t* __restrict__ split, unsigned long long* __restrict__ nlong) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *nlong = 0;        // counted by k_symbolic
     extern __shared__ __align__(16) unsigned char s_dyn[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t* mine = reinterpret_cast<uint32_t*>(s_dyn) + (size_t)w * stride;
@@ -216,16 +222,22 @@ k_row_bitmaps(const P* __restrict__ pos, const I* __restrict__ crd, int64_t rows
         *reinterpret_cast<uint4*>(bits + k * stride + x) = *reinterpret_cast<const uint4*>(mine + x);
 }
 
-// One warp per row of C: the OR of the bitmaps of the rows of B that row i of A names, and its bit count.
+// One warp per row of C: the OR of the bitmaps of the rows of B that row i of A names, and its bit count.  Rows of A
+// of more than `longest` entries are left to k_spmspm, a block each: one full row of 32,768 entries kept its warp busy
+// for 40 ms.
 template <typename P, typename I>
 __global__ void __launch_bounds__(kOrWarps * 32)
 k_symbolic(const P* __restrict__ apos, const I* __restrict__ acrd, const uint32_t* bits, int64_t m, int64_t kdim, int stride,
-           uint32_t* __restrict__ cbits, int64_t* __restrict__ rowlen) {
+           int64_t longest, uint32_t* __restrict__ cbits, int64_t* __restrict__ rowlen, uint32_t* __restrict__ list, unsigned long long* nlong) {
     sp_wait_for_previous_kernel();
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * kOrWarps + (threadIdx.x >> 5);
     if (i >= m) return;
     const int64_t a0 = (int64_t)apos[i], a1 = (int64_t)apos[i + 1];
+    if (a1 - a0 > longest) {
+        if (lane == 0) list[atomicAdd(nlong, 1ull)] = (uint32_t)i;
+        return;
+    }
     constexpr int kQ = 2, kE = 4;                   // 16-byte runs per lane and entry, entries in flight
     uint32_t total = 0;
     for (int x0 = 0; x0 < stride; x0 += 128 * kQ) {
@@ -270,7 +282,7 @@ template <typename P, typename I, bool C32>
 __global__ void __launch_bounds__(kNumWarps * 32)
 k_numeric(const P* __restrict__ apos, const I* __restrict__ acrd, const double* __restrict__ aval,
           const uint32_t* __restrict__ split, const I* __restrict__ bcrd, const double* __restrict__ bval, int64_t m,
-          int nblk, int stride, const uint32_t* __restrict__ cbits, const void* __restrict__ cpos, int cposBits,
+          int nblk, int stride, int64_t longest, const uint32_t* __restrict__ cbits, const void* __restrict__ cpos, int cposBits,
           void* __restrict__ ccrd, int ccrdBits, double* __restrict__ cval, int64_t kdim, int64_t n) {
     // per warp: its columns' sums; the segments of the next 32 entries of A and their factors, read back as
     // broadcasts (a shuffle per word costs the same pipe as a shared-memory access of all of them)
@@ -288,6 +300,7 @@ k_numeric(const P* __restrict__ apos, const I* __restrict__ acrd, const double* 
         const int64_t i = item / nblk;
         const int cb = (int)(item - i * nblk);
         const int64_t a0 = (int64_t)apos[i], a1 = (int64_t)apos[i + 1];
+        if (a1 - a0 > longest) continue;
         const uint32_t* row = cbits + i * stride;
         const int wb = cb * (kColBlk / 32);
         double* accl = acc - cb * kColBlk;              // indexed by column
@@ -421,13 +434,23 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     SP_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t shm_sym = (size_t)((words * 4 + 7) & ~(int64_t)7);
     const size_t shm_num = shm_sym + (size_t)n * sizeof(double);
-    // The bitmap path reads a bitmap row per entry of A where the other one walks a row of B: rows of B
-    // of at least a sixteenth of a bitmap row's words, and bitmaps of at most 256 MB.
+    // The bitmap path reads a bitmap row per entry of A where the other one walks a row of B, and costs something for
+    // every row and block of columns.  It is taken for rows of B of 26 (2048 columns) to 38 entries (8192 and more) on average
+    // (uniform operands, 2048 columns, rows of 20, 30: 61.8, 65.3 us, by blocks 62.2, 71.9; 4096, rows of 24, 40: 93.6, 111,
+    // by blocks 86.6, 145; 8192, rows of 24, 32, 48: 230, 270, 334, by blocks 154, 223, 395; 16,384, rows of 34, 50: 968, 1209,
+    // by blocks 942, 1490) that are also at least a sixteenth of a bitmap row's words, 100 products or more per row and
+    // block of columns (8192 columns, 4 x 40 entries a row, 20 products: 149 us, by blocks 100; 30 x 40, 150 products: 324
+    // and 317), rows of A that leave work for all warps (100 rows of 2000: 1158 us, by blocks 710) and bitmaps of at
+    // most 256 MB.
     const int stride = (int)((words + 3) & ~(int64_t)3);          // words of a bitmap row
     const int64_t kdim = B->dims[0];
-    const bool bitmaps = n <= kMaxCols && m > 0 && kdim > 0 && B->nval < ((int64_t)1 << 32) &&
-                         (m + kdim) * stride * 4 <= ((int64_t)256 << 20) && stride * kdim <= 16 * (B->nval + kdim);
     const int nblk = (int)sp_ceil_div(n, kColBlk);
+    const double products = (double)A->nval * (double)B->nval / (double)std::max<int64_t>(kdim, 1);
+    const bool bitmaps = n <= kMaxCols && m > 0 && m < ((int64_t)1 << 32) && kdim > 0 && B->nval < ((int64_t)1 << 32) &&
+                         (m + kdim) * stride * 4 <= ((int64_t)256 << 20) && stride * kdim <= 16 * (B->nval + kdim) &&
+                         B->nval >= (22 + std::min(stride, 256) / 16) * kdim && products >= 100.0 * (double)m * nblk && A->nval <= m * std::max<int64_t>(m / 8, 128);
+    // rows of A longer than this are not one warp's
+    const int64_t longest = bitmaps ? std::max<int64_t>(512, 4 * (A->nval / m)) : 0;
     const bool in_smem = shm_num + 2048 <= (size_t)smem_max;
     auto blocks_for = [&](size_t shm) {
         int64_t per_sm = (int64_t)((size_t)smem_max / (shm + 1024));
@@ -442,17 +465,19 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     sp_workspace ws(stream);
     double* wsrow = nullptr;
     uint32_t* bm = nullptr;
-    uint32_t *bbits = nullptr, *cbits = nullptr, *split = nullptr;
+    uint32_t *bbits = nullptr, *cbits = nullptr, *split = nullptr, *list = nullptr;
     if (bitmaps) {
         bbits = ws.get<uint32_t>((size_t)kdim * stride);
         cbits = ws.get<uint32_t>((size_t)m * stride);
         split = ws.get<uint32_t>((size_t)kdim * (nblk + 1));
+        list = ws.get<uint32_t>((size_t)(A->nval / (longest + 1)) + 1);
     } else if (!in_smem) {
         wsrow = ws.get<double>((size_t)nblocks * n);
         bm = ws.get<uint32_t>((size_t)nblocks * words);
     }
     int64_t* rowlen = ws.get<int64_t>((size_t)m + 1);
-    int64_t* d_count = ws.get<int64_t>(1);
+    int64_t* d_count = ws.get<int64_t>(2);                        // entries of C; long rows of A
+    unsigned long long* nlong = reinterpret_cast<unsigned long long*>(d_count + 1);
     if (ws.failed) return SP_ERR_ALLOC;
     if (!bitmaps && !in_smem) {
         SP_CUDA(cudaMemsetAsync(wsrow, 0, (size_t)nblocks * n * sizeof(double), stream));
@@ -474,30 +499,33 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
 #define SP_SPMSPM_ARGS                                                                                            \
     static_cast<const P*>(A->pos[1]), static_cast<const I*>(A->crd[1]), A->val, static_cast<const P*>(B->pos[1]), \
         static_cast<const I*>(B->crd[1]), B->val, m, n, wsrow, bm, rowlen, C->pos[1], posBits, C->crd[1], crdBits, C->val, \
-        B->dims[0]
+        B->dims[0], list, nlong
 #define SP_SPMSPM_LAUNCH(NUM)                                                                                     \
     SP_DISPATCH_WIDTHS(A, {                                                                                       \
         if (in_smem) {                                                                                            \
             const size_t shm = NUM ? shm_num : shm_sym;                                                           \
-            if (cudaFuncSetAttribute(k_spmspm<P, I, NUM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
+            if (cudaFuncSetAttribute(k_spmspm<P, I, NUM, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                                      (int)shm) != cudaSuccess)                                                    \
                 return fail(SP_ERR_CUDA);                                                                         \
-            k_spmspm<P, I, NUM, true><<<(unsigned)blocks_for(shm), kPThreads, shm, stream>>>(SP_SPMSPM_ARGS);     \
+            k_spmspm<P, I, NUM, true, false><<<(unsigned)blocks_for(shm), kPThreads, shm, stream>>>(SP_SPMSPM_ARGS);     \
         } else {                                                                                                  \
-            k_spmspm<P, I, NUM, false><<<(unsigned)nblocks, kPThreads, 0, stream>>>(SP_SPMSPM_ARGS);              \
+            k_spmspm<P, I, NUM, false, false><<<(unsigned)nblocks, kPThreads, 0, stream>>>(SP_SPMSPM_ARGS);              \
         }                                                                                                         \
     })
     if (bitmaps) {
         SP_DISPATCH_WIDTHS(A, {
             const size_t shm = (size_t)kBitWarps * stride * sizeof(uint32_t);
             k_row_bitmaps<P, I><<<(unsigned)sp_ceil_div(kdim, kBitWarps), kBitWarps * 32, shm, stream>>>(
-                static_cast<const P*>(B->pos[1]), static_cast<const I*>(B->crd[1]), kdim, n, stride, nblk, bbits, split);
+                static_cast<const P*>(B->pos[1]), static_cast<const I*>(B->crd[1]), kdim, n, stride, nblk, bbits, split, nlong);
             if (sp_launch_dependent(k_symbolic<P, I>, dim3((unsigned)sp_ceil_div(m, kOrWarps)), dim3(kOrWarps * 32), 0, stream,
                                     static_cast<const P*>(A->pos[1]), static_cast<const I*>(A->crd[1]), (const uint32_t*)bbits, m,
-                                    kdim, stride, cbits, rowlen) != cudaSuccess)
+                                    kdim, stride, longest, cbits, rowlen, list, nlong) != cudaSuccess)
+                return fail(SP_ERR_CUDA);
+            if (A->nval > longest &&
+                sp_launch_dependent(k_spmspm<P, I, false, true, true>, dim3((unsigned)(2 * sms)), dim3(kPThreads), shm_sym, stream, SP_SPMSPM_ARGS) != cudaSuccess)
                 return fail(SP_ERR_CUDA);
         });
-        sp_count_launches(1);
+        sp_count_launches(A->nval > longest ? 2 : 1);
     } else if (m > 0) {
         SP_SPMSPM_LAUNCH(false);
     }
@@ -507,10 +535,11 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
     sp_count_launches(2);
     unsigned long long* h_count = sp_host_words();
     if (!h_count) return fail(SP_ERR_ALLOC);
-    if (cudaMemcpyAsync(h_count, d_count, sizeof *h_count, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+    if (cudaMemcpyAsync(h_count, d_count, 2 * sizeof *h_count, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)
         return fail(SP_ERR_CUDA);
-    const int64_t count = (int64_t)*h_count;
+    const int64_t count = (int64_t)h_count[0];
+    const int64_t long_rows = bitmaps && A->nval > longest ? (int64_t)h_count[1] : 0;
     if ((uint64_t)count > sp_width_max(posBits)) return fail(SP_ERR_WIDTH_OVERFLOW);
     C->ncrd[1] = count;
     C->nval = count;
@@ -527,12 +556,34 @@ extern "C" sp_status sp_spmspm(const sp_tensor* A, const sp_tensor* B, int posBi
         if (sp_allow_shared<k_numeric<P, I, C32>>(dev, shm) != cudaSuccess) return fail(SP_ERR_CUDA);                         \
         k_numeric<P, I, C32><<<blocks, kNumWarps * 32, shm, stream>>>(                                                        \
             static_cast<const P*>(A->pos[1]), static_cast<const I*>(A->crd[1]), A->val, split, static_cast<const I*>(B->crd[1]), B->val, m, \
-            nblk, stride, cbits, C->pos[1], posBits, C->crd[1], crdBits, C->val, kdim, n);                                    \
+            nblk, stride, longest, cbits, C->pos[1], posBits, C->crd[1], crdBits, C->val, kdim, n);                                    \
     } while (0)
             SP_DISPATCH_WIDTHS(A, {
                 if (crdBits == 32) SP_NUMERIC(true); else SP_NUMERIC(false);
             });
 #undef SP_NUMERIC
+            if (long_rows > 0) {
+                if (cudaGetLastError() != cudaSuccess) return fail(SP_ERR_CUDA);
+                const unsigned lblocks = (unsigned)std::min<int64_t>(long_rows, in_smem ? blocks_for(shm_num) : (int64_t)sms);
+                if (!in_smem) {
+                    wsrow = ws.get<double>((size_t)lblocks * n);
+                    bm = ws.get<uint32_t>((size_t)lblocks * words);
+                    if (ws.failed) return fail(SP_ERR_ALLOC);
+                    if (cudaMemsetAsync(wsrow, 0, (size_t)lblocks * n * sizeof(double), stream) != cudaSuccess ||
+                        cudaMemsetAsync(bm, 0, (size_t)lblocks * words * sizeof(uint32_t), stream) != cudaSuccess)
+                        return fail(SP_ERR_CUDA);
+                }
+                SP_DISPATCH_WIDTHS(A, {
+                    if (in_smem) {
+                        if (cudaFuncSetAttribute(k_spmspm<P, I, true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm_num) != cudaSuccess)
+                            return fail(SP_ERR_CUDA);
+                        k_spmspm<P, I, true, true, true><<<lblocks, kPThreads, shm_num, stream>>>(SP_SPMSPM_ARGS);
+                    } else {
+                        k_spmspm<P, I, true, false, true><<<lblocks, kPThreads, 0, stream>>>(SP_SPMSPM_ARGS);
+                    }
+                });
+                sp_count_launches(1);
+            }
         } else {
             SP_SPMSPM_LAUNCH(true);
         }
