@@ -50,13 +50,18 @@ LIB_TORCH = os.path.join(HERE, "libsp_torch.so")
 
 
 def build_torch(force: bool = False) -> str:
-    """The binding's torch side (allocator hooks, tensor views); host code only."""
-    src = os.path.join(CSRC, "torch_memory.cpp")
-    if not force and os.path.exists(LIB_TORCH) and os.path.getmtime(LIB_TORCH) >= os.path.getmtime(src):
-        return LIB_TORCH
+    """The binding's torch side (allocator hooks, tensor views); host code only.  Built against one torch: another version,
+    installation or C++ ABI of it gets a library of its own."""
     import sysconfig
 
     import torch
+    src = os.path.join(CSRC, "torch_memory.cpp")
+    stamp = os.path.join(OBJ, "torch_built_for")
+    built_for = f"{torch.__version__} {os.path.dirname(torch.__file__)} {int(torch._C._GLIBCXX_USE_CXX11_ABI)} {sys.version_info[:2]}"
+    if not force and os.path.exists(LIB_TORCH) and os.path.getmtime(LIB_TORCH) >= os.path.getmtime(src) and os.path.exists(stamp):
+        with open(stamp) as f:
+            if f.read() == built_for:
+                return LIB_TORCH
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.sep in _nvcc() else "/usr/local/cuda"
     cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", LIB_TORCH]
@@ -65,6 +70,9 @@ def build_torch(force: bool = False) -> str:
         cmd += ["-isystem", inc]
     cmd += ["-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
     subprocess.check_call(cmd)
+    os.makedirs(OBJ, exist_ok=True)
+    with open(stamp, "w") as f:
+        f.write(built_for)
     return LIB_TORCH
 
 
