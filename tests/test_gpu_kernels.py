@@ -309,7 +309,7 @@ def test_every_kernel_with_wide_positions_and_coordinates(oracle, pb, cb, cbits)
     for lt, od in TENSOR_ENCODINGS.values():
         T = sp().sp_pack(t.dims, tc, tv, lt, od, pb, cb)
         assert_close(sp().sp_mttkrp(T, dev(Bf), dev(Cf)).cpu().numpy(), Mref, Mb, f"mttkrp widths {pb}/{cb}")
-        for R in (5,):      # the generic (odd R) kernel as well
+        for R in (5,):      # one column at a time and idle lanes as well
             B5, C5 = I.dense_operand(3, 12, 96, R), I.dense_operand(3, 13, 96, R)
             r5, b5 = oracle.mttkrp(96, *t.coords, t.vals, B5, C5)
             assert_close(sp().sp_mttkrp(T, dev(B5), dev(C5)).cpu().numpy(), r5, b5, f"mttkrp R=5 widths {pb}/{cb}")
