@@ -107,8 +107,8 @@ k_sddmm(const P* __restrict__ pos, const I* __restrict__ crd, const double* __re
 // carries, and the groups of a warp share the loop's instructions.
 // 2,000,000 samples, K = 128, operands of 134 MB: 262 us with the transpose, 304 us when a warp took one dot
 // product at a time; L = 8, 16, 32: 290, 262, 270 (fewer lanes, fewer copies of the loop in flight; more,
-// more instructions).  Bound: HBM, since the gathered operand does not fit L2 (1.1 GB for 0.3 GB of
-// operands; 64 % of the HBM rate).  Operand rows kept in registers and loaded ahead cost 190 and more
+// more instructions).  Bound: HBM, since the gathered operand does not fit L2 (1.22 GB for 0.3 GB of
+// operands, 73 % of the pin rate, which is what a copy reaches).  Operand rows kept in registers and loaded ahead cost 190 and more
 // registers (342 us); requested through the ring as well, twice the shared memory (273 us).
 constexpr int kDepth = 4;
 
@@ -368,11 +368,16 @@ extern "C" sp_status sp_sddmm(sp_tensor* S, const double* A, int64_t lda, const 
             const P* pos = static_cast<const P*>(S->pos[1]);
             const I* crd = static_cast<const I*>(S->crd[1]);
             const I* outer = dbl ? static_cast<const I*>(S->crd[0]) : nullptr;
+            // K that fills a shape's lanes needs no masks: K = 16, 256, 512 with them 66.0, 414, 546 us, without 59.2, 388,
+            // 532 (2 M, 1 M, 0.5 M samples of a 131,072-square matrix)
             if (pairs) {
-                if (K == 128) SP_SG_LAUNCH(16, 8, 2, true);
+                if (K == 512) SP_SG_LAUNCH(32, 16, 2, true);
+                else if (K == 256) SP_SG_LAUNCH(16, 16, 2, true);
+                else if (K == 128) SP_SG_LAUNCH(16, 8, 2, true);
                 else if (K == 96) SP_SG_LAUNCH(16, 6, 2, true);
                 else if (K == 64) SP_SG_LAUNCH(16, 4, 2, true);
                 else if (K == 32) SP_SG_LAUNCH(8, 4, 2, true);
+                else if (K == 16) SP_SG_LAUNCH(4, 4, 2, true);
                 else if (K <= 16) SP_SG_LAUNCH(4, 4, 2, false);
                 else if (K < 32) SP_SG_LAUNCH(8, 4, 2, false);
                 else if (K < 64) SP_SG_LAUNCH(16, 4, 2, false);
