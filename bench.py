@@ -40,7 +40,7 @@ PACK_PHASES = ("keys", "sort_hist", "sort_scan", "sort_scatter", "count", "emit"
 
 
 def build_probes(force: bool = False) -> str:
-    """Compile bench_probes.cu, plus the product's packer a second time with its phases timed
+    """Compile bench_probes.cu, plus the packer's radix path a second time with its phases timed
     (csrc/pack.cu, -DSP_BENCH_BUILD), into libbench_probes.so next to this file.  It links against
     the product library for the allocator plumbing; nothing in the product links against it."""
     from paper_2202_04305_b200 import build as libbuild
@@ -750,14 +750,14 @@ def main():
     for k, v in first_call.items():
         kernels[k]["ms_first_call_on_a_handle"] = v
 
-    # ---- dominant kernel: the sort's scatter pass inside sp_pack, timed with CUDA events between the
-    #      packer's phases (the bench library's copy of the packer; same kernels, same stream)
+    # ---- dominant kernel: the sort's scatter pass inside sp_pack of the tensor, timed with CUDA events between the
+    #      phases of the radix path (the bench library's copy of it; same kernels, same stream).  Matrices are not
+    #      packed that way: their packs are in `kernels` as whole calls.
     prof = {}
     perm5 = torch.randperm(wl["c5"].nnz, device="cuda", generator=torch.Generator(device="cuda").manual_seed(7))
     c5_rand, v5_rand = [c[perm5].contiguous() for c in suite.c5], suite.v5[perm5].contiguous()
     del perm5
-    for nm, dims, coords, vals, lt, od in [("pack_csc", wl["c3"].dims, suite.c3, suite.v3, (0, 1), (1, 0)),
-                                           ("pack_csf", wl["c5"].dims, suite.c5, suite.v5, (1, 1, 1), None),
+    for nm, dims, coords, vals, lt, od in [("pack_csf", wl["c5"].dims, suite.c5, suite.v5, (1, 1, 1), None),
                                            ("pack_csf_random_input_order", wl["c5"].dims, c5_rand, v5_rand, (1, 1, 1), None)]:
         acc = []
         for _ in range(5):
@@ -769,13 +769,13 @@ def main():
         prof[nm] = {"phases_ms": {k: round(v, 4) for k, v in ph.items()}, "sort_passes": acc[0][1],
                     "total_ms": round(sum(ph.values()), 4)}
     del c5_rand, v5_rand
-    prof["input_order"] = ("pack_csc / pack_csf: the generator's affine index permutation of the sorted list (the order "
+    prof["input_order"] = ("pack_csf: the generator's affine index permutation of the sorted list (the order "
                            "every other number of this report uses); pack_csf_random_input_order: the same entries in a "
                            "seeded uniformly random order")
     n5 = wl["c5"].nnz
     sc_ms = prof["pack_csf"]["phases_ms"]["sort_scatter"] / max(1, prof["pack_csf"]["sort_passes"])
     step_share = {k: v["ms"] for k, v in kernels.items() if not k.startswith("next_") and k != "spmv_csr_powerlaw"}
-    scatter_step_ms = (prof["pack_csf"]["phases_ms"]["sort_scatter"] + 2 * prof["pack_csc"]["phases_ms"]["sort_scatter"])
+    scatter_step_ms = prof["pack_csf"]["phases_ms"]["sort_scatter"]
     dominant = max(step_share, key=step_share.get)
     if scatter_step_ms >= step_share[dominant] * 0.5 or dominant.startswith("pack"):
         per_entry = SORT_PASS_BYTES_PER_ENTRY

@@ -7,8 +7,9 @@
  *     MTTKRP fetch one dense row per stored entry): the rate at which all SMs together fetch
  *     rows of a table at caller-supplied row numbers, the same for single 8-byte elements (the
  *     access SpMV makes to x), and the register-only f64 multiply-add rate;
- *   - spb_pack_timed: the product's packer (the same source file, compiled a second time) with
- *     CUDA events between its phases, which is how bench.py times one radix scatter pass.
+ *   - spb_pack_timed: the radix path of the product's packer (the same source file, compiled a second
+ *     time) with CUDA events between its phases, which is how bench.py times one radix scatter pass.
+ *     sp_pack takes that path for tensors, and for matrices only where their own packer declines.
  * Every call enqueues on `stream` (a cudaStream_t as void*) and returns an sp_status value
  * (0 = ok); all data pointers are DEVICE pointers unless marked host.
  */

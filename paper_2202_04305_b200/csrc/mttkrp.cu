@@ -198,8 +198,8 @@ __device__ __forceinline__ void ld_cols(const char* base, uint32_t off, const ui
 // 20 M entries, R = 32: 479 us with ranges of 128 entries and two entries of each group in flight (one: 481, four: 514
 // to 525; ranges of 64 and 256: 585, 496); 521 us when a warp walked one range in batches of 32, cut at slice ends and
 // closed at every group's last entry.  5 M entries, R = 16, 24, 32: 141, 146, 145 us against 162, 167, 159.  Bound:
-// instruction issue (292 M, 54 % of the slots: eight selects and eight masks per step around eight multiply-adds)
-// and the latency of the row loads at 20 warps per SM together.
+// the L1 pipe (64 %), instruction issue (264 M, 52 % of the slots: eight selects and eight masks per step around eight
+// multiply-adds) and the latency of the row loads at 19 warps per SM together.
 constexpr int kFPer = 128;      // entries per group
 constexpr int kFThreads = 64;
 template <typename P, typename I, int S, bool W256>
@@ -366,8 +366,11 @@ __device__ __forceinline__ void ld_run(const double* p, double* a) {
 }
 
 constexpr int kGThreads = 64;     // 300,000 to 1 M entries: 128 threads 10 % slower, 256 60 %
+// Asked for eight blocks per SM, the compiler spends 116 registers on three single columns a lane, as on the other
+// shapes by itself (116 to 150); unasked it stops at 96 there and the loads wait for one another (3 M entries, R = 17:
+// 113 us, unasked 133).
 template <typename P, typename I, int L, int V, int W, int kU>
-__global__ void __launch_bounds__(kGThreads, L == 8 && V == 3 ? 8 : 1)      // 112 registers there, 96 unasked: 113 us, 133
+__global__ void __launch_bounds__(kGThreads, L == 8 && V == 3 ? 8 : 1)
 k_mttkrp_group(const uint32_t* __restrict__ marks, const I* __restrict__ crd2, const double* __restrict__ val,
                const P* __restrict__ pos1, const I* __restrict__ crd0, const double* __restrict__ F1,
                const double* __restrict__ F2, int64_t R, int64_t cols, double* __restrict__ M, const int64_t* __restrict__ pslice,

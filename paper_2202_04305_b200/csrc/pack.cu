@@ -1291,7 +1291,7 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
 }  // namespace
 
 #ifdef SP_BENCH_BUILD
-// The benchmark's library: the same packer with its phases bracketed by events.
+// The benchmark's library: the radix path with its phases bracketed by events.
 // phase_ms: host, 6 entries (key build, sort histograms, sort scans, sort scatters, node counting,
 // emit + fill); npasses: host, number of radix passes.
 extern "C" sp_status spb_pack_timed(int rank, const int64_t* dims, int64_t nnz, const void* const* coo_coords,

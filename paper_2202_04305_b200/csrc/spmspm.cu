@@ -186,7 +186,7 @@ k_row_offsets(const int64_t* rowlen, int64_t m, void* __restrict__ pos, int posB
 // lanes of an instruction never meet, and no atomic is needed.
 // 8192 x 8192 at density 0.01 (55 M products, 37.5 M results): 463 us for the call, 580 us with one block per row,
 // atomics on a shared-memory row and the bitmap built twice (symbolic 112 -> 48 us with the bitmaps, offsets
-// 26 -> 10, numeric 434 -> 400).  Bound: the shared-memory pipe, 72 % busy: two accesses of 8 bytes per product.
+// 26 -> 10, numeric 434 -> 400).  Bound: the shared-memory pipe, 76 % busy: two accesses of 8 bytes per product.
 constexpr int64_t kMaxCols = 32768;
 constexpr int kColBlk = 1024;                   // columns of a warp of k_numeric (2048, half the warps: 494 us against 463 below)
 constexpr int kBitWarps = 4, kOrWarps = 4, kNumWarps = 4;

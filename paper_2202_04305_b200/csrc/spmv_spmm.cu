@@ -266,8 +266,8 @@ __device__ __forceinline__ void st_vec(double* p, const double* a) {
 // three 53, four 57; with V = 4: four 119 us, six 113, eight 126 on 3.6 M entries and N = 20 - registers).  Pieces being equal, the groups of a warp stay
 // together whatever the row lengths.  A row is stored when its end comes up (rows without entries that
 // end at the same place as zeros); the open last row of a piece is folded into the row's end inside
-// the block, and the one that the block leaves open goes to k_spmm_fixup.  Bound: row-fetch latency and issue (42 %), not
-// traffic (L2 45 %).  The power-law product took 77 us when a warp walked a piece with a lane per column; now 53.
+// the block, and the one that the block leaves open goes to k_spmm_fixup.  Bound: row-fetch latency at 15 warps per SM
+// (issue 35 %, L2 48 %, L1 61 %).  The power-law product took 77 us when a warp walked a piece with a lane per column; now 53.
 template <typename P, typename I, int L, int V, int W, int kU>
 __global__ void __launch_bounds__(kMThreads)
 k_spmm_merge(const P* __restrict__ pos, const I* __restrict__ crd, const double* __restrict__ val,

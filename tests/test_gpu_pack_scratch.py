@@ -22,7 +22,7 @@ class Meter:
 
         def free(ptr, stream, ctx):
             if ptr:
-                self.held -= self.live.pop(ptr)
+                self.held -= self.live.pop(ptr, 0)         # 0: of a handle from before
                 torch.cuda.caching_allocator_delete(ptr)
 
         self._a, self._f = self.b._ALLOC_T(alloc), self.b._FREE_T(free)
