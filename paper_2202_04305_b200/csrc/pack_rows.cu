@@ -1,8 +1,8 @@
 // sp_pack for matrices with a compressed inner level and moderate segments (rows of CSR and DCSR, columns of
 // CSC and DCSC): no sort by key, the entries pass through memory twice.
 //
-//   1. k_rows_count      (where slots of kCap records would not follow the entries, and from kCountFrom entries on)
-//                        entries per bucket, a bucket being a range of outer indices, and where every bucket begins
+//   1. k_rows_count      (where slots of kCap records would not follow the entries) entries per bucket, a bucket being
+//                        a range of outer indices, and where every bucket begins
 //   2. k_rows_partition  (k_rows_partition_tiles from kSmall entries on) range check; entries to their buckets, in any order
 //   3. k_rows_build      a block per bucket: entries per outer index, order inside every segment, and
 //                        everything the bucket contributes to the storage, written in order
@@ -18,21 +18,19 @@
 // and 416; 10,486 entries 62 and 99.  A bucket that overflows (long or very uneven segments) is found on the device
 // too; the kernels after that return and the caller takes the radix path.
 //
-// Without step 1 a bucket has a slot of kCap records, 2.5 times what it holds on average and 16 times in small inputs;
-// with it the scratch is 16 bytes an entry, less than the radix path's, however many rows there are (1,000 entries in
-// 8 M rows: 0.1 MB, 336 MB in slots; 5 M entries: 80 MB, 200 in slots).  It costs 3 us of 40 and more (300,000 entries
-// 43.5 us against 40.0, 1 M 67 against 64) and next to nothing of a large pack, where buckets side by side spare every
-// block the sum over the ones before (5 M entries 194 to 198 us against 195).  An overflow is then known before the
-// entries move: 3.2 M entries with a row of 6,000 284 us against 295, 5 M with a row of 20,000 368 against 373, with a
-// row of 1 M, whose counters collide, 382 against 376 (by radix alone 252, 343, 348).
+// Without step 1 a bucket has a slot of kCap records, 2.5 times what it holds on average and 16 times in small inputs; it
+// runs where slots would take more than 16 records an entry, the rows being many more than the entries, and makes
+// the scratch 16 bytes an entry then (1,000 entries in 8 M rows: 0.1 MB, 336 MB in slots).  For all inputs it would cost 3 us
+// of 40 and more (300,000 entries 43.5 us against 40.0, 1 M 67 against 64, 5 M 198 against 192).
 #include "common.cuh"
+
+#include <stddef.h>
 
 #include <algorithm>
 
 namespace {
 
 constexpr int kCThreads = 1024, kCBlocks = 148; // of k_rows_count
-constexpr int64_t kCountFrom = 2000000;         // entries from which on it runs
 constexpr int kThreads = 512;                   // of k_rows_partition
 constexpr int kBThreads = 512;                  // of k_rows_build and k_rows_outer
 constexpr int kWarps = kBThreads / 32;
@@ -249,10 +247,9 @@ k_rows_partition(const CT* __restrict__ oc, const CT* __restrict__ ic, const dou
 constexpr int kTIpt = 6, kTTile = kThreads * kTIpt;
 struct TileShared {
     Rec rec[kTTile];
-    uint32_t count[kMaxBuckets];                // entries of the tile, then where they begin in rec
-    uint32_t shift[kMaxBuckets];                // place among the records minus place in rec
     uint32_t to[kTTile];                        // where an entry goes among the records
-    uint32_t w[kThreads / 32];
+    uint32_t counters[2 * kMaxBuckets];         // of as many buckets as there are: shared memory not taken is L1 for the loads
+    static constexpr size_t bytes(int nb) { return offsetof(TileShared, counters) + 2 * (size_t)nb * sizeof(uint32_t); }
 };
 
 template <typename CT>
@@ -261,8 +258,11 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
                        uint32_t scale, int inner_bits, int nb, uint32_t slot, uint32_t* cursor, Rec* __restrict__ rec, uint32_t* stop, unsigned long long* host) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     TileShared& s = *reinterpret_cast<TileShared*>(s_raw);
+    uint32_t* const s_count = s.counters;           // entries of the tile per bucket, then where they begin in rec
+    uint32_t* const s_shift = s.counters + nb;      // place of the bucket's entries of this tile among the records minus place in rec
+    __shared__ uint32_t s_w[kThreads / 32];
     const int t = threadIdx.x;
-    for (int b = t; b < nb; b += kThreads) s.count[b] = 0u;
+    for (int b = t; b < nb; b += kThreads) s_count[b] = 0u;
     const int64_t base = (int64_t)blockIdx.x * kTTile;
     const int cnt = (int)(n - base < kTTile ? n - base : kTTile);
     uint32_t o[kTIpt], c[kTIpt], r[kTIpt];
@@ -283,7 +283,7 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
         bad |= out;
         o[i] = out ? 0u : (uint32_t)oo[i];
         c[i] = (uint32_t)cc[i];
-        r[i] = i * kThreads + t < cnt ? atomicAdd(&s.count[__umulhi(o[i], scale)], 1u) : 0u;
+        r[i] = i * kThreads + t < cnt ? atomicAdd(&s_count[__umulhi(o[i], scale)], 1u) : 0u;
     }
     bad = __syncthreads_or(bad) != 0;
     sp_wait_for_previous_kernel();
@@ -298,7 +298,7 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
 #pragma unroll
     for (int q = 0; q < kPerB; ++q) {
         const int b = t + q * kThreads;
-        const uint32_t k = b < nb ? s.count[b] : 0u;
+        const uint32_t k = b < nb ? s_count[b] : 0u;
         at[q] = k ? atomicAdd(cursor + b, k) : 0u;
         mine += k;
     }
@@ -309,20 +309,20 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
         const uint32_t u = __shfl_up_sync(0xffffffffu, incl, d);
         if (lane >= d) incl += u;
     }
-    if (lane == 31) s.w[w] = incl;
+    if (lane == 31) s_w[w] = incl;
     __syncthreads();
     uint32_t from = incl - mine;
 #pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) from += i < w ? s.w[i] : 0u;
+    for (int i = 0; i < kThreads / 32; ++i) from += i < w ? s_w[i] : 0u;
     bool full = false;
 #pragma unroll
     for (int q = 0; q < kPerB; ++q) {
         const int b = t + q * kThreads;
-        const uint32_t k = b < nb ? s.count[b] : 0u;    // read again: registers
+        const uint32_t k = b < nb ? s_count[b] : 0u;    // read again: registers
         if (k) {
             full |= slot && at[q] + k > slot;
-            s.count[b] = from;
-            s.shift[b] = at[q] + (uint32_t)b * slot - from;
+            s_count[b] = from;
+            s_shift[b] = at[q] + (uint32_t)b * slot - from;
             from += k;
         }
     }
@@ -333,9 +333,9 @@ k_rows_partition_tiles(const CT* __restrict__ oc, const CT* __restrict__ ic, con
 #pragma unroll
     for (int i = 0; i < kTIpt; ++i)
         if (i * kThreads + t < cnt) {
-            const uint32_t b = __umulhi(o[i], scale), at = s.count[b] + r[i];
+            const uint32_t b = __umulhi(o[i], scale), at = s_count[b] + r[i];
             s.rec[at] = make_rec(v[i], o[i], blockIdx.x * (uint32_t)kTTile + i * kThreads + t, c[i], inner_bits);
-            s.to[at] = s.shift[b] + at;
+            s.to[at] = s_shift[b] + at;
         }
     __syncthreads();
 #pragma unroll 4
@@ -664,7 +664,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
     const bool dbl = lt[0] == SP_COMPRESSED;
     const size_t pw = posBits / 8, cw = crdBits / 8;
     sp_workspace ws(stream);
-    const bool counted = n >= kCountFrom || (int64_t)nb * kCap > 16 * n + 65536;
+    const bool counted = (int64_t)nb * kCap > 16 * n + 65536;
     const uint32_t slot = counted ? 0u : (uint32_t)kCap;
     const size_t records = counted ? (size_t)n : (size_t)nb * kCap;
     const size_t cursors = sp_workspace::bytes_for<uint32_t>((size_t)nb + 3);
@@ -735,7 +735,7 @@ sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64
         } else {                                                                                                          \
             e = sp_allow_shared<k_rows_partition_tiles<CT>>(t->device, sizeof(TileShared));                               \
             if (e == cudaSuccess)                                                                                         \
-                e = sp_launch_dependent(k_rows_partition_tiles<CT>, dim3((unsigned)sp_ceil_div(n, kTTile)), dim3(kThreads), sizeof(TileShared), \
+                e = sp_launch_dependent(k_rows_partition_tiles<CT>, dim3((unsigned)sp_ceil_div(n, kTTile)), dim3(kThreads), TileShared::bytes(nb), \
                                         stream, oc, ic, vals, n, no, ni, scale, inner_bits, nb, slot, cursor, rec, stop, host);             \
         }                                                                                                                 \
     } while (0)
