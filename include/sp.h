@@ -36,7 +36,8 @@
  *     must be used with the device it was packed on current
  *     (SP_ERR_INVALID_ARG otherwise).
  *   - CUDA graphs: once a kernel call has run on a handle (so its cached tables
- *     exist), later sp_spmv / sp_spmm / sp_sddmm / sp_mttkrp calls on it only
+ *     exist, which are the same for every number of columns), later calls of the
+ *     same kind, sp_spmv / sp_spmm / sp_sddmm / sp_mttkrp, on it only
  *     enqueue stream-ordered work (kernels, memsets and allocator calls for
  *     their scratch) and may be stream-captured, provided the installed
  *     allocator is itself legal during capture (a stream-ordered or caching
