@@ -76,8 +76,13 @@ struct sp_workspace {
     char* pool = nullptr;          // what is left of a reserve()d block
     size_t pool_left = 0;
     explicit sp_workspace(cudaStream_t s) : stream(s) {}
-    ~sp_workspace() {
+    ~sp_workspace() { clear(); }
+    void clear() {
         for (void* p : ptrs) sp_dev_free(p, stream);
+        ptrs.clear();
+        failed = false;
+        pool = nullptr;
+        pool_left = 0;
     }
     static size_t padded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
     template <typename T>
@@ -272,6 +277,15 @@ sp_status sp_get_mttkrp_partition(sp_tensor* t, int64_t nnz_per_chunk, bool with
 // nothing was built, take the general path.
 sp_status sp_pack_rows(const int64_t* dims, const int* ord, const int* lt, int64_t nnz, const void* outer, const void* inner, int coord_bits,
                        const double* vals, int posBits, int crdBits, unsigned flags, cudaStream_t stream, sp_tensor** out);
+
+// Sort of sp_pack for large inputs (pack_sort.cu): enqueues the entries' keys in ascending order, equal ones in the order of the
+// input, and their values; both live in ws.  err (cleared by the caller) receives kSortRange for a coordinate out of range, or
+// kSortFull where some bucket outgrew its room: the arrays hold nothing then.  Level l's coordinates are coords[l], below sizes[l], at shifts[l] of the key.
+constexpr int kSortRange = 1, kSortFull = 4;
+bool sp_sample_sort_takes(int rank, int total_bits, int64_t n);
+sp_status sp_sample_sort(int rank, const int64_t* sizes, const int* shifts, const void* const* coords, int coord_bits, const double* vals, int64_t n,
+                         int total_bits, int device, cudaStream_t stream, sp_workspace& ws, int* err, const uint64_t** keys_out,
+                         const double** vals_out);
 
 // SpMV for rank-2 handles whose inner level is dense (dense_inner.cu).
 sp_status sp_spmv_dense_inner(const sp_tensor* A, const double* x, double* y, cudaStream_t stream);

@@ -4,8 +4,8 @@
 // Pipeline of sp_pack, all on the caller's stream:
 //   1. k_build_keys   level coordinates c_l = coord[dimOrdering[l]] fused into one
 //                     lexicographic key (level 0 in the top bits), range check
-//   2. radix sort     stable LSD, <= 8 bits per pass, (key, entry index) pairs;
-//                     per pass: tile histograms -> per-digit scan -> ranked scatter
+//   2. sort           large inputs: by samples (pack_sort.cu, in the place of step 1 too); others: stable LSD radix sort, <= 8 bits
+//                     per pass, (key, entry index) pairs; per pass: tile histograms -> per-digit scan -> ranked scatter
 //   3. k_count_flags  for every level the flag "key prefix through this level
 //                     differs from the previous entry" = a new stored node;
 //                     per-tile counts, then a scan of the tile counts
@@ -21,7 +21,7 @@
 
 namespace {
 
-constexpr int kErrRange = 1;
+constexpr int kErrRange = kSortRange;
 constexpr int kErrDup = 2;
 
 // Phase timing of the packer: CUDA events on the caller's stream between its kernels.  The product
@@ -1073,88 +1073,127 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
     int* d_err = nullptr;
     int64_t ct_tiles = 0;
 
-    if (n > 0) {
-        const int npasses = (total_bits + kMaxDigitBits - 1) / kMaxDigitBits;
-        // the entry index rides inside the key when both fit in 64 bits; otherwise the values travel
-        // beside the keys (one array per side of the ping-pong; the first pass reads the input's)
-        int idx_bits = 0;
-        while (((int64_t)1 << idx_bits) < n) ++idx_bits;
-        const bool fused = npasses > 0 && idx_bits > 0 && total_bits + idx_bits <= 64;
-        const int shape = !fused ? kShapeValue : n <= kFewTiles * SortShape<kShapeSmall>::kTile ? kShapeSmall : kShapeIndex;
-        const int64_t stiles = sp_ceil_div(n, shape == kShapeValue ? SortShape<kShapeValue>::kTile
-                                              : shape == kShapeSmall ? SortShape<kShapeSmall>::kTile : SortShape<kShapeIndex>::kTile);
+    // Large inputs are split by samples of their keys; should a bucket outgrow its room all the same, they are sorted by digits.
+    bool sampled = false;
+#ifndef SP_BENCH_BUILD
+    sampled = sp_sample_sort_takes(rank, total_bits, n);
+#endif
+    while (n > 0) {
         ct_tiles = sp_ceil_div(n, kCtTile);
-        const size_t nscan = (size_t)sp_ceil_div(stiles, kScanChunk) << kMaxDigitBits;
-        // every buffer of the pack in one allocation
-        ws.reserve(2 * sp_workspace::bytes_for<uint64_t>((size_t)n) +
-                   (fused ? sp_workspace::bytes_for<uint32_t>((size_t)n) : npasses > 0 ? 2 * sp_workspace::bytes_for<uint64_t>((size_t)n) : 0) +
-                   sp_workspace::bytes_for<uint32_t>((size_t)stiles << kMaxDigitBits) +
-                   sp_workspace::bytes_for<uint32_t>((size_t)1 << kMaxDigitBits) + sp_workspace::bytes_for<uint32_t>(nscan) +
-                   sp_workspace::bytes_for<uint64_t>((size_t)ct_tiles) + sp_workspace::bytes_for<int64_t>((size_t)ct_tiles * SP_MAX_RANK) +
-                   sp_workspace::bytes_for<int64_t>(SP_MAX_RANK + 1));
-        uint64_t* kbuf[2] = {ws.get<uint64_t>((size_t)n), ws.get<uint64_t>((size_t)n)};
-        uint64_t* pbuf[2] = {nullptr, nullptr};
-        uint32_t* isorted = nullptr;
-        if (fused) isorted = ws.get<uint32_t>((size_t)n);
-        else if (npasses > 0) { pbuf[0] = ws.get<uint64_t>((size_t)n); pbuf[1] = ws.get<uint64_t>((size_t)n); }
-        uint32_t* tilehist = ws.get<uint32_t>((size_t)stiles << kMaxDigitBits);
-        uint32_t* digit_total = ws.get<uint32_t>((size_t)1 << kMaxDigitBits);
-        uint32_t* chunk_tot = ws.get<uint32_t>(nscan);
-        uint64_t* tilesum = ws.get<uint64_t>((size_t)ct_tiles);
-        tileprefix = ws.get<int64_t>((size_t)ct_tiles * SP_MAX_RANK);
-        int64_t* d_counts = ws.get<int64_t>(SP_MAX_RANK + 1);      // node counts per level, then the error word
-        if (ws.failed) return SP_ERR_ALLOC;
-        d_err = reinterpret_cast<int*>(d_counts + SP_MAX_RANK);
-        SP_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int64_t), stream));
-
-        LevelCoords lc;
-        for (int l = 0; l < SP_MAX_RANK; ++l) lc.p[l] = coo_coords[l < rank ? plan.src[l] : 0];
-        // digit widths as even as possible, the wider ones first
-        int widths[16], shifts[16];
-        for (int ps = 0, kshift = 0; ps < npasses; ++ps) {
-            const int left = npasses - ps;
-            widths[ps] = (total_bits - kshift + left - 1) / left;
-            shifts[ps] = kshift + (fused ? idx_bits : 0);
-            kshift += widths[ps];
-        }
-        const int shift0 = npasses ? shifts[0] : 0;
-        const uint32_t mask0 = npasses ? (1u << widths[0]) - 1u : 0u;
-#define SP_BUILD_KEYS(CT, S)                                                                                       \
-    k_build_keys<CT, S><<<(unsigned)stiles, kSortThreads, 0, stream>>>(lc, n, plan, kbuf[0], fused ? idx_bits : 0,         \
-                                                                        d_err, shift0, mask0, tilehist, stiles)
-        if (shape == kShapeValue) { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeValue); else SP_BUILD_KEYS(int64_t, kShapeValue); }
-        else if (shape == kShapeSmall) { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeSmall); else SP_BUILD_KEYS(int64_t, kShapeSmall); }
-        else { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeIndex); else SP_BUILD_KEYS(int64_t, kShapeIndex); }
-#undef SP_BUILD_KEYS
-        SP_LAUNCH_CHECK();
-        sp_count_launches(1);
-        timer.mark(kPhKeys);
-        int cur = 0;
-        for (int ps = 0; ps < npasses; ++ps) {
-            const bool last = ps == npasses - 1;
-            const int split = (fused && last) ? idx_bits : -1;
-            sp_status ps_st = SP_ERR_UNSUPPORTED;
-#define SP_SORT_PASS_OF(S, B)                                                                                       \
-    sort_pass<S, B>(kbuf[cur], ps == 0 ? reinterpret_cast<const uint64_t*>(coo_vals) : pbuf[cur], kbuf[cur ^ 1],     \
-                    pbuf[cur ^ 1], isorted, n, shifts[ps], tilehist, stiles, digit_total, chunk_tot, split, ps == 0, stream, timer)
-#define SP_SORT_PASS(B)                                                                                             \
-    case B:                                                                                                         \
-        ps_st = shape == kShapeValue ? SP_SORT_PASS_OF(kShapeValue, B)                                               \
-                : shape == kShapeSmall ? SP_SORT_PASS_OF(kShapeSmall, B) : SP_SORT_PASS_OF(kShapeIndex, B);          \
-        break;
-            switch (widths[ps]) {
-                SP_SORT_PASS(1) SP_SORT_PASS(2) SP_SORT_PASS(3) SP_SORT_PASS(4) SP_SORT_PASS(5)
-                SP_SORT_PASS(6) SP_SORT_PASS(7) SP_SORT_PASS(8)
+        const size_t small_bytes = sp_workspace::bytes_for<uint64_t>((size_t)ct_tiles) +
+                                   sp_workspace::bytes_for<int64_t>((size_t)ct_tiles * SP_MAX_RANK) + sp_workspace::bytes_for<int64_t>(SP_MAX_RANK + 1);
+        uint64_t* tilesum = nullptr;
+        int64_t* d_counts = nullptr;               // node counts per level, then the error word
+        auto take_small = [&]() {
+            tilesum = ws.get<uint64_t>((size_t)ct_tiles);
+            tileprefix = ws.get<int64_t>((size_t)ct_tiles * SP_MAX_RANK);
+            d_counts = ws.get<int64_t>(SP_MAX_RANK + 1);
+            if (ws.failed) return SP_ERR_ALLOC;
+            d_err = reinterpret_cast<int*>(d_counts + SP_MAX_RANK);
+            SP_CUDA(cudaMemsetAsync(d_err, 0, sizeof(int64_t), stream));
+            return SP_OK;
+        };
+#ifndef SP_BENCH_BUILD
+        if (sampled) {
+            int device = 0;
+            SP_CUDA(cudaGetDevice(&device));
+            ws.reserve(small_bytes);
+            if (ws.failed) return SP_ERR_ALLOC;
+            const sp_status ts = take_small();
+            if (ts != SP_OK) return ts;
+            const void* coords[SP_MAX_RANK];
+            for (int l = 0; l < rank; ++l) coords[l] = coo_coords[plan.src[l]];
+            const uint64_t* sorted = nullptr;
+            const sp_status ss = sp_sample_sort(rank, plan.sz, plan.shift, coords, coo_coord_bits, coo_vals, n, total_bits, device, stream, ws, d_err,
+                                                &sorted, &vals_sorted);
+            if (ss == SP_ERR_ALLOC) {              // 52 bytes an entry; by digits 33 do
+                ws.clear();
+                sampled = false;
+                continue;
             }
+            if (ss != SP_OK) return ss;
+            keys = const_cast<uint64_t*>(sorted);
+        } else
+#endif
+        {
+            const int npasses = (total_bits + kMaxDigitBits - 1) / kMaxDigitBits;
+            // the entry index rides inside the key when both fit in 64 bits; otherwise the values travel
+            // beside the keys (one array per side of the ping-pong; the first pass reads the input's)
+            int idx_bits = 0;
+            while (((int64_t)1 << idx_bits) < n) ++idx_bits;
+            const bool fused = npasses > 0 && idx_bits > 0 && total_bits + idx_bits <= 64;
+            const int shape = !fused ? kShapeValue : n <= kFewTiles * SortShape<kShapeSmall>::kTile ? kShapeSmall : kShapeIndex;
+            const int64_t stiles = sp_ceil_div(n, shape == kShapeValue ? SortShape<kShapeValue>::kTile
+                                                  : shape == kShapeSmall ? SortShape<kShapeSmall>::kTile : SortShape<kShapeIndex>::kTile);
+            const size_t nscan = (size_t)sp_ceil_div(stiles, kScanChunk) << kMaxDigitBits;
+            // every buffer of the pack in one allocation
+            ws.reserve(2 * sp_workspace::bytes_for<uint64_t>((size_t)n) +
+                       (fused ? sp_workspace::bytes_for<uint32_t>((size_t)n) : npasses > 0 ? 2 * sp_workspace::bytes_for<uint64_t>((size_t)n) : 0) +
+                       sp_workspace::bytes_for<uint32_t>((size_t)stiles << kMaxDigitBits) +
+                       sp_workspace::bytes_for<uint32_t>((size_t)1 << kMaxDigitBits) + sp_workspace::bytes_for<uint32_t>(nscan) +
+                       small_bytes);
+            uint64_t* kbuf[2] = {ws.get<uint64_t>((size_t)n), ws.get<uint64_t>((size_t)n)};
+            uint64_t* pbuf[2] = {nullptr, nullptr};
+            uint32_t* isorted = nullptr;
+            if (fused) isorted = ws.get<uint32_t>((size_t)n);
+            else if (npasses > 0) { pbuf[0] = ws.get<uint64_t>((size_t)n); pbuf[1] = ws.get<uint64_t>((size_t)n); }
+            uint32_t* tilehist = ws.get<uint32_t>((size_t)stiles << kMaxDigitBits);
+            uint32_t* digit_total = ws.get<uint32_t>((size_t)1 << kMaxDigitBits);
+            uint32_t* chunk_tot = ws.get<uint32_t>(nscan);
+            if (ws.failed) return SP_ERR_ALLOC;
+            const sp_status ts = take_small();
+            if (ts != SP_OK) return ts;
+
+            LevelCoords lc;
+            for (int l = 0; l < SP_MAX_RANK; ++l) lc.p[l] = coo_coords[l < rank ? plan.src[l] : 0];
+            // digit widths as even as possible, the wider ones first
+            int widths[16], shifts[16];
+            for (int ps = 0, kshift = 0; ps < npasses; ++ps) {
+                const int left = npasses - ps;
+                widths[ps] = (total_bits - kshift + left - 1) / left;
+                shifts[ps] = kshift + (fused ? idx_bits : 0);
+                kshift += widths[ps];
+            }
+            const int shift0 = npasses ? shifts[0] : 0;
+            const uint32_t mask0 = npasses ? (1u << widths[0]) - 1u : 0u;
+#define SP_BUILD_KEYS(CT, S)                                                                                       \
+        k_build_keys<CT, S><<<(unsigned)stiles, kSortThreads, 0, stream>>>(lc, n, plan, kbuf[0], fused ? idx_bits : 0,         \
+                                                                            d_err, shift0, mask0, tilehist, stiles)
+            if (shape == kShapeValue) { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeValue); else SP_BUILD_KEYS(int64_t, kShapeValue); }
+            else if (shape == kShapeSmall) { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeSmall); else SP_BUILD_KEYS(int64_t, kShapeSmall); }
+            else { if (coo_coord_bits == 32) SP_BUILD_KEYS(int32_t, kShapeIndex); else SP_BUILD_KEYS(int64_t, kShapeIndex); }
+#undef SP_BUILD_KEYS
+            SP_LAUNCH_CHECK();
+            sp_count_launches(1);
+            timer.mark(kPhKeys);
+            int cur = 0;
+            for (int ps = 0; ps < npasses; ++ps) {
+                const bool last = ps == npasses - 1;
+                const int split = (fused && last) ? idx_bits : -1;
+                sp_status ps_st = SP_ERR_UNSUPPORTED;
+#define SP_SORT_PASS_OF(S, B)                                                                                       \
+        sort_pass<S, B>(kbuf[cur], ps == 0 ? reinterpret_cast<const uint64_t*>(coo_vals) : pbuf[cur], kbuf[cur ^ 1],     \
+                        pbuf[cur ^ 1], isorted, n, shifts[ps], tilehist, stiles, digit_total, chunk_tot, split, ps == 0, stream, timer)
+#define SP_SORT_PASS(B)                                                                                             \
+        case B:                                                                                                         \
+            ps_st = shape == kShapeValue ? SP_SORT_PASS_OF(kShapeValue, B)                                               \
+                    : shape == kShapeSmall ? SP_SORT_PASS_OF(kShapeSmall, B) : SP_SORT_PASS_OF(kShapeIndex, B);          \
+            break;
+                switch (widths[ps]) {
+                    SP_SORT_PASS(1) SP_SORT_PASS(2) SP_SORT_PASS(3) SP_SORT_PASS(4) SP_SORT_PASS(5)
+                    SP_SORT_PASS(6) SP_SORT_PASS(7) SP_SORT_PASS(8)
+                }
 #undef SP_SORT_PASS
 #undef SP_SORT_PASS_OF
-            if (ps_st != SP_OK) return ps_st;
-            cur ^= 1;
+                if (ps_st != SP_OK) return ps_st;
+                cur ^= 1;
+            }
+            npasses_done = npasses;
+            keys = kbuf[cur];
+            vals_sorted = nullptr;
+            if (fused) idx = isorted;
+            else vals_sorted = npasses > 0 ? reinterpret_cast<const double*>(pbuf[cur]) : coo_vals;   // no pass: one cell
         }
-        npasses_done = npasses;
-        keys = kbuf[cur];
-        if (fused) idx = isorted;
-        else vals_sorted = npasses > 0 ? reinterpret_cast<const double*>(pbuf[cur]) : coo_vals;   // no pass: one cell
 
         switch (rank) {
             case 1: SP_CUDA(sp_launch_dependent(k_count_flags<1>, dim3((unsigned)ct_tiles), dim3(kCtThreads), 0, stream, (const uint64_t*)keys, n, plan, tilesum)); break;
@@ -1175,7 +1214,13 @@ sp_status pack_impl(int rank, const int64_t* dims, int64_t nnz, const void* cons
         for (int l = 0; l < SP_MAX_RANK; ++l) counts[l] = (int64_t)h_back[l];
         const int h_err = (int)(h_back[SP_MAX_RANK] & 0xffffffff);
         if (h_err & kErrRange) return SP_ERR_OUT_OF_RANGE;
+        if (h_err & kSortFull) {
+            ws.clear();
+            sampled = false;
+            continue;
+        }
         if ((flags & SP_DUP_ERROR) && counts[rank - 1] != n) return SP_ERR_DUPLICATE;
+        break;
     }
 
     // sizes of the level arrays

@@ -1,0 +1,637 @@
+// The sort of sp_pack for large inputs that its packer of matrices does not take: entries in the order of their keys, the values beside them.
+//
+// Entries are split twice by splitters taken from samples, then every bucket is put in order by a block in shared memory:
+//
+//   1. k_first_sample,     a block sorts a sample of the keys: splitters for up to kMaxFirst buckets of about equal size whatever the
+//      k_first_splitters   keys' distribution
+//   2. k_first_split       range check, keys; entries to their buckets, in any order
+//   3. k_second_splitters  a block per bucket sorts a sample of it: splitters for parts of kMean entries
+//   4. k_second_split      entries to their parts, in any order
+//   5. k_sort_parts        a block per part: order in shared memory; keys and values in order
+//
+// An entry passes through memory three times (six to eight times in a radix sort of 42-bit keys).  Between the passes it is
+// a word, the key minus the least key of its first bucket with the entry's number in the input below it, and
+// its value.  The words are distinct, so parts may begin between equal keys, and an entry repeated any number of
+// times does no harm to the second split.
+//
+// 20 M entries of a 16,384^3 tensor: the pack 1335 -> 1057 us.  Splitters 4 + 23 and 31 us, first split 215, second 174, parts 400, then what
+// the sort by digits needs too (186).  The splits are bound by the L1 and shared-memory pipe (81 %: 61 and 44 wavefronts of shared memory to
+// 32 entries), the parts by issue (51 %) and shared memory (46 %) at 31 warps per SM.  Three blocks of k_sort_parts per SM spill (419 us); merge
+// sort in its place 519; splits with 6 entries a thread and three blocks 1086 for the pack, 8 and two 1149, 256 threads 1107.
+#include "common.cuh"
+
+#include <algorithm>
+
+namespace {
+
+constexpr int kMaxFirst = 256;                  // buckets of the first split
+constexpr int kMaxSecond = 128;                 // parts of a bucket
+constexpr int kMean = 2700, kCap = 4096;        // entries of a part: aimed at, and at most
+
+constexpr int kSampleThreads = 1024, kSampleIpt = 8, kSamples = kSampleThreads * kSampleIpt;
+static_assert(kSamples == 1 << 13, "sample_place");
+constexpr int kFetchThreads = 128;              // of k_first_sample: many SMs, for the misses of random accesses
+constexpr int kSecondIpt = 8, kSecondSamples = kSampleThreads * kSecondIpt;
+constexpr int kSplitThreads = 512, kSplitIpt = 4, kSplitTile = kSplitThreads * kSplitIpt;
+constexpr int kPartThreads = 512, kPartIpt = kCap / kPartThreads;
+
+// ------------------------------------------------------------------------------------- sort of the samples
+
+// Bitonic sort over a block of kSampleThreads threads, IPT (a power of two) elements each, thread t's being t * IPT and those after
+// it: exchanges inside a thread, by shuffles, and through shared memory (s, kSampleThreads * IPT words) only between warps.
+// 4096 elements by a merge sort along merge paths took 17 us.
+template <int IPT>
+__device__ __forceinline__ void block_bitonic_sort(uint32_t (&x)[IPT], uint32_t* s) {
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int k = 2; k < IPT; k *= 2)                // runs inside a thread
+#pragma unroll
+        for (int j = k / 2; j > 0; j /= 2)
+#pragma unroll
+            for (int i = 0; i < IPT; ++i)
+                if (!(i & j)) {
+                    const uint32_t a = x[i], b = x[i | j];
+                    x[i] = i & k ? max(a, b) : min(a, b);
+                    x[i | j] = i & k ? min(a, b) : max(a, b);
+                }
+#pragma unroll 1
+    for (int k = 1; k <= kSampleThreads; k *= 2) {  // runs of k threads; a descending one is sorted upwards in its complement
+        const uint32_t flip = t & k ? ~0u : 0u;
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) x[i] ^= flip;
+#pragma unroll 1
+        for (int j = k / 2; j > 0; j /= 2) {
+            const bool lower = !(t & j);
+            if (j < 32) {
+#pragma unroll
+                for (int i = 0; i < IPT; ++i) {
+                    const uint32_t y = __shfl_xor_sync(0xffffffffu, x[i], j);
+                    x[i] = lower ? min(x[i], y) : max(x[i], y);
+                }
+            } else {
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < IPT; ++i) s[i * kSampleThreads + t] = x[i];
+                __syncthreads();
+#pragma unroll
+                for (int i = 0; i < IPT; ++i) {
+                    const uint32_t y = s[i * kSampleThreads + (t ^ j)];
+                    x[i] = lower ? min(x[i], y) : max(x[i], y);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = IPT / 2; j > 0; j /= 2)
+#pragma unroll
+            for (int i = 0; i < IPT; ++i)
+                if (!(i & j)) {
+                    const uint32_t a = x[i], b = x[i | j];
+                    x[i] = min(a, b);
+                    x[i | j] = max(a, b);
+                }
+#pragma unroll
+        for (int i = 0; i < IPT; ++i) x[i] ^= flip;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) s[t * IPT + i] = x[i];
+    __syncthreads();
+}
+
+// ---------------------------------------------------------------------------------------------------- shared
+
+// Exclusive scan over a block of NT threads of one counter per thread; sums: NT / 32 words.
+template <int NT>
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* sums, uint32_t* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) sums[w] = incl;
+    __syncthreads();
+    uint32_t pre = 0, tot = 0;
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) {
+        const uint32_t s = sums[i];
+        if (i < w) pre += s;
+        tot += s;
+    }
+    __syncthreads();
+    *total = tot;
+    return incl - v + pre;
+}
+
+// The i-th of 2^LOG samples of n: a place inside the i-th of as many equal stretches, so that neither an input in order
+// nor one with a period misleads.
+template <int LOG>
+__device__ __forceinline__ int64_t sample_place(int i, int64_t n) {
+    const int64_t from = (int64_t)i * n >> LOG, to = (int64_t)(i + 1) * n >> LOG;
+    uint32_t h = (uint32_t)i * 0x9E3779B1u;
+    h ^= h >> 15; h *= 0x85EBCA77u; h ^= h >> 13;
+    return from + (int64_t)__umulhi(h, (uint32_t)(to - from));
+}
+
+// Number of the N - 1 ascending splitters in s that are at most h (N a power of two).
+template <int N>
+__device__ __forceinline__ uint32_t bucket_of(const uint32_t* s, uint32_t h) {
+    uint32_t at = 0;
+#pragma unroll
+    for (int step = N / 2; step > 0; step /= 2)
+        if (s[at + step - 1] <= h) at += step;
+    return at;
+}
+
+struct SortPlan {
+    int shift[SP_MAX_RANK];         // of a level's coordinate in the key
+    int64_t size[SP_MAX_RANK];
+    const void* coords[SP_MAX_RANK];
+    int total_bits, idx_bits;
+    int shift1;                     // key >> shift1 fits 32 bits
+    int first, grid_bits;           // buckets of the first split, 2^grid_bits - 1 of whose splitters cut the range of keys evenly
+    uint32_t slot;                  // room of a bucket
+    uint32_t max_parts;             // parts in all, at most
+    int64_t n;
+};
+struct __align__(16) PartInfo {
+    uint64_t least;                 // its words begin here
+    uint64_t least_key;             // of its bucket
+    uint32_t top;                   // word - least, shifted right by `shift`, is at most this
+    uint32_t first;                 // the first part of its bucket
+    uint16_t shift, bucket;
+};
+struct SortScratch {
+    uint32_t *sample;               // [kSamples]
+    uint32_t *splitters;            // [kMaxFirst]
+    uint32_t *cursor;               // [kMaxFirst] entries in a bucket
+    uint32_t *second;               // [first][kMaxSecond] splitters inside a bucket
+    uint32_t *filled;               // [max_parts] entries in a part
+    PartInfo *part;                 // [max_parts]
+    int *err;
+    uint64_t *word1, *word2;
+    double *val1, *val2;
+};
+
+__device__ __forceinline__ bool stopped(const int* err) {
+    return __syncthreads_or(threadIdx.x == 0 && (__ldcg(err) & (kSortRange | kSortFull)) != 0) != 0;
+}
+
+__device__ __forceinline__ uint32_t parts_of(uint32_t entries) { return (entries + kMean - 1) / kMean; }
+
+// Bucket b's words are below 2^this.
+__device__ __forceinline__ int word_bits(const SortPlan& p, const uint32_t* splitters, int b) {
+    const uint64_t lo = b ? (uint64_t)splitters[b - 1] << p.shift1 : 0;
+    const uint64_t hi = b + 1 < p.first ? (uint64_t)splitters[b] << p.shift1 : 1ull << p.total_bits;
+    const uint64_t range = hi > lo + 1 ? hi - lo - 1 : 0;
+    return 64 - __clzll((long long)range) + p.idx_bits;
+}
+__device__ __forceinline__ int over_32(int bits) { return bits > 32 ? bits - 32 : 0; }
+
+// --------------------------------------------------------------------------------------------------- kernels
+
+template <typename CT, int RANK>
+__device__ __forceinline__ uint64_t key_of(const SortPlan& p, int64_t e, bool* bad) {
+    CT c[RANK];
+#pragma unroll
+    for (int l = 0; l < RANK; ++l) c[l] = static_cast<const CT*>(p.coords[l])[e];
+    uint64_t key = 0;
+#pragma unroll
+    for (int l = 0; l < RANK; ++l) {
+        if (c[l] < 0 || (int64_t)c[l] >= p.size[l]) { *bad = true; c[l] = 0; }
+        key |= (uint64_t)c[l] << p.shift[l];
+    }
+    return key;
+}
+
+template <typename CT, int RANK>
+__global__ void __launch_bounds__(kFetchThreads)
+k_first_sample(SortPlan p, SortScratch s) {
+    const int i = blockIdx.x * kFetchThreads + threadIdx.x;
+    bool bad = false;                               // reported by k_first_split
+    s.sample[i] = (uint32_t)(key_of<CT, RANK>(p, sample_place<13>(i, p.n), &bad) >> p.shift1);
+    if (i < kMaxFirst) { s.splitters[i] = ~0u; s.cursor[i] = 0u; }
+    for (uint32_t q = i; q < p.max_parts; q += kSamples) s.filled[q] = 0u;
+}
+
+__global__ void __launch_bounds__(kSampleThreads)
+k_first_splitters(SortPlan p, SortScratch s) {
+    sp_wait_for_previous_kernel();
+    __shared__ uint32_t s_sample[kSamples];
+    __shared__ uint32_t s_cut[kMaxFirst];
+    const int t = threadIdx.x;
+    uint32_t x[kSampleIpt];
+#pragma unroll
+    for (int i = 0; i < kSampleIpt; ++i) x[i] = s.sample[i * kSampleThreads + t];
+    block_bitonic_sort(x, s_sample);
+    const int grid = (1 << p.grid_bits) - 1, cuts = p.first - 1, even = cuts - grid;
+    if (t < cuts)
+        s_cut[t] = t < grid ? (uint32_t)(((uint64_t)(t + 1) << (p.total_bits - p.grid_bits)) >> p.shift1)
+                            : s_sample[(int)((int64_t)(t - grid + 1) * kSamples / (even + 1))];
+    __syncthreads();
+    if (t < cuts) {
+        const uint32_t mine = s_cut[t];
+        int rank = 0;
+        for (int i = 0; i < cuts; ++i) rank += s_cut[i] < mine || (s_cut[i] == mine && i < t);
+        s.splitters[rank] = mine;
+    }
+}
+
+struct __align__(16) SplitShared {
+    uint64_t word[kSplitTile];
+    double val[kSplitTile];
+    uint32_t count[kMaxFirst], shift[kMaxFirst];
+    uint32_t cut[kMaxFirst];
+    uint32_t sums[kSplitThreads / 32];
+    uint8_t to[kSplitTile];
+};
+
+// The rest of a split once the tile's entries know their bucket and their rank in it (bucket << 16 | rank): the
+// tile is put in order by bucket in shared memory, so that a bucket's entries leave side by side.  `room`: the size of a
+// bucket's slot.  Returns false when a slot is full.
+template <int N>
+__device__ __forceinline__ bool split_tile(SplitShared& sh, int cnt, const uint64_t (&word)[kSplitIpt], const uint32_t (&br)[kSplitIpt],
+                                           const double* val_in, uint32_t* cursor, uint32_t room, int used,
+                                           uint64_t* word_out, double* val_out) {
+    const int t = threadIdx.x;
+    static_assert(N <= kSplitThreads, "a thread per bucket");
+    const uint32_t k = t < used ? sh.count[t] : 0u;
+    const uint32_t at = k ? atomicAdd(cursor + t, k) : 0u;
+    double v[kSplitIpt];                            // not needed before: requested here they hold no registers through the search
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i) v[i] = i * kSplitThreads + t < cnt ? val_in[i * kSplitThreads + t] : 0.0;
+    uint32_t tot;
+    const uint32_t from = block_scan<kSplitThreads>(k, sh.sums, &tot);
+    if (t < N) {
+        sh.count[t] = from;
+        sh.shift[t] = at + (uint32_t)t * room - from;
+    }
+    if (__syncthreads_or(k && at + k > room)) return false;
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i)
+        if (i * kSplitThreads + t < cnt) {
+            const uint32_t b = br[i] >> 16, j = sh.count[b] + (br[i] & 0xffffu);
+            sh.word[j] = word[i];
+            sh.val[j] = v[i];
+            sh.to[j] = (uint8_t)b;
+        }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i) {
+        const int j = i * kSplitThreads + t;
+        if (j < cnt) {
+            const uint32_t dst = sh.shift[sh.to[j]] + (uint32_t)j;
+            word_out[dst] = sh.word[j];
+            val_out[dst] = sh.val[j];
+        }
+    }
+    return true;
+}
+
+template <typename CT, int RANK>
+__global__ void __launch_bounds__(kSplitThreads, 4)
+k_first_split(SortPlan p, SortScratch s, const double* __restrict__ vals) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    SplitShared& sh = *reinterpret_cast<SplitShared*>(s_raw);
+    const int t = threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * kSplitTile;
+    const int cnt = (int)min((int64_t)kSplitTile, p.n - base);
+    uint64_t word[kSplitIpt];
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i) {
+        const int j = i * kSplitThreads + t;
+        word[i] = j < cnt ? key_of<CT, RANK>(p, base + j, &bad) : 0;
+    }
+    sp_wait_for_previous_kernel();                  // the splitters
+    if (t < kMaxFirst) { sh.cut[t] = s.splitters[t]; sh.count[t] = 0u; }
+    if (__syncthreads_or(bad)) {
+        if (t == 0) atomicOr(s.err, kSortRange);
+        return;
+    }
+    if (stopped(s.err)) return;
+    uint32_t br[kSplitIpt];
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i) {
+        const int j = i * kSplitThreads + t;
+        const uint32_t b = min(bucket_of<kMaxFirst>(sh.cut, (uint32_t)(word[i] >> p.shift1)), (uint32_t)p.first - 1u);
+        br[i] = j < cnt ? b << 16 | atomicAdd(&sh.count[b], 1u) : 0u;
+        word[i] = (word[i] - (b ? (uint64_t)sh.cut[b - 1] << p.shift1 : 0)) << p.idx_bits | (uint64_t)(base + j);
+    }
+    __syncthreads();
+    if (!split_tile<kMaxFirst>(sh, cnt, word, br, vals + base, s.cursor, p.slot, p.first, s.word1, s.val1) && t == 0) atomicOr(s.err, kSortFull);
+}
+
+__global__ void __launch_bounds__(kSampleThreads)
+k_second_splitters(SortPlan p, SortScratch s) {
+    sp_wait_for_previous_kernel();
+    if (stopped(s.err)) return;
+    __shared__ uint32_t sample[kSecondSamples];
+    __shared__ uint32_t s_sums[kSampleThreads / 32];
+    const int t = threadIdx.x, b = blockIdx.x;
+    const uint32_t cnt = s.cursor[b];
+    if (cnt == 0) return;
+    uint32_t parts_before;
+    block_scan<kSampleThreads>(t < b ? parts_of(s.cursor[t]) : 0u, s_sums, &parts_before);
+    const int parts = (int)parts_of(cnt);
+    const uint64_t* word = s.word1 + (size_t)b * p.slot;
+    const int bits = word_bits(p, s.splitters, b), shift = over_32(bits);
+    const int samples = (int)min(cnt, (uint32_t)kSecondSamples);
+    uint32_t x[kSecondIpt];                         // four neighbours at a time: one sector each
+#pragma unroll
+    for (int i = 0; i < kSecondIpt; ++i) {
+        const int j = i * kSampleThreads + t;
+        const int64_t at = samples < kSecondSamples ? j : min(sample_place<11>(j / 4, cnt) / 4 * 4 + j % 4, (int64_t)cnt - 1);
+        x[i] = j < samples ? (uint32_t)(word[at] >> shift) : ~0u;
+    }
+    block_bitonic_sort(x, sample);
+    auto begin_of = [&](int q) { return q ? sample[(int)((int64_t)q * samples / parts)] : 0u; };
+    if (t < kMaxSecond) s.second[b * kMaxSecond + t] = t + 1 < parts ? begin_of(t + 1) : ~0u;
+    if (t < parts) {
+        const uint64_t least = (uint64_t)begin_of(t) << shift;
+        const uint64_t last = t + 1 < parts ? ((uint64_t)begin_of(t + 1) << shift) - 1 : bits < 64 ? (1ull << bits) - 1 : ~0ull;
+        PartInfo info;
+        info.least = least;
+        info.shift = (uint16_t)(last > least ? over_32(64 - __clzll((long long)(last - least))) : 0);
+        info.top = last > least ? (uint32_t)((last - least) >> info.shift) : 0u;
+        info.bucket = (uint16_t)b;
+        info.least_key = b ? (uint64_t)s.splitters[b - 1] << p.shift1 : 0;
+        info.first = parts_before;
+        s.part[parts_before + t] = info;
+    }
+}
+
+__global__ void __launch_bounds__(kSplitThreads, 4)
+k_second_split(SortPlan p, SortScratch s) {
+    sp_wait_for_previous_kernel();
+    const int t = threadIdx.x, b = blockIdx.y;
+    const uint32_t in_bucket = s.cursor[b], base = blockIdx.x * (uint32_t)kSplitTile;
+    if (base >= in_bucket) return;
+    if (stopped(s.err)) return;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    SplitShared& sh = *reinterpret_cast<SplitShared*>(s_raw);
+    const int cnt = (int)min((uint32_t)kSplitTile, in_bucket - base);
+    const size_t from = (size_t)b * p.slot + base;
+    uint64_t word[kSplitIpt];
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i) word[i] = i * kSplitThreads + t < cnt ? s.word1[from + i * kSplitThreads + t] : 0;
+    if (t < kMaxSecond) { sh.cut[t] = s.second[b * kMaxSecond + t]; sh.count[t] = 0u; }
+    uint32_t parts_before;
+    block_scan<kSplitThreads>(t < b ? parts_of(s.cursor[t]) : 0u, sh.sums, &parts_before);
+    const int parts = (int)parts_of(in_bucket), shift = over_32(word_bits(p, s.splitters, b));
+    uint32_t br[kSplitIpt];
+#pragma unroll
+    for (int i = 0; i < kSplitIpt; ++i) {
+        const uint32_t q = min(bucket_of<kMaxSecond>(sh.cut, (uint32_t)(word[i] >> shift)), (uint32_t)parts - 1u);
+        br[i] = i * kSplitThreads + t < cnt ? q << 16 | atomicAdd(&sh.count[q], 1u) : 0u;
+    }
+    __syncthreads();
+    if (!split_tile<kMaxSecond>(sh, cnt, word, br, s.val1 + from, s.filled + parts_before, (uint32_t)kCap, parts, s.word2 + (size_t)parts_before * kCap,
+                                s.val2 + (size_t)parts_before * kCap) && t == 0)
+        atomicOr(s.err, kSortFull);
+}
+
+constexpr int kFew = 4;                         // entries of a bin that are compared by the threads that hold them
+struct PartShared {
+    union {
+        uint64_t word[kCap];
+        struct { uint32_t lo[kCap], hi[kCap]; };        // of the entries in a bin of the first cut
+    };
+    union {
+        double val[kCap];
+        struct { uint32_t bin[kCap + 4], sub[kCap + 4]; };      // entries, then starts, of the bins of the first and the second cut
+    };
+    uint16_t place[kCap];                       // of the entries of crowded bins, at their place in word
+    uint16_t list[kCap / kFew];                 // the crowded bins
+    uint32_t crowded;                           // how many they are
+    uint32_t sums[kPartThreads / 32];
+};
+
+// In-place exclusive scan of s[0 .. kCap), a thread's kPartIpt counters in 16-byte accesses; s[kCap] = the total.
+template <typename F>
+__device__ __forceinline__ void scan_bins(uint32_t* s, uint32_t* sums, F&& each) {
+    static_assert(kPartIpt == 8, "two accesses");
+    const int t = threadIdx.x;
+    uint4 a = reinterpret_cast<const uint4*>(s)[t * 2], b = reinterpret_cast<const uint4*>(s)[t * 2 + 1];
+    uint32_t k[kPartIpt] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}, mine = 0, tot;
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i) mine += k[i];
+    uint32_t at = block_scan<kPartThreads>(mine, sums, &tot);
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i) {
+        const uint32_t v = k[i];
+        each(t * kPartIpt + i, v);
+        k[i] = at;
+        at += v;
+    }
+    reinterpret_cast<uint4*>(s)[t * 2] = make_uint4(k[0], k[1], k[2], k[3]);
+    reinterpret_cast<uint4*>(s)[t * 2 + 1] = make_uint4(k[4], k[5], k[6], k[7]);
+    if (t == 0) s[kCap] = tot;
+    __syncthreads();
+}
+
+// The range of a part's words is cut evenly into bins, and each bin that several entries fall into once more, into as many as
+// there are, between the smallest and the largest of them: a bin then holds two or three entries although keys crowd (20 M
+// entries of a Zipf-skewed tensor: an entry shares its bin with 1.2 others, 36 after the first cut alone).  An entry's place is its
+// bin's start plus the number of smaller words in the bin; where a bin still holds many, a warp counts for all of them.
+__global__ void __launch_bounds__(kPartThreads, 2)
+k_sort_parts(SortPlan p, SortScratch s, uint64_t* __restrict__ keys, double* __restrict__ vals) {
+    sp_wait_for_previous_kernel();
+    if (stopped(s.err)) return;
+    const int cnt = (int)s.filled[blockIdx.x];
+    if (cnt == 0) return;                           // there are fewer parts
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    PartShared& sh = *reinterpret_cast<PartShared*>(s_raw);
+    const int t = threadIdx.x;
+    const size_t slot = (size_t)blockIdx.x * kCap;
+    uint64_t word[kPartIpt];
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i) word[i] = i * kPartThreads + t < cnt ? s.word2[slot + i * kPartThreads + t] : 0;
+    const PartInfo info = s.part[blockIdx.x];
+    uint32_t before = 0, base;                      // entries of the buckets and of the bucket's parts before
+    static_assert(kMaxFirst + kMaxSecond <= kPartThreads, "a load per thread");
+    if (t < info.bucket) before = s.cursor[t];
+    else if (t >= kMaxFirst && info.first + (t - kMaxFirst) < blockIdx.x) before = s.filled[info.first + (t - kMaxFirst)];
+    const float scale = (float)kCap / ((float)info.top + 1.0f);
+    auto offset_of = [&](uint64_t w) { return (uint32_t)((w - info.least) >> info.shift); };
+    if (t == 0) sh.crowded = 0u;
+#pragma unroll
+    for (int i = 0; i < kPartIpt / 4; ++i) {
+        const int j = i * kPartThreads + t;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4*>(sh.bin)[j] = reinterpret_cast<uint4*>(sh.sub)[j] = reinterpret_cast<uint4*>(sh.hi)[j] = zero;
+        reinterpret_cast<uint4*>(sh.lo)[j] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    block_scan<kPartThreads>(before, sh.sums, &base);
+    uint32_t br[kPartIpt];                          // bin; then bin << 16 | rank; then the place
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i)
+        if (i * kPartThreads + t < cnt) {
+            const uint32_t h = offset_of(word[i]);
+            br[i] = min((uint32_t)((float)h * scale), (uint32_t)kCap - 1u);      // not decreasing in the word
+            atomicAdd(&sh.bin[br[i]], 1u);
+            atomicMin(&sh.lo[br[i]], h);
+            atomicMax(&sh.hi[br[i]], h);
+        }
+    __syncthreads();
+    scan_bins(sh.bin, sh.sums, [](int, uint32_t) {});
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i)
+        if (i * kPartThreads + t < cnt) {
+            const uint32_t from = sh.bin[br[i]], k = sh.bin[br[i] + 1] - from;
+            uint32_t g = from;
+            if (k > 1u) {
+                const uint32_t lo = sh.lo[br[i]];
+                g += min((uint32_t)((float)(offset_of(word[i]) - lo) * __fdividef((float)k, (float)(sh.hi[br[i]] - lo) + 1.0f)), k - 1u);
+            }
+            br[i] = g << 16 | atomicAdd(&sh.sub[g], 1u);
+        }
+    __syncthreads();
+    scan_bins(sh.sub, sh.sums, [&](int g, uint32_t k) {
+        if (k > (uint32_t)kFew) sh.list[atomicAdd(&sh.crowded, 1u)] = (uint16_t)g;
+    });
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i)
+        if (i * kPartThreads + t < cnt) sh.word[sh.sub[br[i] >> 16] + (br[i] & 0xffffu)] = word[i];
+    __syncthreads();
+    for (uint32_t c = t >> 5; c < sh.crowded; c += kPartThreads / 32) {        // a warp per crowded bin
+        const uint32_t begin = sh.sub[sh.list[c]], end = sh.sub[sh.list[c] + 1];
+        for (uint32_t e = begin + (t & 31); e < end; e += 32) {
+            const uint64_t w = sh.word[e];
+            uint32_t at = begin;
+#pragma unroll 4
+            for (uint32_t j = begin; j < end; ++j) at += sh.word[j] < w;
+            sh.place[e] = (uint16_t)at;
+        }
+    }
+    __syncthreads();
+    double v[kPartIpt];
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i) v[i] = i * kPartThreads + t < cnt ? s.val2[slot + i * kPartThreads + t] : 0.0;
+    // the bins of a thread's entries side by side: one load of each is on its way at a time
+    uint32_t bin[kPartIpt], most = 0;               // size << 16 | start
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i) {
+        bin[i] = 0;
+        if (i * kPartThreads + t < cnt) {
+            const uint32_t j = sh.sub[br[i] >> 16], k = sh.sub[(br[i] >> 16) + 1] - j;
+            br[i] = k > (uint32_t)kFew ? sh.place[j + (br[i] & 0xffffu)] : j;
+            if (k > 1u && k <= (uint32_t)kFew) {
+                bin[i] = k << 16 | j;
+                most = max(most, k);
+            }
+        }
+    }
+    for (uint32_t q = 0; q < most; ++q)
+#pragma unroll
+        for (int i = 0; i < kPartIpt; ++i)
+            if (q < bin[i] >> 16) br[i] += sh.word[(bin[i] & 0xffffu) + q] < word[i];
+    __syncthreads();                                // the bins are dead from here on
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i)
+        if (i * kPartThreads + t < cnt) {
+            sh.word[br[i]] = word[i];
+            sh.val[br[i]] = v[i];
+        }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPartIpt; ++i) {
+        const int j = i * kPartThreads + t;
+        if (j < cnt) {
+            keys[base + j] = info.least_key + (sh.word[j] >> p.idx_bits);
+            vals[base + j] = sh.val[j];
+        }
+    }
+}
+
+template <typename CT, int RANK>
+cudaError_t launch_first(const SortPlan& p, const SortScratch& s, const double* vals, int device, cudaStream_t stream) {
+    cudaError_t e = sp_allow_shared<k_first_split<CT, RANK>>(device, sizeof(SplitShared));
+    if (e != cudaSuccess) return e;
+    k_first_sample<CT, RANK><<<kSamples / kFetchThreads, kFetchThreads, 0, stream>>>(p, s);
+    e = sp_launch_dependent(k_first_splitters, dim3(1), dim3(kSampleThreads), 0, stream, p, s);
+    if (e != cudaSuccess) return e;
+    return sp_launch_dependent(k_first_split<CT, RANK>, dim3((unsigned)sp_ceil_div(p.n, kSplitTile)), dim3(kSplitThreads), sizeof(SplitShared), stream,
+                               p, s, vals);
+}
+
+}  // namespace
+
+// Whether the sort by samples is the faster one: from kLeast entries on, and from kLeastFused on where key and number fit 64 bits, since the
+// sort by digits then moves 8 bytes a pass instead of 16.  Skewed 16,384^3 tensor, 20 M entries: 1075 us (1345 by digits), 5 M 370 (397);
+// 45- to 49-bit keys, uniform: 2 M 195 (230), 1 M 153 (172), 500,000 135 (142), 200,000 123 (166).  Key and number in 64 bits: 4096^3, 20 M
+// 970 (1169), 13 M 676 (770), 8 M 470 (473), 5 M 340 (319).  Above kMost parts would outgrow their number.  The first split's even splitters make room for five bits of
+// the key beyond 64, no more.
+constexpr int64_t kLeast = 150000, kLeastFused = 10000000, kMost = 50000000;
+constexpr int kMostGridBits = 5;
+
+bool sp_sample_sort_takes(int rank, int total_bits, int64_t n) {
+    if (rank < 2 || n < kLeast || n > kMost) return false;
+    int idx_bits = 0;
+    while (((int64_t)1 << idx_bits) < n) ++idx_bits;
+    return total_bits + idx_bits <= 64 ? n >= kLeastFused : total_bits + idx_bits <= 64 + kMostGridBits;
+}
+
+sp_status sp_sample_sort(int rank, const int64_t* sizes, const int* shifts, const void* const* coords, int coord_bits, const double* vals, int64_t n,
+                         int total_bits, int device, cudaStream_t stream, sp_workspace& ws, int* err, const uint64_t** keys_out,
+                         const double** vals_out) {
+    SortPlan p = {};
+    for (int l = 0; l < rank; ++l) { p.shift[l] = shifts[l]; p.size[l] = sizes[l]; p.coords[l] = coords[l]; }
+    p.n = n;
+    p.total_bits = total_bits;
+    while (((int64_t)1 << p.idx_bits) < n) ++p.idx_bits;
+    p.shift1 = std::max(0, total_bits - 32);
+    p.grid_bits = std::max(0, total_bits + p.idx_bits - 64);
+    int even = 8;
+    while (even < 128 && (int64_t)even * 60000 < n) even *= 2;
+    if (n > 25000000) even = 224;
+    p.first = std::min(kMaxFirst, even + (1 << p.grid_bits) - 1);
+    // 64 samples to a bucket: three quarters more than its share are six standard deviations (36 and its double likewise)
+    const int64_t mean = sp_ceil_div(n, even);
+    p.slot = (uint32_t)std::min<int64_t>(mean + mean * 3 / (even > 128 ? 3 : 4) + 1024, kMaxSecond * kMean);
+    const size_t parts = (size_t)sp_ceil_div(n, kMean) + p.first;
+    p.max_parts = (uint32_t)parts;
+    const size_t slots = (size_t)p.first * p.slot;
+    SortScratch s = {};
+    s.err = err;
+    auto take = [&]() {
+        s.sample = ws.get<uint32_t>(kSamples);
+        s.splitters = ws.get<uint32_t>(kMaxFirst);
+        s.cursor = ws.get<uint32_t>(kMaxFirst);
+        s.second = ws.get<uint32_t>((size_t)p.first * kMaxSecond);
+        s.filled = ws.get<uint32_t>(parts);
+        s.part = ws.get<PartInfo>(parts);
+        s.word1 = ws.get<uint64_t>(slots);
+        s.val1 = ws.get<double>(slots);
+        s.word2 = ws.get<uint64_t>(parts * kCap);
+        s.val2 = ws.get<double>(parts * kCap);
+    };
+    ws.reserve(sp_workspace::bytes_for<uint32_t>(kSamples) + 2 * sp_workspace::bytes_for<uint32_t>(kMaxFirst) +
+               sp_workspace::bytes_for<uint32_t>((size_t)p.first * kMaxSecond) + sp_workspace::bytes_for<uint32_t>(parts) +
+               sp_workspace::bytes_for<PartInfo>(parts) +
+               2 * sp_workspace::bytes_for<double>(slots) + 2 * sp_workspace::bytes_for<double>(parts * kCap));
+    if (ws.failed) return SP_ERR_ALLOC;
+    take();
+    if (ws.failed) return SP_ERR_ALLOC;
+    uint64_t* keys = s.word1;                   // free again once the second split is done
+    double* sorted = s.val1;
+    cudaError_t e = cudaErrorInvalidValue;
+#define SP_FIRST(R) \
+    case R: e = coord_bits == 32 ? launch_first<int32_t, R>(p, s, vals, device, stream) : launch_first<int64_t, R>(p, s, vals, device, stream); break;
+    switch (rank) { SP_FIRST(2) SP_FIRST(3) SP_FIRST(4) SP_FIRST(5) }
+#undef SP_FIRST
+    if (e == cudaSuccess) e = sp_launch_dependent(k_second_splitters, dim3((unsigned)p.first), dim3(kSampleThreads), 0, stream, p, s);
+    if (e == cudaSuccess) e = sp_allow_shared<k_second_split>(device, sizeof(SplitShared));
+    if (e == cudaSuccess)
+        e = sp_launch_dependent(k_second_split, dim3((unsigned)sp_ceil_div(p.slot, kSplitTile), (unsigned)p.first), dim3(kSplitThreads),
+                                sizeof(SplitShared), stream, p, s);
+    if (e == cudaSuccess) e = sp_allow_shared<k_sort_parts>(device, sizeof(PartShared));
+    if (e == cudaSuccess)
+        e = sp_launch_dependent(k_sort_parts, dim3((unsigned)parts), dim3(kPartThreads), sizeof(PartShared), stream, p, s, keys, sorted);
+    if (e != cudaSuccess) return SP_ERR_CUDA;
+    sp_count_launches(6);
+    *keys_out = keys;
+    *vals_out = sorted;
+    return SP_OK;
+}

@@ -1,0 +1,87 @@
+"""sp_pack's sort by samples (150,000 entries and more whose key and number exceed 64 bits) against the oracle: inputs in order and in disorder,
+keys that crowd, repeated coordinates, a bucket that overflows, and what the call reports and asks for."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from gpu_util import assert_storage_equal, dev, sp
+from paper_2202_04305_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+DIMS = (1 << 17, 3 << 15, 1 << 13)          # 47 bits; 18 bits number 150,000 entries
+LEAST = 150_000
+
+
+def draw(n, kind, dims=DIMS, seed=1):
+    """Coordinates and values; duplicates occur, more the more the keys crowd."""
+    rng = np.random.default_rng(seed)
+    u = rng.random((len(dims), n))
+    if kind == "crowded":
+        u = u ** 8
+    c = [np.minimum((x * d).astype(np.int64), d - 1) for x, d in zip(u, dims)]
+    if kind == "fourfold":
+        c = [np.tile(x[: -(-n // 4)], 4)[:n] for x in c]
+    if kind == "one in two":                # more than a bucket holds at one coordinate
+        same = rng.random(n) < 0.5
+        c = [np.where(same, 5, x) for x in c]
+    if kind in ("ascending", "descending"):
+        order = np.lexsort(c[::-1])
+        c = [x[order if kind == "ascending" else order[::-1]] for x in c]
+    return c, rng.standard_normal(n)
+
+
+def pack(c, v, dims=DIMS, lt=(1, 1, 1), od=(0, 1, 2), bits=32, **kw):
+    dt = np.int32 if bits == 32 else np.int64
+    return sp().sp_pack(dims, [dev(x.astype(dt)) for x in c], dev(v), lt, od, bits, bits, **kw)
+
+
+@pytest.mark.parametrize("kind", ["uniform", "crowded", "ascending", "descending", "fourfold", "one in two"])
+@pytest.mark.parametrize("n", [LEAST - 1, LEAST, 262_144, 262_145])
+def test_storage(kind, n):
+    c, v = draw(n, kind)
+    assert_storage_equal(pack(c, v), O.pack(DIMS, c, v, (1, 1, 1), (0, 1, 2)))
+
+
+@pytest.mark.parametrize("lt,od,bits", [((0, 1, 1), (0, 1, 2), 32), ((1, 1, 1), (2, 0, 1), 64), ((1, 1, 1), (0, 2, 1), 32)])
+def test_encodings_and_widths(lt, od, bits):
+    c, v = draw(200_000, "uniform")
+    assert_storage_equal(pack(c, v, lt=lt, od=od, bits=bits), O.pack(DIMS, c, v, lt, od))
+
+
+@pytest.mark.parametrize("dims", [(1 << 24, 1 << 23), (1 << 12, 1 << 11, 1 << 13, 1 << 11), (1 << 10, 1 << 9, 1 << 11, 1 << 10, 1 << 9)])
+def test_ranks(dims):
+    c, v = draw(170_000, "uniform", dims)
+    rank = len(dims)
+    assert_storage_equal(pack(c, v, dims, (1,) * rank, tuple(range(rank))), O.pack(dims, c, v, (1,) * rank, tuple(range(rank))))
+
+
+@pytest.mark.parametrize("bad", [-1, DIMS[1]])
+@pytest.mark.parametrize("at", [0, 100_001, 159_999])
+def test_out_of_range(bad, at):
+    c, v = draw(160_000, "uniform")
+    c[1][at] = bad
+    with pytest.raises(sp().SpError) as e:
+        pack(c, v)
+    assert e.value.code == 3
+
+
+def test_duplicates_reported():
+    c, v = draw(160_000, "fourfold")
+    with pytest.raises(sp().SpError) as e:
+        pack(c, v, flags=1)
+    assert e.value.code == 5
+
+
+def test_refused_scratch_is_asked_for_again_by_the_other_sort():
+    from test_gpu_alloc_failure import FailingAllocator
+    c, v = draw(200_000, "uniform")
+    ref = O.pack(DIMS, c, v, (1, 1, 1), (0, 1, 2))
+    with FailingAllocator() as a:
+        a.arm(2)                            # the small tables, then the sort's scratch
+        t = pack(c, v)
+        assert a.failed
+        assert_storage_equal(t, ref)
+        t.free()
+        assert not a.live
