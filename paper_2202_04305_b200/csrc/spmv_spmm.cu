@@ -476,52 +476,49 @@ k_spmm_rows(const P* __restrict__ pos, const I* __restrict__ crd, const double* 
 
 // Column-major SpMM (CSC, DCSC): C[i,:] += A[i,k] * B[k,:] for every stored entry, as a flat loop
 // over entries.  seg[p] is the column k of entry p (expanded once per handle), crd[p] its row i.
-// A warp takes kScatPer consecutive entries, 32 at a time; lane = output column.  Entries of one
-// column are adjacent, so the B row they share is read from DRAM once and then from L1; C is
-// updated with f64 atomic adds (it was zeroed by the caller).
-constexpr int kScatPer = 256;
-constexpr int kGather = 8;      // B rows in flight per warp
-
-template <typename I, int V>
+// A warp takes 32 consecutive entries; L lanes work on an entry, lane gl of them on the columns gl, L + gl, .., so that the
+// adds of an instruction fall on adjacent words (two adjacent columns a lane leave every second word of a sector to a
+// second instruction: 2.5 M entries, N = 64, 622 us, now 346).  Entries of one column are adjacent, so the B row
+// they share is read from DRAM once and then from L1; C is updated with f64 atomic adds (it was zeroed by the caller).
+// 5 M entries, N = 32: 324 us with 256 entries a warp and 8 rows of B in flight, 302 with 32 and 4 (64 entries 304, 128 311,
+// 16 rows 355); 20,000 entries, N = 32: 38 and 9.  Rows of products added to C by bulk reductions out of shared memory: 350, and 404
+// for N = 64.  Bound: the adds at L2 (258 us by themselves).
+template <typename I, int L, int V, int kRows>
 __global__ void __launch_bounds__(kMThreads)
 k_spmm_scatter(const uint32_t* __restrict__ seg, const I* __restrict__ crd, const double* __restrict__ val,
                int64_t nnz, const double* __restrict__ B, int64_t N, int64_t ldb, double* __restrict__ C,
                int64_t ldc, int64_t m, int64_t n) {
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int64_t p0 = w * kScatPer;
-    if (p0 >= nnz) return;
-    const int64_t p1 = p0 + kScatPer < nnz ? p0 + kScatPer : nnz;
-    for (int64_t cbase = 0; cbase < N; cbase += 32 * V) {
-        const int64_t col = cbase + (int64_t)lane * V;
-        const bool on = col < N;
-        const double* Bc = B + (on ? col : cbase);
-        double* Cc = C + (on ? col : cbase);
-        for (int64_t p = p0; p < p1; p += 32) {
-            const int cnt = p1 - p < 32 ? (int)(p1 - p) : 32;
-            const uint32_t k_l = lane < cnt ? seg[p + lane] : 0u;
-            const I i_l = lane < cnt ? crd[p + lane] : (I)0;
-            const double v_l = lane < cnt ? val[p + lane] : 0.0;
-            for (int g = 0; g < cnt; g += kGather) {
-                vec_t<V> b[kGather];
+    constexpr int kAtOnce = 32 / L;                 // entries that a warp instruction works on; rows in flight: times kRows
+    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32 * 32;
+    if (p >= nnz) return;
+    const int lane = threadIdx.x & 31, gl = lane % L, sub = lane / L;
+    const int cnt = nnz - p < 32 ? (int)(nnz - p) : 32;
+    const uint32_t k_l = lane < cnt ? seg[p + lane] : 0u;
+    const I i_l = lane < cnt ? crd[p + lane] : (I)0;
+    const double v_l = lane < cnt ? val[p + lane] : 0.0;
+    for (int64_t cbase = 0; cbase < N; cbase += L * V) {
+        bool on[V];
 #pragma unroll
-                for (int u = 0; u < kGather; ++u) {
-                    if (g + u < cnt) {
-                        const int64_t k = SP_IDX(__shfl_sync(0xffffffffu, k_l, g + u), n);
-                        b[u] = ld_vec<V>(Bc + k * ldb);
-                    }
-                }
+        for (int q = 0; q < V; ++q) on[q] = cbase + q * L + gl < N;
+        const double* Bc = B + cbase + gl;
+        double* Cc = C + cbase + gl;
+        for (int g = 0; g < cnt; g += kRows * kAtOnce) {
+            double b[kRows][V];
 #pragma unroll
-                for (int u = 0; u < kGather; ++u) {
-                    if (g + u < cnt) {
-                        const int64_t i = SP_IDX(__shfl_sync(0xffffffffu, i_l, g + u), m);
-                        const double vv = __shfl_sync(0xffffffffu, v_l, g + u);
-                        if (on) {
+            for (int u = 0; u < kRows; ++u) {
+                const int e = g + u * kAtOnce + sub;
+                const int64_t k = SP_IDX(__shfl_sync(0xffffffffu, k_l, e & 31), n);
 #pragma unroll
-                            for (int q = 0; q < V; ++q) atomicAdd(Cc + i * ldc + q, vv * b[u].a[q]);
-                        }
-                    }
-                }
+                for (int q = 0; q < V; ++q) b[u][q] = e < cnt && on[q] ? Bc[k * ldb + q * L] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kRows; ++u) {
+                const int e = g + u * kAtOnce + sub;
+                const int64_t i = SP_IDX(__shfl_sync(0xffffffffu, i_l, e & 31), m);
+                const double vv = __shfl_sync(0xffffffffu, v_l, e & 31);
+#pragma unroll
+                for (int q = 0; q < V; ++q)
+                    if (e < cnt && on[q]) atomicAdd(Cc + i * ldc + q * L, vv * b[u][q]);
             }
         }
     }
@@ -715,7 +712,6 @@ extern "C" sp_status sp_spmm(sp_tensor* A, const double* B, int64_t N, int64_t l
     // two columns at a time whenever every operand row starts on a 16-byte boundary
     const bool pairs = N % 2 == 0 && ldb % 2 == 0 && ldc % 2 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0 &&
                        reinterpret_cast<uintptr_t>(C) % 16 == 0;
-    const bool vec2 = pairs && N > 32;
     const int lanes = N <= 16 ? 4 : (N <= 32 || (pairs && N <= 64)) ? 8 : 16;      // of a group of k_spmm_merge
     if (!rowmajor) {
         st = sp_get_segment_ids(A, stream, &segs);
@@ -728,6 +724,7 @@ extern "C" sp_status sp_spmm(sp_tensor* A, const double* B, int64_t N, int64_t l
         if (ws.failed) return SP_ERR_ALLOC;
         carry = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(carry) + 15) & ~(uintptr_t)15);
     }
+#define SP_SCATTER(L, V, R) k_spmm_scatter<I, L, V, R><<<sblocks, kMThreads, 0, stream>>>(segs, crd, A->val, nnz, B, N, ldb, C, ldc, m, A->dims[1])
 #define SP_SPMM_MERGE(L, V, W, U)                                                                                                \
     k_spmm_merge<P, I, L, V, W, U><<<dim3((unsigned)gblocks, (unsigned)sp_ceil_div(N, L * V)), kMThreads, 0, stream>>>( \
         pos, crd, A->val, outer, B, N, ldb, C, ldc, part.row, part.nz, part.nchunks, nseg, carry, crow, m, A->dims[1])
@@ -755,15 +752,21 @@ extern "C" sp_status sp_spmm(sp_tensor* A, const double* B, int64_t N, int64_t l
         } else {
             (void)pos;
             const int64_t nnz = A->ncrd[1];
-            const unsigned sblocks = (unsigned)sp_ceil_div(sp_ceil_div(nnz, kScatPer) * 32, kMThreads);
+            const unsigned sblocks = (unsigned)sp_ceil_div(nnz, kMThreads);
             if (nnz > 0) {
-                if (vec2) k_spmm_scatter<I, 2><<<sblocks, kMThreads, 0, stream>>>(segs, crd, A->val, nnz, B, N, ldb, C, ldc, m, A->dims[1]);
-                else k_spmm_scatter<I, 1><<<sblocks, kMThreads, 0, stream>>>(segs, crd, A->val, nnz, B, N, ldb, C, ldc, m, A->dims[1]);
+                // lanes and columns a lane that N leaves the fewest without work: 17 to 24 go in three rounds of 8 (2 M entries,
+                // N = 20: 86 us, by 32 lanes 97), from 65 on four columns a lane (1 M entries, N = 100: 181, two columns 194)
+                if (N <= 8 || (N > 16 && N <= 24)) SP_SCATTER(8, 1, 4);
+                else if (N <= 16) SP_SCATTER(16, 1, 4);
+                else if (N <= 32) SP_SCATTER(32, 1, 4);
+                else if (N <= 64) SP_SCATTER(32, 2, 4);
+                else SP_SCATTER(32, 4, 2);
                 sp_count_launches(1);
             }
         }
     });
 #undef SP_SPMM_MERGE
+#undef SP_SCATTER
     SP_LAUNCH_CHECK();
     SP_BOUNDS_RETURN(stream);
     return SP_OK;
